@@ -73,9 +73,9 @@ __device__ __forceinline__ uint64_t trial_limit(const uint64_t* table, uint32_t 
 // For fanouts of at most 3 the parts are not computed.  With h the top 32
 // bits of the hash, phi = floor(h * m / 2^32) < k * unit holds exactly when
 // h < T_k = ceil(k * unit * 2^32 / m) (T_k < 2^32 because k * unit < m), so
-// field k - 1 counts the keys with h < T_k, and the split is the one sought
-// iff field k - 1 equals k * unit for k = 1 .. fanout - 1.  This replaces two
-// multiply-highs and a variable shift per key by fanout - 1 compares.
+// the split is the one sought iff m - k * unit keys have h >= T_k for k = 1 ..
+// fanout - 1.  This replaces two multiply-highs and a variable shift per key
+// by fanout - 1 additions with carry.
 // Largest fanout searched by thresholds: with three thresholds (fanout 4) the
 // compares cost about as much as the multiply-highs they replace.
 constexpr uint32_t kMaxThresholdFanout = 3;
@@ -84,27 +84,47 @@ struct SplitParams {
   uint32_t m, unit, fanout, bits, magic;  // magic = ceil(2^32 / unit): exact for m < 2^16, unit >= 2
   uint64_t target, mask;
   uint32_t thr1, thr2;      // T_1, T_2 (threshold modes)
-  uint32_t inc1;            // 1 << B
-  uint32_t cum_target;      // sum over k of k * unit << ((k - 1) * B)
   uint32_t nbits, nmask, ntarget;  // narrow fields (modes 5, 7): 2^nbits > unit
   bool confirm;                    // mode 7: fields can overflow, confirm matches exactly
   uint32_t tail;                   // modes 8..11 on shared nodes: keys of the second phase (0: one phase)
 };
 
 // MODE 0: 32-bit fields + magic; 1: 64-bit fields + magic; 2: 64-bit +
-// division; 3, 4: thresholds for fanout 2, 3 (cumulative 32-bit fields);
+// division; 3, 4: thresholds for fanout 2, 3;
 // 5: 32-bit fields of nbits bits (2^nbits > unit but possibly <= m) + magic.
 // In mode 5 a field can overflow into the next one, so a match may be false,
 // but never missed: when every counted part has exactly unit keys no field
 // overflows.  A match is confirmed with the exact 64-bit count (mode 1).
 // 6: four parts of equal size (m = 4 unit < 256): the part is
-// floor(floor(h m / 2^32) / unit) = floor(4 h / 2^32), the top two bits of h,
-// counted in 8-bit fields with shifts only.
+// floor(floor(h m / 2^32) / unit) = floor(4 h / 2^32), the top two bits of h.
 // 7: F parts of equal size (m = F unit): the part is floor(F h / 2^32), one
 // multiply-high instead of two, counted in nbits-bit fields; when a field
 // can overflow (2^nbits <= m) a match is confirmed exactly as in mode 5.
 // 8..11: mode 7 with nbits = MODE - 3 (5..8) fixed at compile time.
+// Modes 3 and 4: c1 and c2 count the keys with h >= T_1 and h >= T_2, the carry
+// of h + (2^32 - T) added by add-with-carry.  These two additions issue to
+// either pipe (1.4 cycles per warp together); a compare and a predicated
+// add take 2.2.
 template <int MODE>
+__device__ __forceinline__ void count_thresholds(uint32_t h, const SplitParams& p, uint32_t& c1, uint32_t& c2) {
+  asm("{.reg .u32 t; add.cc.u32 t, %1, %2; addc.u32 %0, %0, 0;}" : "+r"(c1) : "r"(h), "r"(0u - p.thr1));
+  if (MODE == 4) asm("{.reg .u32 t; add.cc.u32 t, %1, %2; addc.u32 %0, %0, 0;}" : "+r"(c2) : "r"(h), "r"(0u - p.thr2));
+}
+
+template <int MODE>
+__device__ __forceinline__ bool threshold_match(const SplitParams& p, uint32_t c1, uint32_t c2) {
+  return c1 == p.m - p.unit && (MODE == 3 || c2 == p.m - 2 * p.unit);
+}
+
+template <bool STAGED>
+__device__ __forceinline__ ulonglong2 key_pair(const uint64_t* keys) {
+  if (STAGED) return *reinterpret_cast<const ulonglong2*>(keys);
+  return make_ulonglong2(keys[0], keys[1]);
+}
+
+// STAGED: the keys are in shared memory, 16-byte aligned: modes 3, 4 and 6
+// read them two at a time.
+template <int MODE, bool STAGED>
 __device__ __forceinline__ bool split_trial(const uint64_t* __restrict__ keys, const SplitParams& p,
                                             uint64_t kp) {
   if (MODE >= 8) {
@@ -119,25 +139,52 @@ __device__ __forceinline__ bool split_trial(const uint64_t* __restrict__ keys, c
     for (uint32_t j = 0; j < p.m; j++) acc += shl32(1u, __umulhi(family_top32(keys[j], kp), p.fanout) * NB);
     return (acc & p.nmask) == p.ntarget;
   } else if (MODE == 6) {
-    uint32_t acc = 0;
+    // the two-bit parts are shifted into words of 16 keys (one funnel shift
+    // per key, where counting fields takes four instructions), and the parts
+    // 1, 2 and 3 are counted with population counts; part 0 is implied
+    uint32_t low = 0, high = 0, both = 0;
+    uint32_t j = 0;
+#pragma unroll 1
+    for (; j + 16 <= p.m; j += 16) {
+      uint32_t w = 0;
+#pragma unroll
+      for (uint32_t t = 0; t < 16; t += 2) {
+        const ulonglong2 x = key_pair<STAGED>(keys + j + t);
+        w = __funnelshift_l(family_top32(x.x, kp), w, 2);
+        w = __funnelshift_l(family_top32(x.y, kp), w, 2);
+      }
+      low += __popc(w & 0x55555555u);
+      high += __popc(w & 0xAAAAAAAAu);
+      both += __popc(w & (w >> 1) & 0x55555555u);
+    }
+    if (j < p.m) {
+      uint32_t w = 0;
 #pragma unroll 4
-    for (uint32_t j = 0; j < p.m; j++) acc += 1u << ((family_top32(keys[j], kp) >> 27) & 0x18u);
-    return (acc & 0xFFFFFFu) == p.cum_target;
+      for (; j < p.m; j++) w = __funnelshift_l(family_top32(keys[j], kp), w, 2);
+      low += __popc(w & 0x55555555u);
+      high += __popc(w & 0xAAAAAAAAu);
+      both += __popc(w & (w >> 1) & 0x55555555u);
+    }
+    return low == 2 * p.unit && high == 2 * p.unit && both == p.unit;
   } else if (MODE == 7) {
     uint32_t acc = 0;
 #pragma unroll 4
     for (uint32_t j = 0; j < p.m; j++) acc += shl32(1u, __umulhi(family_top32(keys[j], kp), p.fanout) * p.nbits);
     return (acc & p.nmask) == p.ntarget;
   } else if (MODE == 3 || MODE == 4) {
-    constexpr int F = MODE - 1;
-    uint32_t acc = 0;
-#pragma unroll 4
-    for (uint32_t j = 0; j < p.m; j++) {
-      const uint32_t h = family_top32(keys[j], kp);
-      acc += h < p.thr1 ? 1u : 0u;
-      if (F > 2) acc += h < p.thr2 ? p.inc1 : 0u;
+    uint32_t c1 = 0, c2 = 0, j = 0;
+#pragma unroll 1
+    for (; j + 8 <= p.m; j += 8) {
+#pragma unroll
+      for (uint32_t t = 0; t < 8; t += 2) {
+        const ulonglong2 x = key_pair<STAGED>(keys + j + t);
+        count_thresholds<MODE>(family_top32(x.x, kp), p, c1, c2);
+        count_thresholds<MODE>(family_top32(x.y, kp), p, c1, c2);
+      }
     }
-    return acc == p.cum_target;
+#pragma unroll 1
+    for (; j < p.m; j++) count_thresholds<MODE>(family_top32(keys[j], kp), p, c1, c2);
+    return threshold_match<MODE>(p, c1, c2);
   } else if (MODE == 0) {
     uint32_t acc = 0;
 #pragma unroll 4
@@ -180,7 +227,7 @@ __device__ bool has_duplicate(const uint64_t* keys, uint32_t m, uint32_t lane) {
   return __any_sync(0xFFFFFFFFu, dup);
 }
 
-template <int MODE>
+template <int MODE, bool STAGED>
 __device__ __forceinline__ void split_search_warp(const uint64_t* __restrict__ keys, const SplitParams& sp,
                                                   uint32_t depth, uint32_t wig, uint32_t gwarps, uint32_t lane,
                                                   uint64_t* best, uint64_t stall, uint64_t limit,
@@ -209,8 +256,8 @@ __device__ __forceinline__ void split_search_warp(const uint64_t* __restrict__ k
       }
     }
     const uint64_t kp = family_key(base + lane, depth);
-    bool ok = split_trial<MODE>(keys, sp, kp);
-    if ((MODE == 5 || (MODE >= 7 && sp.confirm)) && ok) ok = split_trial<1>(keys, sp, kp);
+    bool ok = split_trial<MODE, STAGED>(keys, sp, kp);
+    if ((MODE == 5 || (MODE >= 7 && sp.confirm)) && ok) ok = split_trial<1, STAGED>(keys, sp, kp);
     const uint32_t hits = __ballot_sync(0xFFFFFFFFu, ok);
     if (exec && lane == 0) *exec += 32 * sp.m;
     if (hits) {
@@ -220,19 +267,75 @@ __device__ __forceinline__ void split_search_warp(const uint64_t* __restrict__ k
   }
 }
 
+// Threshold nodes that take few trials (a binary split of 100 keys with 96 on
+// one side takes 5): a round of 32 indices is mostly wasted, so four lanes
+// share an index, each counting every fourth key, and a round tests 8.  It
+// saves about 12 of 32 indices per node and costs about 25 instructions per
+// round more (m/4 keys of about 15 instructions each), which pays while the
+// expected trials stay below the node's keys.
+template <int MODE>
+__device__ __forceinline__ void split_search_few(const uint64_t* __restrict__ keys, const SplitParams& sp,
+                                                 uint32_t depth, uint32_t wig, uint32_t gwarps, uint32_t lane,
+                                                 uint64_t* best, uint64_t stall, uint64_t limit, int* err,
+                                                 unsigned long long* exec) {
+  bool checked = false;
+  uint32_t rounds = 0;
+  for (uint64_t base = uint64_t(wig) * 8;; base += uint64_t(gwarps) * 8) {
+    if (gwarps > 1 && __any_sync(0xFFFFFFFFu, base >= volatile_load(best))) break;
+    if ((++rounds & 255) == 0 && __shfl_sync(0xFFFFFFFFu, lane == 0 ? *reinterpret_cast<volatile int*>(err) : 0, 0))
+      break;  // another search failed, or the host cancelled the build
+    if (base >= limit) {
+      if (lane == 0) {
+        set_error(err, RECSPLIT_E_SEARCH_LIMIT);
+        atomicMin(reinterpret_cast<unsigned long long*>(best), 0ull);
+      }
+      break;
+    }
+    if (!checked && base >= stall) {
+      checked = true;
+      if (has_duplicate(keys, sp.m, lane)) {
+        if (lane == 0) {
+          set_error(err, RECSPLIT_E_DUPLICATE);
+          atomicMin(reinterpret_cast<unsigned long long*>(best), 0ull);
+        }
+        break;
+      }
+    }
+    const uint64_t kp = family_key(base + (lane >> 2), depth);
+    uint32_t c1 = 0, c2 = 0;
+#pragma unroll 4
+    for (uint32_t j = lane & 3; j < sp.m; j += 4) count_thresholds<MODE>(family_top32(keys[j], kp), sp, c1, c2);
+    uint32_t c = MODE == 4 ? c1 | (c2 << 16) : c1;  // counts below 2^16
+    c += __shfl_xor_sync(0xFFFFFFFFu, c, 1);
+    c += __shfl_xor_sync(0xFFFFFFFFu, c, 2);
+    const bool ok = threshold_match<MODE>(sp, MODE == 4 ? c & 0xFFFFu : c, c >> 16);
+    const uint32_t hits = __ballot_sync(0xFFFFFFFFu, ok);
+    if (exec && lane == 0) *exec += 8 * sp.m;
+    if (hits) {
+      if (lane == 0) atomicMin(reinterpret_cast<unsigned long long*>(best), base + ((__ffs(hits) - 1) >> 2));
+      break;
+    }
+  }
+}
+
+template <bool STAGED>
 __device__ __forceinline__ void split_search(const uint64_t* __restrict__ keys, const SplitParams& sp, int mode,
                                              uint32_t depth, uint32_t wig, uint32_t gwarps, uint32_t lane,
                                              uint64_t* best, uint64_t stall, uint64_t limit, int* err,
                                              unsigned long long* exec) {
+  if (stall <= uint64_t(sp.m) << 6) {  // stall = 64 times the expected trials
+    if (mode == 3) return split_search_few<3>(keys, sp, depth, wig, gwarps, lane, best, stall, limit, err, exec);
+    if (mode == 4) return split_search_few<4>(keys, sp, depth, wig, gwarps, lane, best, stall, limit, err, exec);
+  }
   switch (mode) {
-    case 0: split_search_warp<0>(keys, sp, depth, wig, gwarps, lane, best, stall, limit, err, exec); break;
-    case 1: split_search_warp<1>(keys, sp, depth, wig, gwarps, lane, best, stall, limit, err, exec); break;
-    case 3: split_search_warp<3>(keys, sp, depth, wig, gwarps, lane, best, stall, limit, err, exec); break;
-    case 4: split_search_warp<4>(keys, sp, depth, wig, gwarps, lane, best, stall, limit, err, exec); break;
-    case 5: split_search_warp<5>(keys, sp, depth, wig, gwarps, lane, best, stall, limit, err, exec); break;
-    case 6: split_search_warp<6>(keys, sp, depth, wig, gwarps, lane, best, stall, limit, err, exec); break;
-    case 7: split_search_warp<7>(keys, sp, depth, wig, gwarps, lane, best, stall, limit, err, exec); break;
-    default: split_search_warp<2>(keys, sp, depth, wig, gwarps, lane, best, stall, limit, err, exec); break;
+    case 0: split_search_warp<0, STAGED>(keys, sp, depth, wig, gwarps, lane, best, stall, limit, err, exec); break;
+    case 1: split_search_warp<1, STAGED>(keys, sp, depth, wig, gwarps, lane, best, stall, limit, err, exec); break;
+    case 3: split_search_warp<3, STAGED>(keys, sp, depth, wig, gwarps, lane, best, stall, limit, err, exec); break;
+    case 4: split_search_warp<4, STAGED>(keys, sp, depth, wig, gwarps, lane, best, stall, limit, err, exec); break;
+    case 5: split_search_warp<5, STAGED>(keys, sp, depth, wig, gwarps, lane, best, stall, limit, err, exec); break;
+    case 6: split_search_warp<6, STAGED>(keys, sp, depth, wig, gwarps, lane, best, stall, limit, err, exec); break;
+    case 7: split_search_warp<7, STAGED>(keys, sp, depth, wig, gwarps, lane, best, stall, limit, err, exec); break;
+    default: split_search_warp<2, STAGED>(keys, sp, depth, wig, gwarps, lane, best, stall, limit, err, exec); break;
   }
 }
 
@@ -296,7 +399,6 @@ __device__ __forceinline__ int split_setup(const Node& nd, const uint64_t* table
   int mode = (nd.m >= 65536 || sp.unit < 2 || sp.magic == 0) ? 2 : (fields * sp.bits <= 32 ? 0 : 1);
   if (sp.fanout == 4 && nd.m == 4 * sp.unit && nd.m < 256) {
     mode = 6;
-    sp.cum_target = sp.unit | (sp.unit << 8) | (sp.unit << 16);
   } else if (sp.fanout >= 5 && nd.m == sp.fanout * sp.unit && sp.unit >= 2 && nd.m < 65536) {
     const uint32_t nb = nd.m < 256 && fields * 8 <= 32 ? 8 : 32 - __clz(sp.unit);
     if (fields * nb <= 32) {
@@ -323,11 +425,15 @@ __device__ __forceinline__ int split_setup(const Node& nd, const uint64_t* table
   }
   if (nd.m < 65536 && sp.fanout >= 2 && sp.fanout <= kMaxThresholdFanout && fields * sp.bits <= 32) {
     mode = 1 + static_cast<int>(sp.fanout);
-    // T_k = ceil(k * unit * 2^32 / m); field k - 1 must count k * unit keys
-    sp.thr1 = static_cast<uint32_t>(((uint64_t(sp.unit) << 32) + nd.m - 1) / nd.m);
-    sp.thr2 = static_cast<uint32_t>(((uint64_t(2 * sp.unit) << 32) + nd.m - 1) / nd.m);
-    sp.cum_target = sp.unit + (fields >= 2 ? (2 * sp.unit) << sp.bits : 0u);
-    sp.inc1 = 1u << sp.bits;
+    // T_k = ceil(k * unit * 2^32 / m), k = 1 on even lanes and 2 on odd ones, in
+    // two 16-bit digits (32-bit divisions: m < 2^16, and k * unit < m where T_k
+    // is used)
+    const uint32_t u = sp.unit << (threadIdx.x & 1);
+    const uint32_t q1 = (u << 16) / nd.m, r1 = (u << 16) % nd.m;
+    const uint32_t q0 = (r1 << 16) / nd.m, r0 = (r1 << 16) % nd.m;
+    const uint32_t thr = (q1 << 16) + q0 + (r0 ? 1u : 0u);
+    sp.thr1 = __shfl_sync(0xFFFFFFFFu, thr, 0);
+    sp.thr2 = __shfl_sync(0xFFFFFFFFu, thr, 1);
   }
   return mode;
 }
@@ -369,19 +475,31 @@ __device__ __forceinline__ void partition_node(const SearchArgs& a, const Node& 
 
 // COUNT: work counting (the evaluations executed go to a.exec_count[1]);
 // without it the counter is compiled out.
+// Warps per node or leaf: the launch shape's, doubled (up to the CTA) while
+// all the work items of the launch then still fit the grid's warps at once.
+// Their number is known on the device only.  A launch of few items lasts as
+// long as its longest search, so idle warps help there (split and leaf phases
+// at l = 8, b = 100: 10^3 keys 87 + 69 -> 51 + 20 us, 10^5 keys 197 + 85 ->
+// 110 + 73 us).
+__device__ __forceinline__ uint32_t group_warps(uint32_t gwarps, uint32_t items) {
+  while (gwarps < kWarps && uint64_t(items) * gwarps * 2 <= gridDim.x * kWarps) gwarps *= 2;
+  return gwarps;
+}
+
 template <bool COUNT>
 __global__ void __launch_bounds__(kThreads, 4) k_split_level(SearchArgs a, uint32_t gwarps, uint32_t cap) {
-  extern __shared__ uint64_t staged[];
+  extern __shared__ __align__(16) uint64_t staged[];
   __shared__ uint64_t best[kWarps];
   __shared__ uint32_t task[kWarps];
   __shared__ uint32_t fill[kWarps][16];
   __shared__ unsigned long long wexec[kWarps];  // work counting: evaluations per warp, flushed at exit
   const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (COUNT && lane == 0) wexec[warp] = 0;
+  const uint32_t total = *a.split_in_count;
+  gwarps = group_warps(gwarps, total);
   const uint32_t gid = warp / gwarps, wig = warp % gwarps;
   const uint32_t tig = wig * 32 + lane, gthreads = gwarps * 32;
   const bool leader = wig == 0 && lane == 0;
-  const uint32_t total = *a.split_in_count;
   uint64_t* mine = staged + size_t(gid) * cap;
 
   for (;;) {
@@ -410,9 +528,9 @@ __global__ void __launch_bounds__(kThreads, 4) k_split_level(SearchArgs a, uint3
 
       unsigned long long* exec = COUNT ? &wexec[warp] : nullptr;
       if (in_smem)
-        split_search(mine, sp, mode, depth, wig, gwarps, lane, &best[gid], stall, limit, a.error, exec);
+        split_search<true>(mine, sp, mode, depth, wig, gwarps, lane, &best[gid], stall, limit, a.error, exec);
       else
-        split_search(src, sp, mode, depth, wig, gwarps, lane, &best[gid], stall, limit, a.error, exec);
+        split_search<false>(src, sp, mode, depth, wig, gwarps, lane, &best[gid], stall, limit, a.error, exec);
       group_sync(gid, gwarps);
     }
 
@@ -505,7 +623,7 @@ __device__ __forceinline__ uint64_t shared_block_two_phase(const uint64_t* __res
       const uint64_t kp = (uint64_t(e.w) << 32) | e.z;
       const uint32_t acc = e.y + split_fields<NB>(keys, sp, kp, head, sp.m);
       ok = (acc & sp.nmask) == sp.ntarget;
-      if (ok && sp.confirm) ok = split_trial<1>(keys, sp, kp);
+      if (ok && sp.confirm) ok = split_trial<1, false>(keys, sp, kp);
     }
     evals += uint64_t(min(32u, ns - t0)) * sp.tail;
     const uint32_t hits = __ballot_sync(0xFFFFFFFFu, ok);
@@ -520,7 +638,7 @@ __device__ __forceinline__ uint64_t shared_block_two_phase(const uint64_t* __res
 
 // Returns the evaluations the warp executed (32 * m per round of 32 indices,
 // or as counted by the two-phase block test).
-template <int MODE>
+template <int MODE, bool STAGED>
 __device__ __forceinline__ uint64_t shared_search_warp(const uint64_t* __restrict__ keys, const SplitParams& sp,
                                                        uint32_t depth, uint32_t lane, uint64_t* best,
                                                        unsigned int* next, uint64_t stall, uint64_t limit,
@@ -563,8 +681,8 @@ __device__ __forceinline__ uint64_t shared_search_warp(const uint64_t* __restric
       const uint64_t base = base0 + r * 32;
       if (r && base >= volatile_load(best)) return evals;
       const uint64_t kp = family_key(base + lane, depth);
-      bool ok = split_trial<MODE>(keys, sp, kp);
-      if ((MODE == 5 || (MODE >= 7 && sp.confirm)) && ok) ok = split_trial<1>(keys, sp, kp);
+      bool ok = split_trial<MODE, STAGED>(keys, sp, kp);
+      if ((MODE == 5 || (MODE >= 7 && sp.confirm)) && ok) ok = split_trial<1, STAGED>(keys, sp, kp);
       const uint32_t hits = __ballot_sync(0xFFFFFFFFu, ok);
       evals += 32 * sp.m;
       if (hits) {
@@ -575,22 +693,23 @@ __device__ __forceinline__ uint64_t shared_search_warp(const uint64_t* __restric
   }
 }
 
+template <bool STAGED>
 __device__ __forceinline__ uint64_t shared_search(const uint64_t* __restrict__ keys, const SplitParams& sp, int mode,
                                                   uint32_t depth, uint32_t lane, uint64_t* best, unsigned int* next,
                                                   uint64_t stall, uint64_t limit, int* err, uint4* surv) {
   switch (mode) {
-    case 0: return shared_search_warp<0>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
-    case 1: return shared_search_warp<1>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
-    case 3: return shared_search_warp<3>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
-    case 4: return shared_search_warp<4>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
-    case 5: return shared_search_warp<5>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
-    case 6: return shared_search_warp<6>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
-    case 7: return shared_search_warp<7>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
-    case 8: return shared_search_warp<8>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
-    case 9: return shared_search_warp<9>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
-    case 10: return shared_search_warp<10>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
-    case 11: return shared_search_warp<11>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
-    default: return shared_search_warp<2>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
+    case 0: return shared_search_warp<0, STAGED>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
+    case 1: return shared_search_warp<1, STAGED>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
+    case 3: return shared_search_warp<3, STAGED>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
+    case 4: return shared_search_warp<4, STAGED>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
+    case 5: return shared_search_warp<5, STAGED>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
+    case 6: return shared_search_warp<6, STAGED>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
+    case 7: return shared_search_warp<7, STAGED>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
+    case 8: return shared_search_warp<8, STAGED>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
+    case 9: return shared_search_warp<9, STAGED>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
+    case 10: return shared_search_warp<10, STAGED>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
+    case 11: return shared_search_warp<11, STAGED>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
+    default: return shared_search_warp<2, STAGED>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
   }
 }
 
@@ -600,7 +719,7 @@ __device__ __forceinline__ uint64_t shared_search(const uint64_t* __restrict__ k
 // once: one per 2^12 expected trials, at most 16.
 template <bool COUNT>
 __global__ void __launch_bounds__(kThreads, 4) k_split_shared(SearchArgs a, SharedNodes st, uint32_t cap) {
-  extern __shared__ uint64_t mine[];
+  extern __shared__ __align__(16) uint64_t mine[];
   __shared__ uint32_t task, owner, closer, drained;
   __shared__ uint32_t fill[16];
   __shared__ uint4 surv[kWarps][kShareRounds * 32];  // two-phase block survivors, per warp
@@ -689,8 +808,12 @@ __global__ void __launch_bounds__(kThreads, 4) k_split_shared(SearchArgs a, Shar
     {
       SplitParams sp;
       const int mode = split_setup(nd, table, sp, /*fixed_width=*/true);
-      const uint64_t done = shared_search(in_smem ? mine : src, sp, mode, depth, lane, &st.best[idx], &st.next[idx],
-                                          stall_threshold(table, nd.m), trial_limit(table, nd.m), a.error, surv[warp]);
+      const uint64_t stall = stall_threshold(table, nd.m), limit = trial_limit(table, nd.m);
+      const uint64_t done =
+          in_smem ? shared_search<true>(mine, sp, mode, depth, lane, &st.best[idx], &st.next[idx], stall, limit,
+                                        a.error, surv[warp])
+                  : shared_search<false>(src, sp, mode, depth, lane, &st.best[idx], &st.next[idx], stall, limit,
+                                         a.error, surv[warp]);
       if (COUNT) evals += done;
     }
     __syncthreads();
@@ -1019,11 +1142,14 @@ __global__ void __launch_bounds__(kThreads, leaf_min_blocks(LMAX)) k_leaves(Sear
   const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   unsigned long long* const exec = a.exec_count ? &wexec[warp] : nullptr;
   if (lane == 0) wexec[warp] = 0;
-  const uint32_t gid = warp / gwarps, wig = warp % gwarps;
-  const bool leader = wig == 0 && lane == 0;
   const bool from_full = FULL || (RANGE && qfull);
   const Node* queue = from_full ? a.full_q[a.cls] : a.part_q[a.cls];
   const uint32_t total = from_full ? a.full_n[a.cls] : a.part_n[a.cls];
+  gwarps = group_warps(gwarps, total);
+  const uint32_t groups = gridDim.x * (kWarps / gwarps);
+  chunk = min(chunk, max(1u, total / (2 * groups)));
+  const uint32_t gid = warp / gwarps, wig = warp % gwarps;
+  const bool leader = wig == 0 && lane == 0;
   const uint32_t extra = RANGE ? a.extra_of[a.cls] : 0;
   const uint64_t* table = a.table[a.cls];
 
@@ -1273,7 +1399,7 @@ int launch_split_level(const SearchArgs& a, uint64_t max_m, uint32_t max_leaf, i
                        const SharedNodes* share) {
   if (share) {
     // one CTA per node at a time, nodes shared once the queue is empty
-    const uint64_t cap = std::max<uint64_t>(1, std::min<uint64_t>(max_m, kSplitSmemBudget / sizeof(uint64_t)));
+    const uint64_t cap = std::min<uint64_t>((max_m + 1) & ~uint64_t(1), kSplitSmemBudget / sizeof(uint64_t));
     const size_t smem = cap * sizeof(uint64_t);
     auto kern = a.exec_count ? k_split_shared<true> : k_split_shared<false>;
     int rc = a.exec_count ? allow_split_smem<k_split_shared<true>>() : allow_split_smem<k_split_shared<false>>();
@@ -1292,8 +1418,8 @@ int launch_split_level(const SearchArgs& a, uint64_t max_m, uint32_t max_leaf, i
   const recsplit_tuning_t t = tuning_for(max_leaf);
   const uint32_t gwarps = t.split_warps[max_m >= 256 ? 2 : (max_m >= 64 ? 1 : 0)];
   const uint32_t groups = kWarps / gwarps;
-  uint64_t cap = std::min<uint64_t>(max_m, kSplitSmemBudget / (groups * sizeof(uint64_t)));
-  if (cap < 1) cap = 1;
+  // an even number of keys per group, so that every group's are 16-byte aligned
+  const uint64_t cap = std::min<uint64_t>((max_m + 1) & ~uint64_t(1), kSplitSmemBudget / (groups * sizeof(uint64_t)));
   const size_t smem = size_t(groups) * cap * sizeof(uint64_t);
   auto kern = a.exec_count ? k_split_level<true> : k_split_level<false>;
   int rc = a.exec_count ? allow_split_smem<k_split_level<true>>() : allow_split_smem<k_split_level<false>>();
