@@ -1290,6 +1290,222 @@ __global__ void __launch_bounds__(kThreads, leaf_min_blocks(LMAX)) k_leaves(Sear
   if (exec && lane == 0 && wexec[warp]) atomicAdd(a.exec_count, wexec[warp]);
 }
 
+// ---------------------------------------------------------------- packed leaves
+// Full leaves of 4 to 8 keys.  A leaf of 8 keys takes 416 trials on
+// average, so a warp that tests 128 indices of one leaf per round tests 64
+// beyond the winner (15%).  Here a warp holds up to four leaves, eight lanes
+// on each: a round tests 8 spl indices per leaf, and the survivors of the
+// first H keys of all four are finished together, 32 at a time, so the second
+// phase's batches stay as full as with one leaf.  A leaf that finishes is
+// replaced at once from nodes the warp has taken ahead (one atomic and one
+// load per chunk).  At the end of the queue, and when there are too few
+// leaves for all warps, the lanes of free slots join the leaves that remain.
+//
+// The keys of the lane's leaf are in its registers, copies in shared memory
+// serve the second phase.  A round covers every index of [base, base +
+// lanes * spl) of its leaf and all survivors are finished, so the smallest
+// success of the round is the leaf's first bijective index.
+//
+// At 8 keys the first four values, 3 bits each, are shifted into one word
+// (one funnel shift per key instead of two shifts and an add) and a table of
+// 4096 bytes in shared memory gives the set of the four values, or 0xFF when
+// two are equal.
+constexpr int kPackedLeaf = 8;
+constexpr uint32_t kPackedSlots = 4;
+
+// Set of the values of a 12-bit index (four 3-bit values), 0xFF when two are
+// equal: four consecutive entries (the index's low 2 bits) per 32-bit word.
+__device__ __forceinline__ void fill_octal_sets(uint32_t* lut) {
+  for (uint32_t w = threadIdx.x; w < 1024; w += kThreads) {
+    const uint32_t e = w * 4;
+    const uint32_t p = (1u << (e >> 9)) | (1u << ((e >> 6) & 7)) | (1u << ((e >> 3) & 7));
+    const bool distinct = __popc(p) == 3;
+    uint32_t v = 0;
+#pragma unroll
+    for (uint32_t t = 0; t < 4; t++) {
+      const uint32_t bit = 1u << ((e + t) & 7);
+      v |= (distinct && !(p & bit) ? p | bit : 0xFFu) << (8 * t);
+    }
+    lut[w] = v;
+  }
+}
+
+// Whether the first H values of index key kp are distinct, and their set.
+template <int L, int H>
+__device__ __forceinline__ bool leaf_head(const uint64_t (&x)[L], uint64_t kp, const uint8_t* lut, uint32_t& seen) {
+  if constexpr (L == 8 && H >= 4) {
+    uint32_t v = family_top32(x[0], kp) >> 29;
+#pragma unroll
+    for (int i = 1; i < 4; i++) v = __funnelshift_l(family_top32(x[i], kp), v, 3);
+    seen = lut[v];
+    bool ok = H > 4 || seen != 0xFFu;
+#pragma unroll
+    for (int i = 4; i < H; i++) {
+      const uint32_t bit = 1u << phi_fixed<L>(x[i], kp);
+      ok = ok && !(seen & bit);
+      seen |= bit;
+    }
+    return ok;
+  } else {
+    seen = 0;
+#pragma unroll
+    for (int i = 0; i < H; i++) seen += 1u << phi_fixed<L>(x[i], kp);
+    return __popc(seen) == H;
+  }
+}
+
+template <int L>
+__global__ void __launch_bounds__(kThreads, 4) k_leaves_packed(SearchArgs a, uint32_t chunk, uint32_t spl) {
+  constexpr int H = leaf_first_part(L);
+  constexpr uint32_t full = (1u << L) - 1;
+  constexpr uint32_t kAll = 0xFFFFFFFFu;
+  __shared__ uint64_t skeys[kWarps][kPackedSlots][L];
+  __shared__ uint64_t sdkey[kWarps][kPackedSlots];
+  __shared__ uint32_t sbase[kWarps][kPackedSlots], sbest[kWarps][kPackedSlots];
+  __shared__ uint2 surv[kWarps][32 * kMaxSpl];  // {index, set of the first values | slot << 16}
+  __shared__ uint32_t lut[L == 8 ? 1024 : 1];
+  const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t total = a.full_n[a.cls];
+  if (L == 8) fill_octal_sets(lut);
+  __syncthreads();
+  const Node* queue = a.full_q[a.cls];
+  const uint32_t below = (1u << lane) - 1;
+  const uint32_t nwarps = gridDim.x * kWarps;
+  const uint32_t slots = total >= kPackedSlots * nwarps ? kPackedSlots : (total >= 2 * nwarps ? 2 : 1);
+  chunk = min(min(chunk, 32u), max(1u, total / (4 * nwarps)));
+  const uint32_t stall = static_cast<uint32_t>(min(stall_threshold(a.table[a.cls], L), uint64_t(1) << 31));
+  const uint32_t limit = static_cast<uint32_t>(min(trial_limit(a.table[a.cls], L), uint64_t(1) << 31));
+
+  Node pend{};                    // lane i: node i of the chunk taken
+  uint32_t pend_at = 0, pend_n = 0;
+  bool more = true;
+  uint32_t act = 0;               // slots in use
+  uint32_t my_slot = 0;           // lanes 0..3: code slot of the leaf in slot `lane`
+  uint32_t rounds = 0;
+  unsigned long long exec = 0;
+
+  for (;;) {
+    // fill free slots
+    for (uint32_t need = ~act & ((1u << slots) - 1); need && more; need &= need - 1) {
+      if (pend_at == pend_n) {
+        uint32_t first = 0;
+        if (lane == 0) first = *reinterpret_cast<volatile int*>(a.error) ? total : atomicAdd(a.work_counter, chunk);
+        first = __shfl_sync(kAll, first, 0);
+        if (first >= total) {
+          more = false;
+          break;
+        }
+        pend_n = min(chunk, total - first);
+        pend_at = 0;
+        if (lane < pend_n) pend = queue[first + lane];
+      }
+      const uint32_t q = __ffs(need) - 1;
+      const uint32_t start = __shfl_sync(kAll, pend.start, pend_at), slot = __shfl_sync(kAll, pend.slot, pend_at);
+      const uint32_t depth = __shfl_sync(kAll, pend.depth, pend_at) & kDepthMask;
+      if (lane == q) my_slot = slot;
+      if (lane < L) skeys[warp][q][lane] = __ldg(a.keys[depth & 1] + start + lane);
+      if (lane == 0) {
+        sdkey[warp][q] = uint64_t(depth) * kWeyl;
+        sbase[warp][q] = 0;
+        sbest[warp][q] = ~0u;
+      }
+      act |= 1u << q;
+      pend_at++;
+    }
+    if (!act) break;
+    __syncwarp();
+    // the four quarters of the warp are dealt to the k slots in use: quarter
+    // -> slot in order, the lanes on that slot, and the quarter's place among them
+    const uint32_t k = __popc(act), quarter = lane >> 3;
+    uint32_t mine = quarter, lanes = 8, place = 0;
+    if (k < kPackedSlots) {
+      const uint32_t rank = k == 3 ? (quarter == 3 ? 0 : quarter) : (k == 2 ? quarter & 1 : 0);
+      mine = __fns(act, 0, static_cast<int>(rank) + 1);
+      lanes = k == 1 ? 32 : (k == 2 || rank == 0 ? 16 : 8);
+      place = k == 1 ? quarter : (k == 2 ? quarter >> 1 : quarter / 3);
+    }
+    uint64_t x[L];
+#pragma unroll
+    for (int j = 0; j < L; j++) x[j] = skeys[warp][mine][j];
+    const uint64_t dkey = sdkey[warp][mine];
+    uint32_t base = sbase[warp][mine];
+    const uint32_t sub = 8 * place + (lane & 7);
+    const uint64_t step = kWeyl64 * lanes;
+    const uint32_t tag = mine << 16;
+    // checked for equal keys in the first round at or beyond the stall point
+    // (again if the lanes were dealt anew since: a round is 32 spl indices at most)
+    uint32_t check = base < stall + 32 * kMaxSpl ? min(stall, limit) : limit;
+
+    bool stop = false, won = false;
+    while (!won) {
+      if ((++rounds & 255) == 0 && __shfl_sync(kAll, lane == 0 ? *reinterpret_cast<volatile int*>(a.error) : 0, 0)) {
+        stop = true;  // another search failed, or the host cancelled the build
+        break;
+      }
+      if (__any_sync(kAll, base >= check)) {
+        bool bad = false;
+        if (base >= limit) {
+          set_error(a.error, RECSPLIT_E_SEARCH_LIMIT);
+          bad = true;
+        } else if (base >= check) {
+          check = limit;
+          bool dup = false;
+#pragma unroll
+          for (int i = 0; i < L; i++)
+#pragma unroll
+            for (int j = i + 1; j < L; j++) dup |= x[i] == x[j];
+          if (dup) set_error(a.error, RECSPLIT_E_DUPLICATE);
+          bad = dup;
+        }
+        if (__any_sync(kAll, bad)) {
+          stop = true;
+          break;
+        }
+      }
+      uint32_t ns = 0, idx = base + sub;
+      uint64_t key = index_key(idx, dkey);
+#pragma unroll 2
+      for (uint32_t j = 0; j < spl; j++, key += step, idx += lanes) {
+        uint32_t seen;
+        const bool ok = leaf_head<L, H>(x, key ^ (key >> 30), reinterpret_cast<const uint8_t*>(lut), seen);
+        const uint32_t b = __ballot_sync(kAll, ok);
+        if (ok) surv[warp][ns + __popc(b & below)] = make_uint2(idx, seen | tag);
+        ns += __popc(b);
+      }
+      base += lanes * spl;
+      __syncwarp();
+      for (uint32_t t0 = 0; t0 < ns; t0 += 32) {
+        const uint32_t t = t0 + lane;
+        bool ok = false;
+        if (t < ns) {
+          const uint2 e = surv[warp][t];
+          const uint32_t s = e.y >> 16;
+          const uint64_t ki = index_key(e.x, sdkey[warp][s]);
+          const uint64_t kp = ki ^ (ki >> 30);
+          uint32_t seen = e.y & 0xFFFFu;
+#pragma unroll
+          for (int i = H; i < L; i++) seen += 1u << phi_fixed<L>(skeys[warp][s][i], kp);
+          ok = seen == full;
+          if (ok) atomicMin(&sbest[warp][s], e.x);
+        }
+        won |= __any_sync(kAll, ok);
+      }
+      if (a.exec_count) exec += spl * 32 * H + ns * (L - H);
+    }
+    if (stop) break;
+    __syncwarp();
+    const uint32_t best = lane < kPackedSlots && (act >> lane & 1) ? sbest[warp][lane] : ~0u;
+    if (best != ~0u) {
+      a.seeds[my_slot] = best;
+      a.sizes[my_slot] = L;
+    }
+    act &= ~__ballot_sync(kAll, best != ~0u);
+    if (sub == 0) sbase[warp][mine] = base;
+    __syncwarp();
+  }
+  if (a.exec_count && lane == 0 && exec) atomicAdd(a.exec_count, exec);
+}
+
 // Dynamic shared memory the split kernels may use: nodes of up to this many
 // bytes of keys are staged, larger ones read from global memory.
 constexpr size_t kSplitSmemBudget = 96 * 1024;
@@ -1340,6 +1556,21 @@ int launch_leaf_kernel(const SearchArgs& a, const recsplit_tuning_t& t, int sm_c
 
 template <int L>
 int launch_full(const SearchArgs& a, const recsplit_tuning_t& t, int sm, cudaStream_t s) {
+  if constexpr (L >= 4 && L <= kPackedLeaf) {
+    auto kern = k_leaves_packed<L>;
+    int blocks = 0;
+    int rc = persistent_grid(kern, 0, sm, &blocks);
+    if (rc) return rc;
+    // (the queue's capacity, keys / L + 1, bounds the leaves; with fewer than
+    // one per four warps the two-phase kernel puts several warps on each)
+    if (t.leaf_two_phase && t.leaf_warps == 1 && uint64_t(a.full_cap[a.cls]) * 4 > uint64_t(blocks) * kWarps) {
+      RS_CUDA(cudaMemsetAsync(a.work_counter, 0, sizeof(uint32_t), s));
+      kern<<<blocks, kThreads, 0, s>>>(a, t.leaf_chunk, t.leaf_seeds_per_lane);
+      count_launch();
+      RS_CUDA(cudaGetLastError());
+      return RECSPLIT_OK;
+    }
+  }
   if (t.leaf_two_phase) return launch_leaf_kernel<L, true, true>(a, t, sm, s);
   return launch_leaf_kernel<L, true, false>(a, t, sm, s);
 }
@@ -1362,20 +1593,22 @@ bool g_tuned[kMaxLeaf + 1] = {};
 }  // namespace
 
 // Seeds per lane that a leaf test mode starts from: one for the one-phase
-// test; for the phased tests four, and the most, eight, from 12 keys on,
-// where a leaf takes thousands of trials and longer rounds spread the
-// per-round checks over more indices (measured faster at l = 12 to 16 with
-// either phased test).
+// test; for the phased tests the fastest measured at each size (leaf phase,
+// b = 100: l = 5: 1; l = 6: 2; l = 7, 8: 4; l = 9, 10: 8, 0.83 and 1.83 ms on 10^6
+// keys against 0.85 and 1.90 with 4; from 12 keys a leaf takes thousands of
+// trials and longer rounds spread the per-round checks).
 uint32_t natural_seeds_per_lane(uint32_t leaf, uint32_t two_phase) {
   if (!two_phase) return 1;
-  return leaf >= 12 ? kMaxSpl : 4;
+  return leaf >= 9 ? kMaxSpl : (leaf >= 7 ? 4 : (leaf == 6 ? 2 : 1));
 }
 
+// (the phased tests are the faster from 4 keys on: leaf phase of 10^7 keys at
+// l = 8, b = 100 3.4 ms with the one-phase test, 2.6 ms with the packed kernel)
 recsplit_tuning_t default_tuning(uint32_t leaf) {
   recsplit_tuning_t t;
   t.leaf_warps = leaf >= 12 ? 4 : 1;
   t.leaf_chunk = leaf >= 12 ? 1 : 4;
-  t.leaf_two_phase = leaf >= 10 ? 1 : 0;
+  t.leaf_two_phase = leaf >= 4 ? 1 : 0;
   t.leaf_seeds_per_lane = natural_seeds_per_lane(leaf, t.leaf_two_phase);
   t.split_warps[0] = 1;
   t.split_warps[1] = leaf >= 12 ? 2 : 1;
