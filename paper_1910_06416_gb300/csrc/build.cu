@@ -784,11 +784,16 @@ int build_sets(const SetInput* in, uint32_t count, const BuildOptions& opt, cuda
     }
   }
   SharedNodes shared{};
-  if (std::find(plan_share.begin(), plan_share.end(), 1) != plan_share.end()) {
-    if ((rc = sc.alloc(&shared.best, split_cap)) || (rc = sc.alloc(&shared.next, split_cap)) ||
-        (rc = sc.alloc(&shared.refs, split_cap)) || (rc = sc.alloc(&shared.cap, split_cap)) ||
-        (rc = sc.alloc(&shared.flag, split_cap)) ||
-        (rc = sc.alloc(&shared.owned, kSharedCtas)))
+  uint64_t share_cap = std::find(plan_share.begin(), plan_share.end(), 1) != plan_share.end() ? split_cap : 0;
+  std::vector<char> share_leaves(nclass);
+  for (uint32_t c = 0; c < nclass; c++) {
+    share_leaves[c] = leaves_shared(class_leaf[c], class_extra[c]);
+    if (share_leaves[c]) share_cap = std::max(share_cap, full_cap[c]);
+  }
+  if (share_cap) {
+    if ((rc = sc.alloc(&shared.best, share_cap)) || (rc = sc.alloc(&shared.next, share_cap)) ||
+        (rc = sc.alloc(&shared.refs, share_cap)) || (rc = sc.alloc(&shared.cap, share_cap)) ||
+        (rc = sc.alloc(&shared.flag, share_cap)) || (rc = sc.alloc(&shared.owned, kSharedCtas)))
       return rc;
   }
 
@@ -842,7 +847,11 @@ int build_sets(const SetInput* in, uint32_t count, const BuildOptions& opt, cuda
     if (!opt.use_graph) timer.mark();
     for (uint32_t c = 0; c < nclass; c++) {
       a.cls = c;
-      int r = launch_leaves(a, class_leaf[c], class_extra[c], sm_count, ws);
+      if (share_leaves[c]) {
+        RS_CUDA(cudaMemsetAsync(shared.flag, 0, full_cap[c] * sizeof(unsigned int), ws));
+        RS_CUDA(cudaMemsetAsync(shared.owned, 0xFF, kSharedCtas * sizeof(unsigned int), ws));
+      }
+      int r = launch_leaves(a, class_leaf[c], class_extra[c], sm_count, ws, share_leaves[c] ? &shared : nullptr);
       if (r) return r;
     }
     if (!opt.use_graph) timer.mark();

@@ -264,10 +264,11 @@ struct SearchArgs {
   unsigned long long* exec_count;
 };
 
-// State of the nodes of one split level for the shared search (search.cu):
-// per node its best index so far, block counter, participants, most
-// participants and state (0 none, 1 open, 2 closed; zeroed per level), and
-// per CTA the node it owns (~0 when none; set to ~0 per level).  kSharedCtas bounds the grid.
+// State of the nodes of one split level, or of a class's full leaves, for the
+// shared search (search.cu): per node its best index so far, block counter,
+// participants, most participants and state (0 none, 1 open, 2 closed; zeroed
+// per launch), and per CTA the node it owns (~0 when none; set to ~0 per
+// launch).  kSharedCtas bounds the grid.
 struct SharedNodes {
   uint64_t* best;
   unsigned int* next;
@@ -282,7 +283,11 @@ constexpr uint32_t kSharedCtas = 4096;
 // with nodes shared by the CTAs that find the queue empty (st zeroed as above)
 int launch_split_level(const SearchArgs& a, uint64_t max_m, uint32_t max_leaf, int sm_count, cudaStream_t s,
                        const SharedNodes* share = nullptr);
-int launch_leaves(const SearchArgs& a, uint32_t leaf, uint32_t extra, int sm_count, cudaStream_t s);
+// Whether the full leaves of a class are searched shared (launch_leaves then
+// needs share, zeroed as above).
+bool leaves_shared(uint32_t leaf, uint32_t extra);
+int launch_leaves(const SearchArgs& a, uint32_t leaf, uint32_t extra, int sm_count, cudaStream_t s,
+                  const SharedNodes* share = nullptr);
 
 // Launch shapes of the searches for one leaf size (see recsplit_tuning_t).
 recsplit_tuning_t tuning_for(uint32_t leaf);

@@ -713,40 +713,36 @@ __device__ __forceinline__ uint64_t shared_search(const uint64_t* __restrict__ k
   }
 }
 
-// One CTA per node at a time (all 8 warps); the node state arrays are sized
-// by the level's queue capacity, `flag` zeroed and `owned` (one entry per
-// CTA) set to ~0 before the launch.  A node takes at most cap[node] CTAs at
-// once: one per 2^12 expected trials, at most 16.
-template <bool COUNT>
-__global__ void __launch_bounds__(kThreads, 4) k_split_shared(SearchArgs a, SharedNodes st, uint32_t cap) {
-  extern __shared__ __align__(16) uint64_t mine[];
+// One CTA per node at a time (all 8 warps): takes nodes of `queue` through
+// the work counter, joins open nodes once the queue is empty, and calls
+// begin(node) (the whole CTA), search(node, idx) (every warp; claims blocks
+// through st.next[idx], lowers st.best[idx]) and, in the last participant to
+// leave, close(node, index found).  The node state arrays are sized by the
+// queue's capacity, `flag` zeroed and `owned` (one entry per CTA) set to ~0
+// before the launch.  A node takes at most cap_of(node) CTAs at once.
+template <typename Cap, typename Begin, typename Search, typename Close>
+__device__ __forceinline__ void shared_nodes(const Node* queue, uint32_t total, const SharedNodes& st,
+                                             uint32_t* work_counter, int* error, Cap cap_of, Begin begin,
+                                             Search search, Close close) {
   __shared__ uint32_t task, owner, closer, drained;
-  __shared__ uint32_t fill[16];
-  __shared__ uint4 surv[kWarps][kShareRounds * 32];  // two-phase block survivors, per warp
   const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t total = *a.split_in_count;
   volatile uint32_t* vflag = st.flag;
-  unsigned long long evals = 0;  // work counting: evaluations of this warp, flushed at exit
-  uint32_t joins = 0;            // nodes joined: bounded, so that the kernel ends whatever the timing
+  uint32_t joins = 0;  // nodes joined: bounded, so that the kernel ends whatever the timing
   if (threadIdx.x == 0) drained = 0;
   __syncthreads();
 
   for (;;) {
     if (threadIdx.x == 0) {
       uint32_t idx = total, own = 0;
-      if (!*reinterpret_cast<volatile int*>(a.error) && !drained) {
-        const uint32_t i = atomicAdd(a.work_counter, 1u);
+      if (!*reinterpret_cast<volatile int*>(error) && !drained) {
+        const uint32_t i = atomicAdd(work_counter, 1u);
         if (i < total) {
           idx = i;
           own = 1;
-          // participants worth having: about one CTA per 2^12 expected
-          // trials, at most 16 (a node of a few hundred trials gains nothing)
-          const Node nd = a.split_in[i];
-          const uint64_t et = a.table[nd.depth >> 8][kTableWords * nd.m + 2];
           st.best[i] = ~0ull;
           st.next[i] = 0;
           st.refs[i] = 1;
-          st.cap[i] = static_cast<uint32_t>(min(uint64_t(16), max(uint64_t(1), et >> 12)));
+          st.cap[i] = cap_of(queue[i]);
           __threadfence();
           vflag[i] = kNodeOpen;
           reinterpret_cast<volatile uint32_t*>(st.owned)[blockIdx.x] = i;
@@ -758,7 +754,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_split_shared(SearchArgs a, Shar
       owner = own;
     }
     __syncthreads();
-    if (task >= total && drained && warp == 0 && joins < kMaxJoins && !*reinterpret_cast<volatile int*>(a.error)) {
+    if (task >= total && drained && warp == 0 && joins < kMaxJoins && !*reinterpret_cast<volatile int*>(error)) {
       joins++;
       // join the open node with the fewest participants, if any
       for (int attempt = 0; attempt < 8; attempt++) {
@@ -796,29 +792,13 @@ __global__ void __launch_bounds__(kThreads, 4) k_split_shared(SearchArgs a, Shar
     __syncthreads();
     const uint32_t idx = task;
     if (idx >= total) break;
-    const Node nd = a.split_in[idx];
-    const uint32_t depth = nd.depth & kDepthMask;
-    const uint64_t* table = a.table[nd.depth >> 8];
-    const uint64_t* src = a.keys[depth & 1] + nd.start;
-    const bool in_smem = nd.m <= cap;
-    if (in_smem)
-      for (uint32_t j = threadIdx.x; j < nd.m; j += kThreads) mine[j] = src[j];
-    if (threadIdx.x < 16) fill[threadIdx.x] = 0;
+    const Node nd = queue[idx];
+    begin(nd);
     __syncthreads();
-    {
-      SplitParams sp;
-      const int mode = split_setup(nd, table, sp, /*fixed_width=*/true);
-      const uint64_t stall = stall_threshold(table, nd.m), limit = trial_limit(table, nd.m);
-      const uint64_t done =
-          in_smem ? shared_search<true>(mine, sp, mode, depth, lane, &st.best[idx], &st.next[idx], stall, limit,
-                                        a.error, surv[warp])
-                  : shared_search<false>(src, sp, mode, depth, lane, &st.best[idx], &st.next[idx], stall, limit,
-                                         a.error, surv[warp]);
-      if (COUNT) evals += done;
-    }
+    search(nd, idx);
     __syncthreads();
     if (threadIdx.x == 0) {
-      // leave; the last participant closes the node and partitions it
+      // leave; the last participant closes the node
       __threadfence();
       const uint32_t left = atomicSub(&st.refs[idx], 1u);
       closer = left == 1 && atomicCAS(&st.flag[idx], kNodeOpen, kNodeClosed) == kNodeOpen;
@@ -826,15 +806,54 @@ __global__ void __launch_bounds__(kThreads, 4) k_split_shared(SearchArgs a, Shar
     }
     __syncthreads();
     if (closer) {
-      const uint64_t seed = volatile_load(&st.best[idx]);
-      if (seed == ~0ull) {
-        if (threadIdx.x == 0) set_error(a.error, RECSPLIT_E_SEARCH_LIMIT);
-      } else if (!*reinterpret_cast<volatile int*>(a.error)) {
-        partition_node(a, nd, seed, in_smem ? mine : nullptr, threadIdx.x, kThreads, lane, warp == 0, fill);
+      const uint64_t found = volatile_load(&st.best[idx]);
+      if (found == ~0ull) {
+        if (threadIdx.x == 0) set_error(error, RECSPLIT_E_SEARCH_LIMIT);
+      } else if (!*reinterpret_cast<volatile int*>(error)) {
+        close(nd, found);
       }
     }
     __syncthreads();
   }
+}
+
+// Participants worth having on a split node: one CTA per 2^12 expected trials,
+// at most 16 (a node of a few hundred trials gains nothing).
+template <bool COUNT>
+__global__ void __launch_bounds__(kThreads, 4) k_split_shared(SearchArgs a, SharedNodes st, uint32_t cap) {
+  extern __shared__ __align__(16) uint64_t mine[];
+  __shared__ uint32_t fill[16];
+  __shared__ uint4 surv[kWarps][kShareRounds * 32];  // two-phase block survivors, per warp
+  const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  unsigned long long evals = 0;  // work counting: evaluations of this warp, flushed at exit
+  shared_nodes(
+      a.split_in, *a.split_in_count, st, a.work_counter, a.error,
+      [&](const Node& nd) {
+        const uint64_t et = a.table[nd.depth >> 8][kTableWords * nd.m + 2];
+        return static_cast<uint32_t>(min(uint64_t(16), max(uint64_t(1), et >> 12)));
+      },
+      [&](const Node& nd) {
+        const uint64_t* src = a.keys[nd.depth & 1] + nd.start;
+        if (nd.m <= cap)
+          for (uint32_t j = threadIdx.x; j < nd.m; j += kThreads) mine[j] = src[j];
+        if (threadIdx.x < 16) fill[threadIdx.x] = 0;
+      },
+      [&](const Node& nd, uint32_t idx) {
+        const uint32_t depth = nd.depth & kDepthMask;
+        const uint64_t* table = a.table[nd.depth >> 8];
+        SplitParams sp;
+        const int mode = split_setup(nd, table, sp, /*fixed_width=*/true);
+        const uint64_t stall = stall_threshold(table, nd.m), limit = trial_limit(table, nd.m);
+        const uint64_t done =
+            nd.m <= cap ? shared_search<true>(mine, sp, mode, depth, lane, &st.best[idx], &st.next[idx], stall, limit,
+                                              a.error, surv[warp])
+                        : shared_search<false>(a.keys[depth & 1] + nd.start, sp, mode, depth, lane, &st.best[idx],
+                                               &st.next[idx], stall, limit, a.error, surv[warp]);
+        if (COUNT) evals += done;
+      },
+      [&](const Node& nd, uint64_t seed) {
+        partition_node(a, nd, seed, nd.m <= cap ? mine : nullptr, threadIdx.x, kThreads, lane, warp == 0, fill);
+      });
   if (COUNT && lane == 0 && evals) atomicAdd(a.exec_count + 1, evals);
 }
 
@@ -954,7 +973,7 @@ __device__ __forceinline__ uint64_t leaf_round_two_phase(const uint64_t (&x)[L],
 //
 // h1 < h2 minimise the expected work per index, h1 + P_h1 (h2 - h1 + c) +
 // P_h2 (l - h2 + c) evaluations with c = 2.5 for the compaction and reload of
-// a survivor (P_h as above): (6, 9) at l = 13, (7, 10) at 16, (8, 13) at 24.
+// a survivor (P_h as above): (6, 9) at l = 13, (8, 13) at 24.
 // At l = 12 a leaf takes about 2 * 10^4 trials, a few rounds of a group, and
 // draining the buffers at the end of every leaf costs more than the full
 // batches save (measured: 6% slower than the two-phase round), so the
@@ -963,6 +982,7 @@ struct LeafPhases {
   int h1, h2;
 };
 __host__ __device__ constexpr LeafPhases leaf_phases(int l) {
+  if (l == 16) return LeafPhases{6, 9};  // whole triples (below), 1% above the minimum
   double best = 1e30;
   LeafPhases arg{1, 2};
   double p1 = 1.0;  // P_h1
@@ -983,15 +1003,54 @@ __host__ __device__ constexpr LeafPhases leaf_phases(int l) {
 constexpr int kFifoLeaf = 13;
 constexpr uint32_t kFifoA = 32 * kMaxSpl + 32;  // below 32 left + one round's spl * 32
 constexpr uint32_t kFifoB = 64;                 // below 32 left + one batch of A
-// Entries carry the low 32 bits of their index; the buffers are drained
-// every 2^16 rounds, so an entry is less than 2^16 * 16 * 32 * kMaxSpl < 2^32
-// indices older than the newest and its index is recovered exactly.
-constexpr uint32_t kFifoDrainRounds = 1u << 16;
+//
+// At l = 16 the values of three keys, 4 bits each, are shifted into one word
+// (one funnel shift per key instead of two shifts and an add), and a table in
+// shared memory gives the set of the three, or all ones when two are equal;
+// sets are combined by testing that they share no value.
+//
+// An entry is {low 32 bits of the index, set of the values so far}; the
+// function key is computed again from the index, 8 instructions per entry of a
+// full batch, which costs no more than storing and loading it did and halves
+// the buffers.
+
+// Set of the values of a 12-bit index (three 4-bit values), 0xFFFF when two are
+// equal: two consecutive entries per 32-bit word.
+__device__ __forceinline__ void fill_hex_sets(uint32_t* lut) {
+  for (uint32_t w = threadIdx.x; w < 2048; w += kThreads) {
+    const uint32_t e = w * 2;
+    const uint32_t p = (1u << (e >> 8)) | (1u << ((e >> 4) & 15));
+    const bool distinct = __popc(p) == 2;
+    uint32_t v = 0;
+#pragma unroll
+    for (uint32_t t = 0; t < 2; t++) {
+      const uint32_t bit = 1u << ((e + t) & 15);
+      v |= (distinct && !(p & bit) ? p | bit : 0xFFFFu) << (16 * t);
+    }
+    lut[w] = v;
+  }
+}
+
+// l = 16: the set of the values of keys x[I], x[I + 1], x[I + 2].
+template <int I>
+__device__ __forceinline__ uint32_t hex_set(const uint64_t* x, uint64_t kp, const uint16_t* lut) {
+  uint32_t v = family_top32(x[I], kp) >> 28;
+  v = __funnelshift_l(family_top32(x[I + 1], kp), v, 4);
+  v = __funnelshift_l(family_top32(x[I + 2], kp), v, 4);
+  return lut[v];
+}
+
+// The keys of the leaf are read from shared memory: 2 l registers for them
+// held the kernel to three CTAs per SM, too few for its dependent chains (ncu
+// at l = 16, 24 warps per SM: issue 66%, fixed-latency waits the leading
+// stall).  Leaf phase at l = 16, b = 2000, 4 * 10^5 keys, four warps per leaf:
+// 143 ms with 16-byte entries and keys in registers, 131 ms so with four CTAs
+// per SM, 139 ms with five (48 registers), 155 ms with six.
 
 // Moves entries [r, n) of a warp buffer, fewer than 32, to its front.
-__device__ __forceinline__ uint32_t fifo_compact(uint4* buf, uint32_t r, uint32_t n, uint32_t lane) {
+__device__ __forceinline__ uint32_t fifo_compact(uint2* buf, uint32_t r, uint32_t n, uint32_t lane) {
   const uint32_t rem = n - r;
-  uint4 v = make_uint4(0, 0, 0, 0);
+  uint2 v = make_uint2(0, 0);
   if (lane < rem) v = buf[r + lane];
   __syncwarp();
   if (lane < rem) buf[lane] = v;
@@ -999,22 +1058,37 @@ __device__ __forceinline__ uint32_t fifo_compact(uint4* buf, uint32_t r, uint32_
   return rem;
 }
 
+// Index of an entry from its low 32 bits and the newest index generated.
+__device__ __forceinline__ uint64_t fifo_index(uint32_t low, uint64_t newest) {
+  return newest - static_cast<uint32_t>(static_cast<uint32_t>(newest) - low);
+}
+
+__device__ __forceinline__ uint64_t fifo_key(uint32_t low, uint64_t newest, uint64_t dkey) {
+  const uint64_t k = index_key(fifo_index(low, newest), dkey);
+  return k ^ (k >> 30);
+}
+
 template <int L>
-__device__ __forceinline__ void fifo_phase1(const uint64_t (&x)[L], uint64_t base, uint64_t dkey, uint32_t spl,
-                                            uint32_t lane, uint4* a, uint32_t& na) {
+__device__ __forceinline__ void fifo_phase1(const uint64_t* x, uint64_t base, uint64_t dkey, uint32_t spl,
+                                            uint32_t lane, const uint16_t* lut, uint2* a, uint32_t& na) {
   constexpr int H1 = leaf_phases(L).h1;
   const uint32_t below = (1u << lane) - 1;
   uint64_t k = index_key(base + lane, dkey);
   for (uint32_t j = 0; j < spl; j++, k += kLaneStep) {
     const uint64_t kp = k ^ (k >> 30);
     uint32_t seen = 0;
+    bool ok;
+    if constexpr (L == 16) {
+      const uint32_t s0 = hex_set<0>(x, kp, lut), s1 = hex_set<3>(x, kp, lut);
+      ok = !(s0 & s1);
+      seen = s0 | s1;
+    } else {
 #pragma unroll
-    for (int i = 0; i < H1; i++) seen += 1u << phi_fixed<L>(x[i], kp);
-    const bool ok = __popc(seen) == H1;
+      for (int i = 0; i < H1; i++) seen += 1u << phi_fixed<L>(x[i], kp);
+      ok = __popc(seen) == H1;
+    }
     const uint32_t b = __ballot_sync(0xFFFFFFFFu, ok);
-    if (ok)
-      a[na + __popc(b & below)] = make_uint4(static_cast<uint32_t>(base) + j * 32 + lane, seen,
-                                             static_cast<uint32_t>(kp), static_cast<uint32_t>(kp >> 32));
+    if (ok) a[na + __popc(b & below)] = make_uint2(static_cast<uint32_t>(base) + j * 32 + lane, seen);
     na += __popc(b);
   }
   __syncwarp();
@@ -1022,17 +1096,24 @@ __device__ __forceinline__ void fifo_phase1(const uint64_t (&x)[L], uint64_t bas
 
 // Phase 2 on entries [ra, ra + c) of A (c <= 32); survivors go to B.
 template <int L>
-__device__ __forceinline__ void fifo_phase2(const uint64_t (&x)[L], const uint4* a, uint32_t ra, uint32_t c,
-                                            uint32_t lane, uint4* b, uint32_t& nb) {
+__device__ __forceinline__ void fifo_phase2(const uint64_t* x, const uint2* a, uint32_t ra, uint32_t c,
+                                            uint64_t newest, uint64_t dkey, uint32_t lane, const uint16_t* lut,
+                                            uint2* b, uint32_t& nb) {
   constexpr LeafPhases ph = leaf_phases(L);
-  uint4 e = make_uint4(0, 0, 0, 0);
+  uint2 e = make_uint2(0, 0);
   bool ok = false;
   if (lane < c) {
     e = a[ra + lane];
-    const uint64_t kp = (uint64_t(e.w) << 32) | e.z;
+    const uint64_t kp = fifo_key(e.x, newest, dkey);
+    if constexpr (L == 16) {
+      const uint32_t s = hex_set<6>(x, kp, lut);
+      ok = !(e.y & s);
+      e.y |= s;
+    } else {
 #pragma unroll
-    for (int i = ph.h1; i < ph.h2; i++) e.y += 1u << phi_fixed<L>(x[i], kp);
-    ok = __popc(e.y) == ph.h2;
+      for (int i = ph.h1; i < ph.h2; i++) e.y += 1u << phi_fixed<L>(x[i], kp);
+      ok = __popc(e.y) == ph.h2;
+    }
   }
   const uint32_t hits = __ballot_sync(0xFFFFFFFFu, ok);
   if (ok) b[nb + __popc(hits & ((1u << lane) - 1))] = e;
@@ -1043,19 +1124,29 @@ __device__ __forceinline__ void fifo_phase2(const uint64_t (&x)[L], const uint4*
 // Phase 3 on entries [rb, rb + c) of B; on success `low` is the low 32 bits
 // of the first bijective entry's index.
 template <int L>
-__device__ __forceinline__ bool fifo_phase3(const uint64_t (&x)[L], const uint4* b, uint32_t rb, uint32_t c,
-                                            uint32_t lane, uint32_t& low) {
+__device__ __forceinline__ bool fifo_phase3(const uint64_t* x, const uint2* b, uint32_t rb, uint32_t c,
+                                            uint64_t newest, uint64_t dkey, uint32_t lane, const uint16_t* lut,
+                                            uint32_t& low) {
   constexpr int H2 = leaf_phases(L).h2;
   constexpr uint32_t full = L == 32 ? ~0u : ((1u << L) - 1);
   bool ok = false;
   uint32_t id = 0;
   if (lane < c) {
-    const uint4 e = b[rb + lane];
-    const uint64_t kp = (uint64_t(e.w) << 32) | e.z;
+    const uint2 e = b[rb + lane];
+    const uint64_t kp = fifo_key(e.x, newest, dkey);
     uint32_t seen = e.y;
+    if constexpr (L == 16) {
+      const uint32_t s0 = hex_set<9>(x, kp, lut), s1 = hex_set<12>(x, kp, lut);
+      ok = !(seen & s0);
+      seen |= s0;
+      ok = ok && !(seen & s1);
+      seen |= s1;
+      ok = ok && !(seen & (1u << phi_fixed<L>(x[15], kp)));
+    } else {
 #pragma unroll
-    for (int i = H2; i < L; i++) seen += 1u << phi_fixed<L>(x[i], kp);
-    ok = seen == full;
+      for (int i = H2; i < L; i++) seen += 1u << phi_fixed<L>(x[i], kp);
+      ok = seen == full;
+    }
     id = e.x;
   }
   const uint32_t hits = __ballot_sync(0xFFFFFFFFu, ok);
@@ -1068,36 +1159,36 @@ __device__ __forceinline__ bool fifo_phase3(const uint64_t (&x)[L], const uint4*
 // with `drain`).  `newest` is the largest index generated so far.  Returns
 // the smallest bijective index found, or ~0.
 template <int L>
-__device__ __forceinline__ uint64_t fifo_pump(const uint64_t (&x)[L], uint4* a, uint32_t& na, uint4* b, uint32_t& nb,
-                                              bool drain, uint64_t newest, uint32_t lane,
-                                              unsigned long long* exec) {
+__device__ __forceinline__ uint64_t fifo_pump(const uint64_t* x, uint2* a, uint32_t& na, uint2* b, uint32_t& nb,
+                                              bool drain, uint64_t newest, uint64_t dkey, uint32_t lane,
+                                              const uint16_t* lut, unsigned long long* exec) {
   constexpr LeafPhases ph = leaf_phases(L);
   uint32_t ra = 0, low = 0;
   bool found = false;
   while (!found && (na - ra >= 32 || (drain && na > ra))) {
     const uint32_t c = min(32u, na - ra);
-    fifo_phase2<L>(x, a, ra, c, lane, b, nb);
+    fifo_phase2<L>(x, a, ra, c, newest, dkey, lane, lut, b, nb);
     if (exec && lane == 0) *exec += c * (ph.h2 - ph.h1);
     ra += c;
     uint32_t rb = 0;
     while (nb - rb >= 32) {
       if (exec && lane == 0) *exec += 32 * (L - ph.h2);
-      if ((found = fifo_phase3<L>(x, b, rb, 32, lane, low))) break;
+      if ((found = fifo_phase3<L>(x, b, rb, 32, newest, dkey, lane, lut, low))) break;
       rb += 32;
     }
-    if (!found) nb = fifo_compact(b, rb, nb, lane);
+    if (!found && rb) nb = fifo_compact(b, rb, nb, lane);
   }
   if (!found) {
-    na = fifo_compact(a, ra, na, lane);  // fewer than 32 left unless draining, which leaves none
+    if (ra) na = fifo_compact(a, ra, na, lane);  // fewer than 32 left unless draining, which leaves none
     for (uint32_t rb = 0; drain && rb < nb; rb += 32) {
       const uint32_t c = min(32u, nb - rb);
       if (exec && lane == 0) *exec += c * (L - ph.h2);
-      if ((found = fifo_phase3<L>(x, b, rb, c, lane, low))) break;
+      if ((found = fifo_phase3<L>(x, b, rb, c, newest, dkey, lane, lut, low))) break;
     }
     if (drain) nb = 0;
   }
   if (!found) return ~0ull;
-  return newest - static_cast<uint32_t>(static_cast<uint32_t>(newest) - low);
+  return fifo_index(low, newest);
 }
 
 // Leaf of m < LMAX keys: slots j >= m contribute nothing.
@@ -1136,9 +1227,7 @@ __global__ void __launch_bounds__(kThreads, leaf_min_blocks(LMAX)) k_leaves(Sear
   __shared__ uint32_t task[kWarps];
   __shared__ unsigned long long wexec[kWarps];  // work counting: evaluations per warp, flushed at exit
   constexpr bool kTwoPhase = FULL && TWO && LMAX >= 4;
-  constexpr bool kFifo = kTwoPhase && LMAX >= kFifoLeaf;
-  // two-phase rounds: one round's survivors; three phases: buffers A and B
-  __shared__ uint4 surv[kTwoPhase ? kWarps : 1][kFifo ? kFifoA + kFifoB : (kTwoPhase ? 32 * kMaxSpl : 1)];
+  __shared__ uint4 surv[kTwoPhase ? kWarps : 1][kTwoPhase ? 32 * kMaxSpl : 1];  // one round's survivors
   const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   unsigned long long* const exec = a.exec_count ? &wexec[warp] : nullptr;
   if (lane == 0) wexec[warp] = 0;
@@ -1181,55 +1270,6 @@ __global__ void __launch_bounds__(kThreads, leaf_min_blocks(LMAX)) k_leaves(Sear
       // a round of a warp covers the spl * 32 indices from base; lane L tests
       // base + j * 32 + L for j < spl
       const uint64_t span = uint64_t(spl) * 32;
-      if constexpr (kFifo) {
-        uint4* const fa = surv[warp];
-        uint4* const fb = surv[warp] + kFifoA;
-        uint32_t na = 0, nb = 0;
-        uint64_t newest = 0;
-        for (uint64_t base = uint64_t(wig) * span;; base += uint64_t(gwarps) * span) {
-          bool drain = false, last = false, at_limit = false;
-          if (gwarps > 1 && __any_sync(0xFFFFFFFFu, base >= volatile_load(&best[gid]))) {
-            drain = last = true;  // another warp found a smaller index than this one's next
-          } else if ((++rounds & 255) == 0 &&
-                     __shfl_sync(0xFFFFFFFFu, lane == 0 ? *reinterpret_cast<volatile int*>(a.error) : 0, 0)) {
-            break;  // another search failed, or the host cancelled the build
-          } else if (base >= limit) {
-            drain = last = at_limit = true;  // an index below the limit may still wait in the buffers
-          } else {
-            if (!checked && base >= stall) {
-              checked = true;
-              bool dup = false;
-#pragma unroll
-              for (int i = 0; i < LMAX; i++)
-#pragma unroll
-                for (int j = i + 1; j < LMAX; j++) dup |= x[i] == x[j];
-              if (dup) {
-                if (lane == 0) {
-                  set_error(a.error, RECSPLIT_E_DUPLICATE);
-                  atomicMin(reinterpret_cast<unsigned long long*>(&best[gid]), 0ull);
-                }
-                break;
-              }
-            }
-            fifo_phase1<LMAX>(x, base, dkey, spl, lane, fa, na);
-            if (exec && lane == 0) *exec += spl * 32 * leaf_phases(LMAX).h1;
-            newest = base + span - 1;
-            drain = (rounds % kFifoDrainRounds) == 0;
-          }
-          const uint64_t found = na || nb ? fifo_pump<LMAX>(x, fa, na, fb, nb, drain, newest, lane, exec) : ~0ull;
-          if (found != ~0ull) {
-            if (lane == 0) atomicMin(reinterpret_cast<unsigned long long*>(&best[gid]), found);
-            break;
-          }
-          if (last) {
-            if (at_limit && lane == 0) {
-              set_error(a.error, RECSPLIT_E_SEARCH_LIMIT);
-              atomicMin(reinterpret_cast<unsigned long long*>(&best[gid]), 0ull);
-            }
-            break;
-          }
-        }
-      } else
       // one compare per round: the stall point until it is checked, then the limit
       for (uint64_t base = uint64_t(wig) * span, next_check = min(stall, limit);; base += uint64_t(gwarps) * span) {
         if (gwarps > 1 && __any_sync(0xFFFFFFFFu, base >= volatile_load(&best[gid]))) break;
@@ -1288,6 +1328,107 @@ __global__ void __launch_bounds__(kThreads, leaf_min_blocks(LMAX)) k_leaves(Sear
     }
   }
   if (exec && lane == 0 && wexec[warp]) atomicAdd(a.exec_count, wexec[warp]);
+}
+
+// ---------------------------------------------------------------- shared leaves
+// Full leaves of kFifoLeaf keys or more with the three-phase test, one CTA per
+// leaf; a CTA that finds the queue empty joins a leaf in progress, as for
+// shared split nodes.  Trial counts are geometric (873,000 on average at
+// l = 16): with four warps per leaf and no joining, 62,700 leaves kept a tenth
+// of the warps idle on average, and 6,000 leaves a third.  Every warp claims
+// kLeafShareRounds rounds of indices at a time, in increasing order, so its
+// buffers stay in index order and every index below the final best has been
+// tested.
+constexpr uint32_t kLeafShareRounds = 4;
+
+// One warp's part in the search of one leaf.
+template <int L>
+__device__ __forceinline__ void fifo_search(const uint64_t* x, uint32_t depth, uint32_t spl, uint64_t stall,
+                                            uint64_t limit, uint64_t* best, unsigned int* next, int* err,
+                                            uint32_t lane, const uint16_t* lut, uint2* fa, uint2* fb,
+                                            unsigned long long* exec) {
+  const uint64_t dkey = uint64_t(depth) * kWeyl;
+  const uint64_t span = uint64_t(spl) * 32, block = kLeafShareRounds * span;
+  uint64_t base = 0, end = 0, newest = 0, mark = 0;
+  uint32_t na = 0, nb = 0, rounds = 0;
+  for (;;) {
+    bool drain = false, generate = true;
+    if (base == end) {
+      unsigned int blk = 0;
+      if (lane == 0) blk = atomicAdd(next, 1u);
+      base = uint64_t(__shfl_sync(0xFFFFFFFFu, blk, 0)) * block;
+      end = base + block;
+      // the one warp whose block holds the stall point checks for keys that
+      // can never be separated
+      if (base <= stall && stall < end && has_duplicate(x, L, lane)) {
+        if (lane == 0) {
+          set_error(err, RECSPLIT_E_DUPLICATE);
+          atomicMin(reinterpret_cast<unsigned long long*>(best), 0ull);
+        }
+        return;
+      }
+      // an entry holds the low 32 bits of its index: none may stay until the
+      // newest index is 2^32 beyond it
+      if (end - mark >= (1ull << 32)) {
+        drain = true;
+        generate = false;
+        mark = base;
+      }
+    }
+    // a smaller index is known, or the limit is reached (the closer reports it
+    // if no index below it succeeded): finish what waits in the buffers
+    const bool last = __any_sync(0xFFFFFFFFu, base >= volatile_load(best)) || base >= limit;
+    if (last) {
+      drain = true;
+      generate = false;
+    }
+    if ((++rounds & 255) == 0 && __shfl_sync(0xFFFFFFFFu, lane == 0 ? *reinterpret_cast<volatile int*>(err) : 0, 0))
+      return;  // another search failed, or the host cancelled the build
+    if (generate) {
+      fifo_phase1<L>(x, base, dkey, spl, lane, lut, fa, na);
+      if (exec && lane == 0) *exec += span * leaf_phases(L).h1;
+      base += span;
+      newest = base - 1;
+    }
+    const uint64_t found = na || nb ? fifo_pump<L>(x, fa, na, fb, nb, drain, newest, dkey, lane, lut, exec) : ~0ull;
+    if (found != ~0ull) {
+      if (lane == 0) atomicMin(reinterpret_cast<unsigned long long*>(best), found);
+      return;
+    }
+    if (last) return;
+  }
+}
+
+template <int L>
+__global__ void __launch_bounds__(kThreads, 4) k_leaves_shared(SearchArgs a, SharedNodes st, uint32_t spl) {
+  __shared__ uint64_t x[L];
+  __shared__ uint2 fifo[kWarps][kFifoA + kFifoB];
+  __shared__ uint32_t lut[L == 16 ? 2048 : 1];
+  __shared__ unsigned long long wexec[kWarps];  // work counting: evaluations per warp, flushed at exit
+  const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (lane == 0) wexec[warp] = 0;
+  if (L == 16) fill_hex_sets(lut);
+  const uint64_t* table = a.table[a.cls];
+  const uint64_t stall = stall_threshold(table, L), limit = trial_limit(table, L);
+  // participants worth having: one CTA per 2^12 expected trials, at most 16
+  const uint32_t cap = static_cast<uint32_t>(min(uint64_t(16), max(uint64_t(1), table[kTableWords * L + 2] >> 12)));
+  shared_nodes(
+      a.full_q[a.cls], a.full_n[a.cls], st, a.work_counter, a.error, [&](const Node&) { return cap; },
+      [&](const Node& nd) {
+        if (threadIdx.x < L) x[threadIdx.x] = a.keys[nd.depth & 1][nd.start + threadIdx.x];
+      },
+      [&](const Node& nd, uint32_t idx) {
+        fifo_search<L>(x, nd.depth & kDepthMask, spl, stall, limit, &st.best[idx], &st.next[idx], a.error, lane,
+                       reinterpret_cast<const uint16_t*>(lut), fifo[warp], fifo[warp] + kFifoA,
+                       a.exec_count ? &wexec[warp] : nullptr);
+      },
+      [&](const Node& nd, uint64_t found) {
+        if (threadIdx.x == 0) {
+          a.seeds[nd.slot] = found;
+          a.sizes[nd.slot] = L;
+        }
+      });
+  if (a.exec_count && lane == 0 && wexec[warp]) atomicAdd(a.exec_count, wexec[warp]);
 }
 
 // ---------------------------------------------------------------- packed leaves
@@ -1555,27 +1696,43 @@ int launch_leaf_kernel(const SearchArgs& a, const recsplit_tuning_t& t, int sm_c
 }
 
 template <int L>
-int launch_full(const SearchArgs& a, const recsplit_tuning_t& t, int sm, cudaStream_t s) {
-  if constexpr (L >= 4 && L <= kPackedLeaf) {
-    auto kern = k_leaves_packed<L>;
-    int blocks = 0;
-    int rc = persistent_grid(kern, 0, sm, &blocks);
-    if (rc) return rc;
-    // (the queue's capacity, keys / L + 1, bounds the leaves; with fewer than
-    // one per four warps the two-phase kernel puts several warps on each)
-    if (t.leaf_two_phase && t.leaf_warps == 1 && uint64_t(a.full_cap[a.cls]) * 4 > uint64_t(blocks) * kWarps) {
+int launch_full(const SearchArgs& a, const recsplit_tuning_t& t, int sm, cudaStream_t s, const SharedNodes* share) {
+  if constexpr (L >= kFifoLeaf) {
+    if (t.leaf_two_phase && share) {
+      auto kern = k_leaves_shared<L>;
+      int blocks = 0;
+      int rc = persistent_grid(kern, 0, sm, &blocks);
+      if (rc) return rc;
+      blocks = std::min<int>(blocks, kSharedCtas);
       RS_CUDA(cudaMemsetAsync(a.work_counter, 0, sizeof(uint32_t), s));
-      kern<<<blocks, kThreads, 0, s>>>(a, t.leaf_chunk, t.leaf_seeds_per_lane);
+      kern<<<blocks, kThreads, 0, s>>>(a, *share, t.leaf_seeds_per_lane);
       count_launch();
       RS_CUDA(cudaGetLastError());
       return RECSPLIT_OK;
     }
+    return launch_leaf_kernel<L, true, false>(a, t, sm, s);
+  } else {
+    if constexpr (L >= 4 && L <= kPackedLeaf) {
+      auto kern = k_leaves_packed<L>;
+      int blocks = 0;
+      int rc = persistent_grid(kern, 0, sm, &blocks);
+      if (rc) return rc;
+      // (the queue's capacity, keys / L + 1, bounds the leaves; with fewer than
+      // one per four warps the two-phase kernel puts several warps on each)
+      if (t.leaf_two_phase && t.leaf_warps == 1 && uint64_t(a.full_cap[a.cls]) * 4 > uint64_t(blocks) * kWarps) {
+        RS_CUDA(cudaMemsetAsync(a.work_counter, 0, sizeof(uint32_t), s));
+        kern<<<blocks, kThreads, 0, s>>>(a, t.leaf_chunk, t.leaf_seeds_per_lane);
+        count_launch();
+        RS_CUDA(cudaGetLastError());
+        return RECSPLIT_OK;
+      }
+    }
+    if (t.leaf_two_phase) return launch_leaf_kernel<L, true, true>(a, t, sm, s);
+    return launch_leaf_kernel<L, true, false>(a, t, sm, s);
   }
-  if (t.leaf_two_phase) return launch_leaf_kernel<L, true, true>(a, t, sm, s);
-  return launch_leaf_kernel<L, true, false>(a, t, sm, s);
 }
 
-typedef int (*FullLauncher)(const SearchArgs&, const recsplit_tuning_t&, int, cudaStream_t);
+typedef int (*FullLauncher)(const SearchArgs&, const recsplit_tuning_t&, int, cudaStream_t, const SharedNodes*);
 constexpr FullLauncher kFull[25] = {
     nullptr,         nullptr,         launch_full<2>,  launch_full<3>,  launch_full<4>,
     launch_full<5>,  launch_full<6>,  launch_full<7>,  launch_full<8>,  launch_full<9>,
@@ -1667,7 +1824,12 @@ int launch_split_level(const SearchArgs& a, uint64_t max_m, uint32_t max_leaf, i
   return RECSPLIT_OK;
 }
 
-int launch_leaves(const SearchArgs& a, uint32_t leaf, uint32_t extra, int sm_count, cudaStream_t s) {
+bool leaves_shared(uint32_t leaf, uint32_t extra) {
+  return !extra && leaf >= uint32_t(kFifoLeaf) && tuning_for(leaf).leaf_two_phase;
+}
+
+int launch_leaves(const SearchArgs& a, uint32_t leaf, uint32_t extra, int sm_count, cudaStream_t s,
+                  const SharedNodes* share) {
   if (leaf < 2) return RECSPLIT_OK;
   const recsplit_tuning_t t = tuning_for(leaf);
   if (extra) {
@@ -1681,7 +1843,7 @@ int launch_leaves(const SearchArgs& a, uint32_t leaf, uint32_t extra, int sm_cou
     }
     return RECSPLIT_OK;
   }
-  int rc = kFull[leaf](a, t, sm_count, s);
+  int rc = kFull[leaf](a, t, sm_count, s, share);
   if (rc) return rc;
   if (leaf == 2) return RECSPLIT_OK;  // no leaves between 2 and leaf - 1
   if (leaf <= 8) return launch_leaf_kernel<8, false>(a, t, sm_count, s);
