@@ -12,7 +12,10 @@
 // result is deterministic and independent of G).  Nodes are handed out by an
 // atomic counter (persistent CTAs), the heaviest levels with larger groups.
 #include <algorithm>
+#include <array>
+#include <climits>
 #include <mutex>
+#include <utility>
 
 #include "device.cuh"
 
@@ -1191,49 +1194,123 @@ __device__ __forceinline__ uint64_t fifo_pump(const uint64_t* x, uint2* a, uint3
   return fifo_index(low, newest);
 }
 
-// Leaf of m < LMAX keys: slots j >= m contribute nothing.
-template <int LMAX>
-__device__ __forceinline__ bool leaf_trial_part(const uint64_t (&x)[LMAX], const uint32_t (&keep)[LMAX], uint32_t m,
-                                                uint64_t kp) {
-  uint32_t seen = 0;
-#pragma unroll
-  for (int j = 0; j < LMAX; j++) seen += (1u << phi_pre(x[j], kp, m)) & keep[j];
-  return seen == (1u << m) - 1;
-}
-
 // Blocks per SM the register budget must allow (keys live in registers).
 __host__ __device__ constexpr int leaf_min_blocks(int l) { return l <= 5 ? 5 : (l <= 12 ? 4 : 3); }
 
-// Leaf of m <= LMAX keys of the perfect, non-minimal variant: the values in
-// [0, m + extra) must be distinct, i.e. the sum of the kept one-hot values
-// must have m one bits (a sum of powers of two loses one bits on every
+// Leaf of M keys of the perfect, non-minimal variant: the values in [0, range),
+// range = M + extra, must be distinct, i.e. the sum of the one-hot values
+// must have M one bits (a sum of powers of two loses one bits on every
 // carry, and a carry out of bit 31 only lowers the count further).
-template <int LMAX>
-__device__ __forceinline__ bool leaf_trial_range(const uint64_t (&x)[LMAX], const uint32_t (&keep)[LMAX], uint32_t m,
-                                                 uint32_t range, uint64_t kp) {
+template <int M>
+__device__ __forceinline__ bool leaf_trial_range(const uint64_t (&x)[M], uint32_t range, uint64_t kp) {
   uint32_t seen = 0;
 #pragma unroll
-  for (int j = 0; j < LMAX; j++) seen += (1u << phi_pre(x[j], kp, range)) & keep[j];
-  return static_cast<uint32_t>(__popc(seen)) == m;
+  for (int j = 0; j < M; j++) seen += 1u << phi_pre(x[j], kp, range);
+  return __popc(seen) == M;
 }
 
-// RANGE: perfect, non-minimal variant (leaf range m + extra of the class);
-// the queue is then the class's full leaves if qfull, else its partial ones.
-template <int LMAX, bool FULL, bool TWO, bool RANGE = false>
-__global__ void __launch_bounds__(kThreads, leaf_min_blocks(LMAX)) k_leaves(SearchArgs a, uint32_t gwarps,
-                                                                            uint32_t chunk, uint32_t spl,
-                                                                            uint32_t qfull) {
+// Search of one leaf of M keys by a group of gwarps warps (this is warp wig):
+// lowers *best (shared memory, ~0 on entry) to the first successful index.
+enum LeafTest { kOnePhase, kTwoPhases, kRangeTest };
+
+template <int M, LeafTest TEST>
+__device__ __forceinline__ void search_leaf(const uint64_t* __restrict__ src, uint32_t depth,
+                                            const uint64_t* table, uint32_t range, uint32_t spl, uint32_t wig,
+                                            uint32_t gwarps, uint32_t lane, uint64_t* best, uint4* surv, int* err,
+                                            unsigned long long* exec) {
+  uint64_t x[M];
+#pragma unroll
+  for (int j = 0; j < M; j++) x[j] = __ldg(src + j);
+  const uint64_t stall = stall_threshold(table, M);
+  const uint64_t limit = trial_limit(table, M);
+  const uint64_t dkey = uint64_t(depth) * kWeyl;
+  uint32_t rounds = 0;
+  // a round of a warp covers the spl * 32 indices from base; lane L tests
+  // base + j * 32 + L for j < spl
+  const uint64_t span = uint64_t(spl) * 32;
+  // one compare per round: the stall point until it is checked, then the limit
+  for (uint64_t base = uint64_t(wig) * span, next_check = min(stall, limit);; base += uint64_t(gwarps) * span) {
+    if (gwarps > 1 && __any_sync(0xFFFFFFFFu, base >= volatile_load(best))) break;
+    if ((++rounds & 255) == 0 && __shfl_sync(0xFFFFFFFFu, lane == 0 ? *reinterpret_cast<volatile int*>(err) : 0, 0))
+      break;  // another search failed, or the host cancelled the build
+    if (base >= next_check) {
+      if (base >= limit) {
+        if (lane == 0) {
+          set_error(err, RECSPLIT_E_SEARCH_LIMIT);
+          atomicMin(reinterpret_cast<unsigned long long*>(best), 0ull);
+        }
+        break;
+      }
+      next_check = limit;
+      bool dup = false;
+#pragma unroll
+      for (int i = 0; i < M; i++)
+#pragma unroll
+        for (int j = i + 1; j < M; j++) dup |= x[i] == x[j];
+      if (dup) {
+        if (lane == 0) {
+          set_error(err, RECSPLIT_E_DUPLICATE);
+          atomicMin(reinterpret_cast<unsigned long long*>(best), 0ull);
+        }
+        break;
+      }
+    }
+    uint64_t found = ~0ull;
+    if constexpr (TEST == kTwoPhases) {
+      found = leaf_round_two_phase<M>(x, base, dkey, spl, lane, surv, exec);
+    } else {
+      uint64_t k = index_key(base + lane, dkey);
+      for (uint32_t j = 0; j < spl; j++, k += kLaneStep) {
+        const uint64_t kp = k ^ (k >> 30);
+        const bool ok = TEST == kRangeTest ? leaf_trial_range<M>(x, range, kp) : leaf_trial_full<M>(x, kp);
+        const uint32_t hits = __ballot_sync(0xFFFFFFFFu, ok);
+        if (hits && found == ~0ull) found = base + j * 32 + __ffs(hits) - 1;
+      }
+      if (exec && lane == 0) *exec += spl * 32 * M;
+    }
+    if (found != ~0ull) {
+      if (lane == 0) atomicMin(reinterpret_cast<unsigned long long*>(best), found);
+      break;
+    }
+  }
+}
+
+// Leaf of m keys, 2 <= m <= LMAX, by the search for exactly m keys (a search
+// over LMAX masked slots evaluates LMAX keys whatever m is: the partial leaves
+// of 2 to 11 keys at l = 12 took 1.87 ms of a batched build so, in 16 slots).
+// From 6 keys on the two-phase test, with the indices per lane that its trial
+// count calls for.
+template <int M, int LMAX, bool RANGE>
+__device__ __forceinline__ void search_leaf_of(uint32_t m, const uint64_t* __restrict__ src, uint32_t depth,
+                                               const uint64_t* table, uint32_t range, uint32_t wig, uint32_t gwarps,
+                                               uint32_t lane, uint64_t* best, uint4* surv, int* err,
+                                               unsigned long long* exec) {
+  if (m == M) {
+    constexpr LeafTest test = RANGE ? kRangeTest : (M >= 6 ? kTwoPhases : kOnePhase);
+    constexpr uint32_t spl = RANGE || M < 6 ? 1 : (M == 6 ? 2 : (M < 9 ? 4 : 8));
+    search_leaf<M, test>(src, depth, table, range, spl, wig, gwarps, lane, best, surv, err, exec);
+  } else if constexpr (M < LMAX) {
+    search_leaf_of<M + 1, LMAX, RANGE>(m, src, depth, table, range, wig, gwarps, lane, best, surv, err, exec);
+  }
+}
+
+// Full leaves of L keys (PART false), or leaves of 2 to L keys of the class's
+// full (qfull) or partial queue.  RANGE: perfect, non-minimal variant (leaf
+// range m + extra of the class).
+template <int L, bool PART, bool TWO, bool RANGE = false>
+__global__ void __launch_bounds__(kThreads, leaf_min_blocks(L)) k_leaves(SearchArgs a, uint32_t gwarps,
+                                                                         uint32_t chunk, uint32_t spl,
+                                                                         uint32_t qfull) {
   __shared__ uint64_t best[kWarps];
   __shared__ uint32_t task[kWarps];
   __shared__ unsigned long long wexec[kWarps];  // work counting: evaluations per warp, flushed at exit
-  constexpr bool kTwoPhase = FULL && TWO && LMAX >= 4;
-  __shared__ uint4 surv[kTwoPhase ? kWarps : 1][kTwoPhase ? 32 * kMaxSpl : 1];  // one round's survivors
+  constexpr bool kSurvivors = PART ? !RANGE && L >= 6 : TWO && L >= 4;
+  __shared__ uint4 surv[kSurvivors ? kWarps : 1][kSurvivors ? 32 * kMaxSpl : 1];  // one round's survivors
   const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   unsigned long long* const exec = a.exec_count ? &wexec[warp] : nullptr;
   if (lane == 0) wexec[warp] = 0;
-  const bool from_full = FULL || (RANGE && qfull);
-  const Node* queue = from_full ? a.full_q[a.cls] : a.part_q[a.cls];
-  const uint32_t total = from_full ? a.full_n[a.cls] : a.part_n[a.cls];
+  const Node* queue = !PART || qfull ? a.full_q[a.cls] : a.part_q[a.cls];
+  const uint32_t total = !PART || qfull ? a.full_n[a.cls] : a.part_n[a.cls];
   gwarps = group_warps(gwarps, total);
   const uint32_t groups = gridDim.x * (kWarps / gwarps);
   chunk = min(chunk, max(1u, total / (2 * groups)));
@@ -1241,6 +1318,7 @@ __global__ void __launch_bounds__(kThreads, leaf_min_blocks(LMAX)) k_leaves(Sear
   const bool leader = wig == 0 && lane == 0;
   const uint32_t extra = RANGE ? a.extra_of[a.cls] : 0;
   const uint64_t* table = a.table[a.cls];
+  uint4* const mine = surv[kSurvivors ? warp : 0];
 
   for (;;) {
     if (leader) task[gid] = *reinterpret_cast<volatile int*>(a.error) ? total : atomicAdd(a.work_counter, chunk);
@@ -1250,79 +1328,20 @@ __global__ void __launch_bounds__(kThreads, leaf_min_blocks(LMAX)) k_leaves(Sear
     const uint32_t last = min(total, first + chunk);
     for (uint32_t idx = first; idx < last; idx++) {
       const Node nd = queue[idx];
-      const uint32_t m = FULL ? LMAX : nd.m;
       const uint32_t depth = nd.depth & kDepthMask;
       const uint64_t* src = a.keys[depth & 1] + nd.start;
-      uint64_t x[LMAX];
-      uint32_t keep[LMAX];
-#pragma unroll
-      for (int j = 0; j < LMAX; j++) {
-        x[j] = (FULL || uint32_t(j) < m) ? __ldg(src + j) : 0;
-        keep[j] = (FULL || uint32_t(j) < m) ? ~0u : 0u;
-      }
       if (leader) best[gid] = ~0ull;
       group_sync(gid, gwarps);
-      const uint64_t stall = stall_threshold(table, m);
-      const uint64_t limit = trial_limit(table, m);
-      const uint64_t dkey = uint64_t(depth) * kWeyl;
-      bool checked = false;
-      uint32_t rounds = 0;
-      // a round of a warp covers the spl * 32 indices from base; lane L tests
-      // base + j * 32 + L for j < spl
-      const uint64_t span = uint64_t(spl) * 32;
-      // one compare per round: the stall point until it is checked, then the limit
-      for (uint64_t base = uint64_t(wig) * span, next_check = min(stall, limit);; base += uint64_t(gwarps) * span) {
-        if (gwarps > 1 && __any_sync(0xFFFFFFFFu, base >= volatile_load(&best[gid]))) break;
-        if ((++rounds & 255) == 0 &&
-            __shfl_sync(0xFFFFFFFFu, lane == 0 ? *reinterpret_cast<volatile int*>(a.error) : 0, 0))
-          break;  // another search failed, or the host cancelled the build
-        if (base >= next_check) {
-          if (base >= limit) {
-            if (lane == 0) {
-              set_error(a.error, RECSPLIT_E_SEARCH_LIMIT);
-              atomicMin(reinterpret_cast<unsigned long long*>(&best[gid]), 0ull);
-            }
-            break;
-          }
-          next_check = limit;
-          bool dup = false;
-#pragma unroll
-          for (int i = 0; i < LMAX; i++)
-#pragma unroll
-            for (int j = i + 1; j < LMAX; j++) dup |= keep[j] && x[i] == x[j];
-          if (dup) {
-            if (lane == 0) {
-              set_error(a.error, RECSPLIT_E_DUPLICATE);
-              atomicMin(reinterpret_cast<unsigned long long*>(&best[gid]), 0ull);
-            }
-            break;
-          }
-        }
-        uint64_t found = ~0ull;
-        if (kTwoPhase) {
-          found = leaf_round_two_phase<LMAX>(x, base, dkey, spl, lane, surv[warp], exec);
-        } else {
-          uint64_t k = index_key(base + lane, dkey);
-          for (uint32_t j = 0; j < spl; j++, k += kLaneStep) {
-            const uint64_t kp = k ^ (k >> 30);
-            const bool ok = RANGE  ? leaf_trial_range<LMAX>(x, keep, m, m + extra, kp)
-                            : FULL ? leaf_trial_full<LMAX>(x, kp)
-                                   : leaf_trial_part<LMAX>(x, keep, m, kp);
-            const uint32_t hits = __ballot_sync(0xFFFFFFFFu, ok);
-            if (hits && found == ~0ull) found = base + j * 32 + __ffs(hits) - 1;
-          }
-          // every slot of the kernel's LMAX is evaluated (masked beyond m)
-          if (exec && lane == 0) *exec += spl * 32 * LMAX;
-        }
-        if (found != ~0ull) {
-          if (lane == 0) atomicMin(reinterpret_cast<unsigned long long*>(&best[gid]), found);
-          break;
-        }
-      }
+      if constexpr (PART)
+        search_leaf_of<2, L, RANGE>(nd.m, src, depth, table, nd.m + extra, wig, gwarps, lane, &best[gid], mine,
+                                    a.error, exec);
+      else
+        search_leaf<L, TWO && L >= 4 ? kTwoPhases : kOnePhase>(src, depth, table, L, spl, wig, gwarps, lane,
+                                                               &best[gid], mine, a.error, exec);
       group_sync(gid, gwarps);
       if (leader) {
         a.seeds[nd.slot] = best[gid];
-        a.sizes[nd.slot] = m;
+        a.sizes[nd.slot] = nd.m;
       }
       group_sync(gid, gwarps);
     }
@@ -1495,21 +1514,26 @@ __device__ __forceinline__ bool leaf_head(const uint64_t (&x)[L], uint64_t kp, c
   }
 }
 
-template <int L>
+// RANGE: perfect, non-minimal variant (range L + extra of the class).  Its
+// leaves, and bijections of at most 5 keys, take a few dozen trials: one phase.
+template <int L, bool RANGE>
 __global__ void __launch_bounds__(kThreads, 4) k_leaves_packed(SearchArgs a, uint32_t chunk, uint32_t spl) {
-  constexpr int H = leaf_first_part(L);
+  constexpr bool kOne = RANGE || L <= 5;
+  constexpr int H = kOne ? L : leaf_first_part(L);
+  constexpr bool kLut = L == 8 && !RANGE;
   constexpr uint32_t full = (1u << L) - 1;
   constexpr uint32_t kAll = 0xFFFFFFFFu;
   __shared__ uint64_t skeys[kWarps][kPackedSlots][L];
   __shared__ uint64_t sdkey[kWarps][kPackedSlots];
   __shared__ uint32_t sbase[kWarps][kPackedSlots], sbest[kWarps][kPackedSlots];
-  __shared__ uint2 surv[kWarps][32 * kMaxSpl];  // {index, set of the first values | slot << 16}
-  __shared__ uint32_t lut[L == 8 ? 1024 : 1];
+  __shared__ uint2 surv[kOne ? 1 : kWarps][kOne ? 1 : 32 * kMaxSpl];  // {index, set of the first values | slot << 16}
+  __shared__ uint32_t lut[kLut ? 1024 : 1];
   const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t total = a.full_n[a.cls];
-  if (L == 8) fill_octal_sets(lut);
+  if (kLut) fill_octal_sets(lut);
   __syncthreads();
   const Node* queue = a.full_q[a.cls];
+  const uint32_t range = L + (RANGE ? a.extra_of[a.cls] : 0);
   const uint32_t below = (1u << lane) - 1;
   const uint32_t nwarps = gridDim.x * kWarps;
   const uint32_t slots = total >= kPackedSlots * nwarps ? kPackedSlots : (total >= 2 * nwarps ? 2 : 1);
@@ -1607,15 +1631,22 @@ __global__ void __launch_bounds__(kThreads, 4) k_leaves_packed(SearchArgs a, uin
       uint64_t key = index_key(idx, dkey);
 #pragma unroll 2
       for (uint32_t j = 0; j < spl; j++, key += step, idx += lanes) {
-        uint32_t seen;
-        const bool ok = leaf_head<L, H>(x, key ^ (key >> 30), reinterpret_cast<const uint8_t*>(lut), seen);
-        const uint32_t b = __ballot_sync(kAll, ok);
-        if (ok) surv[warp][ns + __popc(b & below)] = make_uint2(idx, seen | tag);
-        ns += __popc(b);
+        if constexpr (kOne) {
+          const uint64_t kp = key ^ (key >> 30);
+          const bool ok = RANGE ? leaf_trial_range<L>(x, range, kp) : leaf_trial_full<L>(x, kp);
+          if (ok) atomicMin(&sbest[warp][mine], idx);
+          won |= __any_sync(kAll, ok);
+        } else {
+          uint32_t seen;
+          const bool ok = leaf_head<L, H>(x, key ^ (key >> 30), reinterpret_cast<const uint8_t*>(lut), seen);
+          const uint32_t b = __ballot_sync(kAll, ok);
+          if (ok) surv[warp][ns + __popc(b & below)] = make_uint2(idx, seen | tag);
+          ns += __popc(b);
+        }
       }
       base += lanes * spl;
       __syncwarp();
-      for (uint32_t t0 = 0; t0 < ns; t0 += 32) {
+      for (uint32_t t0 = 0; !kOne && t0 < ns; t0 += 32) {
         const uint32_t t = t0 + lane;
         bool ok = false;
         if (t < ns) {
@@ -1681,64 +1712,74 @@ int persistent_grid(K kernel, size_t smem, int sm_count, int* blocks) {
   return RECSPLIT_OK;
 }
 
-template <int LMAX, bool FULL, bool TWO = false, bool RANGE = false>
-int launch_leaf_kernel(const SearchArgs& a, const recsplit_tuning_t& t, int sm_count, cudaStream_t s,
-                       uint32_t qfull = 0) {
-  auto kern = k_leaves<LMAX, FULL, TWO, RANGE>;
+template <typename K, typename... Args>
+int launch_persistent(K kern, int max_blocks, const SearchArgs& a, int sm_count, cudaStream_t s, Args... args) {
   int blocks = 0;
   int rc = persistent_grid(kern, 0, sm_count, &blocks);
   if (rc) return rc;
   RS_CUDA(cudaMemsetAsync(a.work_counter, 0, sizeof(uint32_t), s));
-  kern<<<blocks, kThreads, 0, s>>>(a, t.leaf_warps, t.leaf_chunk, t.leaf_seeds_per_lane, qfull);
+  kern<<<std::min(blocks, max_blocks), kThreads, 0, s>>>(a, args...);
   count_launch();
   RS_CUDA(cudaGetLastError());
   return RECSPLIT_OK;
 }
 
+// Leaves of 2 to L keys of a queue, each by the search for its size.
+template <int L, bool RANGE>
+int launch_any(const SearchArgs& a, const recsplit_tuning_t& t, int sm, cudaStream_t s, uint32_t qfull) {
+  return launch_persistent(k_leaves<L, true, false, RANGE>, INT_MAX, a, sm, s, t.leaf_warps, t.leaf_chunk, 1u, qfull);
+}
+
+// Whether the packed kernel takes the class's full leaves of L keys.  The
+// queue's capacity (keys / L + 1) bounds the leaves; with fewer than one per
+// four warps of the grid (about four CTAs per SM) the two-phase kernel puts
+// several warps on each.
+template <int L>
+bool packed_leaves(const SearchArgs& a, const recsplit_tuning_t& t, int sm) {
+  return L >= 4 && L <= kPackedLeaf && t.leaf_two_phase && t.leaf_warps == 1 &&
+         uint64_t(a.full_cap[a.cls]) > uint64_t(sm) * kWarps;
+}
+
 template <int L>
 int launch_full(const SearchArgs& a, const recsplit_tuning_t& t, int sm, cudaStream_t s, const SharedNodes* share) {
   if constexpr (L >= kFifoLeaf) {
-    if (t.leaf_two_phase && share) {
-      auto kern = k_leaves_shared<L>;
-      int blocks = 0;
-      int rc = persistent_grid(kern, 0, sm, &blocks);
-      if (rc) return rc;
-      blocks = std::min<int>(blocks, kSharedCtas);
-      RS_CUDA(cudaMemsetAsync(a.work_counter, 0, sizeof(uint32_t), s));
-      kern<<<blocks, kThreads, 0, s>>>(a, *share, t.leaf_seeds_per_lane);
-      count_launch();
-      RS_CUDA(cudaGetLastError());
-      return RECSPLIT_OK;
-    }
-    return launch_leaf_kernel<L, true, false>(a, t, sm, s);
+    if (t.leaf_two_phase && share)
+      return launch_persistent(k_leaves_shared<L>, int(kSharedCtas), a, sm, s, *share, t.leaf_seeds_per_lane);
   } else {
-    if constexpr (L >= 4 && L <= kPackedLeaf) {
-      auto kern = k_leaves_packed<L>;
-      int blocks = 0;
-      int rc = persistent_grid(kern, 0, sm, &blocks);
-      if (rc) return rc;
-      // (the queue's capacity, keys / L + 1, bounds the leaves; with fewer than
-      // one per four warps the two-phase kernel puts several warps on each)
-      if (t.leaf_two_phase && t.leaf_warps == 1 && uint64_t(a.full_cap[a.cls]) * 4 > uint64_t(blocks) * kWarps) {
-        RS_CUDA(cudaMemsetAsync(a.work_counter, 0, sizeof(uint32_t), s));
-        kern<<<blocks, kThreads, 0, s>>>(a, t.leaf_chunk, t.leaf_seeds_per_lane);
-        count_launch();
-        RS_CUDA(cudaGetLastError());
-        return RECSPLIT_OK;
-      }
-    }
-    if (t.leaf_two_phase) return launch_leaf_kernel<L, true, true>(a, t, sm, s);
-    return launch_leaf_kernel<L, true, false>(a, t, sm, s);
+    if constexpr (L >= 4 && L <= kPackedLeaf)
+      if (packed_leaves<L>(a, t, sm))
+        return launch_persistent(k_leaves_packed<L, false>, INT_MAX, a, sm, s, t.leaf_chunk, t.leaf_seeds_per_lane);
+    if (t.leaf_two_phase)
+      return launch_persistent(k_leaves<L, false, true>, INT_MAX, a, sm, s, t.leaf_warps, t.leaf_chunk,
+                               t.leaf_seeds_per_lane, 1u);
   }
+  return launch_persistent(k_leaves<L, false, false>, INT_MAX, a, sm, s, t.leaf_warps, t.leaf_chunk,
+                           t.leaf_seeds_per_lane, 1u);
+}
+
+// Full leaves of the perfect, non-minimal variant.
+template <int L>
+int launch_full_range(const SearchArgs& a, const recsplit_tuning_t& t, int sm, cudaStream_t s, const SharedNodes*) {
+  if constexpr (L >= 4 && L <= kPackedLeaf)
+    if (packed_leaves<L>(a, t, sm))
+      return launch_persistent(k_leaves_packed<L, true>, INT_MAX, a, sm, s, t.leaf_chunk, 1u);
+  if (L <= 8) return launch_any<8, true>(a, t, sm, s, 1);
+  if (L <= 16) return launch_any<16, true>(a, t, sm, s, 1);
+  return launch_any<24, true>(a, t, sm, s, 1);
 }
 
 typedef int (*FullLauncher)(const SearchArgs&, const recsplit_tuning_t&, int, cudaStream_t, const SharedNodes*);
-constexpr FullLauncher kFull[25] = {
-    nullptr,         nullptr,         launch_full<2>,  launch_full<3>,  launch_full<4>,
-    launch_full<5>,  launch_full<6>,  launch_full<7>,  launch_full<8>,  launch_full<9>,
-    launch_full<10>, launch_full<11>, launch_full<12>, launch_full<13>, launch_full<14>,
-    launch_full<15>, launch_full<16>, launch_full<17>, launch_full<18>, launch_full<19>,
-    launch_full<20>, launch_full<21>, launch_full<22>, launch_full<23>, launch_full<24>};
+template <size_t... L>
+constexpr auto full_launchers(std::index_sequence<L...>) {
+  return std::array<FullLauncher, sizeof...(L) + 2>{nullptr, nullptr, launch_full<int(L) + 2>...};
+}
+template <size_t... L>
+constexpr auto range_launchers(std::index_sequence<L...>) {
+  return std::array<FullLauncher, sizeof...(L) + 2>{nullptr, nullptr, launch_full_range<int(L) + 2>...};
+}
+// by leaf size 2 .. kMaxLeaf
+constexpr auto kFull = full_launchers(std::make_index_sequence<kMaxLeaf - 1>{});
+constexpr auto kFullRange = range_launchers(std::make_index_sequence<kMaxLeaf - 1>{});
 
 }  // namespace
 
@@ -1832,23 +1873,16 @@ int launch_leaves(const SearchArgs& a, uint32_t leaf, uint32_t extra, int sm_cou
                   const SharedNodes* share) {
   if (leaf < 2) return RECSPLIT_OK;
   const recsplit_tuning_t t = tuning_for(leaf);
-  if (extra) {
-    // perfect, non-minimal variant: the full and the partial leaves, each
-    // searched over [0, m + extra) by the kernel for leaves of up to LMAX keys
-    for (uint32_t qfull : {1u, 0u}) {
-      const int rc = leaf <= 8    ? launch_leaf_kernel<8, false, false, true>(a, t, sm_count, s, qfull)
-                     : leaf <= 16 ? launch_leaf_kernel<16, false, false, true>(a, t, sm_count, s, qfull)
-                                  : launch_leaf_kernel<24, false, false, true>(a, t, sm_count, s, qfull);
-      if (rc) return rc;
-    }
-    return RECSPLIT_OK;
-  }
-  int rc = kFull[leaf](a, t, sm_count, s, share);
-  if (rc) return rc;
-  if (leaf == 2) return RECSPLIT_OK;  // no leaves between 2 and leaf - 1
-  if (leaf <= 8) return launch_leaf_kernel<8, false>(a, t, sm_count, s);
-  if (leaf <= 16) return launch_leaf_kernel<16, false>(a, t, sm_count, s);
-  return launch_leaf_kernel<24, false>(a, t, sm_count, s);
+  int rc = (extra ? kFullRange : kFull)[leaf](a, t, sm_count, s, share);
+  if (rc || leaf == 2) return rc;  // no leaves between 2 and leaf - 1
+  if (extra)
+    return leaf <= 8    ? launch_any<8, true>(a, t, sm_count, s, 0)
+           : leaf <= 16 ? launch_any<16, true>(a, t, sm_count, s, 0)
+                        : launch_any<24, true>(a, t, sm_count, s, 0);
+  return leaf <= 8    ? launch_any<8, false>(a, t, sm_count, s, 0)
+         : leaf <= 12 ? launch_any<12, false>(a, t, sm_count, s, 0)
+         : leaf <= 16 ? launch_any<16, false>(a, t, sm_count, s, 0)
+                      : launch_any<24, false>(a, t, sm_count, s, 0);
 }
 
 }  // namespace rs
