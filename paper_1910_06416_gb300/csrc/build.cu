@@ -761,9 +761,15 @@ int build_sets(const SetInput* in, uint32_t count, const BuildOptions& opt, cuda
   }
 
   // Level plan: the largest node of every split level, and whether the
-  // level's nodes are heavy enough to be searched shared (a node's expected
-  // trials x keys of at least 2^21 evaluations: a level of such nodes ends
-  // on a few long geometric searches)
+  // level is searched shared.  That costs a few microseconds of CTA-wide steps
+  // per node and removes the level's tail, a few long geometric searches on an
+  // idle device, so it pays where a node's expected trials x keys reach 2^21
+  // evaluations, or 2^16 on a level of fewer than 8 nodes per warp of the device.
+  // Split phase without and with the second clause: l = 12, b = 100: 10^5 keys
+  // 0.84 -> 0.39 ms, 10^6 keys 2.29 -> 1.81 ms (5 * 10^6 keys, above the line: 7.1
+  // against 8.2 ms); l = 13, b = 100, 3 * 10^5 keys 12.6 -> 6.6 ms; l = 12, b = 2000,
+  // 3 * 10^5 keys 4.7 -> 2.8 ms; l = 11, b = 100, 3 * 10^5 keys 1.30 -> 0.69 ms (3 * 10^6
+  // keys: 4.5 against 5.0 ms).
   std::vector<uint64_t> plan_mx;
   std::vector<char> plan_share;
   {
@@ -778,7 +784,8 @@ int build_sets(const SetInput* in, uint32_t count, const BuildOptions& opt, cuda
         }
       if (mx == 0 || plan_mx.size() > kMaxDepth + 1) break;
       plan_mx.push_back(mx);
-      plan_share.push_back(heavy >= double(1 << 21));
+      const bool few = K / mx <= 8ull * 32 * sm_count;
+      plan_share.push_back(heavy >= double(few ? 1 << 16 : 1 << 21));
       for (uint32_t c = 0; c < nclass; c++)
         lm[c] = lm[c] > class_leaf[c] ? next_level_max(make_strategy(class_leaf[c]), lm[c]) : 0;
     }
@@ -821,9 +828,14 @@ int build_sets(const SetInput* in, uint32_t count, const BuildOptions& opt, cuda
   auto search_phase = [&]() -> int {
     int level = 0;
     for (;;) {
-      uint64_t mx = 0;
+      uint64_t mx = 0, trials = 0;
+      bool tables = false;  // nodes of five leaves or more, split in equal parts (leaf sizes from 11)
       for (uint32_t c = 0; c < nclass; c++)
-        if (level_max[c] > class_leaf[c]) mx = std::max(mx, level_max[c]);
+        if (level_max[c] > class_leaf[c]) {
+          mx = std::max(mx, level_max[c]);
+          trials = std::max(trials, T[c].expected_trials[level_max[c]]);
+          tables |= class_leaf[c] >= 11 && level_max[c] >= 5 * class_leaf[c];
+        }
       if (mx == 0) break;
       if (level > kMaxDepth) return fail(RECSPLIT_E_INVALID, "splitting tree deeper than 63 levels");
       const int cur = level & 1;
@@ -837,7 +849,7 @@ int build_sets(const SetInput* in, uint32_t count, const BuildOptions& opt, cuda
         RS_CUDA(cudaMemsetAsync(shared.flag, 0, split_cap * sizeof(unsigned int), ws));
         RS_CUDA(cudaMemsetAsync(shared.owned, 0xFF, kSharedCtas * sizeof(unsigned int), ws));
       }
-      int r = launch_split_level(a, mx, max_leaf, sm_count, ws, share ? &shared : nullptr);
+      int r = launch_split_level(a, mx, trials, max_leaf, tables, sm_count, ws, share ? &shared : nullptr);
       if (r) return r;
       for (uint32_t c = 0; c < nclass; c++)
         level_max[c] = level_max[c] > class_leaf[c] ? next_level_max(make_strategy(class_leaf[c]), level_max[c]) : 0;

@@ -281,8 +281,11 @@ constexpr uint32_t kSharedCtas = 4096;
 
 // share: null for the one-group-per-node search; else the level is searched
 // with nodes shared by the CTAs that find the queue empty (st zeroed as above)
-int launch_split_level(const SearchArgs& a, uint64_t max_m, uint32_t max_leaf, int sm_count, cudaStream_t s,
-                       const SharedNodes* share = nullptr);
+// tables: the level may hold nodes of five to seven equal parts, which are
+// counted by table; trials: the most that a node of the level is expected to
+// take
+int launch_split_level(const SearchArgs& a, uint64_t max_m, uint64_t trials, uint32_t max_leaf, bool tables,
+                       int sm_count, cudaStream_t s, const SharedNodes* share = nullptr);
 // Whether the full leaves of a class are searched shared (launch_leaves then
 // needs share, zeroed as above).
 bool leaves_shared(uint32_t leaf, uint32_t extra);

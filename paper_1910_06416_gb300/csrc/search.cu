@@ -89,8 +89,38 @@ struct SplitParams {
   uint32_t thr1, thr2;      // T_1, T_2 (threshold modes)
   uint32_t nbits, nmask, ntarget;  // narrow fields (modes 5, 7): 2^nbits > unit
   bool confirm;                    // mode 7: fields can overflow, confirm matches exactly
-  uint32_t tail;                   // modes 8..11 on shared nodes: keys of the second phase (0: one phase)
+  const uint32_t* sets;            // modes 8, 9: packed counts of four parts (fill_part_counts)
+  uint32_t tail;                   // modes 8, 9 on shared nodes: keys of the second phase
 };
+
+// Modes 8 and 9: F = 5 .. 7 equal parts (m = F unit).  The part of a key, 3
+// bits, is the top of floor(F 2^29 h / 2^32); the parts of four keys are
+// shifted into one 12-bit word (one funnel shift per key, where counting a
+// part takes a shift-and-add, a shift and an add), and a table of 4096 words in
+// shared memory gives their counts in fields: 6 fields of 5 bits (mode 8: unit <
+// 32) or 4 of 8 bits (mode 9: F = 5, unit < 256).  The last part is implied.
+constexpr uint32_t kPartCounts = 4096;
+
+__device__ __forceinline__ uint32_t part_one(uint32_t part, uint32_t bits, uint32_t fields) {
+  return part < fields ? 1u << (part * bits) : 0u;
+}
+
+// The two tables, 5-bit fields then 8-bit fields, from those of two parts
+// (called by the whole CTA).
+__device__ __forceinline__ void fill_part_counts(uint32_t* t) {
+  __shared__ uint32_t two[2][64];
+  if (threadIdx.x < 64) {
+    const uint32_t p = threadIdx.x & 7, q = threadIdx.x >> 3;
+    two[0][threadIdx.x] = part_one(p, 5, 6) + part_one(q, 5, 6);
+    two[1][threadIdx.x] = part_one(p, 8, 4) + part_one(q, 8, 4);
+  }
+  __syncthreads();
+  for (uint32_t i = threadIdx.x; i < kPartCounts; i += kThreads) {
+    t[i] = two[0][i >> 6] + two[0][i & 63];
+    t[kPartCounts + i] = two[1][i >> 6] + two[1][i & 63];
+  }
+  __syncthreads();
+}
 
 // MODE 0: 32-bit fields + magic; 1: 64-bit fields + magic; 2: 64-bit +
 // division; 3, 4: thresholds for fanout 2, 3;
@@ -103,7 +133,7 @@ struct SplitParams {
 // 7: F parts of equal size (m = F unit): the part is floor(F h / 2^32), one
 // multiply-high instead of two, counted in nbits-bit fields; when a field
 // can overflow (2^nbits <= m) a match is confirmed exactly as in mode 5.
-// 8..11: mode 7 with nbits = MODE - 3 (5..8) fixed at compile time.
+// 8, 9: mode 7 with fields of 5 and 8 bits by table (above).
 // Modes 3 and 4: c1 and c2 count the keys with h >= T_1 and h >= T_2, the carry
 // of h + (2^32 - T) added by add-with-carry.  These two additions issue to
 // either pipe (1.4 cycles per warp together); a compare and a predicated
@@ -125,22 +155,34 @@ __device__ __forceinline__ ulonglong2 key_pair(const uint64_t* keys) {
   return make_ulonglong2(keys[0], keys[1]);
 }
 
-// STAGED: the keys are in shared memory, 16-byte aligned: modes 3, 4 and 6
-// read them two at a time.
+// Fields of modes 8 and 9 of keys [j0, j1) under function kp, j0 even.
+template <int MODE, bool STAGED>
+__device__ __forceinline__ uint32_t split_fields(const uint64_t* __restrict__ keys, const SplitParams& p, uint64_t kp,
+                                                 uint32_t j0, uint32_t j1) {
+  constexpr uint32_t kBits = MODE == 8 ? 5 : 8, kFields = MODE == 8 ? 6 : 4;
+  const uint32_t scale = p.fanout << 29;
+  uint32_t acc = 0, j = j0;
+#pragma unroll 2
+  for (; j + 4 <= j1; j += 4) {
+    const ulonglong2 x = key_pair<STAGED>(keys + j), y = key_pair<STAGED>(keys + j + 2);
+    uint32_t v = __umulhi(family_top32(x.x, kp), scale) >> 29;
+    v = __funnelshift_l(__umulhi(family_top32(x.y, kp), scale), v, 3);
+    v = __funnelshift_l(__umulhi(family_top32(y.x, kp), scale), v, 3);
+    v = __funnelshift_l(__umulhi(family_top32(y.y, kp), scale), v, 3);
+    acc += p.sets[v];
+  }
+#pragma unroll 1
+  for (; j < j1; j++) acc += part_one(__umulhi(family_top32(keys[j], kp), p.fanout), kBits, kFields);
+  return acc;
+}
+
+// STAGED: the keys are in shared memory, 16-byte aligned: modes 3, 4, 6, 8 and
+// 9 read them two at a time.
 template <int MODE, bool STAGED>
 __device__ __forceinline__ bool split_trial(const uint64_t* __restrict__ keys, const SplitParams& p,
                                             uint64_t kp) {
-  if (MODE >= 8) {
-    // mode 7 with the field width fixed at compile time (5..8 bits): the
-    // field offset part * width is a shift-and-add on the ALU pipe instead of
-    // a multiply on the multiply-add pipe, which these nodes saturate (ncu,
-    // 560 -> 5 x 112 and 112 -> 7 x 16 at l = 16: multiply-add pipe 91% busy,
-    // ALU pipe 55%)
-    constexpr uint32_t NB = MODE - 3;
-    uint32_t acc = 0;
-#pragma unroll 4
-    for (uint32_t j = 0; j < p.m; j++) acc += shl32(1u, __umulhi(family_top32(keys[j], kp), p.fanout) * NB);
-    return (acc & p.nmask) == p.ntarget;
+  if constexpr (MODE >= 8) {
+    return (split_fields<MODE, STAGED>(keys, p, kp, 0, p.m) & p.nmask) == p.ntarget;
   } else if (MODE == 6) {
     // the two-bit parts are shifted into words of 16 keys (one funnel shift
     // per key, where counting fields takes four instructions), and the parts
@@ -321,25 +363,34 @@ __device__ __forceinline__ void split_search_few(const uint64_t* __restrict__ ke
   }
 }
 
+// A node too large to be staged (more than 1536 keys) has more keys than the
+// upper unit of any leaf size (1296 at l = 24), so it is split in two: modes 3
+// and 2 are all it needs.
 template <bool STAGED>
 __device__ __forceinline__ void split_search(const uint64_t* __restrict__ keys, const SplitParams& sp, int mode,
                                              uint32_t depth, uint32_t wig, uint32_t gwarps, uint32_t lane,
                                              uint64_t* best, uint64_t stall, uint64_t limit, int* err,
                                              unsigned long long* exec) {
-  if (stall <= uint64_t(sp.m) << 6) {  // stall = 64 times the expected trials
-    if (mode == 3) return split_search_few<3>(keys, sp, depth, wig, gwarps, lane, best, stall, limit, err, exec);
-    if (mode == 4) return split_search_few<4>(keys, sp, depth, wig, gwarps, lane, best, stall, limit, err, exec);
+  if (STAGED) {
+    if (stall <= uint64_t(sp.m) << 6) {  // stall = 64 times the expected trials
+      if (mode == 3) return split_search_few<3>(keys, sp, depth, wig, gwarps, lane, best, stall, limit, err, exec);
+      if (mode == 4) return split_search_few<4>(keys, sp, depth, wig, gwarps, lane, best, stall, limit, err, exec);
+    }
+    switch (mode) {
+      case 0: return split_search_warp<0, true>(keys, sp, depth, wig, gwarps, lane, best, stall, limit, err, exec);
+      case 1: return split_search_warp<1, true>(keys, sp, depth, wig, gwarps, lane, best, stall, limit, err, exec);
+      case 4: return split_search_warp<4, true>(keys, sp, depth, wig, gwarps, lane, best, stall, limit, err, exec);
+      case 5: return split_search_warp<5, true>(keys, sp, depth, wig, gwarps, lane, best, stall, limit, err, exec);
+      case 6: return split_search_warp<6, true>(keys, sp, depth, wig, gwarps, lane, best, stall, limit, err, exec);
+      case 7: return split_search_warp<7, true>(keys, sp, depth, wig, gwarps, lane, best, stall, limit, err, exec);
+      case 8: return split_search_warp<8, true>(keys, sp, depth, wig, gwarps, lane, best, stall, limit, err, exec);
+      case 9: return split_search_warp<9, true>(keys, sp, depth, wig, gwarps, lane, best, stall, limit, err, exec);
+    }
   }
-  switch (mode) {
-    case 0: split_search_warp<0, STAGED>(keys, sp, depth, wig, gwarps, lane, best, stall, limit, err, exec); break;
-    case 1: split_search_warp<1, STAGED>(keys, sp, depth, wig, gwarps, lane, best, stall, limit, err, exec); break;
-    case 3: split_search_warp<3, STAGED>(keys, sp, depth, wig, gwarps, lane, best, stall, limit, err, exec); break;
-    case 4: split_search_warp<4, STAGED>(keys, sp, depth, wig, gwarps, lane, best, stall, limit, err, exec); break;
-    case 5: split_search_warp<5, STAGED>(keys, sp, depth, wig, gwarps, lane, best, stall, limit, err, exec); break;
-    case 6: split_search_warp<6, STAGED>(keys, sp, depth, wig, gwarps, lane, best, stall, limit, err, exec); break;
-    case 7: split_search_warp<7, STAGED>(keys, sp, depth, wig, gwarps, lane, best, stall, limit, err, exec); break;
-    default: split_search_warp<2, STAGED>(keys, sp, depth, wig, gwarps, lane, best, stall, limit, err, exec); break;
-  }
+  if (mode == 3)
+    split_search_warp<3, STAGED>(keys, sp, depth, wig, gwarps, lane, best, stall, limit, err, exec);
+  else
+    split_search_warp<2, STAGED>(keys, sp, depth, wig, gwarps, lane, best, stall, limit, err, exec);
 }
 
 // Emits the children of a split node with at least two keys into the queues
@@ -380,13 +431,10 @@ __device__ void emit_children(const SearchArgs& a, const Node& nd, const uint64_
 }
 
 // Search parameters of a split node; returns the count mode (split_trial).
-// fixed_width: modes 8..11 may be returned (only the shared-node kernel
-// instantiates them: in the one-group-per-node kernel four more search loops
-// made the register allocator spill).
-__device__ __forceinline__ int split_setup(const Node& nd, const uint64_t* table, SplitParams& sp,
-                                           bool fixed_width = false) {
+// counts: the tables of modes 8 and 9, or null if the launch has none.
+__device__ __forceinline__ int split_setup(const Node& nd, const uint64_t* table, const uint32_t* counts,
+                                           SplitParams& sp) {
   const uint64_t w1 = table[kTableWords * nd.m + 1];
-  sp.tail = 0;
   sp.m = nd.m;
   sp.unit = static_cast<uint32_t>(w1);
   sp.fanout = static_cast<uint32_t>(w1 >> 32) & 0xFF;
@@ -403,13 +451,23 @@ __device__ __forceinline__ int split_setup(const Node& nd, const uint64_t* table
   if (sp.fanout == 4 && nd.m == 4 * sp.unit && nd.m < 256) {
     mode = 6;
   } else if (sp.fanout >= 5 && nd.m == sp.fanout * sp.unit && sp.unit >= 2 && nd.m < 65536) {
-    const uint32_t nb = nd.m < 256 && fields * 8 <= 32 ? 8 : 32 - __clz(sp.unit);
+    uint32_t nb = nd.m < 256 && fields * 8 <= 32 ? 8 : 32 - __clz(sp.unit);
+    if (counts && sp.fanout == 5 && sp.unit < 256)
+      mode = 9, nb = 8;
+    else if (counts && sp.fanout <= 7 && sp.unit < 32)
+      mode = 8, nb = 5;
     if (fields * nb <= 32) {
-      mode = fixed_width && nb >= 5 && nb <= 8 ? static_cast<int>(nb) + 3 : 7;  // 8..11: the width at compile time
-      // second-phase keys of the two-phase block search (speed only: any
-      // value from 1 to m - 1 gives the same index); about 1.75 sqrt(m)
-      // minimises the modelled work: 19 of 112 keys, 18 of 96, 42 of 560
-      if (mode >= 8) sp.tail = min(nd.m - 1, static_cast<uint32_t>(1.75f * sqrtf(static_cast<float>(nd.m))) + 1);
+      if (mode >= 8) {
+        sp.sets = counts + (mode == 8 ? 0 : kPartCounts);
+        // second-phase keys of the two-phase block search (speed only: any
+        // value from 1 to m - 1 gives the same index); about 1.75 sqrt(m)
+        // minimises the modelled work (19 of 112 keys, 18 of 96, 42 of 560),
+        // with whole fours in the first phase
+        const uint32_t head = nd.m - static_cast<uint32_t>(1.75f * sqrtf(static_cast<float>(nd.m))) - 1;
+        sp.tail = nd.m - (head & ~3u);
+      } else {
+        mode = 7;
+      }
       sp.confirm = (1u << nb) <= nd.m;
       sp.nbits = nb;
       sp.nmask = fields * nb == 32 ? ~0u : (1u << (fields * nb)) - 1;
@@ -479,19 +537,24 @@ __device__ __forceinline__ void partition_node(const SearchArgs& a, const Node& 
 // COUNT: work counting (the evaluations executed go to a.exec_count[1]);
 // without it the counter is compiled out.
 // Warps per node or leaf: the launch shape's, doubled (up to the CTA) while
-// all the work items of the launch then still fit the grid's warps at once.
-// Their number is known on the device only.  A launch of few items lasts as
-// long as its longest search, so idle warps help there (split and leaf phases
-// at l = 8, b = 100: 10^3 keys 87 + 69 -> 51 + 20 us, 10^5 keys 197 + 85 ->
-// 110 + 73 us).
-__device__ __forceinline__ uint32_t group_warps(uint32_t gwarps, uint32_t items) {
-  while (gwarps < kWarps && uint64_t(items) * gwarps * 2 <= gridDim.x * kWarps) gwarps *= 2;
+// the launch then has at most `spread` groups' worth of work items for the
+// warps of the grid.  Their number is known on the device only.  A launch of
+// few items lasts as long as its longest search, so more warps on each help:
+// split and leaf phases at l = 8, b = 100: 10^3 keys 87 + 69 -> 47 + 21 us, 10^5
+// keys 197 + 85 -> 97 + 75 us; l = 10, b = 100, 3 * 10^5 keys 241 -> 179 us (split,
+// spread 4 against 1).  spread is 4 where a search takes several rounds of 32
+// indices (128 trials) and 2 below, where four warps mostly test past the
+// winner (l = 8, 10^5 keys: split 97 us with 2, 117 us with 4).
+__device__ __forceinline__ uint32_t group_warps(uint32_t gwarps, uint32_t items, uint32_t spread) {
+  while (gwarps < kWarps && uint64_t(items) * gwarps * 2 <= spread * gridDim.x * kWarps) gwarps *= 2;
   return gwarps;
 }
+__host__ __device__ constexpr uint32_t group_spread(uint64_t trials) { return trials >= 128 ? 4 : 2; }
 
 template <bool COUNT>
-__global__ void __launch_bounds__(kThreads, 4) k_split_level(SearchArgs a, uint32_t gwarps, uint32_t cap) {
-  extern __shared__ __align__(16) uint64_t staged[];
+__global__ void __launch_bounds__(kThreads, 4) k_split_level(SearchArgs a, uint32_t gwarps, uint32_t cap,
+                                                             uint32_t tables, uint32_t spread) {
+  extern __shared__ __align__(16) uint64_t dynamic[];  // tables of modes 8 and 9 if any, then the groups' keys
   __shared__ uint64_t best[kWarps];
   __shared__ uint32_t task[kWarps];
   __shared__ uint32_t fill[kWarps][16];
@@ -499,11 +562,13 @@ __global__ void __launch_bounds__(kThreads, 4) k_split_level(SearchArgs a, uint3
   const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (COUNT && lane == 0) wexec[warp] = 0;
   const uint32_t total = *a.split_in_count;
-  gwarps = group_warps(gwarps, total);
+  gwarps = group_warps(gwarps, total, spread);
   const uint32_t gid = warp / gwarps, wig = warp % gwarps;
   const uint32_t tig = wig * 32 + lane, gthreads = gwarps * 32;
   const bool leader = wig == 0 && lane == 0;
-  uint64_t* mine = staged + size_t(gid) * cap;
+  const uint32_t* const counts = tables ? reinterpret_cast<const uint32_t*>(dynamic) : nullptr;
+  if (tables) fill_part_counts(reinterpret_cast<uint32_t*>(dynamic));
+  uint64_t* mine = dynamic + (tables ? kPartCounts : 0) + size_t(gid) * cap;
 
   for (;;) {
     if (leader) task[gid] = *reinterpret_cast<volatile int*>(a.error) ? total : atomicAdd(a.work_counter, 1u);
@@ -517,7 +582,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_split_level(SearchArgs a, uint3
       const uint32_t depth = nd.depth & kDepthMask;
       const uint64_t* table = a.table[nd.depth >> 8];
       SplitParams sp;
-      const int mode = split_setup(nd, table, sp);
+      const int mode = split_setup(nd, table, counts, sp);
       const uint64_t stall = stall_threshold(table, nd.m);
       const uint64_t limit = trial_limit(table, nd.m);
 
@@ -565,18 +630,8 @@ constexpr uint32_t kShareRounds = 4;
 constexpr uint32_t kNodeOpen = 1, kNodeClosed = 2;
 constexpr uint32_t kMaxJoins = 4096;  // nodes one CTA may join in one launch
 
-// Fixed-width fields (modes 8..11) of keys [j0, j1) under function kp.
-template <int NB>
-__device__ __forceinline__ uint32_t split_fields(const uint64_t* __restrict__ keys, const SplitParams& p, uint64_t kp,
-                                                 uint32_t j0, uint32_t j1) {
-  uint32_t acc = 0;
-#pragma unroll 4
-  for (uint32_t j = j0; j < j1; j++) acc += shl32(1u, __umulhi(family_top32(keys[j], kp), p.fanout) * NB);
-  return acc;
-}
-
 // Two-phase test of one claimed block (kShareRounds * 32 indices from base0)
-// for the equal-part modes 8..11: phase 1 counts the first m - tail keys of
+// for the equal-part modes 8 and 9: phase 1 counts the first m - tail keys of
 // every index and keeps, in index order, those whose parts all still hold at
 // most unit keys; phase 2 adds the last tail keys of the survivors, 32 at a
 // time, and applies the one-phase test to the sum (the same fields: the
@@ -587,11 +642,11 @@ __device__ __forceinline__ uint32_t split_fields(const uint64_t* __restrict__ ke
 // fields read in phase 1 are exact for the indices that are kept; an index
 // whose fields overflowed has a part beyond unit and may be kept or dropped.
 // Returns the evaluations executed; `hit` the smallest successful index, if any.
-template <int MODE>
+template <int MODE, bool STAGED>
 __device__ __forceinline__ uint64_t shared_block_two_phase(const uint64_t* __restrict__ keys, const SplitParams& sp,
                                                            uint32_t depth, uint32_t lane, uint64_t base0,
                                                            uint64_t* best, uint4* surv, uint64_t* hit) {
-  constexpr uint32_t NB = MODE - 3;
+  constexpr uint32_t NB = MODE == 8 ? 5 : 8;
   const uint32_t head = sp.m - sp.tail, fmask = (1u << NB) - 1;
   const uint32_t below = (1u << lane) - 1;
   uint64_t evals = 0;
@@ -600,7 +655,7 @@ __device__ __forceinline__ uint64_t shared_block_two_phase(const uint64_t* __res
     const uint64_t base = base0 + r * 32;
     if (r && base >= volatile_load(best)) break;  // a smaller index is known: the rest cannot win
     const uint64_t kp = family_key(base + lane, depth);
-    const uint32_t acc = split_fields<NB>(keys, sp, kp, 0, head);
+    const uint32_t acc = split_fields<MODE, STAGED>(keys, sp, kp, 0, head);
     uint32_t counted = 0;
     bool keep = true;
     for (uint32_t t = 0; t + 1 < sp.fanout; t++) {
@@ -624,9 +679,9 @@ __device__ __forceinline__ uint64_t shared_block_two_phase(const uint64_t* __res
     if (t < ns) {
       const uint4 e = surv[t];
       const uint64_t kp = (uint64_t(e.w) << 32) | e.z;
-      const uint32_t acc = e.y + split_fields<NB>(keys, sp, kp, head, sp.m);
+      const uint32_t acc = e.y + split_fields<MODE, STAGED>(keys, sp, kp, head, sp.m);
       ok = (acc & sp.nmask) == sp.ntarget;
-      if (ok && sp.confirm) ok = split_trial<1, false>(keys, sp, kp);
+      if (ok && sp.confirm) ok = split_trial<1, STAGED>(keys, sp, kp);
     }
     evals += uint64_t(min(32u, ns - t0)) * sp.tail;
     const uint32_t hits = __ballot_sync(0xFFFFFFFFu, ok);
@@ -671,9 +726,9 @@ __device__ __forceinline__ uint64_t shared_search_warp(const uint64_t* __restric
         return evals;
       }
     }
-    if (MODE >= 8 && sp.tail) {
+    if constexpr (MODE >= 8) {
       uint64_t hit;
-      evals += shared_block_two_phase<MODE >= 8 ? MODE : 8>(keys, sp, depth, lane, base0, best, surv, &hit);
+      evals += shared_block_two_phase<MODE, STAGED>(keys, sp, depth, lane, base0, best, surv, &hit);
       if (hit != ~0ull) {
         if (lane == 0) atomicMin(reinterpret_cast<unsigned long long*>(best), hit);
         return evals;
@@ -700,20 +755,20 @@ template <bool STAGED>
 __device__ __forceinline__ uint64_t shared_search(const uint64_t* __restrict__ keys, const SplitParams& sp, int mode,
                                                   uint32_t depth, uint32_t lane, uint64_t* best, unsigned int* next,
                                                   uint64_t stall, uint64_t limit, int* err, uint4* surv) {
-  switch (mode) {
-    case 0: return shared_search_warp<0, STAGED>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
-    case 1: return shared_search_warp<1, STAGED>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
-    case 3: return shared_search_warp<3, STAGED>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
-    case 4: return shared_search_warp<4, STAGED>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
-    case 5: return shared_search_warp<5, STAGED>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
-    case 6: return shared_search_warp<6, STAGED>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
-    case 7: return shared_search_warp<7, STAGED>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
-    case 8: return shared_search_warp<8, STAGED>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
-    case 9: return shared_search_warp<9, STAGED>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
-    case 10: return shared_search_warp<10, STAGED>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
-    case 11: return shared_search_warp<11, STAGED>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
-    default: return shared_search_warp<2, STAGED>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
+  if (STAGED) {
+    switch (mode) {
+      case 0: return shared_search_warp<0, true>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
+      case 1: return shared_search_warp<1, true>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
+      case 4: return shared_search_warp<4, true>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
+      case 5: return shared_search_warp<5, true>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
+      case 6: return shared_search_warp<6, true>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
+      case 7: return shared_search_warp<7, true>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
+      case 8: return shared_search_warp<8, true>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
+      case 9: return shared_search_warp<9, true>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
+    }
   }
+  if (mode == 3) return shared_search_warp<3, STAGED>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
+  return shared_search_warp<2, STAGED>(keys, sp, depth, lane, best, next, stall, limit, err, surv);
 }
 
 // One CTA per node at a time (all 8 warps): takes nodes of `queue` through
@@ -823,12 +878,16 @@ __device__ __forceinline__ void shared_nodes(const Node* queue, uint32_t total, 
 // Participants worth having on a split node: one CTA per 2^12 expected trials,
 // at most 16 (a node of a few hundred trials gains nothing).
 template <bool COUNT>
-__global__ void __launch_bounds__(kThreads, 4) k_split_shared(SearchArgs a, SharedNodes st, uint32_t cap) {
-  extern __shared__ __align__(16) uint64_t mine[];
+__global__ void __launch_bounds__(kThreads, 4) k_split_shared(SearchArgs a, SharedNodes st, uint32_t cap,
+                                                              uint32_t tables) {
+  extern __shared__ __align__(16) uint64_t dynamic[];  // tables of modes 8 and 9 if any, then the node's keys
   __shared__ uint32_t fill[16];
   __shared__ uint4 surv[kWarps][kShareRounds * 32];  // two-phase block survivors, per warp
   const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   unsigned long long evals = 0;  // work counting: evaluations of this warp, flushed at exit
+  const uint32_t* const counts = tables ? reinterpret_cast<const uint32_t*>(dynamic) : nullptr;
+  if (tables) fill_part_counts(reinterpret_cast<uint32_t*>(dynamic));
+  uint64_t* const mine = dynamic + (tables ? kPartCounts : 0);
   shared_nodes(
       a.split_in, *a.split_in_count, st, a.work_counter, a.error,
       [&](const Node& nd) {
@@ -845,7 +904,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_split_shared(SearchArgs a, Shar
         const uint32_t depth = nd.depth & kDepthMask;
         const uint64_t* table = a.table[nd.depth >> 8];
         SplitParams sp;
-        const int mode = split_setup(nd, table, sp, /*fixed_width=*/true);
+        const int mode = split_setup(nd, table, counts, sp);
         const uint64_t stall = stall_threshold(table, nd.m), limit = trial_limit(table, nd.m);
         const uint64_t done =
             nd.m <= cap ? shared_search<true>(mine, sp, mode, depth, lane, &st.best[idx], &st.next[idx], stall, limit,
@@ -1311,7 +1370,7 @@ __global__ void __launch_bounds__(kThreads, leaf_min_blocks(L)) k_leaves(SearchA
   if (lane == 0) wexec[warp] = 0;
   const Node* queue = !PART || qfull ? a.full_q[a.cls] : a.part_q[a.cls];
   const uint32_t total = !PART || qfull ? a.full_n[a.cls] : a.part_n[a.cls];
-  gwarps = group_warps(gwarps, total);
+  gwarps = group_warps(gwarps, total, PART ? 2 : group_spread(a.table[a.cls][kTableWords * L + 2]));
   const uint32_t groups = gridDim.x * (kWarps / gwarps);
   chunk = min(chunk, max(1u, total / (2 * groups)));
   const uint32_t gid = warp / gwarps, wig = warp % gwarps;
@@ -1678,9 +1737,11 @@ __global__ void __launch_bounds__(kThreads, 4) k_leaves_packed(SearchArgs a, uin
   if (a.exec_count && lane == 0 && exec) atomicAdd(a.exec_count, exec);
 }
 
-// Dynamic shared memory the split kernels may use: nodes of up to this many
-// bytes of keys are staged, larger ones read from global memory.
+// Dynamic shared memory the split kernels may use: nodes of up to
+// kSplitSmemBudget bytes of keys are staged, larger ones read from global
+// memory; the tables of modes 8 and 9 come on top.
 constexpr size_t kSplitSmemBudget = 96 * 1024;
+constexpr size_t kSplitTableBytes = 2 * kPartCounts * sizeof(uint32_t);
 
 // Raises the kernel's dynamic shared memory limit to the budget, once per
 // kernel and process.  Setting it per launch to the launch's own size would
@@ -1697,7 +1758,8 @@ int allow_split_smem() {
   RS_CUDA(cudaGetDevice(&dev));
   if (dev < 0 || dev >= 64) return fail(RECSPLIT_E_INVALID, "device ordinal above 63");
   std::call_once(once[dev], [&] {
-    status[dev] = cudaFuncSetAttribute(KERNEL, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSplitSmemBudget));
+    status[dev] = cudaFuncSetAttribute(KERNEL, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        int(kSplitSmemBudget + kSplitTableBytes));
   });
   if (status[dev] != cudaSuccess) return cuda_fail(status[dev], "cudaFuncSetAttribute");
   return RECSPLIT_OK;
@@ -1826,12 +1888,13 @@ void set_tuning_for(uint32_t leaf, const recsplit_tuning_t& t) {
   g_tuned[leaf] = true;
 }
 
-int launch_split_level(const SearchArgs& a, uint64_t max_m, uint32_t max_leaf, int sm_count, cudaStream_t s,
-                       const SharedNodes* share) {
+int launch_split_level(const SearchArgs& a, uint64_t max_m, uint64_t trials, uint32_t max_leaf, bool tables,
+                       int sm_count, cudaStream_t s, const SharedNodes* share) {
+  const size_t table_bytes = tables ? kSplitTableBytes : 0;
   if (share) {
     // one CTA per node at a time, nodes shared once the queue is empty
     const uint64_t cap = std::min<uint64_t>((max_m + 1) & ~uint64_t(1), kSplitSmemBudget / sizeof(uint64_t));
-    const size_t smem = cap * sizeof(uint64_t);
+    const size_t smem = table_bytes + cap * sizeof(uint64_t);
     auto kern = a.exec_count ? k_split_shared<true> : k_split_shared<false>;
     int rc = a.exec_count ? allow_split_smem<k_split_shared<true>>() : allow_split_smem<k_split_shared<false>>();
     if (rc) return rc;
@@ -1840,7 +1903,7 @@ int launch_split_level(const SearchArgs& a, uint64_t max_m, uint32_t max_leaf, i
     if (rc) return rc;
     blocks = std::min<int>(blocks, kSharedCtas);
     RS_CUDA(cudaMemsetAsync(a.work_counter, 0, sizeof(uint32_t), s));
-    kern<<<blocks, kThreads, smem, s>>>(a, *share, static_cast<uint32_t>(cap));
+    kern<<<blocks, kThreads, smem, s>>>(a, *share, static_cast<uint32_t>(cap), uint32_t(tables));
     count_launch();
     RS_CUDA(cudaGetLastError());
     return RECSPLIT_OK;
@@ -1851,7 +1914,7 @@ int launch_split_level(const SearchArgs& a, uint64_t max_m, uint32_t max_leaf, i
   const uint32_t groups = kWarps / gwarps;
   // an even number of keys per group, so that every group's are 16-byte aligned
   const uint64_t cap = std::min<uint64_t>((max_m + 1) & ~uint64_t(1), kSplitSmemBudget / (groups * sizeof(uint64_t)));
-  const size_t smem = size_t(groups) * cap * sizeof(uint64_t);
+  const size_t smem = table_bytes + size_t(groups) * cap * sizeof(uint64_t);
   auto kern = a.exec_count ? k_split_level<true> : k_split_level<false>;
   int rc = a.exec_count ? allow_split_smem<k_split_level<true>>() : allow_split_smem<k_split_level<false>>();
   if (rc) return rc;
@@ -1859,7 +1922,7 @@ int launch_split_level(const SearchArgs& a, uint64_t max_m, uint32_t max_leaf, i
   rc = persistent_grid(kern, smem, sm_count, &blocks);
   if (rc) return rc;
   RS_CUDA(cudaMemsetAsync(a.work_counter, 0, sizeof(uint32_t), s));
-  kern<<<blocks, kThreads, smem, s>>>(a, gwarps, static_cast<uint32_t>(cap));
+  kern<<<blocks, kThreads, smem, s>>>(a, gwarps, static_cast<uint32_t>(cap), uint32_t(tables), group_spread(trials));
   count_launch();
   RS_CUDA(cudaGetLastError());
   return RECSPLIT_OK;
