@@ -764,7 +764,9 @@ int build_sets(const SetInput* in, uint32_t count, const BuildOptions& opt, cuda
   // level is searched shared.  That costs a few microseconds of CTA-wide steps
   // per node and removes the level's tail, a few long geometric searches on an
   // idle device, so it pays where a node's expected trials x keys reach 2^21
-  // evaluations, or 2^16 on a level of fewer than 8 nodes per warp of the device.
+  // evaluations, or 2^16 on a level of few nodes: 8 of the largest size per warp
+  // of the device, counting the keys of every class over its largest node
+  // (half of it, since parts are smaller; at the roots, the buckets).
   // Split phase without and with the second clause: l = 12, b = 100: 10^5 keys
   // 0.84 -> 0.39 ms, 10^6 keys 2.29 -> 1.81 ms (5 * 10^6 keys, above the line: 7.1
   // against 8.2 ms); l = 13, b = 100, 3 * 10^5 keys 12.6 -> 6.6 ms; l = 12, b = 2000,
@@ -775,16 +777,17 @@ int build_sets(const SetInput* in, uint32_t count, const BuildOptions& opt, cuda
   {
     std::vector<uint64_t> lm = level_max;
     for (;;) {
-      uint64_t mx = 0;
+      uint64_t mx = 0, nodes = 0;
       double heavy = 0;
       for (uint32_t c = 0; c < nclass; c++)
         if (lm[c] > class_leaf[c]) {
           mx = std::max(mx, lm[c]);
+          nodes += plan_mx.empty() ? nb_c[c] : 2 * keys_c[c] / lm[c];
           heavy = std::max(heavy, double(T[c].expected_trials[lm[c]]) * double(lm[c]));
         }
       if (mx == 0 || plan_mx.size() > kMaxDepth + 1) break;
       plan_mx.push_back(mx);
-      const bool few = K / mx <= 8ull * 32 * sm_count;
+      const bool few = nodes <= 16ull * 32 * sm_count;
       plan_share.push_back(heavy >= double(few ? 1 << 16 : 1 << 21));
       for (uint32_t c = 0; c < nclass; c++)
         lm[c] = lm[c] > class_leaf[c] ? next_level_max(make_strategy(class_leaf[c]), lm[c]) : 0;
