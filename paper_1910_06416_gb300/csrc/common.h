@@ -136,6 +136,11 @@ struct View {
   const uint64_t* table;  // kTableWords words per size
   const LookupRecord* rec;  // one lookup record per size
   const uint64_t* so;  // s_i, o_i of every bucket decoded beforehand, or null
+  const uint64_t* flat;  // function key of every code decoded beforehand (lookup.cu), or null: so then
+                         // holds s_i and the size of every bucket
+  uint64_t range;      // size of the output range
+  uint64_t codes;      // stored codes
+  uint64_t log_group;  // parts that a bucket's codes are decoded in (lookup.cu), log2
   uint64_t tree_words32;  // 32-bit words of the tree section (code scans stop there)
   uint64_t mmax;       // largest bucket (the tables cover sizes 0 .. mmax)
   uint32_t extra;      // leaf range extra (0: minimal)
@@ -214,16 +219,18 @@ int build_sets(const SetInput* sets, uint32_t count, const BuildOptions& opt, cu
 int lookup_structure(const Handle& h, const KeyInput& q, uint64_t* d_out, cudaStream_t s, bool allow_scratch = true);
 // Lookups of keys[i] in views[ids[i]] (count views); an id not below count
 // gives 2^64 - 1.  any_range: some view has a leaf range extra (perfect,
-// non-minimal variant)
+// non-minimal variant); flat: every view with buckets has flat set
 int lookup_many(const View* d_views, uint32_t count, const uint32_t* d_ids, const uint64_t* d_keys, uint64_t q,
-                uint64_t* d_out, cudaStream_t s, bool any_range = true);
-// Batched lookups over several structures with at least as many queries as
-// the structures have buckets: s_i, o_i of every bucket of every structure
-// are decoded into one pooled array *so (the caller frees it, stream-ordered,
-// after the lookups) and views[i].so (host views) points at structure i's
-// part.  Otherwise, or if the memory is not available, *so stays null and the
+                uint64_t* d_out, cudaStream_t s, bool any_range = true, bool flat = false);
+// Batched lookups over several structures with several times as many queries
+// as the structures have codes: the function key of every code and s_i and the
+// size of every bucket of every structure are decoded into one pooled array
+// *scratch (the caller frees it, stream-ordered, after the lookups), and
+// views[i].flat and .so (host views) point at structure i's parts.  With fewer
+// queries, but at least as many as buckets, s_i and o_i alone (views[i].so).
+// Otherwise, or if the memory is not available, *scratch stays null and the
 // views are unchanged (the lookups then select in the lists per query).
-int decode_views(View* views, uint32_t count, uint64_t q, cudaStream_t s, uint64_t** so);
+int decode_views(View* views, uint32_t count, uint64_t q, cudaStream_t s, uint64_t** scratch, bool* flat);
 int lookup_many_bytes(const View* d_views, uint32_t count, const uint32_t* d_ids, const uint8_t* d_bytes,
                       const uint64_t* d_offsets, uint64_t q, uint64_t* d_out, cudaStream_t s);
 

@@ -7,6 +7,7 @@
 // bijection's value is added to the keys left behind (c) and to s_b.
 #include <nvtx3/nvToolsExt.h>
 
+#include <algorithm>
 #include <vector>
 
 #include "device.cuh"
@@ -244,6 +245,212 @@ __device__ __forceinline__ uint64_t descend(const View& v, uint64_t s0, uint32_t
   }
 }
 
+// ---------------------------------------------------------------- flat codes
+// A batch with several times as many queries as the structure has codes
+// (flat_pays) decodes every code once: the function key K ^ (K >> 30) of code c (preorder) of the
+// bucket that starts at s_b is stored at flat[s_b + c] (a bucket of m keys has
+// fewer than m codes), and so holds s_b and the bucket's size.  A level of the
+// descent then loads its key and steps over the earlier siblings' codes with
+// one multiply-add, where it otherwise reads a fixed part, finds a unary part
+// and selects past the siblings in the bit vector.
+
+// Key of code c of a bucket of m keys (fixed parts from bit `fixed` of t, unary
+// part un): the path to node c of the preorder gives its size, depth and the
+// position of its fixed part.
+__device__ __forceinline__ uint64_t code_key(const View& v, const uint32_t* __restrict__ t, uint32_t end,
+                                             uint32_t fixed, uint32_t m, uint32_t c, uint32_t un) {
+  const uint4* __restrict__ rec = reinterpret_cast<const uint4*>(v.rec);
+  uint32_t depth = 0, r;
+  for (;;) {
+    const uint4 nd = __ldg(rec + m);
+    r = (nd.w >> kLookupCodeBits) & 31;
+    if (c == 0) break;
+    c--;
+    const uint32_t codes = nd.w & ((1u << kLookupCodeBits) - 1), fanout = nd.w >> 28;
+    const uint32_t j = codes ? min(c / codes, fanout - 1) : fanout - 1;
+    c -= j * codes;
+    fixed += r + j * nd.z;
+    m = j + 1 < fanout ? nd.x : m - nd.x * (fanout - 1);
+    depth++;
+  }
+  const uint32_t w = fixed >> 5;
+  const uint32_t f0 = __ldg(t + w), f1 = w + 1 < end ? __ldg(t + w + 1) : 0u;
+  const uint32_t low = __funnelshift_r(f0, f1, fixed & 31) & ((1u << r) - 1u);
+  return family_key((uint64_t(un) << r) | low, depth);
+}
+
+// Part g of 2^log_group of the decode of bucket b: codes g, g + 2^log_group, ...
+// Every part reads the lists for itself and scans the unary part with a cursor
+// of its own, so parts need nothing from each other.
+template <bool RANGE>
+__device__ __forceinline__ void flat_bucket(const View& v, uint64_t b, uint32_t g, uint32_t log_group) {
+  uint64_t* so = const_cast<uint64_t*>(v.so);
+  const uint64_t s0 = ef_prefix(v, b);
+  const uint32_t m = size_of_range<RANGE>(v, ef_prefix(v, b + 1) - s0);
+  if (g == 0) {
+    so[2 * b] = s0;
+    so[2 * b + 1] = m;
+  }
+  if (m < 2) return;
+  const uint64_t w0 = __ldg(v.table + kTableWords * m);
+  const uint32_t codes = static_cast<uint32_t>(w0 >> 32);
+  if (g >= codes) return;
+  const uint64_t o = ef_offset(v, b, s0);
+  const uint32_t* __restrict__ t = reinterpret_cast<const uint32_t*>(v.tree) + (o >> 5);
+  const uint64_t left = v.tree_words32 - (o >> 5);
+  const uint32_t end = left < 0xFFFFFFFFull ? static_cast<uint32_t>(left) : 0xFFFFFFFFu;
+  const uint32_t fixed = static_cast<uint32_t>(o & 31);
+  uint64_t* flat = const_cast<uint64_t*>(v.flat) + s0;
+  const uint32_t u0 = fixed + static_cast<uint32_t>(w0);  // first bit of the unary part
+  // cursor: `rank` ones lie in [u0, word w), `word` holds the ones of word w
+  // from u0 on
+  uint32_t w = u0 >> 5, rank = 0;
+  uint32_t word = __ldg(t + w) & (~0u << (u0 & 31));
+  for (uint32_t c = g; c < codes; c += 1u << log_group) {
+    uint32_t from = u0;  // the bit after the one of code c - 1
+    if (c) {
+      uint32_t ones = __popc(word);
+      while (rank + ones < c) {
+        if (++w >= end) return;
+        rank += ones;
+        word = __ldg(t + w);
+        ones = __popc(word);
+      }
+      from = (w << 5) + select_in_word32(word, c - 1 - rank) + 1;
+    }
+    const uint32_t one = code_next_one(t, from, end);
+    if (one == ~0u) return;
+    flat[c] = code_key(v, t, end, fixed, m, c, one - from);
+  }
+}
+
+// Parts (log2) that the buckets of a structure are decoded in, `per` codes or
+// more to a part on average.  One thread per bucket left 10^4 buckets of 18
+// codes waiting on dependent loads (13 us).
+uint32_t flat_log_group(uint64_t codes, uint64_t nb, uint64_t per) {
+  uint32_t lg = 0;
+  while (lg < 10 && codes >= (nb * per) << (lg + 1)) lg++;
+  return lg;
+}
+
+// Codes per part: two, or as many as keep all parts to 2^19 (about the
+// threads the device holds).
+uint64_t codes_per_part(uint64_t codes) { return std::max<uint64_t>(2, codes >> 19); }
+
+// Whether a batch of q queries decodes the codes first: the decode costs
+// about as much as three queries per code gain (l = 8, b = 100, 10^7 keys: 3.6 *
+// 10^6 queries 97 us either way, 7.1 * 10^6 187 -> 155 us; l = 12, b = 2000, 3 *
+// 10^6 keys: 2.0 codes' worth of queries 54 -> 38 us), a few microseconds at
+// least, and buckets of a few codes have nothing to skip (l = 5, b = 5: 1.6 codes,
+// 517 us without and 546 with it for ten queries per code).
+bool flat_pays(uint64_t q, uint64_t codes, uint64_t nb) {
+  return q >= 3 * codes && q >= (1u << 18) && codes >= 2 * nb;
+}
+
+template <bool RANGE>
+__global__ void __launch_bounds__(256) k_flat_decode(const __grid_constant__ View v, uint32_t log_group) {
+  const uint64_t i = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x;
+  if (i >> log_group < v.nb) flat_bucket<RANGE>(v, i >> log_group, i & ((1u << log_group) - 1), log_group);
+}
+
+// Buckets of every structure: part p of the global index space belongs to the
+// structure i with base[i] <= p < base[i + 1].
+__global__ void __launch_bounds__(256) k_flat_decode_views(const View* __restrict__ views,
+                                                           const uint64_t* __restrict__ base, uint32_t count,
+                                                           uint64_t total) {
+  const uint64_t p = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x;
+  if (p >= total) return;
+  uint32_t lo = 0, hi = count;  // last i with base[i] <= p
+  while (hi - lo > 1) {
+    const uint32_t mid = (lo + hi) / 2;
+    if (__ldg(base + mid) <= p) lo = mid; else hi = mid;
+  }
+  const View& v = views[lo];
+  const uint64_t i = p - __ldg(base + lo);
+  flat_bucket<true>(v, i >> v.log_group, i & ((1u << v.log_group) - 1), v.log_group);
+}
+
+// What a flat lookup reads of a structure.
+struct FlatView {
+  uint64_t nb;
+  const ulonglong2* so;
+  const uint64_t* flat;
+  const uint4* rec;
+  const uint64_t* table;  // output ranges (RANGE)
+  uint64_t extra;
+};
+
+__host__ __device__ __forceinline__ FlatView flat_view(const View& v) {
+  return FlatView{v.nb, reinterpret_cast<const ulonglong2*>(v.so), v.flat, reinterpret_cast<const uint4*>(v.rec),
+                  v.table, v.extra};
+}
+
+template <bool RANGE>
+__device__ __forceinline__ uint64_t lookup_flat(const FlatView& v, uint64_t hi, uint64_t lo) {
+  if (v.nb == 0) return 0;
+  const ulonglong2 p = __ldg(v.so + bucket_of(hi, v.nb));
+  uint32_t m = static_cast<uint32_t>(p.y);
+  if (m <= 1) return p.x;
+  const uint64_t* __restrict__ code = v.flat + p.x;
+  const uint64_t xpre = pre_key(lo);
+  uint32_t c = 0;  // keys (or output ranges) of the siblings left behind
+  for (;;) {
+    const uint64_t kp = __ldg(code);
+    const uint4 nd = __ldg(v.rec + m);
+    const uint32_t h = family_top32(xpre, kp);
+    const uint32_t fanout = nd.w >> 28;
+    if (fanout == 0) return p.x + c + __umulhi(h, RANGE ? m + static_cast<uint32_t>(v.extra) : m);
+    const uint32_t val = __umulhi(h, m);
+    const uint32_t part = min(nd.y ? __umulhi(val, nd.y) : val / nd.x, fanout - 1);
+    code += 1 + part * (nd.w & ((1u << kLookupCodeBits) - 1));
+    c += RANGE ? part * static_cast<uint32_t>(__ldg(v.table + kTableWords * nd.x + 3) >> 32) : part * nd.x;
+    m = part + 1 < fanout ? nd.x : m - nd.x * (fanout - 1);
+    if (m <= 1) return p.x + c;
+  }
+}
+
+template <bool RANGE>
+__global__ void __launch_bounds__(256, 8) k_lookup_u64_flat(FlatView v, const uint64_t* __restrict__ keys, uint64_t q,
+                                                            uint64_t* __restrict__ out) {
+  for (uint64_t i = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; i < q; i += uint64_t(gridDim.x) * blockDim.x) {
+    uint64_t hi, lo;
+    signature_u64(__ldg(keys + i), hi, lo);
+    out[i] = lookup_flat<RANGE>(v, hi, lo);
+  }
+}
+
+template <bool RANGE>
+__global__ void __launch_bounds__(256, 8) k_lookup_bytes_flat(FlatView v, const uint8_t* __restrict__ bytes,
+                                                              const uint64_t* __restrict__ offsets, uint64_t q,
+                                                              uint64_t* __restrict__ out) {
+  const uint64_t last = __ldg(offsets + q);  // the bytes span [0, offsets[q])
+  for (uint64_t i = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; i < q; i += uint64_t(gridDim.x) * blockDim.x) {
+    const uint64_t o0 = __ldg(offsets + i), o1 = __ldg(offsets + i + 1);
+    uint64_t hi, lo;
+    const bool ok = o0 <= o1 && o1 <= last;  // else read as the empty string
+    signature_bytes(bytes + (ok ? o0 : 0), ok ? o1 - o0 : 0, hi, lo);
+    out[i] = lookup_flat<RANGE>(v, hi, lo);
+  }
+}
+
+template <bool ANY_RANGE>
+__global__ void __launch_bounds__(256, 8) k_lookup_many_flat(const View* __restrict__ views, uint32_t count,
+                                                             const uint32_t* __restrict__ ids,
+                                                             const uint64_t* __restrict__ keys, uint64_t q,
+                                                             uint64_t* __restrict__ out) {
+  for (uint64_t i = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; i < q; i += uint64_t(gridDim.x) * blockDim.x) {
+    const uint32_t id = __ldg(ids + i);
+    if (id >= count) {
+      out[i] = ~0ull;
+      continue;
+    }
+    uint64_t hi, lo;
+    signature_u64(__ldg(keys + i), hi, lo);
+    const FlatView v = flat_view(views[id]);
+    out[i] = ANY_RANGE && v.extra ? lookup_flat<true>(v, hi, lo) : lookup_flat<false>(v, hi, lo);
+  }
+}
+
 // s_i and o_i of every bucket, one thread per element.
 __global__ void k_ef_decode(View v, uint64_t* __restrict__ so) {
   for (uint64_t i = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; i <= v.nb; i += uint64_t(gridDim.x) * blockDim.x) {
@@ -365,8 +572,7 @@ int lookup_many_bytes(const View* d_views, uint32_t count, const uint32_t* d_ids
 }
 
 int lookup_many(const View* d_views, uint32_t count, const uint32_t* d_ids, const uint64_t* d_keys, uint64_t q,
-                uint64_t* d_out,
-                cudaStream_t s, bool any_range) {
+                uint64_t* d_out, cudaStream_t s, bool any_range, bool flat) {
   if (q == 0) return RECSPLIT_OK;
   LookupRange range;
   int dev = 0, sms = 0;
@@ -375,26 +581,54 @@ int lookup_many(const View* d_views, uint32_t count, const uint32_t* d_ids, cons
   const int block = 256;
   const uint64_t want = (q + block - 1) / block;
   const unsigned grid = static_cast<unsigned>(want < uint64_t(sms) * 64 ? want : uint64_t(sms) * 64);
-  (any_range ? k_lookup_many<true> : k_lookup_many<false>)<<<grid, block, 0, s>>>(d_views, count, d_ids, d_keys, q,
-                                                                                  d_out);
+  auto kern = flat ? (any_range ? k_lookup_many_flat<true> : k_lookup_many_flat<false>)
+                   : (any_range ? k_lookup_many<true> : k_lookup_many<false>);
+  kern<<<grid, block, 0, s>>>(d_views, count, d_ids, d_keys, q, d_out);
   count_launch();
   RS_CUDA(cudaGetLastError());
   return RECSPLIT_OK;
 }
 
-int decode_views(View* views, uint32_t count, uint64_t q, cudaStream_t s, uint64_t** so) {
-  *so = nullptr;
+int decode_views(View* views, uint32_t count, uint64_t q, cudaStream_t s, uint64_t** scratch, bool* flat) {
+  *scratch = nullptr;
+  *flat = false;
+  // elements 0 .. N of every list, or the N buckets of every structure
+  // (or their parts)
   std::vector<uint64_t> base(count + 1);
+  uint64_t elements = 0, buckets = 0, codes = 0, range = 0;
+  for (uint32_t i = 0; i < count; i++) {
+    elements += views[i].nb ? views[i].nb + 1 : 0;
+    buckets += views[i].nb;
+    codes += views[i].codes;
+    range += views[i].range;
+  }
+  if (buckets == 0 || q < elements + count) return RECSPLIT_OK;
+  *flat = flat_pays(q, codes, buckets);
+  void *d_scratch = nullptr, *d_views = nullptr, *d_base = nullptr;
+  if (*flat && pool_alloc(&d_scratch, 16 * buckets + 8 * range, s) != RECSPLIT_OK) *flat = false;
+  if (!*flat && pool_alloc(&d_scratch, 16 * elements, s) != RECSPLIT_OK)
+    return RECSPLIT_OK;  // fall back to per-query selects
+  uint64_t* so = static_cast<uint64_t*>(d_scratch);
+  uint64_t* keys = so + 2 * buckets;
+  uint64_t* next_so = so;
   uint64_t total = 0;
   for (uint32_t i = 0; i < count; i++) {
+    View& v = views[i];
     base[i] = total;
-    total += views[i].nb ? views[i].nb + 1 : 0;
+    if (!v.nb) continue;
+    v.so = next_so;
+    if (*flat) {
+      v.flat = keys;
+      v.log_group = flat_log_group(v.codes, v.nb, codes_per_part(codes));
+      keys += v.range;
+      next_so += 2 * v.nb;
+      total += v.nb << v.log_group;
+    } else {
+      next_so += 2 * (v.nb + 1);
+      total += v.nb + 1;
+    }
   }
   base[count] = total;
-  if (total == 0 || q < total + count) return RECSPLIT_OK;
-  void *d_so = nullptr, *d_views = nullptr, *d_base = nullptr;
-  if (pool_alloc(&d_so, 16 * total, s) != RECSPLIT_OK) return RECSPLIT_OK;  // fall back to per-query selects
-  for (uint32_t i = 0; i < count; i++) views[i].so = views[i].nb ? static_cast<uint64_t*>(d_so) + 2 * base[i] : nullptr;
   int rc = pool_alloc(&d_views, sizeof(View) * count, s);
   if (!rc) rc = pool_alloc(&d_base, sizeof(uint64_t) * (count + 1), s);
   cudaError_t e = cudaSuccess;
@@ -403,8 +637,12 @@ int decode_views(View* views, uint32_t count, uint64_t q, cudaStream_t s, uint64
                                                    cudaMemcpyHostToDevice, s);
   if (!rc && e == cudaSuccess) {
     const uint64_t blocks = (total + 255) / 256;
-    k_ef_decode_views<<<static_cast<unsigned>(blocks < 65535 ? blocks : 65535), 256, 0, s>>>(
-        static_cast<const View*>(d_views), static_cast<const uint64_t*>(d_base), count, total);
+    if (*flat)
+      k_flat_decode_views<<<static_cast<unsigned>(blocks), 256, 0, s>>>(
+          static_cast<const View*>(d_views), static_cast<const uint64_t*>(d_base), count, total);
+    else
+      k_ef_decode_views<<<static_cast<unsigned>(blocks < 65535 ? blocks : 65535), 256, 0, s>>>(
+          static_cast<const View*>(d_views), static_cast<const uint64_t*>(d_base), count, total);
     count_launch();
     e = cudaGetLastError();
   }
@@ -413,18 +651,23 @@ int decode_views(View* views, uint32_t count, uint64_t q, cudaStream_t s, uint64
   if (d_views) cudaFreeAsync(d_views, s);
   if (d_base) cudaFreeAsync(d_base, s);
   if (rc || e != cudaSuccess) {
-    for (uint32_t i = 0; i < count; i++) views[i].so = nullptr;
-    cudaFreeAsync(d_so, s);
+    for (uint32_t i = 0; i < count; i++) views[i].so = views[i].flat = nullptr;
+    *flat = false;
+    cudaFreeAsync(d_scratch, s);
     if (rc) return rc;
-    return cuda_fail(e, "decode of the Elias-Fano lists");
+    return cuda_fail(e, "decode of the structures");
   }
-  *so = static_cast<uint64_t*>(d_so);
+  *scratch = so;
   return RECSPLIT_OK;
 }
 
 View make_view(const Handle& h) {
   View v;
   v.so = nullptr;
+  v.flat = nullptr;
+  v.range = h.range_size;
+  v.codes = h.ncodes;
+  v.log_group = 0;
   v.mmax = h.header[H_MMAX];
   v.extra = header_extra(h.header);
   const uint64_t* H = h.header;
@@ -457,10 +700,31 @@ int lookup_structure(const Handle& h, const KeyInput& q, uint64_t* d_out, cudaSt
   const int block = 256;
   const uint64_t want = (q.n + block - 1) / block;
   const unsigned grid = static_cast<unsigned>(want < uint64_t(sms) * 64 ? want : uint64_t(sms) * 64);
-  // With at least as many queries as buckets, the prefix sums and offsets of
-  // all buckets are decoded once instead of selected per query (the stored
-  // structure does not change).  The scratch is allocated only then.
+  // With several times as many queries as codes, every code is decoded once;
+  // with at least as many as buckets, the prefix sums and offsets of all buckets are
+  // decoded once instead of selected per query (the stored structure does not
+  // change).  The scratch is allocated only then.
   uint64_t* so = nullptr;
+  if (allow_scratch && v.nb && flat_pays(q.n, v.codes, v.nb) &&
+      pool_alloc(reinterpret_cast<void**>(&so), 16 * v.nb + 8 * v.range, s) == RECSPLIT_OK) {
+    View f = v;
+    f.so = so;
+    f.flat = so + 2 * v.nb;
+    const FlatView fv = flat_view(f);
+    const uint32_t lg = flat_log_group(v.codes, v.nb, codes_per_part(v.codes));
+    const unsigned dg = static_cast<unsigned>(((v.nb << lg) + block - 1) / block);
+    (v.extra ? k_flat_decode<true> : k_flat_decode<false>)<<<dg, block, 0, s>>>(f, lg);
+    if (q.u64)
+      (v.extra ? k_lookup_u64_flat<true> : k_lookup_u64_flat<false>)<<<grid, block, 0, s>>>(fv, q.u64, q.n, d_out);
+    else
+      (v.extra ? k_lookup_bytes_flat<true> : k_lookup_bytes_flat<false>)<<<grid, block, 0, s>>>(fv, q.bytes, q.offsets,
+                                                                                              q.n, d_out);
+    count_launch(2);
+    const cudaError_t e = cudaGetLastError();
+    cudaFreeAsync(so, s);
+    if (e != cudaSuccess) return cuda_fail(e, "lookup launch");
+    return RECSPLIT_OK;
+  }
   if (allow_scratch && v.nb && q.n >= v.nb + 1 && pool_alloc(reinterpret_cast<void**>(&so), 16 * (v.nb + 1), s) == RECSPLIT_OK) {
     const uint64_t dg = (v.nb + 1 + block - 1) / block;
     k_ef_decode<<<static_cast<unsigned>(dg < 65535 ? dg : 65535), block, 0, s>>>(v, so);
