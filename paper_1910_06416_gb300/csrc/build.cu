@@ -100,12 +100,13 @@ __global__ void __launch_bounds__(kBlock) k_signature(const DevSet* __restrict__
   }
 }
 
-// Per bucket: its set, and the per-class largest / per-set smallest bucket.
+// Per bucket: its set, and the per-class largest / per-set smallest bucket
+// (the smallest as the largest complement, so that all start from 0).
 __global__ void __launch_bounds__(kBlock) k_bucket_sets(const DevSet* __restrict__ sets, uint32_t count,
                                                         const uint64_t* __restrict__ counts,
                                                         uint32_t* __restrict__ bset,
                                                         unsigned long long* __restrict__ cls_max,
-                                                        unsigned long long* __restrict__ set_min,
+                                                        unsigned long long* __restrict__ set_cmin,
                                                         unsigned long long* __restrict__ set_max) {
   const uint32_t si = set_of_block(sets, count, blockIdx.x, 1);
   const DevSet st = sets[si];
@@ -130,21 +131,7 @@ __global__ void __launch_bounds__(kBlock) k_bucket_sets(const DevSet* __restrict
       atomicMax(cls_max + st.cls, mx);
       atomicMax(set_max + si, mx);
     }
-    if (mn != ~0ull) atomicMin(set_min + si, mn);
-  }
-}
-
-// Per set: tree bits and number of codes (differences of the global scans at
-// the set's first and one-past-last bucket).
-__global__ void k_set_scalars(const DevSet* __restrict__ sets, uint32_t count, const uint64_t* __restrict__ off,
-                              const uint64_t* __restrict__ cbase, const uint64_t* __restrict__ rstart,
-                              uint64_t* __restrict__ tree_bits, uint64_t* __restrict__ ncodes,
-                              uint64_t* __restrict__ nrange) {
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) {
-    const uint64_t b0 = sets[i].bucket_base, b1 = b0 + sets[i].nb;
-    tree_bits[i] = off[b1] - off[b0];
-    ncodes[i] = cbase[b1] - cbase[b0];
-    nrange[i] = rstart[b1] - rstart[b0];
+    if (mn != ~0ull) atomicMax(set_cmin + si, ~mn);
   }
 }
 
@@ -269,20 +256,38 @@ __device__ __forceinline__ uint64_t beta_of(uint64_t tree_bits, uint64_t n) {
   return (q << 32) + (r << 32) / n;
 }
 
-// Per set: the smallest difference of consecutive values o_i - beta s_i.
+// Signed 64-bit value as an unsigned one that grows as the value falls, above
+// 0: the largest over values that start at 0 is the smallest value.
+__host__ __device__ inline unsigned long long falling(long long v) {
+  return ~(static_cast<unsigned long long>(v) ^ (1ull << 63));
+}
+
+// Per set: the smallest difference of consecutive values o_i - beta s_i (as
+// falling()), and its tree bits, codes and output range (differences of the
+// global scans at the set's first and one-past-last bucket).
 // rstart: prefix sums of the bucket output ranges (of the bucket sizes when
 // the leaf range extra is 0), global over all sets.
+struct SetResults {
+  uint64_t *tree_bits, *codes, *range;
+  unsigned long long* delta;  // 0 until the set's buckets are seen
+};
 __global__ void __launch_bounds__(kBlock) k_ef_prepare(const DevSet* __restrict__ sets, uint32_t count,
                                                        const uint64_t* __restrict__ rstart,
                                                        const uint64_t* __restrict__ off,
-                                                       long long* __restrict__ set_db) {
+                                                       const uint64_t* __restrict__ cbase, SetResults res) {
   const uint32_t si = set_of_block(sets, count, blockIdx.x, 1);
   const DevSet st = sets[si];
   const uint64_t bb = st.bucket_base;
   const uint64_t T = off[bb + st.nb] - off[bb];
   const uint64_t r0 = rstart[bb];
-  const uint64_t beta = beta_of(T, rstart[bb + st.nb] - r0);
+  const uint64_t range = rstart[bb + st.nb] - r0;
+  const uint64_t beta = beta_of(T, range);
   const uint64_t t0 = (blockIdx.x - st.bucket_tile_base) * kTile;
+  if (t0 == 0 && threadIdx.x == 0) {
+    res.tree_bits[si] = T;
+    res.codes[si] = cbase[bb + st.nb] - cbase[bb];
+    res.range[si] = range;
+  }
   long long mn = LLONG_MAX;
   for (int k = 0; k < kTileItems; k++) {
     const uint64_t j = t0 + uint64_t(k) * kBlock + threadIdx.x;
@@ -294,7 +299,7 @@ __global__ void __launch_bounds__(kBlock) k_ef_prepare(const DevSet* __restrict_
     }
   }
   for (int o = 16; o; o >>= 1) mn = min(mn, __shfl_xor_sync(0xFFFFFFFFu, mn, o));
-  if ((threadIdx.x & 31) == 0 && mn != LLONG_MAX) atomicMin(set_db + si, mn);
+  if ((threadIdx.x & 31) == 0 && mn != LLONG_MAX) atomicMax(res.delta + si, falling(mn));
 }
 
 // ---------------------------------------------------------------- A6
@@ -334,6 +339,8 @@ struct BitSink {
 
 // Per-set output parameters (after the structure layout is known).
 struct DevOut {
+  uint64_t* blob;
+  uint64_t header[kHeaderWords];
   uint64_t* tree;
   uint64_t* lower;
   uint64_t* upper_a;
@@ -388,15 +395,17 @@ __device__ __forceinline__ void ef_values(const DevSet& st, const DevOut& p, con
 }
 
 // Elements 0 .. nb of every set: interleaved lower bits, upper bits, and the
-// u64 / u16 inventories of both lists.
+// u64 / u16 inventories of both lists; and the header (every set has an
+// element, so a first block).
 __global__ void __launch_bounds__(kBlock) k_ef_write(const DevSet* __restrict__ sets, uint32_t count,
                                                      const DevOut* __restrict__ outs,
                                                      const uint64_t* __restrict__ rstart,
                                                      const uint64_t* __restrict__ off) {
   const uint32_t si = set_of_block(sets, count, blockIdx.x, 2);
   const DevSet st = sets[si];
-  const DevOut p = outs[si];
+  const DevOut& p = outs[si];
   const uint64_t t0 = (blockIdx.x - st.elem_tile_base) * kTile;
+  if (t0 == 0 && threadIdx.x < kHeaderWords) p.blob[threadIdx.x] = p.header[threadIdx.x];
   for (int k = 0; k < kTileItems; k++) {
     const uint64_t i = t0 + uint64_t(k) * kBlock + threadIdx.x;
     if (i > st.nb) break;
@@ -421,13 +430,6 @@ __global__ void __launch_bounds__(kBlock) k_ef_write(const DevSet* __restrict__ 
       p.subs[2 * (i >> kInvLo) + 1] = static_cast<uint16_t>(db < 0xFFFF ? db : 0xFFFF);
     }
   }
-}
-
-__global__ void k_headers(const uint64_t* __restrict__ headers, const uint64_t* __restrict__ blob_off,
-                          uint32_t count, uint64_t* __restrict__ arena) {
-  for (uint64_t i = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; i < uint64_t(count) * kHeaderWords;
-       i += uint64_t(gridDim.x) * blockDim.x)
-    arena[blob_off[i / kHeaderWords] + i % kHeaderWords] = headers[i];
 }
 
 // ---------------------------------------------------------------- tracing
@@ -496,20 +498,71 @@ struct PhaseTimer {
 };
 
 // ---------------------------------------------------------------- host
+// Stream-ordered scratch of a build.  plan() lists the arrays of one
+// allocation (256-byte aligned each) and alloc() makes it: the small per-bucket
+// and per-set arrays share allocations, since thirty of them, and as many
+// frees, took about a tenth of the time of a build of 10^3 keys.
 struct Scratch {
   cudaStream_t s;
   std::vector<void*> ptrs;
+  std::vector<std::pair<void**, size_t>> planned;
+  size_t bytes = 0;
   ~Scratch() {
     for (void* p : ptrs) cudaFreeAsync(p, s);
   }
   template <typename T>
-  int alloc(T** p, uint64_t count) {
+  void plan(T** p, uint64_t count) {
+    planned.emplace_back(reinterpret_cast<void**>(p), bytes);
+    bytes += (std::max<uint64_t>(count, 1) * sizeof(T) + 255) & ~size_t(255);
+  }
+  // `zero` set: the whole allocation starts as zeros
+  int alloc(bool zero = false) {
     void* q = nullptr;
-    int rc = pool_alloc(&q, std::max<uint64_t>(count, 1) * sizeof(T), s);
+    const size_t n = bytes;
+    std::vector<std::pair<void**, size_t>> list;
+    list.swap(planned);
+    bytes = 0;
+    int rc = pool_alloc(&q, n, s);
     if (rc) return rc;
     ptrs.push_back(q);
-    *p = static_cast<T*>(q);
+    for (auto& e : list) *e.first = static_cast<char*>(q) + e.second;
+    if (zero) RS_CUDA(cudaMemsetAsync(q, 0, n, s));
     return RECSPLIT_OK;
+  }
+  template <typename T>
+  int alloc(T** p, uint64_t count) {
+    plan(p, count);
+    return alloc();
+  }
+};
+
+// Results a build reads back from the device: one copy, into page-locked
+// memory of the host thread where they fit (a copy to pageable memory waits
+// for the stream by itself and is staged).
+struct Readback {
+  static constexpr size_t kBytes = 64 << 10;
+  struct Pinned {
+    void* p = nullptr;
+    bool tried = false;
+    ~Pinned() {
+      if (p) cudaFreeHost(p);
+    }
+  };
+  std::vector<uint64_t> pageable;
+  uint64_t* words = nullptr;
+  bool pinned = false;
+  explicit Readback(size_t n) {
+    static thread_local Pinned mine;
+    if (!mine.tried) {
+      mine.tried = true;
+      if (cudaHostAlloc(&mine.p, kBytes, cudaHostAllocDefault) != cudaSuccess) {
+        cudaGetLastError();
+        mine.p = nullptr;
+      }
+    }
+    pinned = mine.p && n * sizeof(uint64_t) <= kBytes;
+    if (!pinned) pageable.resize(n);
+    words = pinned ? static_cast<uint64_t*>(mine.p) : pageable.data();
   }
 };
 
@@ -581,30 +634,87 @@ int build_sets(const SetInput* in, uint32_t count, const BuildOptions& opt, cuda
   if (K >= (1ull << 32)) return fail(RECSPLIT_E_INVALID, "at most 2^32 - 1 keys per build");
   const uint32_t nclass = static_cast<uint32_t>(class_leaf.size());
 
+  // classes by key count (queue capacities): a split node has more keys than
+  // its leaf size, and each split node or bucket yields at most one partial leaf
+  std::vector<uint64_t> keys_c(nclass, 0), nb_c(nclass, 0), full_cap(nclass), part_cap(nclass);
+  for (const DevSet& d : hs) {
+    keys_c[d.cls] += d.n;
+    nb_c[d.cls] += d.nb;
+  }
+  uint64_t split_cap = 1, qtotal = 0;
+  for (uint32_t c = 0; c < nclass; c++) {
+    split_cap += keys_c[c] / (class_leaf[c] + 1);
+    full_cap[c] = keys_c[c] / class_leaf[c] + 1;
+    part_cap[c] = nb_c[c] + keys_c[c] / (class_leaf[c] + 1) + 1;
+    qtotal += full_cap[c] + part_cap[c];
+  }
+  qtotal += 2 * split_cap;
+
   Scratch sc{s};
   PhaseTimer timer(profiling_enabled(), s);
   const uint64_t launch0 = launch_mark();
   uint32_t split_levels = 0;
   timer.mark();
   int rc;
+  const bool count_work = timer.on && work_counting_enabled();
+  // what starts as zeros, in one allocation and one memset
+  uint64_t* counts;
+  uint32_t *cursor, *sizes;
+  uint64_t* back1;  // read back after the histogram: class maxima, bad offsets, set minima (complements), set maxima
+  uint64_t* back2;  // and after the lengths: tree bits, codes, ranges, smallest deltas, error
+  const uint64_t n_back1 = kMaxClasses + 1 + 2 * uint64_t(count), n_back2 = 4 * uint64_t(count) + 1;
+  // one counter per use, so that none is zeroed between launches: nodes of
+  // every split level, work counters of the split and leaf launches, leaves
+  constexpr uint32_t kLevels = kMaxDepth + 3;
+  uint32_t* counters;
+  unsigned long long* exec = nullptr;  // work counting: evaluations executed
+  sc.plan(&counts, NB + 1);
+  sc.plan(&cursor, NB + 1);
+  sc.plan(&sizes, K + 1);
+  sc.plan(&back1, n_back1);
+  sc.plan(&back2, n_back2);
+  sc.plan(&counters, 2 * kLevels + 4 * kMaxClasses);
+  if (count_work) sc.plan(&exec, 2);
+  if ((rc = sc.alloc(/*zero=*/true))) return rc;
+  unsigned long long* cls_max = reinterpret_cast<unsigned long long*>(back1);
+  int* bad_offsets = reinterpret_cast<int*>(back1 + kMaxClasses);
+  unsigned long long* set_cmin = cls_max + kMaxClasses + 1;
+  unsigned long long* set_max = set_cmin + count;
+  SetResults results{back2, back2 + count, back2 + 2 * uint64_t(count),
+                     reinterpret_cast<unsigned long long*>(back2 + 3 * uint64_t(count))};
+  int* d_error = reinterpret_cast<int*>(back2 + 4 * uint64_t(count));
+  uint32_t* const level_n = counters;                 // split nodes per level
+  uint32_t* const level_work = counters + kLevels;    // and the work counter of its launch
+  uint32_t* const leaf_work = level_work + kLevels;   // two leaf launches per class
+  uint32_t* const full_n = leaf_work + 2 * kMaxClasses;
+  uint32_t* const part_n = full_n + kMaxClasses;
+
   DevSet* d_sets;
+  DevOut* d_outs;
   uint32_t *bucket, *bset;
-  uint64_t *lo, *counts, *bstart, *codes, *cbase;
-  unsigned long long *cls_max, *set_min, *set_max;
-  int* bad_offsets;
-  if ((rc = sc.alloc(&d_sets, count)) || (rc = sc.alloc(&bucket, K)) || (rc = sc.alloc(&lo, K)) ||
-      (rc = sc.alloc(&counts, NB + 1)) || (rc = sc.alloc(&bstart, NB + 1)) || (rc = sc.alloc(&codes, NB + 1)) ||
-      (rc = sc.alloc(&cbase, NB + 1)) || (rc = sc.alloc(&bset, NB + 1)) || (rc = sc.alloc(&cls_max, kMaxClasses)) ||
-      (rc = sc.alloc(&set_min, count)) || (rc = sc.alloc(&set_max, count)) || (rc = sc.alloc(&bad_offsets, 1)))
-    return rc;
+  uint64_t *lo, *bstart, *codes, *cbase, *bits, *off, *scan_tmp, *ranges = nullptr;
+  // prefix sums of the bucket output ranges: s_i itself unless a set has a
+  // leaf range extra
+  uint64_t* rstart = nullptr;
+  sc.plan(&d_sets, count);
+  sc.plan(&d_outs, count);
+  if ((rc = sc.alloc())) return rc;
+  sc.plan(&bstart, NB + 1);
+  sc.plan(&codes, NB + 1);
+  sc.plan(&cbase, NB + 1);
+  sc.plan(&bset, NB + 1);
+  sc.plan(&bits, NB + 1);
+  sc.plan(&off, NB + 1);
+  sc.plan(&scan_tmp, scan_scratch(NB));
+  if (any_extra) {
+    sc.plan(&ranges, NB + 1);
+    sc.plan(&rstart, NB + 1);
+  }
+  if ((rc = sc.alloc()) || (rc = sc.alloc(&bucket, K)) || (rc = sc.alloc(&lo, K))) return rc;
+  if (!any_extra) rstart = bstart;
   RS_CUDA(cudaMemcpyAsync(d_sets, hs.data(), count * sizeof(DevSet), cudaMemcpyHostToDevice, s));
 
   // A1 + A2: signatures, bucket ids, histogram; bucket -> set; extremes
-  RS_CUDA(cudaMemsetAsync(counts, 0, (NB + 1) * sizeof(uint64_t), s));
-  RS_CUDA(cudaMemsetAsync(cls_max, 0, kMaxClasses * sizeof(unsigned long long), s));
-  RS_CUDA(cudaMemsetAsync(set_min, 0xFF, count * sizeof(unsigned long long), s));
-  RS_CUDA(cudaMemsetAsync(set_max, 0, count * sizeof(unsigned long long), s));
-  RS_CUDA(cudaMemsetAsync(bad_offsets, 0, sizeof(int), s));
   if (key_tiles) {
     k_signature<<<static_cast<unsigned>(key_tiles), kBlock, 0, s>>>(
         d_sets, count, bucket, lo, reinterpret_cast<unsigned long long*>(counts), bad_offsets);
@@ -612,20 +722,21 @@ int build_sets(const SetInput* in, uint32_t count, const BuildOptions& opt, cuda
   }
   if (bucket_tiles) {
     k_bucket_sets<<<static_cast<unsigned>(bucket_tiles), kBlock, 0, s>>>(d_sets, count, counts, bset, cls_max,
-                                                                         set_min, set_max);
+                                                                         set_cmin, set_max);
     count_launch();
   }
   RS_CUDA(cudaGetLastError());
   timer.mark();
-  std::vector<unsigned long long> h_cls_max(kMaxClasses), h_set_min(count), h_set_max(count);
-  RS_CUDA(cudaMemcpyAsync(h_cls_max.data(), cls_max, kMaxClasses * sizeof(unsigned long long), cudaMemcpyDeviceToHost,
-                          s));
-  RS_CUDA(cudaMemcpyAsync(h_set_min.data(), set_min, count * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
-  RS_CUDA(cudaMemcpyAsync(h_set_max.data(), set_max, count * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
-  int h_bad = 0;
-  RS_CUDA(cudaMemcpyAsync(&h_bad, bad_offsets, sizeof(int), cudaMemcpyDeviceToHost, s));
-  RS_CUDA(cudaStreamSynchronize(s));  // sync 1: largest bucket per class
-  if (h_bad) return fail(RECSPLIT_E_INVALID, "byte-string offsets must not decrease");
+  std::vector<uint64_t> h_cls_max(kMaxClasses), h_set_min(count), h_set_max(count);
+  {
+    Readback back(n_back1);
+    RS_CUDA(cudaMemcpyAsync(back.words, back1, n_back1 * sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
+    RS_CUDA(cudaStreamSynchronize(s));  // sync 1: largest bucket per class
+    if (static_cast<int>(back.words[kMaxClasses])) return fail(RECSPLIT_E_INVALID, "byte-string offsets must not decrease");
+    std::copy_n(back.words, kMaxClasses, h_cls_max.begin());
+    for (uint32_t i = 0; i < count; i++) h_set_min[i] = ~back.words[kMaxClasses + 1 + i];
+    std::copy_n(back.words + kMaxClasses + 1 + count, count, h_set_max.begin());
+  }
 
   // tables per class, in one buffer
   std::vector<Tables> T(nclass);
@@ -652,71 +763,33 @@ int build_sets(const SetInput* in, uint32_t count, const BuildOptions& opt, cuda
   }
 
   // prefix sums s_i and code-slot bases (global over all sets)
-  if ((rc = exclusive_scan_u64(counts, bstart, NB, s))) return rc;
+  if ((rc = exclusive_scan_u64(counts, bstart, NB, scan_tmp, s))) return rc;
   if (NB) {
     k_bucket_codes<<<grid_for(NB), kBlock, 0, s>>>(counts, bset, d_sets, NB, ct, codes);
     count_launch();
   }
-  if ((rc = exclusive_scan_u64(codes, cbase, NB, s))) return rc;
-  // prefix sums of the bucket output ranges: s_i itself unless a set has a
-  // leaf range extra
-  uint64_t* rstart = bstart;
+  if ((rc = exclusive_scan_u64(codes, cbase, NB, scan_tmp, s))) return rc;
   if (any_extra) {
-    uint64_t* ranges;
-    if ((rc = sc.alloc(&ranges, NB + 1)) || (rc = sc.alloc(&rstart, NB + 1))) return rc;
     if (NB) {
       k_bucket_ranges<<<grid_for(NB), kBlock, 0, s>>>(counts, bset, d_sets, NB, ct, ranges);
       count_launch();
     }
-    if ((rc = exclusive_scan_u64(ranges, rstart, NB, s))) return rc;
+    if ((rc = exclusive_scan_u64(ranges, rstart, NB, scan_tmp, s))) return rc;
   }
 
-  // grouping
+  // grouping; queues: two split levels (ping-pong) shared by all classes, full
+  // and partial leaves per class
   uint64_t* keys[2];
-  uint32_t* cursor;
-  if ((rc = sc.alloc(&keys[0], K)) || (rc = sc.alloc(&keys[1], K)) || (rc = sc.alloc(&cursor, NB + 1))) return rc;
-  RS_CUDA(cudaMemsetAsync(cursor, 0, (NB + 1) * sizeof(uint32_t), s));
+  Node* qmem;
+  uint64_t* seeds;
+  if ((rc = sc.alloc(&keys[0], K)) || (rc = sc.alloc(&keys[1], K)) || (rc = sc.alloc(&qmem, qtotal)) ||
+      (rc = sc.alloc(&seeds, K + 1)))
+    return rc;
   if (K) {
     k_scatter<<<std::min<unsigned>(grid_for(K), sm_count * 16), kBlock, 0, s>>>(bucket, lo, K, bstart, cursor,
                                                                                  keys[0]);
     count_launch();
   }
-
-  // queues: two split levels (ping-pong) shared by all classes; full and
-  // partial leaves per class.  A split node has more keys than its leaf size,
-  // and each split node or bucket yields at most one partial leaf.
-  std::vector<uint64_t> keys_c(nclass, 0), nb_c(nclass, 0);
-  for (const DevSet& d : hs) {
-    keys_c[d.cls] += d.n;
-    nb_c[d.cls] += d.nb;
-  }
-  uint64_t split_cap = 1;
-  std::vector<uint64_t> full_cap(nclass), part_cap(nclass);
-  for (uint32_t c = 0; c < nclass; c++) {
-    split_cap += keys_c[c] / (class_leaf[c] + 1);
-    full_cap[c] = keys_c[c] / class_leaf[c] + 1;
-    part_cap[c] = nb_c[c] + keys_c[c] / (class_leaf[c] + 1) + 1;
-  }
-  uint64_t qtotal = 2 * split_cap;
-  for (uint32_t c = 0; c < nclass; c++) qtotal += full_cap[c] + part_cap[c];
-  Node* qmem;
-  uint32_t* counters;  // split[0], split[1], work, full[kMaxClasses], part[kMaxClasses]
-  int* d_error;
-  uint64_t* seeds;
-  uint32_t* sizes;
-  if ((rc = sc.alloc(&qmem, qtotal)) || (rc = sc.alloc(&counters, 3 + 2 * kMaxClasses)) ||
-      (rc = sc.alloc(&d_error, 1)) || (rc = sc.alloc(&seeds, K + 1)) || (rc = sc.alloc(&sizes, K + 1)))
-    return rc;
-  RS_CUDA(cudaMemsetAsync(counters, 0, (3 + 2 * kMaxClasses) * sizeof(uint32_t), s));
-  RS_CUDA(cudaMemsetAsync(d_error, 0, sizeof(int), s));
-  // work counting: the searches also count the evaluations they execute
-  const bool count_work = timer.on && work_counting_enabled();
-  unsigned long long* exec = nullptr;
-  if (count_work) {
-    if ((rc = sc.alloc(&exec, 2))) return rc;
-    RS_CUDA(cudaMemsetAsync(exec, 0, 2 * sizeof(unsigned long long), s));
-  }
-  RS_CUDA(cudaMemsetAsync(sizes, 0, (K + 1) * sizeof(uint32_t), s));
   SearchArgs a{};
   a.keys[0] = keys[0];
   a.keys[1] = keys[1];
@@ -738,13 +811,12 @@ int build_sets(const SetInput* in, uint32_t count, const BuildOptions& opt, cuda
     }
   }
   a.split_cap = static_cast<uint32_t>(split_cap);
-  a.work_counter = counters + 2;
-  a.full_n = counters + 3;
-  a.part_n = counters + 3 + kMaxClasses;
+  a.full_n = full_n;
+  a.part_n = part_n;
   a.error = d_error;
   a.exec_count = exec;
   a.split_in = q_split[0];
-  a.split_in_count = counters + 0;
+  a.split_in_count = level_n;
   if (NB) {
     k_roots<<<grid_for(NB), kBlock, 0, s>>>(counts, bstart, cbase, bset, d_sets, NB, a);
     count_launch();
@@ -801,18 +873,18 @@ int build_sets(const SetInput* in, uint32_t count, const BuildOptions& opt, cuda
     if (share_leaves[c]) share_cap = std::max(share_cap, full_cap[c]);
   }
   if (share_cap) {
-    if ((rc = sc.alloc(&shared.best, share_cap)) || (rc = sc.alloc(&shared.next, share_cap)) ||
-        (rc = sc.alloc(&shared.refs, share_cap)) || (rc = sc.alloc(&shared.cap, share_cap)) ||
-        (rc = sc.alloc(&shared.flag, share_cap)) || (rc = sc.alloc(&shared.owned, kSharedCtas)))
-      return rc;
+    // (flag and owned are zeroed once: every launch has its own epoch)
+    sc.plan(&shared.flag, share_cap);
+    sc.plan(&shared.owned, kSharedCtas);
+    if ((rc = sc.alloc(/*zero=*/true))) return rc;
+    sc.plan(&shared.best, share_cap);
+    sc.plan(&shared.next, share_cap);
+    sc.plan(&shared.refs, share_cap);
+    sc.plan(&shared.cap, share_cap);
+    if ((rc = sc.alloc())) return rc;
   }
 
   // A3 (split levels), A4 (leaves), A5 (lengths): optionally one CUDA graph
-  uint64_t *bits, *off, *set_T, *set_codes, *set_R;
-  long long* set_db;
-  if ((rc = sc.alloc(&bits, NB + 1)) || (rc = sc.alloc(&off, NB + 1)) || (rc = sc.alloc(&set_db, count)) ||
-      (rc = sc.alloc(&set_T, count)) || (rc = sc.alloc(&set_codes, count)) || (rc = sc.alloc(&set_R, count)))
-    return rc;
   // The graph is captured on a stream of its own (the caller's stream may be
   // the legacy default stream, which cannot be captured) and launched on s.
   cudaGraph_t graph = nullptr;
@@ -843,15 +915,12 @@ int build_sets(const SetInput* in, uint32_t count, const BuildOptions& opt, cuda
       if (level > kMaxDepth) return fail(RECSPLIT_E_INVALID, "splitting tree deeper than 63 levels");
       const int cur = level & 1;
       a.split_in = q_split[cur];
-      a.split_in_count = counters + cur;
+      a.split_in_count = level_n + level;
       a.split_out = q_split[cur ^ 1];
-      a.split_out_count = counters + (cur ^ 1);
-      RS_CUDA(cudaMemsetAsync(a.split_out_count, 0, sizeof(uint32_t), ws));
+      a.split_out_count = level_n + level + 1;
+      a.work_counter = level_work + level;
       const bool share = size_t(level) < plan_share.size() && plan_share[level];
-      if (share) {
-        RS_CUDA(cudaMemsetAsync(shared.flag, 0, split_cap * sizeof(unsigned int), ws));
-        RS_CUDA(cudaMemsetAsync(shared.owned, 0xFF, kSharedCtas * sizeof(unsigned int), ws));
-      }
+      if (share) shared.epoch++;
       int r = launch_split_level(a, mx, trials, max_leaf, tables, sm_count, ws, share ? &shared : nullptr);
       if (r) return r;
       for (uint32_t c = 0; c < nclass; c++)
@@ -862,10 +931,8 @@ int build_sets(const SetInput* in, uint32_t count, const BuildOptions& opt, cuda
     if (!opt.use_graph) timer.mark();
     for (uint32_t c = 0; c < nclass; c++) {
       a.cls = c;
-      if (share_leaves[c]) {
-        RS_CUDA(cudaMemsetAsync(shared.flag, 0, full_cap[c] * sizeof(unsigned int), ws));
-        RS_CUDA(cudaMemsetAsync(shared.owned, 0xFF, kSharedCtas * sizeof(unsigned int), ws));
-      }
+      a.work_counter = leaf_work + 2 * c;
+      if (share_leaves[c]) shared.epoch++;
       int r = launch_leaves(a, class_leaf[c], class_extra[c], sm_count, ws, share_leaves[c] ? &shared : nullptr);
       if (r) return r;
     }
@@ -875,15 +942,12 @@ int build_sets(const SetInput* in, uint32_t count, const BuildOptions& opt, cuda
                                                      bits);
       count_launch();
     }
-    int r = exclusive_scan_u64(bits, off, NB, ws);
+    int r = exclusive_scan_u64(bits, off, NB, scan_tmp, ws);
     if (r) return r;
-    RS_CUDA(cudaMemsetAsync(set_db, 0x7F, count * sizeof(long long), ws));
     if (bucket_tiles) {
-      k_ef_prepare<<<static_cast<unsigned>(bucket_tiles), kBlock, 0, ws>>>(d_sets, count, rstart, off, set_db);
+      k_ef_prepare<<<static_cast<unsigned>(bucket_tiles), kBlock, 0, ws>>>(d_sets, count, rstart, off, cbase, results);
       count_launch();
     }
-    k_set_scalars<<<grid_for(count), kBlock, 0, ws>>>(d_sets, count, off, cbase, rstart, set_T, set_codes, set_R);
-    count_launch();
     RS_CUDA(cudaGetLastError());
     return RECSPLIT_OK;
   };
@@ -909,18 +973,27 @@ int build_sets(const SetInput* in, uint32_t count, const BuildOptions& opt, cuda
   }
 
   // sync 2: per-set tree size and minimum delta of the offsets list
-  std::vector<long long> h_db(count);
+  std::vector<long long> h_db(count, 0);
   std::vector<uint64_t> h_T(count), h_codes(count), h_R(count);
   int herr = 0;
-  // the deadline wait comes first: a copy into pageable host memory would
-  // itself wait for the whole search
-  if ((rc = wait_stream(s, d_error, timeout_ms(), t_call))) return rc;
-  RS_CUDA(cudaMemcpyAsync(h_T.data(), set_T, count * sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
-  RS_CUDA(cudaMemcpyAsync(h_codes.data(), set_codes, count * sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
-  RS_CUDA(cudaMemcpyAsync(h_R.data(), set_R, count * sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
-  RS_CUDA(cudaMemcpyAsync(h_db.data(), set_db, count * sizeof(long long), cudaMemcpyDeviceToHost, s));
-  RS_CUDA(cudaMemcpyAsync(&herr, d_error, sizeof(int), cudaMemcpyDeviceToHost, s));
-  RS_CUDA(cudaStreamSynchronize(s));
+  {
+    // the deadline wait comes before a copy into pageable memory, which would
+    // itself wait for the whole search
+    Readback back(n_back2);
+    if (!back.pinned && (rc = wait_stream(s, d_error, timeout_ms(), t_call))) return rc;
+    RS_CUDA(cudaMemcpyAsync(back.words, back2, n_back2 * sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
+    if (back.pinned)
+      rc = wait_stream(s, d_error, timeout_ms(), t_call);
+    else
+      RS_CUDA(cudaStreamSynchronize(s));
+    if (rc) return rc;
+    std::copy_n(back.words, count, h_T.begin());
+    std::copy_n(back.words + count, count, h_codes.begin());
+    std::copy_n(back.words + 2 * uint64_t(count), count, h_R.begin());
+    for (uint32_t i = 0; i < count; i++)
+      if (const uint64_t d = back.words[3 * uint64_t(count) + i]) h_db[i] = static_cast<long long>(~d ^ (1ull << 63));
+    herr = static_cast<int>(back.words[4 * uint64_t(count)]);
+  }
   if (herr == RECSPLIT_E_DUPLICATE) return fail(herr, "two keys share their lower signature half (duplicate keys)");
   if (herr == RECSPLIT_E_SEARCH_LIMIT) return fail(herr, "seed search exceeded its limit");
   if (herr) return fail(herr, "a queue capacity or bucket code length check failed");
@@ -975,6 +1048,8 @@ int build_sets(const SetInput* in, uint32_t count, const BuildOptions& opt, cuda
   for (uint32_t i = 0; i < count; i++) {
     uint64_t* blob = d_arena + blob_off[i];
     DevOut& o = houts[i];
+    o.blob = blob;
+    std::copy_n(headers.data() + uint64_t(i) * kHeaderWords, kHeaderWords, o.header);
     o.tree = blob + layouts[i].tree;
     o.lower = blob + layouts[i].lower;
     o.upper_a = blob + layouts[i].upper_a;
@@ -982,17 +1057,8 @@ int build_sets(const SetInput* in, uint32_t count, const BuildOptions& opt, cuda
     o.anchors = blob + layouts[i].anchors;
     o.subs = reinterpret_cast<uint16_t*>(blob + layouts[i].subs);
   }
-  DevOut* d_outs;
-  uint64_t *d_headers, *d_blob_off;
-  if ((rc = sc.alloc(&d_outs, count)) || (rc = sc.alloc(&d_headers, headers.size())) ||
-      (rc = sc.alloc(&d_blob_off, count + 1)))
-    return rc;
   RS_CUDA(cudaMemsetAsync(d_arena, 0, blob_off[count] * sizeof(uint64_t), s));
   RS_CUDA(cudaMemcpyAsync(d_outs, houts.data(), count * sizeof(DevOut), cudaMemcpyHostToDevice, s));
-  RS_CUDA(cudaMemcpyAsync(d_headers, headers.data(), headers.size() * sizeof(uint64_t), cudaMemcpyHostToDevice, s));
-  RS_CUDA(cudaMemcpyAsync(d_blob_off, blob_off.data(), (count + 1) * sizeof(uint64_t), cudaMemcpyHostToDevice, s));
-  k_headers<<<grid_for(uint64_t(count) * kHeaderWords), kBlock, 0, s>>>(d_headers, d_blob_off, count, d_arena);
-  count_launch();
 
   // A6: Golomb-Rice codes; A7: Elias-Fano
   if (NB) {

@@ -188,9 +188,9 @@ int cuda_fail(cudaError_t e, const char* what);
 
 // ---------------------------------------------------------------- launchers
 // Exclusive scan of `count` uint64 values: out[0..count] with out[count] =
-// total.  `in` and `out` may alias.  Temporary storage comes from the
-// stream-ordered allocator.
-int exclusive_scan_u64(const uint64_t* in, uint64_t* out, uint64_t count, cudaStream_t s);
+// total.  `in` and `out` may alias.  scratch: scan_scratch(count) words.
+uint64_t scan_scratch(uint64_t count);
+int exclusive_scan_u64(const uint64_t* in, uint64_t* out, uint64_t count, uint64_t* scratch, cudaStream_t s);
 
 // Kinds of key input.
 struct KeyInput {
@@ -259,7 +259,7 @@ struct SearchArgs {
   uint32_t* full_n;                       // per class
   Node* part_q[kMaxClasses];              // leaves of 2 .. leaf-1 keys
   uint32_t* part_n;                       // per class
-  uint32_t* work_counter;                 // dynamic scheduling counter (zeroed per launch)
+  uint32_t* work_counter;                 // dynamic scheduling counter of the launch, zero (launch_leaves: two)
   int* error;                             // first error code
   uint32_t cls;                           // class of a leaf launch
   uint32_t extra_of[kMaxClasses];         // leaf range extra per class
@@ -273,9 +273,10 @@ struct SearchArgs {
 
 // State of the nodes of one split level, or of a class's full leaves, for the
 // shared search (search.cu): per node its best index so far, block counter,
-// participants, most participants and state (0 none, 1 open, 2 closed; zeroed
-// per launch), and per CTA the node it owns (~0 when none; set to ~0 per
-// launch).  kSharedCtas bounds the grid.
+// participants, most participants and state (2 epoch - 1 open, 2 epoch closed,
+// smaller none), and per CTA the node it owns plus 1 (0 when none: as it leaves
+// it).  flag and owned start as zeros; every launch has an epoch of its own,
+// from 1.  kSharedCtas bounds the grid.
 struct SharedNodes {
   uint64_t* best;
   unsigned int* next;
@@ -283,6 +284,7 @@ struct SharedNodes {
   unsigned int* cap;  // most participants a node takes
   unsigned int* flag;
   unsigned int* owned;
+  unsigned int epoch;
 };
 constexpr uint32_t kSharedCtas = 4096;
 
@@ -294,7 +296,7 @@ constexpr uint32_t kSharedCtas = 4096;
 int launch_split_level(const SearchArgs& a, uint64_t max_m, uint64_t trials, uint32_t max_leaf, bool tables,
                        int sm_count, cudaStream_t s, const SharedNodes* share = nullptr);
 // Whether the full leaves of a class are searched shared (launch_leaves then
-// needs share, zeroed as above).
+// needs share).
 bool leaves_shared(uint32_t leaf, uint32_t extra);
 int launch_leaves(const SearchArgs& a, uint32_t leaf, uint32_t extra, int sm_count, cudaStream_t s,
                   const SharedNodes* share = nullptr);

@@ -71,7 +71,13 @@ __global__ void __launch_bounds__(kThreads) k_tile_scan(const uint64_t* in, uint
 
 }  // namespace
 
-int exclusive_scan_u64(const uint64_t* in, uint64_t* out, uint64_t count, cudaStream_t s) {
+// Words of temporary storage a scan of `count` values takes.
+uint64_t scan_scratch(uint64_t count) {
+  const uint64_t tiles = (count + kTile - 1) / kTile;
+  return tiles <= 1 ? 0 : tiles + 1 + scan_scratch(tiles);
+}
+
+int exclusive_scan_u64(const uint64_t* in, uint64_t* out, uint64_t count, uint64_t* scratch, cudaStream_t s) {
   if (count == 0) {
     RS_CUDA(cudaMemsetAsync(out, 0, sizeof(uint64_t), s));
     return RECSPLIT_OK;
@@ -83,18 +89,14 @@ int exclusive_scan_u64(const uint64_t* in, uint64_t* out, uint64_t count, cudaSt
     RS_CUDA(cudaGetLastError());
     return RECSPLIT_OK;
   }
-  uint64_t* sums = nullptr;
-  int rc0 = pool_alloc(reinterpret_cast<void**>(&sums), (tiles + 1) * sizeof(uint64_t), s);
-  if (rc0) return rc0;
-  k_tile_sums<<<static_cast<unsigned>(tiles), kThreads, 0, s>>>(in, count, sums);
+  k_tile_sums<<<static_cast<unsigned>(tiles), kThreads, 0, s>>>(in, count, scratch);
   count_launch();
   RS_CUDA(cudaGetLastError());
-  int rc = exclusive_scan_u64(sums, sums, tiles, s);
+  int rc = exclusive_scan_u64(scratch, scratch, tiles, scratch + tiles + 1, s);
   if (rc) return rc;
-  k_tile_scan<<<static_cast<unsigned>(tiles), kThreads, 0, s>>>(in, out, count, sums);
+  k_tile_scan<<<static_cast<unsigned>(tiles), kThreads, 0, s>>>(in, out, count, scratch);
   count_launch();
   RS_CUDA(cudaGetLastError());
-  RS_CUDA(cudaFreeAsync(sums, s));
   return RECSPLIT_OK;
 }
 

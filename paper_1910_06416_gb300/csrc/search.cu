@@ -562,7 +562,9 @@ __global__ void __launch_bounds__(kThreads, 4) k_split_level(SearchArgs a, uint3
   const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (COUNT && lane == 0) wexec[warp] = 0;
   const uint32_t total = *a.split_in_count;
-  gwarps = group_warps(gwarps, total, spread);
+  // (a counting build keeps the launch shape: with one warp per node its count is
+  // the same in every build)
+  if (!COUNT) gwarps = group_warps(gwarps, total, spread);
   const uint32_t gid = warp / gwarps, wig = warp % gwarps;
   const uint32_t tig = wig * 32 + lane, gthreads = gwarps * 32;
   const bool leader = wig == 0 && lane == 0;
@@ -627,7 +629,6 @@ __global__ void __launch_bounds__(kThreads, 4) k_split_level(SearchArgs a, uint3
 // The last participant to leave (refs drops to 0 and it closes the node)
 // partitions the keys and queues the children.
 constexpr uint32_t kShareRounds = 4;
-constexpr uint32_t kNodeOpen = 1, kNodeClosed = 2;
 constexpr uint32_t kMaxJoins = 4096;  // nodes one CTA may join in one launch
 
 // Two-phase test of one claimed block (kShareRounds * 32 indices from base0)
@@ -776,8 +777,7 @@ __device__ __forceinline__ uint64_t shared_search(const uint64_t* __restrict__ k
 // begin(node) (the whole CTA), search(node, idx) (every warp; claims blocks
 // through st.next[idx], lowers st.best[idx]) and, in the last participant to
 // leave, close(node, index found).  The node state arrays are sized by the
-// queue's capacity, `flag` zeroed and `owned` (one entry per CTA) set to ~0
-// before the launch.  A node takes at most cap_of(node) CTAs at once.
+// queue's capacity.  A node takes at most cap_of(node) CTAs at once.
 template <typename Cap, typename Begin, typename Search, typename Close>
 __device__ __forceinline__ void shared_nodes(const Node* queue, uint32_t total, const SharedNodes& st,
                                              uint32_t* work_counter, int* error, Cap cap_of, Begin begin,
@@ -785,6 +785,7 @@ __device__ __forceinline__ void shared_nodes(const Node* queue, uint32_t total, 
   __shared__ uint32_t task, owner, closer, drained;
   const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   volatile uint32_t* vflag = st.flag;
+  const uint32_t kNodeOpen = 2 * st.epoch - 1, kNodeClosed = 2 * st.epoch;
   uint32_t joins = 0;  // nodes joined: bounded, so that the kernel ends whatever the timing
   if (threadIdx.x == 0) drained = 0;
   __syncthreads();
@@ -803,7 +804,7 @@ __device__ __forceinline__ void shared_nodes(const Node* queue, uint32_t total, 
           st.cap[i] = cap_of(queue[i]);
           __threadfence();
           vflag[i] = kNodeOpen;
-          reinterpret_cast<volatile uint32_t*>(st.owned)[blockIdx.x] = i;
+          reinterpret_cast<volatile uint32_t*>(st.owned)[blockIdx.x] = i + 1;
         } else {
           drained = 1;
         }
@@ -819,7 +820,7 @@ __device__ __forceinline__ void shared_nodes(const Node* queue, uint32_t total, 
         uint32_t pick = total, fewest = ~0u;
         for (uint32_t k0 = 0; k0 < gridDim.x; k0 += 32) {
           const uint32_t k = k0 + lane;
-          const uint32_t j = k < gridDim.x ? reinterpret_cast<volatile uint32_t*>(st.owned)[k] : ~0u;
+          const uint32_t j = k < gridDim.x ? reinterpret_cast<volatile uint32_t*>(st.owned)[k] - 1 : ~0u;
           uint32_t r = ~0u;
           if (j < total && vflag[j] == kNodeOpen) {
             const uint32_t refs = reinterpret_cast<volatile uint32_t*>(st.refs)[j];
@@ -860,7 +861,7 @@ __device__ __forceinline__ void shared_nodes(const Node* queue, uint32_t total, 
       __threadfence();
       const uint32_t left = atomicSub(&st.refs[idx], 1u);
       closer = left == 1 && atomicCAS(&st.flag[idx], kNodeOpen, kNodeClosed) == kNodeOpen;
-      if (owner) reinterpret_cast<volatile uint32_t*>(st.owned)[blockIdx.x] = ~0u;
+      if (owner) reinterpret_cast<volatile uint32_t*>(st.owned)[blockIdx.x] = 0;
     }
     __syncthreads();
     if (closer) {
@@ -1779,7 +1780,6 @@ int launch_persistent(K kern, int max_blocks, const SearchArgs& a, int sm_count,
   int blocks = 0;
   int rc = persistent_grid(kern, 0, sm_count, &blocks);
   if (rc) return rc;
-  RS_CUDA(cudaMemsetAsync(a.work_counter, 0, sizeof(uint32_t), s));
   kern<<<std::min(blocks, max_blocks), kThreads, 0, s>>>(a, args...);
   count_launch();
   RS_CUDA(cudaGetLastError());
@@ -1902,7 +1902,6 @@ int launch_split_level(const SearchArgs& a, uint64_t max_m, uint64_t trials, uin
     rc = persistent_grid(kern, smem, sm_count, &blocks);
     if (rc) return rc;
     blocks = std::min<int>(blocks, kSharedCtas);
-    RS_CUDA(cudaMemsetAsync(a.work_counter, 0, sizeof(uint32_t), s));
     kern<<<blocks, kThreads, smem, s>>>(a, *share, static_cast<uint32_t>(cap), uint32_t(tables));
     count_launch();
     RS_CUDA(cudaGetLastError());
@@ -1921,7 +1920,6 @@ int launch_split_level(const SearchArgs& a, uint64_t max_m, uint64_t trials, uin
   int blocks = 0;
   rc = persistent_grid(kern, smem, sm_count, &blocks);
   if (rc) return rc;
-  RS_CUDA(cudaMemsetAsync(a.work_counter, 0, sizeof(uint32_t), s));
   kern<<<blocks, kThreads, smem, s>>>(a, gwarps, static_cast<uint32_t>(cap), uint32_t(tables), group_spread(trials));
   count_launch();
   RS_CUDA(cudaGetLastError());
@@ -1938,14 +1936,16 @@ int launch_leaves(const SearchArgs& a, uint32_t leaf, uint32_t extra, int sm_cou
   const recsplit_tuning_t t = tuning_for(leaf);
   int rc = (extra ? kFullRange : kFull)[leaf](a, t, sm_count, s, share);
   if (rc || leaf == 2) return rc;  // no leaves between 2 and leaf - 1
+  SearchArgs b = a;
+  b.work_counter++;
   if (extra)
-    return leaf <= 8    ? launch_any<8, true>(a, t, sm_count, s, 0)
-           : leaf <= 16 ? launch_any<16, true>(a, t, sm_count, s, 0)
-                        : launch_any<24, true>(a, t, sm_count, s, 0);
-  return leaf <= 8    ? launch_any<8, false>(a, t, sm_count, s, 0)
-         : leaf <= 12 ? launch_any<12, false>(a, t, sm_count, s, 0)
-         : leaf <= 16 ? launch_any<16, false>(a, t, sm_count, s, 0)
-                      : launch_any<24, false>(a, t, sm_count, s, 0);
+    return leaf <= 8    ? launch_any<8, true>(b, t, sm_count, s, 0)
+           : leaf <= 16 ? launch_any<16, true>(b, t, sm_count, s, 0)
+                        : launch_any<24, true>(b, t, sm_count, s, 0);
+  return leaf <= 8    ? launch_any<8, false>(b, t, sm_count, s, 0)
+         : leaf <= 12 ? launch_any<12, false>(b, t, sm_count, s, 0)
+         : leaf <= 16 ? launch_any<16, false>(b, t, sm_count, s, 0)
+                      : launch_any<24, false>(b, t, sm_count, s, 0);
 }
 
 }  // namespace rs
