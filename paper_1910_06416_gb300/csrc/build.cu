@@ -23,6 +23,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "device.cuh"
+#include "lookback.cuh"
 
 namespace rs {
 
@@ -49,6 +50,8 @@ struct DevSet {
   uint64_t n, key_base, nb, bucket_base;
   uint32_t cls, leaf;
   uint64_t key_tile_base, bucket_tile_base, elem_tile_base;  // first block of the set in each tiling
+  uint64_t lane_base;     // first lane of the set in the kernels over codes (bucket_lane)
+  uint32_t warp_buckets;  // a warp per bucket there, else a lane
 };
 
 // Set whose tile range contains block `blk` (tile bases are non-decreasing).
@@ -141,22 +144,6 @@ struct ClassTables {
   uint32_t leaf[kMaxClasses];
 };
 
-__global__ void k_bucket_codes(const uint64_t* __restrict__ counts, const uint32_t* __restrict__ bset,
-                               const DevSet* __restrict__ sets, uint64_t nbt, ClassTables ct,
-                               uint64_t* __restrict__ codes) {
-  for (uint64_t b = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; b < nbt; b += uint64_t(gridDim.x) * blockDim.x)
-    codes[b] = ct.t[sets[bset[b]].cls][kTableWords * counts[b]] >> 32;
-}
-
-// Output range of every bucket (table word 3, upper half): the sum of its
-// leaves' ranges, which is the bucket size when the leaf range extra is 0.
-__global__ void k_bucket_ranges(const uint64_t* __restrict__ counts, const uint32_t* __restrict__ bset,
-                                const DevSet* __restrict__ sets, uint64_t nbt, ClassTables ct,
-                                uint64_t* __restrict__ ranges) {
-  for (uint64_t b = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; b < nbt; b += uint64_t(gridDim.x) * blockDim.x)
-    ranges[b] = ct.t[sets[bset[b]].cls][kTableWords * counts[b] + 3] >> 32;
-}
-
 // Sec. 9: grouping by bucket; the order inside a bucket does not matter
 // (every search depends on the set only).  Keys are stored as x ^ (x >> 30)
 // of their lower half, the form the searches consume.
@@ -170,78 +157,164 @@ __global__ void k_scatter(const uint32_t* __restrict__ bucket, const uint64_t* _
   }
 }
 
-// Every bucket of two or more keys is appended to the queue of its kind
-// (split node, full leaf, partial leaf).  The lanes of a warp that append to
-// the same queue take their slots with one atomic: with buckets of a few keys
-// there are millions of appends to a handful of counters, and one atomic per
-// bucket on the same address serialises them.
-__global__ void k_roots(const uint64_t* __restrict__ counts, const uint64_t* __restrict__ bstart,
-                        const uint64_t* __restrict__ cbase, const uint32_t* __restrict__ bset,
-                        const DevSet* __restrict__ sets, uint64_t nbt, SearchArgs a) {
-  const uint32_t lane = threadIdx.x & 31;
-  const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
-  // the loop bound is uniform across the warp: every lane reaches the ballot
-  for (uint64_t w0 = blockIdx.x * uint64_t(blockDim.x) + (threadIdx.x & ~31u); w0 < nbt; w0 += stride) {
-    const uint64_t b = w0 + lane;
-    const uint64_t m = b < nbt ? counts[b] : 0;
-    const bool want = m >= 2;
-    Node nd{};
-    Node* q = nullptr;
-    uint32_t* cnt = nullptr;
-    uint32_t cap = 0;
-    if (want) {
-      const DevSet& st = sets[bset[b]];
-      nd = Node{static_cast<uint32_t>(bstart[b]), static_cast<uint32_t>(m), static_cast<uint32_t>(cbase[b]),
-                st.cls << 8};
-      if (m > st.leaf)
-        q = a.split_in, cnt = a.split_in_count, cap = a.split_cap;
-      else if (m == st.leaf)
-        q = a.full_q[st.cls], cnt = a.full_n + st.cls, cap = a.full_cap[st.cls];
-      else
-        q = a.part_q[st.cls], cnt = a.part_n + st.cls, cap = a.part_cap[st.cls];
+// Prefix sums over the buckets of all sets of their keys (s_i, bstart), codes
+// (first code slot, cbase) and, with RANGE, output ranges (table word 3, upper
+// half: the sum of the leaves' ranges), and the first queue entries, in one
+// launch: every bucket of two or more keys is appended to the queue of its
+// kind (split node, full leaf, partial leaf).  The lanes of a warp that append
+// to the same queue take their slots with one atomic: with buckets of a few
+// keys there are millions of appends to a handful of counters, and one atomic
+// per bucket on the same address serialises them.
+constexpr int kGroupItems = 4;
+constexpr uint64_t kGroupTile = uint64_t(kBlock) * kGroupItems;
+
+template <bool RANGE>
+__global__ void __launch_bounds__(kBlock) k_group_scan(const uint64_t* __restrict__ counts,
+                                                       const uint32_t* __restrict__ bset,
+                                                       const DevSet* __restrict__ sets, uint64_t nbt, ClassTables ct,
+                                                       uint64_t* __restrict__ bstart, uint64_t* __restrict__ cbase,
+                                                       uint64_t* __restrict__ rstart, LookState st, SearchArgs a) {
+  constexpr int N = RANGE ? 3 : 2;
+  __shared__ uint32_t tile_s;
+  __shared__ uint64_t before_s[N];
+  if (threadIdx.x == 0) tile_s = atomicAdd(st.ticket, 1u);
+  __syncthreads();
+  const uint32_t tile = tile_s, lane = threadIdx.x & 31;
+  const uint64_t base = tile * kGroupTile + threadIdx.x * uint64_t(kGroupItems);
+  uint32_t m[kGroupItems], cls[kGroupItems], codes[kGroupItems], range[kGroupItems];
+  uint64_t s[N] = {}, run[N], total[N];
+#pragma unroll
+  for (int k = 0; k < kGroupItems; k++) {
+    const uint64_t b = base + k;
+    m[k] = cls[k] = codes[k] = range[k] = 0;
+    if (b < nbt) {
+      m[k] = static_cast<uint32_t>(counts[b]);  // at most 2^32 - 1 keys in all
+      cls[k] = sets[bset[b]].cls;
+      const uint64_t* t = ct.t[cls[k]] + kTableWords * uint64_t(m[k]);
+      codes[k] = static_cast<uint32_t>(t[0] >> 32);
+      if (RANGE) range[k] = static_cast<uint32_t>(t[3] >> 32);
     }
+    s[0] += m[k];
+    s[1] += codes[k];
+    if (RANGE) s[N - 1] += range[k];
+  }
+  block_scan<N, kBlock>(s, run, total);
+  if (threadIdx.x < 32) {
+    uint64_t before[N];
+    look_back<N>(st, tile, total, before, a.error);
+    if (threadIdx.x == 0)
+      for (int k = 0; k < N; k++) before_s[k] = before[k];
+  }
+  __syncthreads();
+  uint64_t at = run[0] + before_s[0], slot = run[1] + before_s[1], rat = RANGE ? run[N - 1] + before_s[N - 1] : 0;
+#pragma unroll
+  for (int k = 0; k < kGroupItems; k++) {
+    const uint64_t b = base + k;
+    if (b < nbt) {
+      bstart[b] = at;
+      cbase[b] = slot;
+      if (RANGE) rstart[b] = rat;
+    }
+    const bool want = m[k] >= 2;
     const uint32_t active = __ballot_sync(0xFFFFFFFFu, want);
-    if (!want) continue;
-    const uint32_t peers = __match_any_sync(active, reinterpret_cast<unsigned long long>(cnt));
-    const uint32_t leader = __ffs(peers) - 1;
-    uint32_t base = 0;
-    if (lane == leader) base = atomicAdd(cnt, static_cast<uint32_t>(__popc(peers)));
-    base = __shfl_sync(peers, base, leader);
-    const uint32_t at = base + __popc(peers & ((1u << lane) - 1));
-    if (at < cap)
-      q[at] = nd;
-    else
-      atomicCAS(a.error, 0, RECSPLIT_E_INVALID);
+    if (want) {
+      const uint32_t c = cls[k], leaf = a.leaf_of[c];
+      Node* q;
+      uint32_t *cnt, cap;
+      if (m[k] > leaf)
+        q = a.split_in, cnt = a.split_in_count, cap = a.split_cap;
+      else if (m[k] == leaf)
+        q = a.full_q[c], cnt = a.full_n + c, cap = a.full_cap[c];
+      else
+        q = a.part_q[c], cnt = a.part_n + c, cap = a.part_cap[c];
+      const uint32_t peers = __match_any_sync(active, reinterpret_cast<unsigned long long>(cnt));
+      const uint32_t leader = __ffs(peers) - 1;
+      uint32_t first = 0;
+      if (lane == leader) first = atomicAdd(cnt, static_cast<uint32_t>(__popc(peers)));
+      first = __shfl_sync(peers, first, leader);
+      const uint32_t e = first + __popc(peers & ((1u << lane) - 1));
+      if (e < cap)
+        q[e] = Node{static_cast<uint32_t>(at), m[k], static_cast<uint32_t>(slot), c << 8};
+      else
+        atomicCAS(a.error, 0, RECSPLIT_E_INVALID);
+    }
+    __syncwarp();
+    at += m[k];
+    slot += codes[k];
+    rat += range[k];
+  }
+  if (threadIdx.x == kBlock - 1 && (tile + 1) * kGroupTile >= nbt) {
+    bstart[nbt] = at;
+    cbase[nbt] = slot;
+    if (RANGE) rstart[nbt] = rat;
   }
 }
 
 // ---------------------------------------------------------------- A5
+// The kernels over the codes of buckets take a lane per bucket where buckets
+// have a few codes and a warp per bucket where they have more: one lane walking
+// the 360 codes of a bucket (l = 12, b = 2000) held the lengths of a batched
+// build at 0.35 ms and the writing at 0.45 ms.  Lanes are numbered per set from
+// a multiple of 32; lane_set finds the set of a warp.
+// A warp pays from 64 codes, and from 8 on few buckets, where the time is one
+// lane's chain of loads (10 buckets of 18 codes: lengths and writing 9 + 12 -> 4
+// + 4 us); on 10^5 such buckets the lanes are the faster (34 us against 81 us,
+// for the atomic per code of the warp's writing).
+constexpr uint64_t kWarpCodes = 64, kFewWarpCodes = 8, kFewBuckets = 8192;
+
+struct BucketLane {
+  uint32_t set;     // ~0: no bucket
+  uint64_t bucket;  // global index
+  bool whole_warp;
+};
+__device__ __forceinline__ BucketLane bucket_lane(const DevSet* sets, uint32_t count) {
+  const uint64_t t = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x;
+  uint32_t lo = 0, hi = count;  // last set with lane_base <= the warp's first lane
+  while (hi - lo > 1) {
+    const uint32_t mid = (lo + hi) >> 1;
+    if (sets[mid].lane_base <= (t & ~uint64_t(31))) lo = mid; else hi = mid;
+  }
+  const DevSet& st = sets[lo];
+  const bool whole = st.warp_buckets != 0;
+  const uint64_t j = (t - st.lane_base) >> (whole ? 5 : 0);
+  return BucketLane{t >= st.lane_base && j < st.nb ? lo : ~0u, st.bucket_base + j, whole};
+}
+
 // Bits of bucket b: fixed bits of its tree (table) + unary parts (i >> r) + 1.
 // After a failed search (error set) the slots of unsearched nodes were never
 // written: the lengths are then not computed (the build reports the error).
 // Lookups address the bits of a bucket with 32-bit offsets, so a bucket whose
 // code reaches 2^32 bits (more than a billion keys in one bucket) fails the
 // build with RECSPLIT_E_INVALID.
-__global__ void k_bucket_bits(const uint64_t* __restrict__ counts, const uint64_t* __restrict__ cbase,
-                              const uint64_t* __restrict__ seeds, const uint32_t* __restrict__ sizes,
-                              const uint32_t* __restrict__ bset, const DevSet* __restrict__ sets, ClassTables ct,
-                              uint64_t nbt, int* __restrict__ error, uint64_t* __restrict__ bits) {
+__global__ void __launch_bounds__(kBlock) k_bucket_bits(const uint64_t* __restrict__ counts,
+                                                        const uint64_t* __restrict__ cbase,
+                                                        const uint64_t* __restrict__ seeds,
+                                                        const uint32_t* __restrict__ sizes,
+                                                        const DevSet* __restrict__ sets, uint32_t count,
+                                                        ClassTables ct, int* __restrict__ error,
+                                                        uint64_t* __restrict__ bits) {
   const bool failed = *reinterpret_cast<const volatile int*>(error) != 0;
-  for (uint64_t b = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; b < nbt; b += uint64_t(gridDim.x) * blockDim.x) {
-    const uint32_t cls = sets[bset[b]].cls;
-    const uint64_t* table = ct.t[cls];
-    const uint64_t m = counts[b];
-    uint64_t len = static_cast<uint32_t>(table[kTableWords * m]);
-    if (!failed) {
-      for (uint64_t c = cbase[b], e = cbase[b + 1]; c < e; c++) {
-        const uint32_t sz = sizes[c];
-        const uint32_t r = sz <= ct.mmax[cls] ? static_cast<uint32_t>(table[kTableWords * sz + 1] >> 40) & 31 : 0;
-        len += (seeds[c] >> r) + 1;
-      }
-      if (len >= (1ull << 32)) atomicCAS(error, 0, RECSPLIT_E_INVALID);
+  const BucketLane bl = bucket_lane(sets, count);
+  if (bl.set == ~0u) return;  // whole warps, or single lanes
+  const uint32_t cls = sets[bl.set].cls;
+  const uint64_t* table = ct.t[cls];
+  const uint64_t mmax = ct.mmax[cls];
+  const uint32_t step = bl.whole_warp ? 32 : 1;
+  uint64_t len = 0;
+  if (!failed)
+    for (uint64_t c = cbase[bl.bucket] + (bl.whole_warp ? threadIdx.x & 31 : 0), e = cbase[bl.bucket + 1]; c < e;
+         c += step) {
+      const uint32_t sz = sizes[c];
+      const uint32_t r = sz <= mmax ? static_cast<uint32_t>(table[kTableWords * sz + 1] >> 40) & 31 : 0;
+      len += (seeds[c] >> r) + 1;
     }
-    bits[b] = len;
+  if (bl.whole_warp) {
+    for (int o = 16; o; o >>= 1) len += __shfl_xor_sync(0xFFFFFFFFu, len, o);
+    if (threadIdx.x & 31) return;
   }
+  len += static_cast<uint32_t>(table[kTableWords * counts[bl.bucket]]);
+  if (!failed && len >= (1ull << 32)) atomicCAS(error, 0, RECSPLIT_E_INVALID);
+  bits[bl.bucket] = len;
 }
 
 __device__ __forceinline__ uint64_t mulhi32_shift(uint64_t a, uint64_t b) {
@@ -353,24 +426,30 @@ struct DevOut {
 };
 
 // Per bucket: fixed parts of all codes in preorder from o_b, then the unary
-// parts from o_b + F(m) (Sec. 6.2).
-__global__ void k_write_codes(const uint64_t* __restrict__ counts, const uint64_t* __restrict__ cbase,
-                              const uint64_t* __restrict__ seeds, const uint32_t* __restrict__ sizes,
-                              const uint32_t* __restrict__ bset, const DevSet* __restrict__ sets,
-                              const DevOut* __restrict__ outs, ClassTables ct, const uint64_t* __restrict__ off,
-                              uint64_t nbt) {
-  for (uint64_t b = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; b < nbt; b += uint64_t(gridDim.x) * blockDim.x) {
-    const uint64_t m = counts[b];
-    if (m < 2) continue;
-    const uint32_t si = bset[b];
-    const uint64_t* table = ct.t[sets[si].cls];
-    uint64_t* tree = outs[si].tree;
-    const uint64_t base = off[b] - off[sets[si].bucket_base];
-    uint64_t fpos = base;
-    uint64_t upos = base + static_cast<uint32_t>(table[kTableWords * m]);
+// parts from o_b + F(m) (Sec. 6.2).  A warp places 32 codes at a time with
+// prefix sums of their fixed and unary lengths.
+__global__ void __launch_bounds__(kBlock) k_write_codes(const uint64_t* __restrict__ counts,
+                                                        const uint64_t* __restrict__ cbase,
+                                                        const uint64_t* __restrict__ seeds,
+                                                        const uint32_t* __restrict__ sizes,
+                                                        const DevSet* __restrict__ sets, uint32_t count,
+                                                        const DevOut* __restrict__ outs, ClassTables ct,
+                                                        const uint64_t* __restrict__ off) {
+  const BucketLane bl = bucket_lane(sets, count);
+  if (bl.set == ~0u) return;  // whole warps, or single lanes
+  const uint64_t m = counts[bl.bucket];
+  if (m < 2) return;
+  const DevSet& st = sets[bl.set];
+  const uint64_t* table = ct.t[st.cls];
+  const uint64_t mmax = ct.mmax[st.cls];
+  uint64_t* tree = outs[bl.set].tree;
+  const uint64_t base = off[bl.bucket] - off[st.bucket_base];
+  uint64_t fpos = base;
+  uint64_t upos = base + static_cast<uint32_t>(table[kTableWords * m]);
+  const uint64_t first = cbase[bl.bucket], e = cbase[bl.bucket + 1];
+  if (!bl.whole_warp) {
     BitSink fixed{tree}, unary{tree};
-    const uint64_t mmax = ct.mmax[sets[si].cls];
-    for (uint64_t c = cbase[b], e = cbase[b + 1]; c < e; c++) {
+    for (uint64_t c = first; c < e; c++) {
       const uint32_t sz = sizes[c];
       const uint32_t r = sz <= mmax ? static_cast<uint32_t>(table[kTableWords * sz + 1] >> 40) & 31 : 0;
       const uint64_t s = seeds[c];
@@ -382,6 +461,35 @@ __global__ void k_write_codes(const uint64_t* __restrict__ counts, const uint64_
     }
     fixed.flush();
     unary.flush();
+    return;
+  }
+  const uint32_t lane = threadIdx.x & 31;
+  for (uint64_t c0 = first; c0 < e; c0 += 32) {
+    const uint64_t c = c0 + lane;
+    uint32_t r = 0;
+    uint64_t s = 0, u = 0;  // unary length
+    if (c < e) {
+      const uint32_t sz = sizes[c];
+      r = sz <= mmax ? static_cast<uint32_t>(table[kTableWords * sz + 1] >> 40) & 31 : 0;
+      s = seeds[c];
+      u = (s >> r) + 1;
+    }
+    uint32_t fr = r;
+    uint64_t ur = u;
+    for (uint32_t d = 1; d < 32; d <<= 1) {
+      const uint32_t x = __shfl_up_sync(0xFFFFFFFFu, fr, d);
+      const uint64_t y = __shfl_up_sync(0xFFFFFFFFu, ur, d);
+      if (lane >= d) {
+        fr += x;
+        ur += y;
+      }
+    }
+    if (c < e) {
+      or_bits(tree, fpos + fr - r, r ? (s & ((1ull << r) - 1)) : 0, r);
+      or_bits(tree, upos + ur - 1, 1, 1);
+    }
+    fpos += __shfl_sync(0xFFFFFFFFu, fr, 31);
+    upos += __shfl_sync(0xFFFFFFFFu, ur, 31);
   }
 }
 
@@ -673,7 +781,11 @@ int build_sets(const SetInput* in, uint32_t count, const BuildOptions& opt, cuda
   sc.plan(&sizes, K + 1);
   sc.plan(&back1, n_back1);
   sc.plan(&back2, n_back2);
-  sc.plan(&counters, 2 * kLevels + 4 * kMaxClasses);
+  sc.plan(&counters, 2 * kLevels + 4 * kMaxClasses + 2);
+  // scans: group_scan's tiles, then those of the lengths
+  const uint64_t group_tiles = (NB + kGroupTile - 1) / kGroupTile, bit_tiles = scan_tiles(NB);
+  uint32_t* look_flags;
+  sc.plan(&look_flags, group_tiles + bit_tiles);
   if (count_work) sc.plan(&exec, 2);
   if ((rc = sc.alloc(/*zero=*/true))) return rc;
   unsigned long long* cls_max = reinterpret_cast<unsigned long long*>(back1);
@@ -688,11 +800,12 @@ int build_sets(const SetInput* in, uint32_t count, const BuildOptions& opt, cuda
   uint32_t* const leaf_work = level_work + kLevels;   // two leaf launches per class
   uint32_t* const full_n = leaf_work + 2 * kMaxClasses;
   uint32_t* const part_n = full_n + kMaxClasses;
+  uint32_t* const tickets = part_n + kMaxClasses;
 
   DevSet* d_sets;
   DevOut* d_outs;
   uint32_t *bucket, *bset;
-  uint64_t *lo, *bstart, *codes, *cbase, *bits, *off, *scan_tmp, *ranges = nullptr;
+  uint64_t *lo, *bstart, *cbase, *bits, *off, *look;
   // prefix sums of the bucket output ranges: s_i itself unless a set has a
   // leaf range extra
   uint64_t* rstart = nullptr;
@@ -700,16 +813,12 @@ int build_sets(const SetInput* in, uint32_t count, const BuildOptions& opt, cuda
   sc.plan(&d_outs, count);
   if ((rc = sc.alloc())) return rc;
   sc.plan(&bstart, NB + 1);
-  sc.plan(&codes, NB + 1);
   sc.plan(&cbase, NB + 1);
   sc.plan(&bset, NB + 1);
   sc.plan(&bits, NB + 1);
   sc.plan(&off, NB + 1);
-  sc.plan(&scan_tmp, scan_scratch(NB));
-  if (any_extra) {
-    sc.plan(&ranges, NB + 1);
-    sc.plan(&rstart, NB + 1);
-  }
+  sc.plan(&look, 6 * std::max(group_tiles, bit_tiles));
+  if (any_extra) sc.plan(&rstart, NB + 1);
   if ((rc = sc.alloc()) || (rc = sc.alloc(&bucket, K)) || (rc = sc.alloc(&lo, K))) return rc;
   if (!any_extra) rstart = bstart;
   RS_CUDA(cudaMemcpyAsync(d_sets, hs.data(), count * sizeof(DevSet), cudaMemcpyHostToDevice, s));
@@ -762,20 +871,16 @@ int build_sets(const SetInput* in, uint32_t count, const BuildOptions& opt, cuda
     ct.leaf[c] = class_leaf[c];
   }
 
-  // prefix sums s_i and code-slot bases (global over all sets)
-  if ((rc = exclusive_scan_u64(counts, bstart, NB, scan_tmp, s))) return rc;
-  if (NB) {
-    k_bucket_codes<<<grid_for(NB), kBlock, 0, s>>>(counts, bset, d_sets, NB, ct, codes);
-    count_launch();
+  // lanes of the kernels over codes: by the codes of a mean bucket
+  uint64_t lanes = 0;
+  for (uint32_t i = 0; i < count; i++) {
+    DevSet& d = hs[i];
+    const uint64_t mean = d.nb ? std::min(T[d.cls].mmax, d.n / d.nb) : 0;
+    d.warp_buckets = T[d.cls].codes[mean] >= (NB <= kFewBuckets ? kFewWarpCodes : kWarpCodes);
+    d.lane_base = lanes;
+    lanes += d.warp_buckets ? d.nb * 32 : (d.nb + 31) & ~uint64_t(31);
   }
-  if ((rc = exclusive_scan_u64(codes, cbase, NB, scan_tmp, s))) return rc;
-  if (any_extra) {
-    if (NB) {
-      k_bucket_ranges<<<grid_for(NB), kBlock, 0, s>>>(counts, bset, d_sets, NB, ct, ranges);
-      count_launch();
-    }
-    if ((rc = exclusive_scan_u64(ranges, rstart, NB, scan_tmp, s))) return rc;
-  }
+  RS_CUDA(cudaMemcpyAsync(d_sets, hs.data(), count * sizeof(DevSet), cudaMemcpyHostToDevice, s));
 
   // grouping; queues: two split levels (ping-pong) shared by all classes, full
   // and partial leaves per class
@@ -785,11 +890,6 @@ int build_sets(const SetInput* in, uint32_t count, const BuildOptions& opt, cuda
   if ((rc = sc.alloc(&keys[0], K)) || (rc = sc.alloc(&keys[1], K)) || (rc = sc.alloc(&qmem, qtotal)) ||
       (rc = sc.alloc(&seeds, K + 1)))
     return rc;
-  if (K) {
-    k_scatter<<<std::min<unsigned>(grid_for(K), sm_count * 16), kBlock, 0, s>>>(bucket, lo, K, bstart, cursor,
-                                                                                 keys[0]);
-    count_launch();
-  }
   SearchArgs a{};
   a.keys[0] = keys[0];
   a.keys[1] = keys[1];
@@ -817,8 +917,20 @@ int build_sets(const SetInput* in, uint32_t count, const BuildOptions& opt, cuda
   a.exec_count = exec;
   a.split_in = q_split[0];
   a.split_in_count = level_n;
+  // prefix sums s_i, code-slot bases (global over all sets), first queue entries
   if (NB) {
-    k_roots<<<grid_for(NB), kBlock, 0, s>>>(counts, bstart, cbase, bset, d_sets, NB, a);
+    const LookState st{look_flags, look, look + 3 * std::max(group_tiles, bit_tiles), tickets};
+    (any_extra ? k_group_scan<true> : k_group_scan<false>)<<<static_cast<unsigned>(group_tiles), kBlock, 0, s>>>(
+        counts, bset, d_sets, NB, ct, bstart, cbase, rstart, st, a);
+    count_launch();
+  } else {
+    RS_CUDA(cudaMemsetAsync(bstart, 0, sizeof(uint64_t), s));
+    RS_CUDA(cudaMemsetAsync(cbase, 0, sizeof(uint64_t), s));
+    RS_CUDA(cudaMemsetAsync(rstart, 0, sizeof(uint64_t), s));
+  }
+  if (K) {
+    k_scatter<<<std::min<unsigned>(grid_for(K), sm_count * 16), kBlock, 0, s>>>(bucket, lo, K, bstart, cursor,
+                                                                                 keys[0]);
     count_launch();
   }
   RS_CUDA(cudaGetLastError());
@@ -938,11 +1050,11 @@ int build_sets(const SetInput* in, uint32_t count, const BuildOptions& opt, cuda
     }
     if (!opt.use_graph) timer.mark();
     if (NB) {
-      k_bucket_bits<<<grid_for(NB), kBlock, 0, ws>>>(counts, cbase, seeds, sizes, bset, d_sets, ct, NB, d_error,
-                                                     bits);
+      k_bucket_bits<<<grid_for(lanes), kBlock, 0, ws>>>(counts, cbase, seeds, sizes, d_sets, count, ct, d_error, bits);
       count_launch();
     }
-    int r = exclusive_scan_u64(bits, off, NB, scan_tmp, ws);
+    const LookState st{look_flags + group_tiles, look, look + 3 * std::max(group_tiles, bit_tiles), tickets + 1};
+    int r = exclusive_scan_u64(bits, off, NB, st, d_error, ws);
     if (r) return r;
     if (bucket_tiles) {
       k_ef_prepare<<<static_cast<unsigned>(bucket_tiles), kBlock, 0, ws>>>(d_sets, count, rstart, off, cbase, results);
@@ -1062,7 +1174,7 @@ int build_sets(const SetInput* in, uint32_t count, const BuildOptions& opt, cuda
 
   // A6: Golomb-Rice codes; A7: Elias-Fano
   if (NB) {
-    k_write_codes<<<grid_for(NB), kBlock, 0, s>>>(counts, cbase, seeds, sizes, bset, d_sets, d_outs, ct, off, NB);
+    k_write_codes<<<grid_for(lanes), kBlock, 0, s>>>(counts, cbase, seeds, sizes, d_sets, count, d_outs, ct, off);
     count_launch();
   }
   k_ef_write<<<static_cast<unsigned>(elem_tiles), kBlock, 0, s>>>(d_sets, count, d_outs, rstart, off);

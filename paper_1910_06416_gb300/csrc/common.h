@@ -188,9 +188,12 @@ int cuda_fail(cudaError_t e, const char* what);
 
 // ---------------------------------------------------------------- launchers
 // Exclusive scan of `count` uint64 values: out[0..count] with out[count] =
-// total.  `in` and `out` may alias.  scratch: scan_scratch(count) words.
-uint64_t scan_scratch(uint64_t count);
-int exclusive_scan_u64(const uint64_t* in, uint64_t* out, uint64_t count, uint64_t* scratch, cudaStream_t s);
+// total, in one launch.  `in` and `out` do not alias.  st: state of one value
+// for scan_tiles(count) tiles (lookback.cuh); *error is set if it cannot end.
+struct LookState;
+uint64_t scan_tiles(uint64_t count);
+int exclusive_scan_u64(const uint64_t* in, uint64_t* out, uint64_t count, const LookState& st, int* error,
+                       cudaStream_t s);
 
 // Kinds of key input.
 struct KeyInput {
