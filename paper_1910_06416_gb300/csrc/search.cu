@@ -544,12 +544,16 @@ __device__ __forceinline__ void partition_node(const SearchArgs& a, const Node& 
 // keys 197 + 85 -> 97 + 75 us; l = 10, b = 100, 3 * 10^5 keys 241 -> 179 us (split,
 // spread 4 against 1).  spread is 4 where a search takes several rounds of 32
 // indices (128 trials) and 2 below, where four warps mostly test past the
-// winner (l = 8, 10^5 keys: split 97 us with 2, 117 us with 4).
+// winner (l = 8, 10^5 keys: split 97 us with 2, 117 us with 4), and 32 where it
+// takes long (2048 trials, leaves from l = 10: 3 * 10^5 keys at l = 11, b = 100 take
+// 1.64 ms with one warp per leaf and 1.34 ms with four, 3 * 10^6 keys 10.8 and 11.3).
 __device__ __forceinline__ uint32_t group_warps(uint32_t gwarps, uint32_t items, uint32_t spread) {
   while (gwarps < kWarps && uint64_t(items) * gwarps * 2 <= spread * gridDim.x * kWarps) gwarps *= 2;
   return gwarps;
 }
-__host__ __device__ constexpr uint32_t group_spread(uint64_t trials) { return trials >= 128 ? 4 : 2; }
+__host__ __device__ constexpr uint32_t group_spread(uint64_t trials) {
+  return trials >= 2048 ? 32 : (trials >= 128 ? 4 : 2);
+}
 
 template <bool COUNT>
 __global__ void __launch_bounds__(kThreads, 4) k_split_level(SearchArgs a, uint32_t gwarps, uint32_t cap,
