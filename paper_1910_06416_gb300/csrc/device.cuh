@@ -14,28 +14,27 @@ constexpr uint64_t kMixB = 0x94D049BB133111EBull;
 constexpr uint64_t kSigHi = 0x6A09E667F3BCC909ull;
 constexpr uint64_t kSigLo = 0xBB67AE8584CAA73Bull;
 
-// z >> S (0 < S < 32) for the signature mixer: the low word is a funnel shift
-// (integer ALU pipe), the high word the multiply-high floor(hi * 2^(32-S) /
-// 2^32), which issues to the multiply-add pipe.  The kernels that hash keys
-// are bound by the ALU pipe (ncu, 10^6 string lookups: ALU pipe 75% busy,
-// multiply-add pipe 21%), so this moves one instruction of every shift off
-// it; measured on 10^8 string lookups: 3.78 -> 3.61 ms.  The same form in
-// the search hash (family_top32) made the searches 3-6% slower: their
-// multiply-add pipe already carries the hash's 64-bit multiplies.
-template <int S>
-__device__ __forceinline__ uint64_t shr_mix(uint64_t z) {
-  const uint32_t lo = static_cast<uint32_t>(z), hi = static_cast<uint32_t>(z >> 32);
-  uint32_t h;
-  asm volatile("mul.hi.u32 %0, %1, %2;" : "=r"(h) : "r"(hi), "r"(1u << (32 - S)));
-  return (uint64_t(h) << 32) | __funnelshift_r(lo, hi, S);
+// z * C mod 2^64 as the three 32-bit multiplies it needs, the high word's sum
+// folded into the multiply-adds (the compiler's own adds an add or a move):
+// 10^8 string lookups 2.01 -> 1.96 ms.  With it, plain shifts in the mixer are
+// the faster again; high words by a multiply-high (to take them off the ALU
+// pipe) cost 1.99 ms.
+template <uint64_t C>
+__device__ __forceinline__ uint64_t mul_const(uint64_t z) {
+  uint32_t lo, hi;
+  asm("{.reg .u64 t; mul.wide.u32 t, %2, %4; mov.b64 {%0, %1}, t; mad.lo.u32 %1, %2, %5, %1; mad.lo.u32 %1, %3, %4, %1;}"
+      : "=&r"(lo), "=&r"(hi)
+      : "r"(static_cast<uint32_t>(z)), "r"(static_cast<uint32_t>(z >> 32)), "n"(static_cast<uint32_t>(C)),
+        "n"(static_cast<uint32_t>(C >> 32)));
+  return (uint64_t(hi) << 32) | lo;
 }
 
 // splitmix64 finalizer (Steele, Lea, Flood 2014).
 __host__ __device__ __forceinline__ uint64_t mix64(uint64_t z) {
 #ifdef __CUDA_ARCH__
-  z = (z ^ shr_mix<30>(z)) * kMixA;
-  z = (z ^ shr_mix<27>(z)) * kMixB;
-  return z ^ shr_mix<31>(z);
+  z = mul_const<kMixA>(z ^ (z >> 30));
+  z = mul_const<kMixB>(z ^ (z >> 27));
+  return z ^ (z >> 31);
 #else
   z = (z ^ (z >> 30)) * kMixA;
   z = (z ^ (z >> 27)) * kMixB;
