@@ -249,7 +249,8 @@ __device__ __forceinline__ uint64_t descend(const View& v, uint64_t s0, uint32_t
 // A batch with several times as many queries as the structure has codes
 // (flat_pays) decodes every code once: the function key K ^ (K >> 30) of code c (preorder) of the
 // bucket that starts at s_b is stored at flat[s_b + c] (a bucket of m keys has
-// fewer than m codes), and so holds s_b and the bucket's size.  A level of the
+// fewer than m codes), and so holds s_b, the bucket's size and the key of its
+// first code in 16 bytes: {s_b | m << 40, key}.  A level of the
 // descent then loads its key and steps over the earlier siblings' codes with
 // one multiply-add, where it otherwise reads a fixed part, finds a unary part
 // and selects past the siblings in the bit vector.
@@ -279,6 +280,10 @@ __device__ __forceinline__ uint64_t code_key(const View& v, const uint32_t* __re
   return family_key((uint64_t(un) << r) | low, depth);
 }
 
+// so packs values below 2^kFlatSizeShift and sizes below 2^24.
+constexpr int kFlatSizeShift = 40;
+bool flat_fits(uint64_t range, uint64_t mmax) { return range < (1ull << kFlatSizeShift) && mmax < (1ull << 24); }
+
 // Part g of 2^log_group of the decode of bucket b: codes g, g + 2^log_group, ...
 // Every part reads the lists for itself and scans the unary part with a cursor
 // of its own, so parts need nothing from each other.
@@ -287,10 +292,7 @@ __device__ __forceinline__ void flat_bucket(const View& v, uint64_t b, uint32_t 
   uint64_t* so = const_cast<uint64_t*>(v.so);
   const uint64_t s0 = ef_prefix(v, b);
   const uint32_t m = size_of_range<RANGE>(v, ef_prefix(v, b + 1) - s0);
-  if (g == 0) {
-    so[2 * b] = s0;
-    so[2 * b + 1] = m;
-  }
+  if (g == 0) so[2 * b] = s0 | (uint64_t(m) << kFlatSizeShift);
   if (m < 2) return;
   const uint64_t w0 = __ldg(v.table + kTableWords * m);
   const uint32_t codes = static_cast<uint32_t>(w0 >> 32);
@@ -320,7 +322,9 @@ __device__ __forceinline__ void flat_bucket(const View& v, uint64_t b, uint32_t 
     }
     const uint32_t one = code_next_one(t, from, end);
     if (one == ~0u) return;
-    flat[c] = code_key(v, t, end, fixed, m, c, one - from);
+    const uint64_t key = code_key(v, t, end, fixed, m, c, one - from);
+    flat[c] = key;
+    if (c == 0) so[2 * b + 1] = key;
   }
 }
 
@@ -389,23 +393,23 @@ template <bool RANGE>
 __device__ __forceinline__ uint64_t lookup_flat(const FlatView& v, uint64_t hi, uint64_t lo) {
   if (v.nb == 0) return 0;
   const ulonglong2 p = __ldg(v.so + bucket_of(hi, v.nb));
-  uint32_t m = static_cast<uint32_t>(p.y);
-  if (m <= 1) return p.x;
-  const uint64_t* __restrict__ code = v.flat + p.x;
+  const uint64_t s0 = p.x & ((1ull << kFlatSizeShift) - 1);
+  uint32_t m = static_cast<uint32_t>(p.x >> kFlatSizeShift);
+  if (m <= 1) return s0;
+  const uint64_t* __restrict__ code = v.flat + s0;
   const uint64_t xpre = pre_key(lo);
   uint32_t c = 0;  // keys (or output ranges) of the siblings left behind
-  for (;;) {
-    const uint64_t kp = __ldg(code);
+  for (uint64_t kp = p.y;; kp = __ldg(code)) {
     const uint4 nd = __ldg(v.rec + m);
     const uint32_t h = family_top32(xpre, kp);
     const uint32_t fanout = nd.w >> 28;
-    if (fanout == 0) return p.x + c + __umulhi(h, RANGE ? m + static_cast<uint32_t>(v.extra) : m);
+    if (fanout == 0) return s0 + c + __umulhi(h, RANGE ? m + static_cast<uint32_t>(v.extra) : m);
     const uint32_t val = __umulhi(h, m);
     const uint32_t part = min(nd.y ? __umulhi(val, nd.y) : val / nd.x, fanout - 1);
     code += 1 + part * (nd.w & ((1u << kLookupCodeBits) - 1));
     c += RANGE ? part * static_cast<uint32_t>(__ldg(v.table + kTableWords * nd.x + 3) >> 32) : part * nd.x;
     m = part + 1 < fanout ? nd.x : m - nd.x * (fanout - 1);
-    if (m <= 1) return p.x + c;
+    if (m <= 1) return s0 + c;
   }
 }
 
@@ -596,14 +600,16 @@ int decode_views(View* views, uint32_t count, uint64_t q, cudaStream_t s, uint64
   // (or their parts)
   std::vector<uint64_t> base(count + 1);
   uint64_t elements = 0, buckets = 0, codes = 0, range = 0;
+  bool fits = true;
   for (uint32_t i = 0; i < count; i++) {
     elements += views[i].nb ? views[i].nb + 1 : 0;
     buckets += views[i].nb;
     codes += views[i].codes;
     range += views[i].range;
+    fits &= flat_fits(views[i].range, views[i].mmax);
   }
   if (buckets == 0 || q < elements + count) return RECSPLIT_OK;
-  *flat = flat_pays(q, codes, buckets);
+  *flat = fits && flat_pays(q, codes, buckets);
   void *d_scratch = nullptr, *d_views = nullptr, *d_base = nullptr;
   if (*flat && pool_alloc(&d_scratch, 16 * buckets + 8 * range, s) != RECSPLIT_OK) *flat = false;
   if (!*flat && pool_alloc(&d_scratch, 16 * elements, s) != RECSPLIT_OK)
@@ -705,7 +711,7 @@ int lookup_structure(const Handle& h, const KeyInput& q, uint64_t* d_out, cudaSt
   // decoded once instead of selected per query (the stored structure does not
   // change).  The scratch is allocated only then.
   uint64_t* so = nullptr;
-  if (allow_scratch && v.nb && flat_pays(q.n, v.codes, v.nb) &&
+  if (allow_scratch && v.nb && flat_pays(q.n, v.codes, v.nb) && flat_fits(v.range, v.mmax) &&
       pool_alloc(reinterpret_cast<void**>(&so), 16 * v.nb + 8 * v.range, s) == RECSPLIT_OK) {
     View f = v;
     f.so = so;
