@@ -350,7 +350,7 @@ int recsplit_lookup_batch(const recsplit_t* const* hs, uint32_t count, const uin
   int rc;
   // large batches: every bucket, or every code, decoded once (freed on return)
   uint64_t* d_so = nullptr;
-  bool flat = false;
+  FlatBatch flat;
   if ((rc = decode_views(views.data(), count, q, s, &d_so, &flat))) return rc;
   so.dev = d_so;
   so.owned = d_so != nullptr;
@@ -370,7 +370,7 @@ int recsplit_lookup_batch(const recsplit_t* const* hs, uint32_t count, const uin
   bool any_range = false;
   for (uint32_t i = 0; i < count; i++) any_range |= views[i].extra != 0;
   if ((rc = lookup_many(static_cast<const View*>(v.dev), count, static_cast<const uint32_t*>(d.dev),
-                        static_cast<const uint64_t*>(k.dev), q, static_cast<uint64_t*>(o.dev), s, any_range, flat)))
+                        static_cast<const uint64_t*>(k.dev), q, static_cast<uint64_t*>(o.dev), s, any_range, &flat)))
     return rc;
   if (!dev) RS_CUDA(cudaMemcpyAsync(out, o.dev, q * sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
   RS_CUDA(cudaStreamSynchronize(s));  // the staged views are released after the lookups

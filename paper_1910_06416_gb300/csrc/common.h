@@ -220,20 +220,25 @@ struct BuildOptions {
 int build_sets(const SetInput* sets, uint32_t count, const BuildOptions& opt, cudaStream_t s, Handle** out);
 // allow_scratch = false: allocate nothing (no per-batch decode of the lists)
 int lookup_structure(const Handle& h, const KeyInput& q, uint64_t* d_out, cudaStream_t s, bool allow_scratch = true);
+// Flat views of a batch's structures on the device (lookup.cu), or null.
+struct FlatBatch {
+  const void* views = nullptr;
+  bool steps = false;
+};
 // Lookups of keys[i] in views[ids[i]] (count views); an id not below count
 // gives 2^64 - 1.  any_range: some view has a leaf range extra (perfect,
-// non-minimal variant); flat: every view with buckets has flat set
+// non-minimal variant); flat: from decode_views
 int lookup_many(const View* d_views, uint32_t count, const uint32_t* d_ids, const uint64_t* d_keys, uint64_t q,
-                uint64_t* d_out, cudaStream_t s, bool any_range = true, bool flat = false);
+                uint64_t* d_out, cudaStream_t s, bool any_range = true, const FlatBatch* flat = nullptr);
 // Batched lookups over several structures with several times as many queries
 // as the structures have codes: the function key of every code and s_i and the
 // size of every bucket of every structure are decoded into one pooled array
 // *scratch (the caller frees it, stream-ordered, after the lookups), and
-// views[i].flat and .so (host views) point at structure i's parts.  With fewer
-// queries, but at least as many as buckets, s_i and o_i alone (views[i].so).
-// Otherwise, or if the memory is not available, *scratch stays null and the
-// views are unchanged (the lookups then select in the lists per query).
-int decode_views(View* views, uint32_t count, uint64_t q, cudaStream_t s, uint64_t** scratch, bool* flat);
+// *flat describes them.  With fewer queries, but at least as many as buckets,
+// s_i and o_i alone (views[i].so, host views).  Otherwise, or if the memory is
+// not available, *scratch stays null and the views are unchanged (the lookups
+// then select in the lists per query).
+int decode_views(View* views, uint32_t count, uint64_t q, cudaStream_t s, uint64_t** scratch, FlatBatch* flat);
 int lookup_many_bytes(const View* d_views, uint32_t count, const uint32_t* d_ids, const uint8_t* d_bytes,
                       const uint64_t* d_offsets, uint64_t q, uint64_t* d_out, cudaStream_t s);
 

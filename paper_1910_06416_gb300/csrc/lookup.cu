@@ -374,22 +374,44 @@ __global__ void __launch_bounds__(256) k_flat_decode_views(const View* __restric
   flat_bucket<true>(v, i >> v.log_group, i & ((1u << v.log_group) - 1), v.log_group);
 }
 
-// What a flat lookup reads of a structure.
-struct FlatView {
-  uint64_t nb;
+// What a flat lookup reads of a structure (16-byte loads where it is read per
+// query).
+struct alignas(16) FlatView {
   const ulonglong2* so;
   const uint64_t* flat;
-  const uint4* rec;
+  uint64_t nb;
   const uint64_t* table;  // output ranges (RANGE)
+  // sizes of the splitting strategy (Sec. 5.4), their reciprocals ceil(2^32 / u)
+  // and the codes of subtrees of `lower` and `upper` keys
+  uint32_t leaf, lower, upper, leaf_magic;
+  uint32_t lower_magic, upper_magic, lower_codes, upper_codes;
+  const uint4* rec;
   uint64_t extra;
 };
 
-__host__ __device__ __forceinline__ FlatView flat_view(const View& v) {
-  return FlatView{v.nb, reinterpret_cast<const ulonglong2*>(v.so), v.flat, reinterpret_cast<const uint4*>(v.rec),
-                  v.table, v.extra};
+FlatView flat_view(const View& v) {
+  const Strategy st = make_strategy(v.leaf);
+  auto magic = [](uint64_t u) { return static_cast<uint32_t>(((1ull << 32) + u - 1) / u); };
+  const uint32_t lower_codes = static_cast<uint32_t>(1 + st.lower / st.leaf);
+  return FlatView{reinterpret_cast<const ulonglong2*>(v.so), v.flat, v.nb, v.table, v.leaf,
+                  static_cast<uint32_t>(st.lower), static_cast<uint32_t>(st.upper),
+                  v.leaf >= 2 ? magic(st.leaf) : 0, magic(st.lower), magic(st.upper), lower_codes,
+                  static_cast<uint32_t>(1 + st.upper / st.lower * lower_codes),
+                  reinterpret_cast<const uint4*>(v.rec), v.extra};
 }
 
-template <bool RANGE>
+// Whether the steps of a descent can be computed (lookup_flat): the
+// reciprocals are exact for values below 2^16, and leaves of one key have no
+// code.
+bool steps_computed(const View& v) { return v.mmax < 65536 && v.leaf >= 2; }
+
+// STEPS: the part, its size and the codes to step over are computed from the
+// strategy's sizes instead of loaded by node size.  About 12 instructions
+// replace a load that is scattered over the lanes: 64-bit keys, which are bound
+// by such loads, gain (l = 8, b = 100, ten queries per code 280 -> 266 us; l = 12,
+// b = 2000 85 -> 73 us; 256 structures 355 -> 319 us), strings, whose signatures
+// keep the ALU pipe busy, lose (1.91 against 1.94 ms) and load.
+template <bool RANGE, bool STEPS>
 __device__ __forceinline__ uint64_t lookup_flat(const FlatView& v, uint64_t hi, uint64_t lo) {
   if (v.nb == 0) return 0;
   const ulonglong2 p = __ldg(v.so + bucket_of(hi, v.nb));
@@ -400,26 +422,49 @@ __device__ __forceinline__ uint64_t lookup_flat(const FlatView& v, uint64_t hi, 
   const uint64_t xpre = pre_key(lo);
   uint32_t c = 0;  // keys (or output ranges) of the siblings left behind
   for (uint64_t kp = p.y;; kp = __ldg(code)) {
-    const uint4 nd = __ldg(v.rec + m);
     const uint32_t h = family_top32(xpre, kp);
-    const uint32_t fanout = nd.w >> 28;
-    if (fanout == 0) return s0 + c + __umulhi(h, RANGE ? m + static_cast<uint32_t>(v.extra) : m);
-    const uint32_t val = __umulhi(h, m);
-    const uint32_t part = min(nd.y ? __umulhi(val, nd.y) : val / nd.x, fanout - 1);
-    code += 1 + part * (nd.w & ((1u << kLookupCodeBits) - 1));
-    c += RANGE ? part * static_cast<uint32_t>(__ldg(v.table + kTableWords * nd.x + 3) >> 32) : part * nd.x;
-    m = part + 1 < fanout ? nd.x : m - nd.x * (fanout - 1);
+    uint32_t unit, codes, part;  // of every child but the last; the key's child
+    if constexpr (STEPS) {
+      if (m <= v.leaf) return s0 + c + __umulhi(h, RANGE ? m + static_cast<uint32_t>(v.extra) : m);
+      const uint32_t val = __umulhi(h, m);
+      const bool low = m <= v.lower;
+      unit = low ? v.leaf : v.lower;
+      codes = low ? 1u : v.lower_codes;
+      part = __umulhi(val, low ? v.leaf_magic : v.lower_magic);
+      if (m > v.upper) {
+        // two children, the first of k * upper keys: k subtrees of `upper` under
+        // k - 1 binary splits
+        const uint32_t k = __umulhi((m >> 1) + v.upper - 1, v.upper_magic);
+        unit = k * v.upper;
+        codes = k * v.upper_codes + k - 1;
+        part = val >= unit;
+        m = part ? m - unit : unit;
+      } else {
+        m = min(unit, m - part * unit);
+      }
+    } else {
+      const uint4 nd = __ldg(v.rec + m);
+      const uint32_t fanout = nd.w >> 28;
+      if (fanout == 0) return s0 + c + __umulhi(h, RANGE ? m + static_cast<uint32_t>(v.extra) : m);
+      const uint32_t val = __umulhi(h, m);
+      unit = nd.x;
+      codes = nd.w & ((1u << kLookupCodeBits) - 1);
+      part = min(nd.y ? __umulhi(val, nd.y) : val / nd.x, fanout - 1);
+      m = part + 1 < fanout ? unit : m - unit * (fanout - 1);
+    }
+    code += 1 + part * codes;
+    c += RANGE ? part * static_cast<uint32_t>(__ldg(v.table + kTableWords * unit + 3) >> 32) : part * unit;
     if (m <= 1) return s0 + c;
   }
 }
 
-template <bool RANGE>
+template <bool RANGE, bool STEPS>
 __global__ void __launch_bounds__(256, 8) k_lookup_u64_flat(FlatView v, const uint64_t* __restrict__ keys, uint64_t q,
                                                             uint64_t* __restrict__ out) {
   for (uint64_t i = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; i < q; i += uint64_t(gridDim.x) * blockDim.x) {
     uint64_t hi, lo;
     signature_u64(__ldg(keys + i), hi, lo);
-    out[i] = lookup_flat<RANGE>(v, hi, lo);
+    out[i] = lookup_flat<RANGE, STEPS>(v, hi, lo);
   }
 }
 
@@ -433,12 +478,12 @@ __global__ void __launch_bounds__(256, 8) k_lookup_bytes_flat(FlatView v, const 
     uint64_t hi, lo;
     const bool ok = o0 <= o1 && o1 <= last;  // else read as the empty string
     signature_bytes(bytes + (ok ? o0 : 0), ok ? o1 - o0 : 0, hi, lo);
-    out[i] = lookup_flat<RANGE>(v, hi, lo);
+    out[i] = lookup_flat<RANGE, false>(v, hi, lo);
   }
 }
 
-template <bool ANY_RANGE>
-__global__ void __launch_bounds__(256, 8) k_lookup_many_flat(const View* __restrict__ views, uint32_t count,
+template <bool ANY_RANGE, bool STEPS>
+__global__ void __launch_bounds__(256, 8) k_lookup_many_flat(const FlatView* __restrict__ views, uint32_t count,
                                                              const uint32_t* __restrict__ ids,
                                                              const uint64_t* __restrict__ keys, uint64_t q,
                                                              uint64_t* __restrict__ out) {
@@ -450,8 +495,8 @@ __global__ void __launch_bounds__(256, 8) k_lookup_many_flat(const View* __restr
     }
     uint64_t hi, lo;
     signature_u64(__ldg(keys + i), hi, lo);
-    const FlatView v = flat_view(views[id]);
-    out[i] = ANY_RANGE && v.extra ? lookup_flat<true>(v, hi, lo) : lookup_flat<false>(v, hi, lo);
+    const FlatView v = views[id];
+    out[i] = ANY_RANGE && v.extra ? lookup_flat<true, STEPS>(v, hi, lo) : lookup_flat<false, STEPS>(v, hi, lo);
   }
 }
 
@@ -576,7 +621,7 @@ int lookup_many_bytes(const View* d_views, uint32_t count, const uint32_t* d_ids
 }
 
 int lookup_many(const View* d_views, uint32_t count, const uint32_t* d_ids, const uint64_t* d_keys, uint64_t q,
-                uint64_t* d_out, cudaStream_t s, bool any_range, bool flat) {
+                uint64_t* d_out, cudaStream_t s, bool any_range, const FlatBatch* flat) {
   if (q == 0) return RECSPLIT_OK;
   LookupRange range;
   int dev = 0, sms = 0;
@@ -585,45 +630,52 @@ int lookup_many(const View* d_views, uint32_t count, const uint32_t* d_ids, cons
   const int block = 256;
   const uint64_t want = (q + block - 1) / block;
   const unsigned grid = static_cast<unsigned>(want < uint64_t(sms) * 64 ? want : uint64_t(sms) * 64);
-  auto kern = flat ? (any_range ? k_lookup_many_flat<true> : k_lookup_many_flat<false>)
-                   : (any_range ? k_lookup_many<true> : k_lookup_many<false>);
-  kern<<<grid, block, 0, s>>>(d_views, count, d_ids, d_keys, q, d_out);
+  if (flat && flat->views) {
+    auto kern = flat->steps ? (any_range ? k_lookup_many_flat<true, true> : k_lookup_many_flat<false, true>)
+                            : (any_range ? k_lookup_many_flat<true, false> : k_lookup_many_flat<false, false>);
+    kern<<<grid, block, 0, s>>>(static_cast<const FlatView*>(flat->views), count, d_ids, d_keys, q, d_out);
+  } else {
+    (any_range ? k_lookup_many<true> : k_lookup_many<false>)<<<grid, block, 0, s>>>(d_views, count, d_ids, d_keys, q,
+                                                                                    d_out);
+  }
   count_launch();
   RS_CUDA(cudaGetLastError());
   return RECSPLIT_OK;
 }
 
-int decode_views(View* views, uint32_t count, uint64_t q, cudaStream_t s, uint64_t** scratch, bool* flat) {
+int decode_views(View* views, uint32_t count, uint64_t q, cudaStream_t s, uint64_t** scratch, FlatBatch* batch) {
   *scratch = nullptr;
-  *flat = false;
+  *batch = FlatBatch{};
   // elements 0 .. N of every list, or the N buckets of every structure
   // (or their parts)
   std::vector<uint64_t> base(count + 1);
   uint64_t elements = 0, buckets = 0, codes = 0, range = 0;
-  bool fits = true;
+  bool fits = true, steps = true;
   for (uint32_t i = 0; i < count; i++) {
     elements += views[i].nb ? views[i].nb + 1 : 0;
     buckets += views[i].nb;
     codes += views[i].codes;
     range += views[i].range;
     fits &= flat_fits(views[i].range, views[i].mmax);
+    steps &= steps_computed(views[i]);
   }
   if (buckets == 0 || q < elements + count) return RECSPLIT_OK;
-  *flat = fits && flat_pays(q, codes, buckets);
+  bool flat = fits && flat_pays(q, codes, buckets);
   void *d_scratch = nullptr, *d_views = nullptr, *d_base = nullptr;
-  if (*flat && pool_alloc(&d_scratch, 16 * buckets + 8 * range, s) != RECSPLIT_OK) *flat = false;
-  if (!*flat && pool_alloc(&d_scratch, 16 * elements, s) != RECSPLIT_OK)
+  // flat: the flat views, then s_i and sizes, then the keys
+  const uint64_t view_words = (sizeof(FlatView) * count + 7) / 8;
+  if (flat && pool_alloc(&d_scratch, 8 * (view_words + 2 * buckets + range), s) != RECSPLIT_OK) flat = false;
+  if (!flat && pool_alloc(&d_scratch, 16 * elements, s) != RECSPLIT_OK)
     return RECSPLIT_OK;  // fall back to per-query selects
-  uint64_t* so = static_cast<uint64_t*>(d_scratch);
-  uint64_t* keys = so + 2 * buckets;
-  uint64_t* next_so = so;
+  uint64_t* next_so = static_cast<uint64_t*>(d_scratch) + (flat ? view_words : 0);
+  uint64_t* keys = next_so + 2 * buckets;
   uint64_t total = 0;
   for (uint32_t i = 0; i < count; i++) {
     View& v = views[i];
     base[i] = total;
     if (!v.nb) continue;
     v.so = next_so;
-    if (*flat) {
+    if (flat) {
       v.flat = keys;
       v.log_group = flat_log_group(v.codes, v.nb, codes_per_part(codes));
       keys += v.range;
@@ -635,15 +687,19 @@ int decode_views(View* views, uint32_t count, uint64_t q, cudaStream_t s, uint64
     }
   }
   base[count] = total;
+  std::vector<FlatView> flat_views(flat ? count : 0);
+  for (uint32_t i = 0; flat && i < count; i++) flat_views[i] = flat_view(views[i]);
   int rc = pool_alloc(&d_views, sizeof(View) * count, s);
   if (!rc) rc = pool_alloc(&d_base, sizeof(uint64_t) * (count + 1), s);
   cudaError_t e = cudaSuccess;
   if (!rc) e = cudaMemcpyAsync(d_views, views, sizeof(View) * count, cudaMemcpyHostToDevice, s);
   if (!rc && e == cudaSuccess) e = cudaMemcpyAsync(d_base, base.data(), sizeof(uint64_t) * (count + 1),
                                                    cudaMemcpyHostToDevice, s);
+  if (!rc && e == cudaSuccess && flat)
+    e = cudaMemcpyAsync(d_scratch, flat_views.data(), sizeof(FlatView) * count, cudaMemcpyHostToDevice, s);
   if (!rc && e == cudaSuccess) {
     const uint64_t blocks = (total + 255) / 256;
-    if (*flat)
+    if (flat)
       k_flat_decode_views<<<static_cast<unsigned>(blocks), 256, 0, s>>>(
           static_cast<const View*>(d_views), static_cast<const uint64_t*>(d_base), count, total);
     else
@@ -658,12 +714,12 @@ int decode_views(View* views, uint32_t count, uint64_t q, cudaStream_t s, uint64
   if (d_base) cudaFreeAsync(d_base, s);
   if (rc || e != cudaSuccess) {
     for (uint32_t i = 0; i < count; i++) views[i].so = views[i].flat = nullptr;
-    *flat = false;
     cudaFreeAsync(d_scratch, s);
     if (rc) return rc;
     return cuda_fail(e, "decode of the structures");
   }
-  *scratch = so;
+  *scratch = static_cast<uint64_t*>(d_scratch);
+  if (flat) *batch = FlatBatch{d_scratch, steps};
   return RECSPLIT_OK;
 }
 
@@ -721,7 +777,9 @@ int lookup_structure(const Handle& h, const KeyInput& q, uint64_t* d_out, cudaSt
     const unsigned dg = static_cast<unsigned>(((v.nb << lg) + block - 1) / block);
     (v.extra ? k_flat_decode<true> : k_flat_decode<false>)<<<dg, block, 0, s>>>(f, lg);
     if (q.u64)
-      (v.extra ? k_lookup_u64_flat<true> : k_lookup_u64_flat<false>)<<<grid, block, 0, s>>>(fv, q.u64, q.n, d_out);
+      (steps_computed(v) ? (v.extra ? k_lookup_u64_flat<true, true> : k_lookup_u64_flat<false, true>)
+                         : (v.extra ? k_lookup_u64_flat<true, false> : k_lookup_u64_flat<false, false>))
+          <<<grid, block, 0, s>>>(fv, q.u64, q.n, d_out);
     else
       (v.extra ? k_lookup_bytes_flat<true> : k_lookup_bytes_flat<false>)<<<grid, block, 0, s>>>(fv, q.bytes, q.offsets,
                                                                                               q.n, d_out);
