@@ -681,16 +681,6 @@ int ef_width(uint64_t u, uint64_t count) {
   return q ? floor_log2_u64(q) : 0;
 }
 
-// Largest node of the next level, given the largest of this one.
-uint64_t next_level_max(const Strategy& st, uint64_t cur) {
-  uint64_t best = 0;
-  for (uint64_t m = st.leaf + 1; m <= cur; m++) {
-    const Shape sh = shape_of(st, m);
-    best = std::max(best, std::max(sh.unit, sh.last));
-  }
-  return best;
-}
-
 uint64_t tiles(uint64_t items) { return (items + kTile - 1) / kTile; }
 
 }  // namespace
@@ -974,7 +964,7 @@ int build_sets(const SetInput* in, uint32_t count, const BuildOptions& opt, cuda
       const bool few = nodes <= 16ull * 32 * sm_count;
       plan_share.push_back(heavy >= double(few ? 1 << 16 : 1 << 21));
       for (uint32_t c = 0; c < nclass; c++)
-        lm[c] = lm[c] > class_leaf[c] ? next_level_max(make_strategy(class_leaf[c]), lm[c]) : 0;
+        lm[c] = lm[c] > class_leaf[c] ? T[c].next_max[lm[c]] : 0;
     }
   }
   SharedNodes shared{};
@@ -1036,7 +1026,7 @@ int build_sets(const SetInput* in, uint32_t count, const BuildOptions& opt, cuda
       int r = launch_split_level(a, mx, trials, max_leaf, tables, sm_count, ws, share ? &shared : nullptr);
       if (r) return r;
       for (uint32_t c = 0; c < nclass; c++)
-        level_max[c] = level_max[c] > class_leaf[c] ? next_level_max(make_strategy(class_leaf[c]), level_max[c]) : 0;
+        level_max[c] = level_max[c] > class_leaf[c] ? T[c].next_max[level_max[c]] : 0;
       level++;
       split_levels++;
     }

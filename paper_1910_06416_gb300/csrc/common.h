@@ -73,6 +73,7 @@ struct Tables {
   std::vector<uint64_t> fixed_bits;
   std::vector<uint64_t> codes;
   std::vector<uint64_t> expected_trials;  // 1/p rounded up (search stall detection)
+  std::vector<uint64_t> next_max;         // largest child of the split nodes of up to m keys
   std::vector<uint64_t> range;            // output range of a subtree (m when extra = 0)
   std::vector<uint64_t> device_words;     // kTableWords per size
 };
