@@ -221,9 +221,10 @@ __global__ void __launch_bounds__(kBlock) k_group_scan(const uint64_t* __restric
       const uint32_t c = cls[k], leaf = a.leaf_of[c];
       Node* q;
       uint32_t *cnt, cap;
-      if (m[k] > leaf)
-        q = a.split_in, cnt = a.split_in_count, cap = a.split_cap;
-      else if (m[k] == leaf)
+      if (m[k] > leaf) {
+        const int heavy = a.heavy_flag < 2 && heavy_flag(ct.t[c][kTableWords * uint64_t(m[k]) + 1], 0, a.heavy_flag);
+        q = a.split_in[heavy], cnt = a.split_in_count[heavy], cap = a.split_cap[heavy];
+      } else if (m[k] == leaf)
         q = a.full_q[c], cnt = a.full_n + c, cap = a.full_cap[c];
       else
         q = a.part_q[c], cnt = a.part_n + c, cap = a.part_cap[c];
@@ -746,7 +747,6 @@ int build_sets(const SetInput* in, uint32_t count, const BuildOptions& opt, cuda
     part_cap[c] = nb_c[c] + keys_c[c] / (class_leaf[c] + 1) + 1;
     qtotal += full_cap[c] + part_cap[c];
   }
-  qtotal += 2 * split_cap;
 
   Scratch sc{s};
   PhaseTimer timer(profiling_enabled(), s);
@@ -771,7 +771,7 @@ int build_sets(const SetInput* in, uint32_t count, const BuildOptions& opt, cuda
   sc.plan(&sizes, K + 1);
   sc.plan(&back1, n_back1);
   sc.plan(&back2, n_back2);
-  sc.plan(&counters, 2 * kLevels + 4 * kMaxClasses + 2);
+  sc.plan(&counters, 4 * kLevels + 4 * kMaxClasses + 2);
   // scans: group_scan's tiles, then those of the lengths
   const uint64_t group_tiles = (NB + kGroupTile - 1) / kGroupTile, bit_tiles = scan_tiles(NB);
   uint32_t* look_flags;
@@ -785,9 +785,9 @@ int build_sets(const SetInput* in, uint32_t count, const BuildOptions& opt, cuda
   SetResults results{back2, back2 + count, back2 + 2 * uint64_t(count),
                      reinterpret_cast<unsigned long long*>(back2 + 3 * uint64_t(count))};
   int* d_error = reinterpret_cast<int*>(back2 + 4 * uint64_t(count));
-  uint32_t* const level_n = counters;                 // split nodes per level
-  uint32_t* const level_work = counters + kLevels;    // and the work counter of its launch
-  uint32_t* const leaf_work = level_work + kLevels;   // two leaf launches per class
+  uint32_t* const level_n = counters;                     // split nodes per level, light and heavy
+  uint32_t* const level_work = counters + 2 * kLevels;    // and the work counters of its launches
+  uint32_t* const leaf_work = level_work + 2 * kLevels;   // two leaf launches per class
   uint32_t* const full_n = leaf_work + 2 * kMaxClasses;
   uint32_t* const part_n = full_n + kMaxClasses;
   uint32_t* const tickets = part_n + kMaxClasses;
@@ -872,6 +872,72 @@ int build_sets(const SetInput* in, uint32_t count, const BuildOptions& opt, cuda
   }
   RS_CUDA(cudaMemcpyAsync(d_sets, hs.data(), count * sizeof(DevSet), cudaMemcpyHostToDevice, s));
 
+  // Heavy nodes are searched shared: that costs a few microseconds of CTA-wide
+  // steps per node and removes the tail of a level, a few long geometric
+  // searches on an idle device, so it pays where a node's expected trials x keys
+  // reach 2^21 evaluations, or 2^16 in a build of few such nodes: 8 per warp of
+  // the device, counting the keys of a class over its smallest such node.
+  // Split phase without and with the second clause: l = 12, b = 100: 10^5 keys
+  // 0.84 -> 0.31 ms, 10^6 keys 2.29 -> 1.69 ms (5 * 10^6 keys, above the line: 7.1
+  // against 8.2 ms); l = 13, b = 100, 3 * 10^5 keys 12.6 -> 4.5 ms; l = 16, b = 100, 3 *
+  // 10^4 keys 26 -> 5.4 ms; l = 12, b = 2000, 3 * 10^5 keys 4.7 -> 2.1 ms.  Light nodes of
+  // the same level have a queue of their own (48 sets with l = 5, 8, 12: all
+  // nodes of four such levels shared took 9.2 ms, the heavy ones alone 7.2).
+  std::vector<uint64_t> level_max(nclass);
+  uint32_t max_leaf = 0;
+  double heavy_keys = 0;  // keys over the smallest node of 2^16
+  bool any_heavy = false;
+  for (uint32_t c = 0; c < nclass; c++) {
+    level_max[c] = h_cls_max[c];
+    max_leaf = std::max(max_leaf, class_leaf[c]);
+    if (h_cls_max[c] <= class_leaf[c] || T[c].heaviest[h_cls_max[c]] < double(kHeavyEvals[0])) continue;
+    any_heavy = true;
+    const auto& hv = T[c].heaviest;
+    heavy_keys += double(keys_c[c]) / double(std::lower_bound(hv.begin(), hv.end(), double(kHeavyEvals[0])) - hv.begin());
+  }
+  const uint32_t heavy_flag_index = heavy_keys <= 8.0 * 32 * sm_count ? 0 : 1;
+  const uint64_t heavy_min = kHeavyEvals[heavy_flag_index];
+  // the levels that may hold heavy nodes: sizes that occur, from the bucket
+  // sizes down
+  std::vector<char> level_heavy;
+  if (any_heavy) {
+    std::vector<std::vector<uint32_t>> sizes_at(nclass);
+    for (uint32_t c = 0; c < nclass; c++) {
+      if (T[c].heaviest[h_cls_max[c]] < double(heavy_min)) continue;
+      uint64_t least = h_cls_max[c];
+      for (uint32_t i = 0; i < count; i++)
+        if (hs[i].cls == c && hs[i].nb) least = std::min(least, h_set_min[i]);
+      for (uint64_t m = std::max<uint64_t>(least, class_leaf[c] + 1); m <= h_cls_max[c]; m++)
+        sizes_at[c].push_back(static_cast<uint32_t>(m));
+    }
+    std::vector<char> seen;
+    for (bool some = true; some && level_heavy.size() <= kMaxDepth + 1;) {
+      bool heavy = false;
+      some = false;
+      for (uint32_t c = 0; c < nclass; c++) {
+        if (sizes_at[c].empty()) continue;
+        const Strategy st = make_strategy(class_leaf[c]);
+        seen.assign(h_cls_max[c] + 1, 0);
+        std::vector<uint32_t> next;
+        for (uint32_t m : sizes_at[c]) {
+          const uint64_t e = T[c].expected_trials[m];
+          heavy |= is_heavy(e, m, heavy_min);
+          const Shape sh = shape_of(st, m);
+          for (uint64_t k : {sh.unit, sh.last})
+            if (k > class_leaf[c] && !seen[k]) {
+              seen[k] = 1;
+              next.push_back(static_cast<uint32_t>(k));
+            }
+        }
+        sizes_at[c].swap(next);
+        some |= !sizes_at[c].empty();
+      }
+      level_heavy.push_back(heavy);
+    }
+  }
+  const uint64_t heavy_cap = any_heavy ? split_cap : 0;
+  qtotal += 2 * (split_cap + heavy_cap);
+
   // grouping; queues: two split levels (ping-pong) shared by all classes, full
   // and partial leaves per class
   uint64_t* keys[2];
@@ -885,9 +951,9 @@ int build_sets(const SetInput* in, uint32_t count, const BuildOptions& opt, cuda
   a.keys[1] = keys[1];
   a.seeds = seeds;
   a.sizes = sizes;
-  Node* q_split[2] = {qmem, qmem + split_cap};
+  Node* q_split[2][2] = {{qmem, qmem + split_cap}, {qmem + 2 * split_cap, qmem + 2 * split_cap + heavy_cap}};
   {
-    Node* q = qmem + 2 * split_cap;
+    Node* q = qmem + 2 * (split_cap + heavy_cap);
     for (uint32_t c = 0; c < nclass; c++) {
       a.table[c] = ct.t[c];
       a.leaf_of[c] = class_leaf[c];
@@ -900,13 +966,17 @@ int build_sets(const SetInput* in, uint32_t count, const BuildOptions& opt, cuda
       q += part_cap[c];
     }
   }
-  a.split_cap = static_cast<uint32_t>(split_cap);
+  a.split_cap[0] = static_cast<uint32_t>(split_cap);
+  a.split_cap[1] = static_cast<uint32_t>(heavy_cap);
+  a.heavy_flag = any_heavy ? heavy_flag_index : 2;
   a.full_n = full_n;
   a.part_n = part_n;
   a.error = d_error;
   a.exec_count = exec;
-  a.split_in = q_split[0];
-  a.split_in_count = level_n;
+  for (int h = 0; h < 2; h++) {
+    a.split_in[h] = q_split[h][0];
+    a.split_in_count[h] = level_n + h;
+  }
   // prefix sums s_i, code-slot bases (global over all sets), first queue entries
   if (NB) {
     const LookState st{look_flags, look, look + 3 * std::max(group_tiles, bit_tiles), tickets};
@@ -926,49 +996,8 @@ int build_sets(const SetInput* in, uint32_t count, const BuildOptions& opt, cuda
   RS_CUDA(cudaGetLastError());
   timer.mark();
 
-  // level plan: largest node per level over all classes
-  std::vector<uint64_t> level_max(nclass);
-  uint32_t max_leaf = 0;
-  for (uint32_t c = 0; c < nclass; c++) {
-    level_max[c] = h_cls_max[c];
-    max_leaf = std::max(max_leaf, class_leaf[c]);
-  }
-
-  // Level plan: the largest node of every split level, and whether the
-  // level is searched shared.  That costs a few microseconds of CTA-wide steps
-  // per node and removes the level's tail, a few long geometric searches on an
-  // idle device, so it pays where a node's expected trials x keys reach 2^21
-  // evaluations, or 2^16 on a level of few nodes: 8 of the largest size per warp
-  // of the device, counting the keys of every class over its largest node
-  // (half of it, since parts are smaller; at the roots, the buckets).
-  // Split phase without and with the second clause: l = 12, b = 100: 10^5 keys
-  // 0.84 -> 0.39 ms, 10^6 keys 2.29 -> 1.81 ms (5 * 10^6 keys, above the line: 7.1
-  // against 8.2 ms); l = 13, b = 100, 3 * 10^5 keys 12.6 -> 6.6 ms; l = 12, b = 2000,
-  // 3 * 10^5 keys 4.7 -> 2.8 ms; l = 11, b = 100, 3 * 10^5 keys 1.30 -> 0.69 ms (3 * 10^6
-  // keys: 4.5 against 5.0 ms).
-  std::vector<uint64_t> plan_mx;
-  std::vector<char> plan_share;
-  {
-    std::vector<uint64_t> lm = level_max;
-    for (;;) {
-      uint64_t mx = 0, nodes = 0;
-      double heavy = 0;
-      for (uint32_t c = 0; c < nclass; c++)
-        if (lm[c] > class_leaf[c]) {
-          mx = std::max(mx, lm[c]);
-          nodes += plan_mx.empty() ? nb_c[c] : 2 * keys_c[c] / lm[c];
-          heavy = std::max(heavy, double(T[c].expected_trials[lm[c]]) * double(lm[c]));
-        }
-      if (mx == 0 || plan_mx.size() > kMaxDepth + 1) break;
-      plan_mx.push_back(mx);
-      const bool few = nodes <= 16ull * 32 * sm_count;
-      plan_share.push_back(heavy >= double(few ? 1 << 16 : 1 << 21));
-      for (uint32_t c = 0; c < nclass; c++)
-        lm[c] = lm[c] > class_leaf[c] ? T[c].next_max[lm[c]] : 0;
-    }
-  }
   SharedNodes shared{};
-  uint64_t share_cap = std::find(plan_share.begin(), plan_share.end(), 1) != plan_share.end() ? split_cap : 0;
+  uint64_t share_cap = heavy_cap;
   std::vector<char> share_leaves(nclass);
   for (uint32_t c = 0; c < nclass; c++) {
     share_leaves[c] = leaves_shared(class_leaf[c], class_extra[c]);
@@ -1016,14 +1045,19 @@ int build_sets(const SetInput* in, uint32_t count, const BuildOptions& opt, cuda
       if (mx == 0) break;
       if (level > kMaxDepth) return fail(RECSPLIT_E_INVALID, "splitting tree deeper than 63 levels");
       const int cur = level & 1;
-      a.split_in = q_split[cur];
-      a.split_in_count = level_n + level;
-      a.split_out = q_split[cur ^ 1];
-      a.split_out_count = level_n + level + 1;
-      a.work_counter = level_work + level;
-      const bool share = size_t(level) < plan_share.size() && plan_share[level];
-      if (share) shared.epoch++;
-      int r = launch_split_level(a, mx, trials, max_leaf, tables, sm_count, ws, share ? &shared : nullptr);
+      for (int h = 0; h < 2; h++) {
+        a.split_in[h] = q_split[h][cur];
+        a.split_in_count[h] = level_n + 2 * level + h;
+        a.split_out[h] = q_split[h][cur ^ 1];
+        a.split_out_count[h] = level_n + 2 * (level + 1) + h;
+      }
+      a.work_counter = level_work + 2 * level;
+      int r = launch_split_level(a, mx, trials, max_leaf, tables, sm_count, ws);
+      if (!r && size_t(level) < level_heavy.size() && level_heavy[level]) {
+        a.work_counter++;
+        shared.epoch++;
+        r = launch_split_level(a, mx, trials, max_leaf, tables, sm_count, ws, &shared);
+      }
       if (r) return r;
       for (uint32_t c = 0; c < nclass; c++)
         level_max[c] = level_max[c] > class_leaf[c] ? T[c].next_max[level_max[c]] : 0;

@@ -63,10 +63,19 @@ int golomb_rice_param(const Strategy& st, uint64_t m);
 
 // Per-size tables for node sizes 0 .. mmax.  Device form: four words per size
 //   w0 = fixed_bits(subtree) | codes(subtree) << 32
-//   w1 = unit | fanout << 32 | r << 40
+//   w1 = unit | fanout << 32 | r << 40 | heavy flags << 48: for each of the node
+//        itself, its children of `unit` keys and its last child (2 bits each),
+//        whether it is a split node of kHeavyEvals[0], [1] expected evaluations
+//        and kHeavyTrials trials
 //   w2 = expected number of trials (1/p rounded up)
 //   w3 = ceil(2^32 / unit) for unit >= 2 (exact floor(v / unit) for v < m < 2^16), else 0
 constexpr int kTableWords = 4;
+constexpr uint64_t kHeavyEvals[2] = {1ull << 16, 1ull << 21};
+constexpr uint64_t kHeavyTrials = 1024;  // the warps of a CTA test 1024 indices at a time
+constexpr int kHeavyShift = 48;
+inline bool is_heavy(uint64_t trials, uint64_t m, uint64_t evals) {
+  return trials >= kHeavyTrials && (trials >= evals || trials * m >= evals);
+}
 struct Tables {
   uint64_t mmax = 0;
   std::vector<uint8_t> r;
@@ -74,6 +83,8 @@ struct Tables {
   std::vector<uint64_t> codes;
   std::vector<uint64_t> expected_trials;  // 1/p rounded up (search stall detection)
   std::vector<uint64_t> next_max;         // largest child of the split nodes of up to m keys
+  std::vector<double> heaviest;           // most expected trials x keys of the split nodes of up to m keys that take
+                                          // kHeavyTrials trials
   std::vector<uint64_t> range;            // output range of a subtree (m when extra = 0)
   std::vector<uint64_t> device_words;     // kTableWords per size
 };
@@ -260,10 +271,13 @@ struct SearchArgs {
   uint32_t* sizes;                        // node size per code slot
   const uint64_t* table[kMaxClasses];     // device tables per class
   uint32_t leaf_of[kMaxClasses];          // leaf size per class
-  Node* split_in;                         // split nodes of this level
-  uint32_t* split_in_count;
-  Node* split_out;                        // split nodes of the next level
-  uint32_t* split_out_count;
+  // split nodes of this level and of the next, [0] light and [1] heavy (searched
+  // shared): by the heavy flag of its table word, 0 or 1 (2: none is heavy)
+  Node* split_in[2];
+  uint32_t* split_in_count[2];
+  Node* split_out[2];
+  uint32_t* split_out_count[2];
+  uint32_t heavy_flag;
   Node* full_q[kMaxClasses];              // leaves of exactly the class's leaf size
   uint32_t* full_n;                       // per class
   Node* part_q[kMaxClasses];              // leaves of 2 .. leaf-1 keys
@@ -274,7 +288,7 @@ struct SearchArgs {
   uint32_t extra_of[kMaxClasses];         // leaf range extra per class
   // queue capacities: an append beyond one sets RECSPLIT_E_INVALID in *error
   // instead of writing (the sizes are computed to suffice; this guards them)
-  uint32_t split_cap, full_cap[kMaxClasses], part_cap[kMaxClasses];
+  uint32_t split_cap[2], full_cap[kMaxClasses], part_cap[kMaxClasses];
   // work counting (null unless counting): [0] hash evaluations the leaf
   // searches executed, [1] those of the split searches
   unsigned long long* exec_count;
@@ -297,8 +311,8 @@ struct SharedNodes {
 };
 constexpr uint32_t kSharedCtas = 4096;
 
-// share: null for the one-group-per-node search; else the level is searched
-// with nodes shared by the CTAs that find the queue empty (st zeroed as above)
+// share: null for the level's light nodes, a group of warps each; else its
+// heavy nodes, shared by the CTAs that find the queue empty
 // tables: the level may hold nodes of five to seven equal parts, which are
 // counted by table; trials: the most that a node of the level is expected to
 // take

@@ -157,6 +157,12 @@ __device__ __forceinline__ uint32_t phi_fixed(uint64_t xpre, uint64_t kpre) {
     return __umulhi(h, static_cast<uint32_t>(M));
 }
 
+// Heavy flag of a table word 1: of the node itself (which = 0), its children of
+// `unit` keys (1) or its last child (2).
+__device__ __forceinline__ bool heavy_flag(uint64_t w1, uint32_t which, uint32_t flag) {
+  return flag < 2 && (w1 >> (kHeavyShift + 2 * which + flag) & 1);
+}
+
 // ---------------------------------------------------------------- bit arrays
 // Bit k of an array is bit (k mod 64) of word k / 64.
 __device__ __forceinline__ uint64_t read_bits(const uint64_t* a, uint64_t pos, uint32_t width) {

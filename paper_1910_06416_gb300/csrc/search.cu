@@ -394,13 +394,16 @@ __device__ __forceinline__ void split_search(const uint64_t* __restrict__ keys, 
 }
 
 // Emits the children of a split node with at least two keys into the queues
-// of full leaves, partial leaves or next-level splits (one warp).
-__device__ void emit_children(const SearchArgs& a, const Node& nd, const uint64_t* table, uint32_t leaf,
-                              uint32_t unit, uint32_t fanout, uint32_t lane) {
+// of full leaves, partial leaves or next-level splits, light or heavy (one
+// warp).
+__device__ void emit_children(const SearchArgs& a, const Node& nd, const uint64_t* table, uint64_t w1, uint32_t leaf,
+                              uint32_t lane) {
+  const uint32_t unit = static_cast<uint32_t>(w1), fanout = static_cast<uint32_t>(w1 >> 32) & 0xFF;
   const uint32_t t = lane;
   const uint32_t k = t + 1 < fanout ? unit : nd.m - unit * (fanout - 1);
   const bool valid = t < fanout && k >= 2;
-  const uint32_t kind = k == leaf ? 0 : (k < leaf ? 1 : 2);
+  const uint32_t kind =
+      !valid ? 4 : (k == leaf ? 0 : (k < leaf ? 1 : (heavy_flag(w1, t + 1 < fanout ? 1 : 2, a.heavy_flag) ? 3 : 2)));
   const uint32_t c_of_node = nd.depth >> 8;
   const uint32_t unit_codes = static_cast<uint32_t>(table[kTableWords * unit] >> 32);
   Node child;
@@ -409,14 +412,14 @@ __device__ void emit_children(const SearchArgs& a, const Node& nd, const uint64_
   child.slot = nd.slot + 1 + t * unit_codes;
   child.depth = nd.depth + 1;
 #pragma unroll
-  for (uint32_t c = 0; c < 3; c++) {
-    const bool mine = valid && kind == c;
+  for (uint32_t c = 0; c < 4; c++) {
+    const bool mine = kind == c;
     const uint32_t ballot = __ballot_sync(0xFFFFFFFFu, mine);
     if (!ballot) continue;
     const uint32_t leader = __ffs(ballot) - 1;
-    Node* q = c == 0 ? a.full_q[c_of_node] : (c == 1 ? a.part_q[c_of_node] : a.split_out);
-    uint32_t* cnt = c == 0 ? a.full_n + c_of_node : (c == 1 ? a.part_n + c_of_node : a.split_out_count);
-    const uint32_t cap = c == 0 ? a.full_cap[c_of_node] : (c == 1 ? a.part_cap[c_of_node] : a.split_cap);
+    Node* q = c == 0 ? a.full_q[c_of_node] : (c == 1 ? a.part_q[c_of_node] : a.split_out[c - 2]);
+    uint32_t* cnt = c == 0 ? a.full_n + c_of_node : (c == 1 ? a.part_n + c_of_node : a.split_out_count[c - 2]);
+    const uint32_t cap = c == 0 ? a.full_cap[c_of_node] : (c == 1 ? a.part_cap[c_of_node] : a.split_cap[c - 2]);
     uint32_t base = 0;
     if (lane == leader) base = atomicAdd(cnt, __popc(ballot));
     base = __shfl_sync(0xFFFFFFFFu, base, leader);
@@ -462,9 +465,10 @@ __device__ __forceinline__ int split_setup(const Node& nd, const uint64_t* table
         // second-phase keys of the two-phase block search (speed only: any
         // value from 1 to m - 1 gives the same index); about 1.75 sqrt(m)
         // minimises the modelled work (19 of 112 keys, 18 of 96, 42 of 560),
-        // with whole fours in the first phase
+        // with whole fours in the first phase; below 90 keys too many indices
+        // reach the second phase (three of five at 60 keys)
         const uint32_t head = nd.m - static_cast<uint32_t>(1.75f * sqrtf(static_cast<float>(nd.m))) - 1;
-        sp.tail = nd.m - (head & ~3u);
+        sp.tail = nd.m < 90 ? 0 : nd.m - (head & ~3u);
       } else {
         mode = 7;
       }
@@ -531,7 +535,7 @@ __device__ __forceinline__ void partition_node(const SearchArgs& a, const Node& 
     else
       set_error(a.error, RECSPLIT_E_INVALID);  // unreachable for a correct split
   }
-  if (first_warp) emit_children(a, nd, table, a.leaf_of[cls], unit, fanout, lane);
+  if (first_warp) emit_children(a, nd, table, w1, a.leaf_of[cls], lane);
 }
 
 // COUNT: work counting (the evaluations executed go to a.exec_count[1]);
@@ -565,7 +569,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_split_level(SearchArgs a, uint3
   __shared__ unsigned long long wexec[kWarps];  // work counting: evaluations per warp, flushed at exit
   const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (COUNT && lane == 0) wexec[warp] = 0;
-  const uint32_t total = *a.split_in_count;
+  const uint32_t total = *a.split_in_count[0];
   // (a counting build keeps the launch shape: with one warp per node its count is
   // the same in every build)
   if (!COUNT) gwarps = group_warps(gwarps, total, spread);
@@ -584,7 +588,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_split_level(SearchArgs a, uint3
     {
       // search: the parameters live only for this scope, so the registers
       // of the search loops are not shared with the partition step's state
-      const Node nd = a.split_in[idx];
+      const Node nd = a.split_in[0][idx];
       const uint32_t depth = nd.depth & kDepthMask;
       const uint64_t* table = a.table[nd.depth >> 8];
       SplitParams sp;
@@ -610,7 +614,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_split_level(SearchArgs a, uint3
 
     const uint64_t seed = best[gid];
     if (!*reinterpret_cast<volatile int*>(a.error)) {
-      const Node nd = a.split_in[idx];
+      const Node nd = a.split_in[0][idx];
       partition_node(a, nd, seed, nd.m <= cap ? mine : nullptr, tig, gthreads, lane, wig == 0, fill[gid]);
     }
     group_sync(gid, gwarps);
@@ -732,13 +736,15 @@ __device__ __forceinline__ uint64_t shared_search_warp(const uint64_t* __restric
       }
     }
     if constexpr (MODE >= 8) {
-      uint64_t hit;
-      evals += shared_block_two_phase<MODE, STAGED>(keys, sp, depth, lane, base0, best, surv, &hit);
-      if (hit != ~0ull) {
-        if (lane == 0) atomicMin(reinterpret_cast<unsigned long long*>(best), hit);
-        return evals;
+      if (sp.tail) {
+        uint64_t hit;
+        evals += shared_block_two_phase<MODE, STAGED>(keys, sp, depth, lane, base0, best, surv, &hit);
+        if (hit != ~0ull) {
+          if (lane == 0) atomicMin(reinterpret_cast<unsigned long long*>(best), hit);
+          return evals;
+        }
+        continue;
       }
-      continue;
     }
     for (uint32_t r = 0; r < kShareRounds; r++) {
       const uint64_t base = base0 + r * 32;
@@ -880,8 +886,10 @@ __device__ __forceinline__ void shared_nodes(const Node* queue, uint32_t total, 
   }
 }
 
-// Participants worth having on a split node: one CTA per 2^12 expected trials,
-// at most 16 (a node of a few hundred trials gains nothing).
+// Participants worth having on a split node: one CTA per 2^10 expected trials
+// (a CTA's warps test 1024 indices at a time), at most 16: what more of them
+// test lies beyond the index found and takes issue slots from other nodes (16
+// on nodes of 3679 trials, l = 12, b = 2000: split phase 2.8 -> 4.7 ms).
 template <bool COUNT>
 __global__ void __launch_bounds__(kThreads, 4) k_split_shared(SearchArgs a, SharedNodes st, uint32_t cap,
                                                               uint32_t tables) {
@@ -894,10 +902,10 @@ __global__ void __launch_bounds__(kThreads, 4) k_split_shared(SearchArgs a, Shar
   if (tables) fill_part_counts(reinterpret_cast<uint32_t*>(dynamic));
   uint64_t* const mine = dynamic + (tables ? kPartCounts : 0);
   shared_nodes(
-      a.split_in, *a.split_in_count, st, a.work_counter, a.error,
+      a.split_in[1], *a.split_in_count[1], st, a.work_counter, a.error,
       [&](const Node& nd) {
         const uint64_t et = a.table[nd.depth >> 8][kTableWords * nd.m + 2];
-        return static_cast<uint32_t>(min(uint64_t(16), max(uint64_t(1), et >> 12)));
+        return static_cast<uint32_t>(min(uint64_t(16), max(uint64_t(1), et >> 10)));
       },
       [&](const Node& nd) {
         const uint64_t* src = a.keys[nd.depth & 1] + nd.start;

@@ -123,6 +123,7 @@ int build_tables(uint32_t leaf, uint32_t extra, uint64_t mmax, Tables* T, std::s
   T->expected_trials.assign(mmax + 1, 0);
   T->range.assign(mmax + 1, 0);
   T->next_max.assign(mmax + 1, 0);
+  T->heaviest.assign(mmax + 1, 0.0);
   LogTerms terms;
   // the search tables, then the lookup records (two words per size)
   T->device_words.assign((kTableWords + 2) * (mmax + 1), 0);
@@ -152,13 +153,24 @@ int build_tables(uint32_t leaf, uint32_t extra, uint64_t mmax, Tables* T, std::s
     }
     const double et = std::exp(-lp);
     T->expected_trials[m] = et > 1e18 ? ~0ull : static_cast<uint64_t>(std::ceil(et));
+    T->heaviest[m] =
+        std::max(T->heaviest[m - 1], sh.fanout && et >= kHeavyTrials ? et * static_cast<double>(m) : 0.0);
     if (fb >= (1ull << 32) || nc >= (1ull << 32) || r >= 32 || sh.unit >= (1ull << 32)) {
       if (err) *err = "node size too large for the device tables";
       return RECSPLIT_E_INVALID;
     }
     T->device_words[kTableWords * m] = fb | (nc << 32);
-    T->device_words[kTableWords * m + 1] =
-        sh.unit | (static_cast<uint64_t>(sh.fanout) << 32) | (static_cast<uint64_t>(r) << 40);
+    auto heavy_flags = [&](uint64_t k) {
+      const uint64_t e = T->expected_trials[k];
+      uint64_t f = 0;
+      for (int i = 0; i < 2; i++)
+        if (k > leaf && is_heavy(e, k, kHeavyEvals[i])) f |= 1ull << i;
+      return f;
+    };
+    uint64_t flags = heavy_flags(m);
+    if (sh.fanout) flags |= heavy_flags(sh.unit) << 2 | heavy_flags(sh.last) << 4;
+    T->device_words[kTableWords * m + 1] = sh.unit | (static_cast<uint64_t>(sh.fanout) << 32) |
+                                           (static_cast<uint64_t>(r) << 40) | (flags << kHeavyShift);
     T->device_words[kTableWords * m + 2] = T->expected_trials[m];
     // word 3, lower half: M = ceil(2^32 / unit), with which floor(v * M / 2^32)
     // = floor(v / unit) for every v < m when (m - 1) * (M * unit - 2^32) < 2^32
