@@ -355,7 +355,10 @@ int recsplit_lookup_batch(const recsplit_t* const* hs, uint32_t count, const uin
   so.dev = d_so;
   so.owned = d_so != nullptr;
   so.s = s;
-  if ((rc = v.from(views.data(), count * sizeof(View), false, s))) return rc;
+  if (flat.decoded)
+    v.dev = const_cast<View*>(flat.decoded);
+  else if ((rc = v.from(views.data(), count * sizeof(View), false, s)))
+    return rc;
   if (!dev) {
     if ((rc = k.from(keys, q * sizeof(uint64_t), false, s)) || (rc = d.from(ids, q * sizeof(uint32_t), false, s)))
       return rc;

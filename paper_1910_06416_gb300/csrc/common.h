@@ -232,8 +232,10 @@ struct BuildOptions {
 int build_sets(const SetInput* sets, uint32_t count, const BuildOptions& opt, cudaStream_t s, Handle** out);
 // allow_scratch = false: allocate nothing (no per-batch decode of the lists)
 int lookup_structure(const Handle& h, const KeyInput& q, uint64_t* d_out, cudaStream_t s, bool allow_scratch = true);
-// Flat views of a batch's structures on the device (lookup.cu), or null.
+// A batch's structures on the device, decoded (lookup.cu): their views and, if
+// their codes are decoded too, their flat views; null otherwise.
 struct FlatBatch {
+  const View* decoded = nullptr;
   const void* views = nullptr;
   bool steps = false;
 };
@@ -242,12 +244,12 @@ struct FlatBatch {
 // non-minimal variant); flat: from decode_views
 int lookup_many(const View* d_views, uint32_t count, const uint32_t* d_ids, const uint64_t* d_keys, uint64_t q,
                 uint64_t* d_out, cudaStream_t s, bool any_range = true, const FlatBatch* flat = nullptr);
-// Batched lookups over several structures with several times as many queries
-// as the structures have codes: the function key of every code and s_i and the
-// size of every bucket of every structure are decoded into one pooled array
-// *scratch (the caller frees it, stream-ordered, after the lookups), and
-// *flat describes them.  With fewer queries, but at least as many as buckets,
-// s_i and o_i alone (views[i].so, host views).  Otherwise, or if the memory is
+// Batched lookups over several structures with more queries than the structures
+// have codes: the function key of every code and s_i and the size of every
+// bucket of every structure are decoded into one pooled array *scratch (the
+// caller frees it, stream-ordered, after the lookups), and *flat describes
+// them.  With fewer queries, but enough for the buckets, s_i, the size and o_i of
+// every bucket alone (views[i].so).  Otherwise, or if the memory is
 // not available, *scratch stays null and the views are unchanged (the lookups
 // then select in the lists per query).
 int decode_views(View* views, uint32_t count, uint64_t q, cudaStream_t s, uint64_t** scratch, FlatBatch* flat);

@@ -8,6 +8,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include <algorithm>
+#include <cstring>
 #include <vector>
 
 #include "device.cuh"
@@ -15,13 +16,7 @@
 namespace rs {
 namespace {
 
-// Sec. 6.3 / 7.4: s_b and o_b of bucket b from the two Elias-Fano lists.
-__device__ __forceinline__ uint64_t ef_prefix(const View& v, uint64_t b) {
-  const uint64_t pa = ef_select(v, 0, b);
-  const uint64_t xa = ((pa - b) << v.low_a) | read_bits(v.lower, b * (v.low_a + v.low_b), v.low_a);
-  return xa + static_cast<uint64_t>(static_cast<int64_t>(b) * v.delta_a);
-}
-
+// Sec. 6.3 / 7.4: o_b of bucket b, whose prefix s_b is s0, from the second Elias-Fano list.
 __device__ __forceinline__ uint64_t ef_offset(const View& v, uint64_t b, uint64_t s0) {
   const uint64_t pb = ef_select(v, 1, b);
   const uint64_t xb = ((pb - b) << v.low_b) | read_bits(v.lower, b * (v.low_a + v.low_b) + v.low_a, v.low_b);
@@ -58,10 +53,14 @@ __device__ __forceinline__ uint32_t size_of_range(const View& v, uint64_t R) {
   return static_cast<uint32_t>(a);
 }
 
+// Decoded buckets are {s_i | size << kSizeShift, o_i or a key}: values below 2^40,
+// sizes below 2^24.
+constexpr int kSizeShift = 40;
+bool decode_fits(uint64_t range, uint64_t mmax) { return range < (1ull << kSizeShift) && mmax < (1ull << 24); }
+
+// s_b and the size of bucket b (two consecutive elements of the first list).
 template <bool RANGE>
-__device__ __forceinline__ uint64_t lookup_one(const View& v, uint64_t hi, uint64_t lo) {
-  if (v.nb == 0) return 0;
-  const uint64_t b = bucket_of(hi, v.nb);
+__device__ __forceinline__ uint64_t bucket_start(const View& v, uint64_t b, uint32_t& m) {
   const uint32_t rec_w = v.low_a + v.low_b;
   const uint64_t rec = b * rec_w;
   const uint64_t pa = ef_select(v, 0, b);
@@ -70,32 +69,57 @@ __device__ __forceinline__ uint64_t lookup_one(const View& v, uint64_t hi, uint6
   const uint64_t xa1 = ((pa1 - b - 1) << v.low_a) | read_bits(v.lower, rec + rec_w, v.low_a);
   const uint64_t s0 = xa0 + static_cast<uint64_t>(static_cast<int64_t>(b) * v.delta_a);
   const uint64_t s1 = xa1 + static_cast<uint64_t>(static_cast<int64_t>(b + 1) * v.delta_a);
-  const uint32_t m = size_of_range<RANGE>(v, s1 - s0);
+  m = size_of_range<RANGE>(v, s1 - s0);
+  return s0;
+}
+
+template <bool RANGE>
+__device__ __forceinline__ uint64_t lookup_one(const View& v, uint64_t hi, uint64_t lo) {
+  if (v.nb == 0) return 0;
+  const uint64_t b = bucket_of(hi, v.nb);
+  uint32_t m;
+  const uint64_t s0 = bucket_start<RANGE>(v, b, m);
   if (m <= 1) return s0;
   return descend<RANGE>(v, s0, m, ef_offset(v, b, s0), lo);
 }
 
-// The same lookup with s_i, o_i of every bucket decoded beforehand (so[2i],
-// so[2i+1]; so[2N] = n): for batches with more queries than buckets.
+// Loads of what a decode launch before the lookup wrote.  The lookup's grid can
+// start before that launch ends (launch_lookup), so these are neither read-only
+// loads nor free to move above the wait for it.
+__device__ __forceinline__ uint64_t load_decoded(const uint64_t* p) {
+  uint64_t x;
+  asm volatile("ld.global.u64 %0, [%1];" : "=l"(x) : "l"(p));
+  return x;
+}
+__device__ __forceinline__ ulonglong2 load_decoded(const ulonglong2* p) {
+  ulonglong2 x;
+  asm volatile("ld.global.v2.u64 {%0, %1}, [%2];" : "=l"(x.x), "=l"(x.y) : "l"(p));
+  return x;
+}
+
+// The same lookup with s_i, the size and o_i of every bucket decoded beforehand:
+// for batches with at least as many queries as buckets.
 template <bool RANGE>
-__device__ __forceinline__ uint64_t lookup_decoded(const View& v, const uint64_t* __restrict__ so, uint64_t hi,
+__device__ __forceinline__ uint64_t lookup_decoded(const View& v, const uint64_t* so, uint64_t hi,
                                                    uint64_t lo) {
   if (v.nb == 0) return 0;
   const uint64_t b = bucket_of(hi, v.nb);
-  const ulonglong2 p = __ldg(reinterpret_cast<const ulonglong2*>(so) + b);
-  const uint64_t s1 = __ldg(so + 2 * b + 2);
-  const uint32_t m = size_of_range<RANGE>(v, s1 - p.x);
-  if (m <= 1) return p.x;
-  return descend<RANGE>(v, p.x, m, p.y, lo);
+  const ulonglong2 p = load_decoded(reinterpret_cast<const ulonglong2*>(so) + b);
+  const uint64_t s0 = p.x & ((1ull << kSizeShift) - 1);
+  const uint32_t m = static_cast<uint32_t>(p.x >> kSizeShift);
+  if (m <= 1) return s0;
+  return descend<RANGE>(v, s0, m, p.y, lo);
 }
 
-// Bit reads inside one bucket's code.  The tree bits are read as 32-bit
-// little-endian words (bit k of the vector is bit k mod 32 of 32-bit word
-// k / 32, the same bits as the 64-bit layout), with positions relative to the
-// 32-bit word `t` that holds the code's first bit.  A bucket's code takes about
-// two bits per key and the build rejects one that reaches 2^32 bits, so
-// positions fit 32-bit registers.  32-bit words make every mask, shift, find
-// and count a single instruction.
+// Bit reads inside one bucket's code, with positions relative to the word `t` that
+// holds the code's first bit.  A bucket's code takes about two bits per key and
+// the build rejects one that reaches 2^32 bits, so positions fit 32-bit registers.
+// The descent reads 64-bit words: its loads are scattered over the lanes, a fixed part
+// lies in one such word nine times in ten and a window in two (32-bit words took two
+// and three).  With {s_b | size, o_b} of a decoded bucket in 16 bytes: l = 8, b =
+// 100, 10^7 keys, 10^6 queries 37.2 -> 37.0 us; with a leaf range extra, whose bucket
+// sizes each query searched for before, 43.8 -> 38.0.  Scans beyond the window
+// read the same bits as 32-bit little-endian words.
 //
 // Scans stop at `end`, the 32-bit words from t to the end of the tree
 // section, and then return 2^32 - 1: the structure check of deserialize
@@ -146,13 +170,21 @@ __device__ __forceinline__ uint32_t select_in_word64(uint64_t x, uint32_t k) {
   return (up ? 32u : 0u) + select_in_word32(up ? static_cast<uint32_t>(x >> 32) : lo, up ? k - c : k);
 }
 
-// The 64 bits of the code from bit pos (relative to t), zero past `end`.
-__device__ __forceinline__ uint64_t window64(const uint32_t* __restrict__ t, uint32_t pos, uint32_t end) {
-  const uint32_t w = pos >> 5, sh = pos & 31;
-  const uint32_t a0 = w < end ? __ldg(t + w) : 0u;
-  const uint32_t a1 = w + 1 < end ? __ldg(t + w + 1) : 0u;
-  const uint32_t a2 = w + 2 < end ? __ldg(t + w + 2) : 0u;
-  return (uint64_t(__funnelshift_r(a1, a2, sh)) << 32) | __funnelshift_r(a0, a1, sh);
+// The 64 bits of the code from bit pos (relative to t), zero past the `end`
+// 64-bit words.
+__device__ __forceinline__ uint64_t window64(const uint64_t* __restrict__ t, uint32_t pos, uint32_t end) {
+  const uint32_t w = pos >> 6, sh = pos & 63;
+  const uint64_t a0 = w < end ? __ldg(t + w) : 0ull;
+  const uint64_t a1 = sh && w + 1 < end ? __ldg(t + w + 1) : 0ull;
+  return (a0 >> sh) | ((a1 << 1) << (63 - sh));
+}
+
+// The r < 32 bits of the code from bit pos on.
+__device__ __forceinline__ uint32_t code_bits(const uint64_t* __restrict__ t, uint32_t pos, uint32_t r, uint32_t end) {
+  const uint32_t w = pos >> 6, sh = pos & 63;
+  uint64_t x = __ldg(t + w) >> sh;
+  if (sh + r > 64 && w + 1 < end) x |= __ldg(t + w + 1) << (64 - sh);
+  return static_cast<uint32_t>(x) & ((1u << r) - 1u);
 }
 
 // (i * 64 + d) * W = i * (64 W) + d * W: the family key of index i at depth d
@@ -166,25 +198,24 @@ constexpr uint64_t kWeyl64 = kWeyl << 6;
 // subtree (to skip the earlier siblings).  The unary part of the bucket's
 // code (one code per node, about 1.5 bits each) is held in a 64-bit register
 // window from its first bit, so reading a unary code is a find-first-set and
-// skipping j * codes(unit) codes a select inside the window.  Where the
-// window runs out (buckets of thousands of keys), a scan of the code words
+// skipping j * codes(unit) codes a select inside the window, which is shifted past
+// what is read.  Where the window runs out (buckets of thousands of keys), a scan of the code words
 // finds the position and the window is reloaded there: the chosen subtree's
-// codes follow it, so the rest of the descent reads the new window.  Fixed parts
-// are read with two loads and a funnel shift, without a branch.  With a leaf
+// codes follow it, so the rest of the descent reads the new window.  With a leaf
 // range extra e (RANGE), a leaf of m keys maps into m + e values and the
 // siblings left behind contribute their output ranges (table word 3) instead
 // of their keys.
 template <bool RANGE>
 __device__ __forceinline__ uint64_t descend(const View& v, uint64_t s0, uint32_t m, uint64_t o, uint64_t lo) {
-  const uint32_t* __restrict__ t = reinterpret_cast<const uint32_t*>(v.tree) + (o >> 5);
-  const uint64_t left = v.tree_words32 - (o >> 5);
-  const uint32_t end = left < 0xFFFFFFFFull ? static_cast<uint32_t>(left) : 0xFFFFFFFFu;
-  uint32_t fixed = static_cast<uint32_t>(o & 31);
+  const uint64_t* __restrict__ t = v.tree + (o >> 6);
+  const uint32_t* __restrict__ t32 = reinterpret_cast<const uint32_t*>(t);
+  const uint64_t left = v.tree_words32 / 2 - (o >> 6);
+  const uint32_t end = left < 0x7FFFFFFFull ? static_cast<uint32_t>(left) : 0x7FFFFFFFu;
+  uint32_t fixed = static_cast<uint32_t>(o & 63);
   // the unary part starts after the fixed parts of all the bucket's codes
   const uint32_t u0 = fixed + static_cast<uint32_t>(__ldg(v.table + kTableWords * m));
-  uint32_t wb = 0;  // first bit of the window, relative to u0
-  uint64_t win = window64(t, u0, end);
-  uint32_t up = 0;  // bit of the next unary code, relative to u0
+  uint32_t up = u0;  // bit of the next unary code
+  uint64_t win = window64(t, u0, end);  // bits from `up` on, zeros past the window
   const uint64_t xpre = pre_key(lo);
   uint64_t dkey = 0;  // depth * W
   uint32_t c = 0;     // keys of the siblings left behind
@@ -192,25 +223,22 @@ __device__ __forceinline__ uint64_t descend(const View& v, uint64_t s0, uint32_t
   uint4 nd = __ldg(rec + m);
   for (;;) {
     const uint32_t r = (nd.w >> kLookupCodeBits) & 31, fanout = nd.w >> 28;
-    const uint32_t fw = fixed >> 5;
-    const uint32_t f0 = __ldg(t + fw);
-    const uint32_t f1 = fw + 1 < end ? __ldg(t + fw + 1) : 0u;
-    const uint32_t low = __funnelshift_r(f0, f1, fixed & 31) & ((1u << r) - 1u);
+    const uint32_t low = code_bits(t, fixed, r, end);
     fixed += r;
-    const uint32_t rel = up - wb;
-    const uint64_t rest = rel < 64 ? win >> rel : 0ull;
-    uint32_t one;  // the unary code's one bit, relative to u0
-    if (rest) {
-      one = up + static_cast<uint32_t>(__ffsll(static_cast<long long>(rest)) - 1);
-    } else {
-      const uint32_t a = code_next_one(t, u0 + up, end);
+    uint32_t unary;  // zeros of the unary code
+    if (!win) {
+      // no one bit is left in the window: the rest of the descent reads from the next one on
+      const uint32_t a = code_next_one(t32, up, 2 * end);
       if (a == ~0u) return ~0ull;
-      one = a - u0;
-      wb = one;  // the rest of the descent reads from here on
-      win = window64(t, u0 + wb, end);
+      unary = a - up;
+      win = window64(t, a, end);
+    } else {
+      unary = static_cast<uint32_t>(__ffsll(static_cast<long long>(win)) - 1);
+      win >>= unary;
     }
-    const uint64_t seed = (uint64_t(one - up) << r) | low;
-    up = one + 1;
+    win >>= 1;
+    const uint64_t seed = (uint64_t(unary) << r) | low;
+    up += unary + 1;
     const uint64_t k = seed * kWeyl64 + dkey;
     const uint32_t h = family_top32(xpre, k ^ (k >> 30));
     if (fanout == 0) return s0 + c + __umulhi(h, RANGE ? m + v.extra : m);
@@ -223,16 +251,15 @@ __device__ __forceinline__ uint64_t descend(const View& v, uint64_t s0, uint32_t
       // one of rank part * codes(unit) - 1
       const uint32_t skip = part * (nd.w & ((1u << kLookupCodeBits) - 1));
       if (skip) {
-        const uint32_t rel = up - wb;
-        const uint64_t x = rel < 64 ? win & (~0ull << rel) : 0ull;
-        if (static_cast<uint32_t>(__popcll(x)) >= skip) {
-          up = wb + select_in_word64(x, skip - 1) + 1;
+        if (static_cast<uint32_t>(__popcll(win)) >= skip) {
+          const uint32_t past = select_in_word64(win, skip - 1);
+          win = (win >> past) >> 1;
+          up += past + 1;
         } else {
-          const uint32_t a = code_select(t, u0 + up, skip - 1, end);
+          const uint32_t a = code_select(t32, up, skip - 1, 2 * end);
           if (a == ~0u) return ~0ull;
-          up = a - u0 + 1;
-          wb = up;  // the chosen subtree's codes start here
-          win = window64(t, u0 + wb, end);
+          up = a + 1;
+          win = window64(t, up, end);  // the chosen subtree's codes start here
         }
       }
       // keys (or, with a leaf range extra, output ranges) of the siblings left behind
@@ -246,9 +273,8 @@ __device__ __forceinline__ uint64_t descend(const View& v, uint64_t s0, uint32_t
 }
 
 // ---------------------------------------------------------------- flat codes
-// A batch with several times as many queries as the structure has codes
-// (flat_pays) decodes every code once: the function key K ^ (K >> 30) of code c (preorder) of the
-// bucket that starts at s_b is stored at flat[s_b + c] (a bucket of m keys has
+// A batch with more queries than the structure has codes (flat_pays) decodes every
+// code once: the function key K ^ (K >> 30) of code c (preorder) of the bucket that starts at s_b is stored at flat[s_b + c] (a bucket of m keys has
 // fewer than m codes), and so holds s_b, the bucket's size and the key of its
 // first code in 16 bytes: {s_b | m << 40, key}.  A level of the
 // descent then loads its key and steps over the earlier siblings' codes with
@@ -280,19 +306,15 @@ __device__ __forceinline__ uint64_t code_key(const View& v, const uint32_t* __re
   return family_key((uint64_t(un) << r) | low, depth);
 }
 
-// so packs values below 2^kFlatSizeShift and sizes below 2^24.
-constexpr int kFlatSizeShift = 40;
-bool flat_fits(uint64_t range, uint64_t mmax) { return range < (1ull << kFlatSizeShift) && mmax < (1ull << 24); }
-
 // Part g of 2^log_group of the decode of bucket b: codes g, g + 2^log_group, ...
 // Every part reads the lists for itself and scans the unary part with a cursor
 // of its own, so parts need nothing from each other.
 template <bool RANGE>
 __device__ __forceinline__ void flat_bucket(const View& v, uint64_t b, uint32_t g, uint32_t log_group) {
   uint64_t* so = const_cast<uint64_t*>(v.so);
-  const uint64_t s0 = ef_prefix(v, b);
-  const uint32_t m = size_of_range<RANGE>(v, ef_prefix(v, b + 1) - s0);
-  if (g == 0) so[2 * b] = s0 | (uint64_t(m) << kFlatSizeShift);
+  uint32_t m;
+  const uint64_t s0 = bucket_start<RANGE>(v, b, m);
+  if (g == 0) so[2 * b] = s0 | (uint64_t(m) << kSizeShift);
   if (m < 2) return;
   const uint64_t w0 = __ldg(v.table + kTableWords * m);
   const uint32_t codes = static_cast<uint32_t>(w0 >> 32);
@@ -341,18 +363,25 @@ uint32_t flat_log_group(uint64_t codes, uint64_t nb, uint64_t per) {
 // threads the device holds).
 uint64_t codes_per_part(uint64_t codes) { return std::max<uint64_t>(2, codes >> 19); }
 
-// Whether a batch of q queries decodes the codes first: the decode costs
-// about as much as three queries per code gain (l = 8, b = 100, 10^7 keys: 3.6 *
-// 10^6 queries 97 us either way, 7.1 * 10^6 187 -> 155 us; l = 12, b = 2000, 3 *
-// 10^6 keys: 2.0 codes' worth of queries 54 -> 38 us), a few microseconds at
-// least, and buckets of a few codes have nothing to skip (l = 5, b = 5: 1.6 codes,
+// Whether a batch of q queries decodes the codes first, at 1.5 queries per code: l =
+// 8, b = 100, 10^7 keys (1.78 * 10^6 codes), with the lists decoded alone and with the
+// codes: 1.0 queries per code 53 and 58 us, 1.5 73 and 70, 3.0 135 and 105; l = 12, b =
+// 2000, 3 * 10^6 keys: 1.5 45 and 27 us.  Below 200000 queries the two paths are equal
+// within 3 us, and buckets of a few codes have nothing to skip (l = 5, b = 5: 1.6 codes,
 // 517 us without and 546 with it for ten queries per code).
 bool flat_pays(uint64_t q, uint64_t codes, uint64_t nb) {
-  return q >= 3 * codes && q >= (1u << 18) && codes >= 2 * nb;
+  return 2 * q >= 3 * codes && q >= 3 * (1u << 16) && codes >= 2 * nb;
 }
+
+// Whether a batch of q queries decodes the buckets of the lists first: l = 8, b = 100,
+// 10^5 buckets: without and with it 2 * 10^5 queries 16.5 and 16.2 us, 4 * 10^5 25.2
+// and 20.7, 10^6 51.5 and 34.7; l = 5, b = 5, 2 * 10^6 buckets: 10^6 queries 53.5 and
+// 55.6 us, 3.2 * 10^6 150 and 87.
+bool decode_pays(uint64_t q, uint64_t nb) { return q >= nb / 2 + (1u << 18); }
 
 template <bool RANGE>
 __global__ void __launch_bounds__(256) k_flat_decode(const __grid_constant__ View v, uint32_t log_group) {
+  cudaTriggerProgrammaticLaunchCompletion();
   const uint64_t i = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x;
   if (i >> log_group < v.nb) flat_bucket<RANGE>(v, i >> log_group, i & ((1u << log_group) - 1), log_group);
 }
@@ -414,14 +443,14 @@ bool steps_computed(const View& v) { return v.mmax < 65536 && v.leaf >= 2; }
 template <bool RANGE, bool STEPS>
 __device__ __forceinline__ uint64_t lookup_flat(const FlatView& v, uint64_t hi, uint64_t lo) {
   if (v.nb == 0) return 0;
-  const ulonglong2 p = __ldg(v.so + bucket_of(hi, v.nb));
-  const uint64_t s0 = p.x & ((1ull << kFlatSizeShift) - 1);
-  uint32_t m = static_cast<uint32_t>(p.x >> kFlatSizeShift);
+  const ulonglong2 p = load_decoded(v.so + bucket_of(hi, v.nb));
+  const uint64_t s0 = p.x & ((1ull << kSizeShift) - 1);
+  uint32_t m = static_cast<uint32_t>(p.x >> kSizeShift);
   if (m <= 1) return s0;
   const uint64_t* __restrict__ code = v.flat + s0;
   const uint64_t xpre = pre_key(lo);
   uint32_t c = 0;  // keys (or output ranges) of the siblings left behind
-  for (uint64_t kp = p.y;; kp = __ldg(code)) {
+  for (uint64_t kp = p.y;; kp = load_decoded(code)) {
     const uint32_t h = family_top32(xpre, kp);
     uint32_t unit, codes, part;  // of every child but the last; the key's child
     if constexpr (STEPS) {
@@ -464,6 +493,7 @@ __global__ void __launch_bounds__(256, 8) k_lookup_u64_flat(FlatView v, const ui
   for (uint64_t i = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; i < q; i += uint64_t(gridDim.x) * blockDim.x) {
     uint64_t hi, lo;
     signature_u64(__ldg(keys + i), hi, lo);
+    cudaGridDependencySynchronize();  // the decode's results are read from here on
     out[i] = lookup_flat<RANGE, STEPS>(v, hi, lo);
   }
 }
@@ -478,6 +508,7 @@ __global__ void __launch_bounds__(256, 8) k_lookup_bytes_flat(FlatView v, const 
     uint64_t hi, lo;
     const bool ok = o0 <= o1 && o1 <= last;  // else read as the empty string
     signature_bytes(bytes + (ok ? o0 : 0), ok ? o1 - o0 : 0, hi, lo);
+    cudaGridDependencySynchronize();
     out[i] = lookup_flat<RANGE, false>(v, hi, lo);
   }
 }
@@ -500,43 +531,54 @@ __global__ void __launch_bounds__(256, 8) k_lookup_many_flat(const FlatView* __r
   }
 }
 
-// s_i and o_i of every bucket, one thread per element.
-__global__ void k_ef_decode(View v, uint64_t* __restrict__ so) {
-  for (uint64_t i = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; i <= v.nb; i += uint64_t(gridDim.x) * blockDim.x) {
-    const uint64_t s = ef_prefix(v, i);
-    so[2 * i] = s;
-    so[2 * i + 1] = ef_offset(v, i, s);
-  }
+template <bool RANGE>
+__device__ __forceinline__ void decode_bucket(const View& v, uint64_t b) {
+  uint64_t* so = const_cast<uint64_t*>(v.so);
+  uint32_t m;
+  const uint64_t s0 = bucket_start<RANGE>(v, b, m);
+  reinterpret_cast<ulonglong2*>(so)[b] = make_ulonglong2(s0 | (uint64_t(m) << kSizeShift), ef_offset(v, b, s0));
 }
 
+// Every bucket, one thread each.
 template <bool RANGE>
-__global__ void k_lookup_u64(View v, const uint64_t* __restrict__ so, const uint64_t* __restrict__ keys, uint64_t q,
-                             uint64_t* __restrict__ out) {
+__global__ void k_ef_decode(View v) {
+  cudaTriggerProgrammaticLaunchCompletion();
+  for (uint64_t i = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; i < v.nb; i += uint64_t(gridDim.x) * blockDim.x)
+    decode_bucket<RANGE>(v, i);
+}
+
+template <bool RANGE, bool DECODED>
+__global__ void __launch_bounds__(256, 6) k_lookup_u64(View v, const uint64_t* so,
+                                                       const uint64_t* __restrict__ keys, uint64_t q,
+                                                       uint64_t* __restrict__ out) {
   for (uint64_t i = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; i < q; i += uint64_t(gridDim.x) * blockDim.x) {
     uint64_t hi, lo;
     signature_u64(__ldg(keys + i), hi, lo);
-    out[i] = so ? lookup_decoded<RANGE>(v, so, hi, lo) : lookup_one<RANGE>(v, hi, lo);
+    if (DECODED) cudaGridDependencySynchronize();  // the decode's results are read from here on
+    out[i] = DECODED ? lookup_decoded<RANGE>(v, so, hi, lo) : lookup_one<RANGE>(v, hi, lo);
   }
 }
 
 // 32 registers (8 blocks of 256 threads per SM): the kernel is bound by
 // instruction issue, and full occupancy outweighs a few spilled registers
 // (measured: 4.09 -> 4.01 ms for 10^8 string lookups).
-template <bool RANGE>
-__global__ void __launch_bounds__(256, 8) k_lookup_bytes(View v, const uint64_t* __restrict__ so, const uint8_t* __restrict__ bytes,
-                               const uint64_t* __restrict__ offsets, uint64_t q, uint64_t* __restrict__ out) {
+template <bool RANGE, bool DECODED>
+__global__ void __launch_bounds__(256, 8) k_lookup_bytes(View v, const uint64_t* so,
+                                                         const uint8_t* __restrict__ bytes,
+                                                         const uint64_t* __restrict__ offsets, uint64_t q, uint64_t* __restrict__ out) {
   const uint64_t last = __ldg(offsets + q);  // the bytes span [0, offsets[q])
   for (uint64_t i = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; i < q; i += uint64_t(gridDim.x) * blockDim.x) {
     const uint64_t o0 = __ldg(offsets + i), o1 = __ldg(offsets + i + 1);
     uint64_t hi, lo;
     const bool ok = o0 <= o1 && o1 <= last;  // else read as the empty string
     signature_bytes(bytes + (ok ? o0 : 0), ok ? o1 - o0 : 0, hi, lo);
-    out[i] = so ? lookup_decoded<RANGE>(v, so, hi, lo) : lookup_one<RANGE>(v, hi, lo);
+    if (DECODED) cudaGridDependencySynchronize();
+    out[i] = DECODED ? lookup_decoded<RANGE>(v, so, hi, lo) : lookup_one<RANGE>(v, hi, lo);
   }
 }
 
-// s_i and o_i of every bucket of every structure: element g of the global
-// index space belongs to the structure i with base[i] <= g < base[i + 1].
+// Buckets of every structure: bucket g of the global index space belongs to the
+// structure i with base[i] <= g < base[i + 1].
 __global__ void k_ef_decode_views(const View* __restrict__ views, const uint64_t* __restrict__ base, uint32_t count,
                                   uint64_t total) {
   for (uint64_t g = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; g < total; g += uint64_t(gridDim.x) * blockDim.x) {
@@ -546,11 +588,7 @@ __global__ void k_ef_decode_views(const View* __restrict__ views, const uint64_t
       if (__ldg(base + mid) <= g) lo = mid; else hi = mid;
     }
     const View& v = views[lo];
-    const uint64_t e = g - __ldg(base + lo);
-    uint64_t* so = const_cast<uint64_t*>(v.so);
-    const uint64_t s = ef_prefix(v, e);
-    so[2 * e] = s;
-    so[2 * e + 1] = ef_offset(v, e, s);
+    decode_bucket<true>(v, g - __ldg(base + lo));
   }
 }
 
@@ -646,80 +684,77 @@ int lookup_many(const View* d_views, uint32_t count, const uint32_t* d_ids, cons
 int decode_views(View* views, uint32_t count, uint64_t q, cudaStream_t s, uint64_t** scratch, FlatBatch* batch) {
   *scratch = nullptr;
   *batch = FlatBatch{};
-  // elements 0 .. N of every list, or the N buckets of every structure
-  // (or their parts)
-  std::vector<uint64_t> base(count + 1);
-  uint64_t elements = 0, buckets = 0, codes = 0, range = 0;
+  // the buckets of every structure, or their parts
+  uint64_t buckets = 0, codes = 0, range = 0;
   bool fits = true, steps = true;
   for (uint32_t i = 0; i < count; i++) {
-    elements += views[i].nb ? views[i].nb + 1 : 0;
     buckets += views[i].nb;
     codes += views[i].codes;
     range += views[i].range;
-    fits &= flat_fits(views[i].range, views[i].mmax);
+    fits &= decode_fits(views[i].range, views[i].mmax);
     steps &= steps_computed(views[i]);
   }
-  if (buckets == 0 || q < elements + count) return RECSPLIT_OK;
-  bool flat = fits && flat_pays(q, codes, buckets);
-  void *d_scratch = nullptr, *d_views = nullptr, *d_base = nullptr;
-  // flat: the flat views, then s_i and sizes, then the keys
-  const uint64_t view_words = (sizeof(FlatView) * count + 7) / 8;
-  if (flat && pool_alloc(&d_scratch, 8 * (view_words + 2 * buckets + range), s) != RECSPLIT_OK) flat = false;
-  if (!flat && pool_alloc(&d_scratch, 16 * elements, s) != RECSPLIT_OK)
+  if (buckets == 0 || !decode_pays(q, buckets) || !fits) return RECSPLIT_OK;
+  bool flat = flat_pays(q, codes, buckets);
+  // one allocation: the views, the flat views, the first part of every view (one
+  // copy), then the decoded buckets and, with the codes, their keys
+  constexpr uint64_t kViewWords = sizeof(View) / 8, kFlatWords = sizeof(FlatView) / 8;
+  static_assert(sizeof(View) % 8 == 0 && sizeof(FlatView) % 16 == 0, "views are copied as words");
+  auto flat_at = [&] { return (count * kViewWords + 1) & ~uint64_t(1); };  // 16-byte aligned
+  auto base_at = [&] { return flat_at() + (flat ? count * kFlatWords : 0); };
+  auto so_at = [&] { return (base_at() + count + 2) & ~uint64_t(1); };
+  void* d_scratch = nullptr;
+  if (flat && pool_alloc(&d_scratch, 8 * (so_at() + 2 * buckets + range), s) != RECSPLIT_OK) flat = false;
+  if (!flat && pool_alloc(&d_scratch, 8 * (so_at() + 2 * buckets), s) != RECSPLIT_OK)
     return RECSPLIT_OK;  // fall back to per-query selects
-  uint64_t* next_so = static_cast<uint64_t*>(d_scratch) + (flat ? view_words : 0);
+  uint64_t* const d = static_cast<uint64_t*>(d_scratch);
+  std::vector<uint64_t> host(base_at() + count + 1);
+  uint64_t* const base = host.data() + base_at();
+  uint64_t* next_so = d + so_at();
   uint64_t* keys = next_so + 2 * buckets;
   uint64_t total = 0;
   for (uint32_t i = 0; i < count; i++) {
     View& v = views[i];
     base[i] = total;
-    if (!v.nb) continue;
-    v.so = next_so;
-    if (flat) {
-      v.flat = keys;
-      v.log_group = flat_log_group(v.codes, v.nb, codes_per_part(codes));
-      keys += v.range;
+    if (v.nb) {
+      v.so = next_so;
       next_so += 2 * v.nb;
+      if (flat) {
+        v.flat = keys;
+        v.log_group = flat_log_group(v.codes, v.nb, codes_per_part(codes));
+        keys += v.range;
+      }
       total += v.nb << v.log_group;
-    } else {
-      next_so += 2 * (v.nb + 1);
-      total += v.nb + 1;
+    }
+    memcpy(host.data() + i * kViewWords, &v, sizeof(View));
+    if (flat) {
+      const FlatView f = flat_view(v);
+      memcpy(host.data() + flat_at() + i * kFlatWords, &f, sizeof(FlatView));
     }
   }
   base[count] = total;
-  std::vector<FlatView> flat_views(flat ? count : 0);
-  for (uint32_t i = 0; flat && i < count; i++) flat_views[i] = flat_view(views[i]);
-  int rc = pool_alloc(&d_views, sizeof(View) * count, s);
-  if (!rc) rc = pool_alloc(&d_base, sizeof(uint64_t) * (count + 1), s);
-  cudaError_t e = cudaSuccess;
-  if (!rc) e = cudaMemcpyAsync(d_views, views, sizeof(View) * count, cudaMemcpyHostToDevice, s);
-  if (!rc && e == cudaSuccess) e = cudaMemcpyAsync(d_base, base.data(), sizeof(uint64_t) * (count + 1),
-                                                   cudaMemcpyHostToDevice, s);
-  if (!rc && e == cudaSuccess && flat)
-    e = cudaMemcpyAsync(d_scratch, flat_views.data(), sizeof(FlatView) * count, cudaMemcpyHostToDevice, s);
-  if (!rc && e == cudaSuccess) {
+  // (a pageable copy has left the host array when cudaMemcpyAsync returns)
+  cudaError_t e = cudaMemcpyAsync(d, host.data(), host.size() * sizeof(uint64_t), cudaMemcpyHostToDevice, s);
+  const View* const d_views = reinterpret_cast<const View*>(d);
+  if (e == cudaSuccess) {
     const uint64_t blocks = (total + 255) / 256;
     if (flat)
-      k_flat_decode_views<<<static_cast<unsigned>(blocks), 256, 0, s>>>(
-          static_cast<const View*>(d_views), static_cast<const uint64_t*>(d_base), count, total);
+      k_flat_decode_views<<<static_cast<unsigned>(blocks), 256, 0, s>>>(d_views, d + base_at(), count, total);
     else
-      k_ef_decode_views<<<static_cast<unsigned>(blocks < 65535 ? blocks : 65535), 256, 0, s>>>(
-          static_cast<const View*>(d_views), static_cast<const uint64_t*>(d_base), count, total);
+      k_ef_decode_views<<<static_cast<unsigned>(blocks < 65535 ? blocks : 65535), 256, 0, s>>>(d_views, d + base_at(),
+                                                                                              count, total);
     count_launch();
     e = cudaGetLastError();
   }
-  // the pageable copies above complete before cudaMemcpyAsync returns, so the
-  // host arrays may go out of scope
-  if (d_views) cudaFreeAsync(d_views, s);
-  if (d_base) cudaFreeAsync(d_base, s);
-  if (rc || e != cudaSuccess) {
+  if (e != cudaSuccess) {
     for (uint32_t i = 0; i < count; i++) views[i].so = views[i].flat = nullptr;
     cudaFreeAsync(d_scratch, s);
-    if (rc) return rc;
     return cuda_fail(e, "decode of the structures");
   }
-  *scratch = static_cast<uint64_t*>(d_scratch);
-  if (flat) *batch = FlatBatch{d_scratch, steps};
+  *scratch = d;
+  batch->decoded = d_views;
+  if (flat) batch->views = d + flat_at();
+  batch->steps = steps;
   return RECSPLIT_OK;
 }
 
@@ -752,6 +787,25 @@ View make_view(const Handle& h) {
   return v;
 }
 
+// Launch of a lookup.  `early`: the launch before it in the stream is the decode of
+// the structure, whose blocks let this grid start once all of them run; it
+// reads its keys and computes their signatures meanwhile and waits
+// for the decode's end before it reads the decode's results (10^7 keys, l = 8,
+// b = 100: 10^6 queries 37.0 -> 34.8 us).
+template <typename... P, typename... A>
+cudaError_t launch_lookup(bool early, void (*kernel)(P...), unsigned grid, int block, cudaStream_t s, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1] = {};
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = early ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 int lookup_structure(const Handle& h, const KeyInput& q, uint64_t* d_out, cudaStream_t s, bool allow_scratch) {
   if (q.n == 0) return RECSPLIT_OK;
   LookupRange range;
@@ -762,12 +816,11 @@ int lookup_structure(const Handle& h, const KeyInput& q, uint64_t* d_out, cudaSt
   const int block = 256;
   const uint64_t want = (q.n + block - 1) / block;
   const unsigned grid = static_cast<unsigned>(want < uint64_t(sms) * 64 ? want : uint64_t(sms) * 64);
-  // With several times as many queries as codes, every code is decoded once;
-  // with at least as many as buckets, the prefix sums and offsets of all buckets are
-  // decoded once instead of selected per query (the stored structure does not
-  // change).  The scratch is allocated only then.
+  // With enough queries every code is decoded once (flat_pays), or else the prefix
+  // sums and offsets of all buckets (decode_pays) instead of selected per query (the
+  // stored structure does not change).  The scratch is allocated only then.
   uint64_t* so = nullptr;
-  if (allow_scratch && v.nb && flat_pays(q.n, v.codes, v.nb) && flat_fits(v.range, v.mmax) &&
+  if (allow_scratch && v.nb && flat_pays(q.n, v.codes, v.nb) && decode_fits(v.range, v.mmax) &&
       pool_alloc(reinterpret_cast<void**>(&so), 16 * v.nb + 8 * v.range, s) == RECSPLIT_OK) {
     View f = v;
     f.so = so;
@@ -776,33 +829,42 @@ int lookup_structure(const Handle& h, const KeyInput& q, uint64_t* d_out, cudaSt
     const uint32_t lg = flat_log_group(v.codes, v.nb, codes_per_part(v.codes));
     const unsigned dg = static_cast<unsigned>(((v.nb << lg) + block - 1) / block);
     (v.extra ? k_flat_decode<true> : k_flat_decode<false>)<<<dg, block, 0, s>>>(f, lg);
-    if (q.u64)
-      (steps_computed(v) ? (v.extra ? k_lookup_u64_flat<true, true> : k_lookup_u64_flat<false, true>)
-                         : (v.extra ? k_lookup_u64_flat<true, false> : k_lookup_u64_flat<false, false>))
-          <<<grid, block, 0, s>>>(fv, q.u64, q.n, d_out);
-    else
-      (v.extra ? k_lookup_bytes_flat<true> : k_lookup_bytes_flat<false>)<<<grid, block, 0, s>>>(fv, q.bytes, q.offsets,
-                                                                                              q.n, d_out);
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess)
+      e = q.u64 ? launch_lookup(true,
+                                steps_computed(v)
+                                    ? (v.extra ? k_lookup_u64_flat<true, true> : k_lookup_u64_flat<false, true>)
+                                    : (v.extra ? k_lookup_u64_flat<true, false> : k_lookup_u64_flat<false, false>),
+                                grid, block, s, fv, q.u64, q.n, d_out)
+                : launch_lookup(true, v.extra ? k_lookup_bytes_flat<true> : k_lookup_bytes_flat<false>, grid, block, s,
+                                fv, q.bytes, q.offsets, q.n, d_out);
     count_launch(2);
-    const cudaError_t e = cudaGetLastError();
     cudaFreeAsync(so, s);
     if (e != cudaSuccess) return cuda_fail(e, "lookup launch");
     return RECSPLIT_OK;
   }
-  if (allow_scratch && v.nb && q.n >= v.nb + 1 && pool_alloc(reinterpret_cast<void**>(&so), 16 * (v.nb + 1), s) == RECSPLIT_OK) {
-    const uint64_t dg = (v.nb + 1 + block - 1) / block;
-    k_ef_decode<<<static_cast<unsigned>(dg < 65535 ? dg : 65535), block, 0, s>>>(v, so);
+  if (allow_scratch && v.nb && decode_pays(q.n, v.nb) && decode_fits(v.range, v.mmax) &&
+      pool_alloc(reinterpret_cast<void**>(&so), 16 * v.nb, s) == RECSPLIT_OK) {
+    View d = v;
+    d.so = so;
+    const uint64_t dg = (v.nb + block - 1) / block;
+    (v.extra ? k_ef_decode<true> : k_ef_decode<false>)<<<static_cast<unsigned>(dg < 65535 ? dg : 65535), block, 0,
+                                                         s>>>(d);
     count_launch();
   } else {
     so = nullptr;
   }
-  if (q.u64)
-    (v.extra ? k_lookup_u64<true> : k_lookup_u64<false>)<<<grid, block, 0, s>>>(v, so, q.u64, q.n, d_out);
-  else
-    (v.extra ? k_lookup_bytes<true> : k_lookup_bytes<false>)<<<grid, block, 0, s>>>(v, so, q.bytes, q.offsets, q.n,
-                                                                                    d_out);
+  cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess)
+    e = q.u64 ? launch_lookup(so != nullptr,
+                              so ? (v.extra ? k_lookup_u64<true, true> : k_lookup_u64<false, true>)
+                                 : (v.extra ? k_lookup_u64<true, false> : k_lookup_u64<false, false>),
+                              grid, block, s, v, so, q.u64, q.n, d_out)
+              : launch_lookup(so != nullptr,
+                              so ? (v.extra ? k_lookup_bytes<true, true> : k_lookup_bytes<false, true>)
+                                 : (v.extra ? k_lookup_bytes<true, false> : k_lookup_bytes<false, false>),
+                              grid, block, s, v, so, q.bytes, q.offsets, q.n, d_out);
   count_launch();
-  const cudaError_t e = cudaGetLastError();
   if (so) cudaFreeAsync(so, s);
   if (e != cudaSuccess) return cuda_fail(e, "lookup launch");
   return RECSPLIT_OK;
