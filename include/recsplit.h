@@ -217,7 +217,7 @@ typedef struct recsplit_profile {
 
 /* Per-build profiling for the calling host thread: 0 off; 1 phase events
  * and the algorithmic work counts (two small kernels after the build's last
- * phase, and counters the searches update per round); 2 phase events only
+ * phase, and counters of the searches); 2 phase events only
  * (the work fields of the profile are 0).  Other values fail with
  * RECSPLIT_E_INVALID. */
 int recsplit_set_profiling(int enabled);
@@ -327,12 +327,17 @@ int recsplit_lookup_u64_static(const recsplit_t* h, const uint64_t* keys, uint64
  *  leaf_chunk:   leaves a group takes from the work queue at a time (1..64)
  *  leaf_seeds_per_lane: indices each lane tests per round (1, 2, 4 or 8)
  *  split_warps[k]: warps per split node for levels whose largest node has
- *                <64 (k=0), <256 (k=1) or more (k=2) keys (1, 2, 4 or 8)
+ *                <64 (k=0), <256 (k=1) or more (k=2) keys (1, 2, 4 or 8);
+ *                searches with fewer nodes or leaves than the device has warps
+ *                use more warps each than leaf_warps and split_warps say
  *  leaf_two_phase: 1 = phased test: map the first keys of a leaf for all of
  *                a round's indices and finish only the survivors (two phases
  *                up to 12 keys; from 13, three phases whose survivors wait in
  *                per-warp queues across rounds), 0 = test every index on
- *                all keys */
+ *                all keys.  The phased test of leaves of 4 to 8 keys with
+ *                leaf_warps 1 puts four leaves on a warp; that of full leaves of 13
+ *                keys or more uses a CTA per leaf, which idle CTAs join, whatever
+ *                leaf_warps and leaf_chunk say */
 typedef struct recsplit_tuning {
   uint32_t leaf_warps;
   uint32_t leaf_chunk;

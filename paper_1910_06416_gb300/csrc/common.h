@@ -68,7 +68,8 @@ int golomb_rice_param(const Strategy& st, uint64_t m);
 //        whether it is a split node of kHeavyEvals[0], [1] expected evaluations
 //        and kHeavyTrials trials
 //   w2 = expected number of trials (1/p rounded up)
-//   w3 = ceil(2^32 / unit) for unit >= 2 (exact floor(v / unit) for v < m < 2^16), else 0
+//   w3 = ceil(2^32 / unit) for unit >= 2 (exact floor(v / unit) for v < m < 2^16), else 0,
+//        | subtree output range << 32
 constexpr int kTableWords = 4;
 constexpr uint64_t kHeavyEvals[2] = {1ull << 16, 1ull << 21};
 constexpr uint64_t kHeavyTrials = 1024;  // the warps of a CTA test 1024 indices at a time
@@ -88,9 +89,6 @@ struct Tables {
   std::vector<uint64_t> range;            // output range of a subtree (m when extra = 0)
   std::vector<uint64_t> device_words;     // kTableWords per size
 };
-// Device words per node size m: w0 = subtree fixed bits | subtree codes << 32;
-// w1 = unit | fanout << 32 | r << 40; w2 = expected trials;
-// w3 = ceil(2^32 / unit) | subtree output range << 32.
 // After the kTableWords * (mmax + 1) words come the lookup records, one
 // 16-byte LookupRecord per node size 0 .. mmax (lookup_records()).
 int build_tables(uint32_t leaf, uint32_t extra, uint64_t mmax, Tables* out, std::string* err);

@@ -3,14 +3,23 @@
 // (Sec. 5.1), and for every leaf the first index that maps the leaf's keys
 // onto [0, m) (Sec. 5.2).
 //
-// Work unit: one node, searched by a group of G warps (G = 1, 2, 4 or 8 of the
-// 8 warps of a CTA).  Lane L of warp w of a group tests indices
+// Work unit of the light nodes: one node, searched by a group of G warps (G = 1, 2,
+// 4 or 8 of the 8 warps of a CTA).  Lane L of warp w of a group tests indices
 // w*32 + L, w*32 + L + 32G, ...; a warp stops after the round in which one of
 // its lanes succeeds, or as soon as the group's best success so far is below
 // its next round.  Every index below the final minimum has then been tested
 // by its owner, so the group minimum is the first successful index (the
 // result is deterministic and independent of G).  Nodes are handed out by an
-// atomic counter (persistent CTAs), the heaviest levels with larger groups.
+// atomic counter (persistent CTAs), in larger groups where there are fewer nodes
+// than warps.  Leaves of 4 to 8 keys share a warp four at a time
+// (k_leaves_packed); heavy split nodes and leaves of 13 keys or more are
+// searched by all CTAs that would otherwise idle (shared_nodes).
+//
+// What bounds the searches: an evaluation of the hash family alone takes 20.5 to
+// 21.5 cycles per warp and sub-partition (six 32-bit multiplies on one pipe, seven
+// shifts and xors on the other; occupancy, uniform registers and other forms of the
+// products made no difference), so a search's floor is its evaluations times
+// that, and what it adds per evaluation is kept to the counting of one value.
 #include <algorithm>
 #include <array>
 #include <climits>
@@ -538,8 +547,6 @@ __device__ __forceinline__ void partition_node(const SearchArgs& a, const Node& 
   if (first_warp) emit_children(a, nd, table, w1, a.leaf_of[cls], lane);
 }
 
-// COUNT: work counting (the evaluations executed go to a.exec_count[1]);
-// without it the counter is compiled out.
 // Warps per node or leaf: the launch shape's, doubled (up to the CTA) while
 // the launch then has at most `spread` groups' worth of work items for the
 // warps of the grid.  Their number is known on the device only.  A launch of
@@ -559,6 +566,8 @@ __host__ __device__ constexpr uint32_t group_spread(uint64_t trials) {
   return trials >= 2048 ? 32 : (trials >= 128 ? 4 : 2);
 }
 
+// Light split nodes of a level.  COUNT: work counting (the evaluations executed go to a.exec_count[1]);
+// without it the counter is compiled out.
 template <bool COUNT>
 __global__ void __launch_bounds__(kThreads, 4) k_split_level(SearchArgs a, uint32_t gwarps, uint32_t cap,
                                                              uint32_t tables, uint32_t spread) {
