@@ -145,11 +145,12 @@ struct View {
   const uint16_t* subs;
   const uint64_t* table;  // kTableWords words per size
   const LookupRecord* rec;  // one lookup record per size
-  const uint64_t* so;  // s_i, o_i of every bucket decoded beforehand, or null
+  const uint64_t* so;  // s_i and size, o_i of every bucket decoded beforehand, or null
   const uint64_t* flat;  // function key of every code decoded beforehand (lookup.cu), or null: so then
-                         // holds s_i and the size of every bucket
+                         // holds the first code's key in place of o_i
   uint64_t range;      // size of the output range
   uint64_t codes;      // stored codes
+  uint32_t flat_slope;  // places of `flat` per value of the output range, in units of 2^-32 (lookup.cu)
   uint64_t log_group;  // parts that a bucket's codes are decoded in (lookup.cu), log2
   uint64_t tree_words32;  // 32-bit words of the tree section (code scans stop there)
   uint64_t mmax;       // largest bucket (the tables cover sizes 0 .. mmax)

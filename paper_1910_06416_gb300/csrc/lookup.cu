@@ -274,12 +274,52 @@ __device__ __forceinline__ uint64_t descend(const View& v, uint64_t s0, uint32_t
 
 // ---------------------------------------------------------------- flat codes
 // A batch with more queries than the structure has codes (flat_pays) decodes every
-// code once: the function key K ^ (K >> 30) of code c (preorder) of the bucket that starts at s_b is stored at flat[s_b + c] (a bucket of m keys has
-// fewer than m codes), and so holds s_b, the bucket's size and the key of its
+// code once: the function key K ^ (K >> 30) of code c (preorder) of bucket b is stored
+// at place flat_base(s_b, b) + c, and so holds s_b, the bucket's size and the key of its
 // first code in 16 bytes: {s_b | m << 40, key}.  A level of the
 // descent then loads its key and steps over the earlier siblings' codes with
 // one multiply-add, where it otherwise reads a fixed part, finds a unary part
 // and selects past the siblings in the bit vector.
+//
+// A bucket of m keys has at most rho m + 3 codes, rho = 1 / l + 1 / lower + 2 / upper (a leaf
+// and a node of each kind per so many keys, two at the top, and of each kind at
+// most one that is not full), and fewer than m, so the places floor(rho s_b) + 4 b .. of
+// different buckets are disjoint and nearly all are used: the keys of a lookup's
+// level share sectors.
+// (One place per value of the range: 4 * 10^7 keys, l = 8, b = 100, three queries per
+// code 0.69 ms against 0.38; 3.4 * 10^7 keys in 256 structures, 7 * 10^7 queries 2.7
+// against 1.9 ms.)
+constexpr uint32_t kFlatSlack = 4;  // places per bucket beyond rho s_b
+
+// rho in units of 2^-32 (below 1: a bucket has fewer codes than keys), by leaf size: a table,
+// since a batch asks for it per structure.
+struct FlatSlopes {
+  uint32_t of[kMaxLeaf + 1];
+  FlatSlopes() : of{} {
+    for (uint32_t leaf = 1; leaf <= kMaxLeaf; leaf++) {
+      const Strategy st = make_strategy(leaf);
+      uint64_t slope = 0;
+      for (uint64_t u : {uint64_t(st.leaf), st.lower, st.upper, st.upper}) slope += ((1ull << 32) + u - 1) / u;
+      of[leaf] = static_cast<uint32_t>(std::min<uint64_t>(slope, 0xFFFFFFFFull));
+    }
+  }
+};
+uint32_t flat_slope(uint32_t leaf) {
+  static const FlatSlopes slopes;
+  return slopes.of[leaf];
+}
+
+// Places of a structure; with at most kFlatPlaces of them s_b, b and the places fit
+// 32 bits (rho is at least 1 / 24).
+uint64_t flat_places(const View& v) {
+  const uint64_t range = std::min<uint64_t>(v.range, 1ull << 40), nb = std::min<uint64_t>(v.nb, 1ull << 40);
+  const uint64_t high = (range >> 16) * v.flat_slope, low = (range & 0xFFFF) * v.flat_slope;  // range * slope in halves
+  return (high >> 16) + (low >> 32) + 1 + kFlatSlack * nb;
+}
+
+__device__ __forceinline__ uint32_t flat_base(uint32_t slope, uint64_t s, uint64_t b) {
+  return __umulhi(static_cast<uint32_t>(s), slope) + kFlatSlack * static_cast<uint32_t>(b);
+}
 
 // Key of code c of a bucket of m keys (fixed parts from bit `fixed` of t, unary
 // part un): the path to node c of the preorder gives its size, depth and the
@@ -324,7 +364,7 @@ __device__ __forceinline__ void flat_bucket(const View& v, uint64_t b, uint32_t 
   const uint64_t left = v.tree_words32 - (o >> 5);
   const uint32_t end = left < 0xFFFFFFFFull ? static_cast<uint32_t>(left) : 0xFFFFFFFFu;
   const uint32_t fixed = static_cast<uint32_t>(o & 31);
-  uint64_t* flat = const_cast<uint64_t*>(v.flat) + s0;
+  uint64_t* flat = const_cast<uint64_t*>(v.flat) + flat_base(v.flat_slope, s0, b);
   const uint32_t u0 = fixed + static_cast<uint32_t>(w0);  // first bit of the unary part
   // cursor: `rank` ones lie in [u0, word w), `word` holds the ones of word w
   // from u0 on
@@ -363,14 +403,20 @@ uint32_t flat_log_group(uint64_t codes, uint64_t nb, uint64_t per) {
 // threads the device holds).
 uint64_t codes_per_part(uint64_t codes) { return std::max<uint64_t>(2, codes >> 19); }
 
+// Most places of the flat keys, 128 MiB: beyond, they are read from HBM, while the code bits of the
+// same structures stay in L2.  l = 8, b = 100, three queries per code, lists alone and codes:
+// 4 * 10^7 keys (70 MB of flat keys) 0.52 and 0.38 ms, 10^8 (174 MB) 1.26 and 1.35,
+// 3 * 10^8 4.1 and 7.1.
+constexpr uint64_t kFlatPlaces = 1ull << 24;
+
 // Whether a batch of q queries decodes the codes first, at 1.5 queries per code: l =
 // 8, b = 100, 10^7 keys (1.78 * 10^6 codes), with the lists decoded alone and with the
 // codes: 1.0 queries per code 53 and 58 us, 1.5 73 and 70, 3.0 135 and 105; l = 12, b =
 // 2000, 3 * 10^6 keys: 1.5 45 and 27 us.  Below 200000 queries the two paths are equal
 // within 3 us, and buckets of a few codes have nothing to skip (l = 5, b = 5: 1.6 codes,
 // 517 us without and 546 with it for ten queries per code).
-bool flat_pays(uint64_t q, uint64_t codes, uint64_t nb) {
-  return 2 * q >= 3 * codes && q >= 3 * (1u << 16) && codes >= 2 * nb;
+bool flat_pays(uint64_t q, uint64_t codes, uint64_t nb, uint64_t places) {
+  return places <= kFlatPlaces && 2 * q >= 3 * codes && q >= 3 * (1u << 16) && codes >= 2 * nb;
 }
 
 // Whether a batch of q queries decodes the buckets of the lists first: l = 8, b = 100,
@@ -415,7 +461,7 @@ struct alignas(16) FlatView {
   uint32_t leaf, lower, upper, leaf_magic;
   uint32_t lower_magic, upper_magic, lower_codes, upper_codes;
   const uint4* rec;
-  uint64_t extra;
+  uint32_t extra, slope;
 };
 
 FlatView flat_view(const View& v) {
@@ -426,7 +472,7 @@ FlatView flat_view(const View& v) {
                   static_cast<uint32_t>(st.lower), static_cast<uint32_t>(st.upper),
                   v.leaf >= 2 ? magic(st.leaf) : 0, magic(st.lower), magic(st.upper), lower_codes,
                   static_cast<uint32_t>(1 + st.upper / st.lower * lower_codes),
-                  reinterpret_cast<const uint4*>(v.rec), v.extra};
+                  reinterpret_cast<const uint4*>(v.rec), v.extra, v.flat_slope};
 }
 
 // Whether the steps of a descent can be computed (lookup_flat): the
@@ -443,18 +489,19 @@ bool steps_computed(const View& v) { return v.mmax < 65536 && v.leaf >= 2; }
 template <bool RANGE, bool STEPS>
 __device__ __forceinline__ uint64_t lookup_flat(const FlatView& v, uint64_t hi, uint64_t lo) {
   if (v.nb == 0) return 0;
-  const ulonglong2 p = load_decoded(v.so + bucket_of(hi, v.nb));
+  const uint64_t b = bucket_of(hi, v.nb);
+  const ulonglong2 p = load_decoded(v.so + b);
   const uint64_t s0 = p.x & ((1ull << kSizeShift) - 1);
   uint32_t m = static_cast<uint32_t>(p.x >> kSizeShift);
   if (m <= 1) return s0;
-  const uint64_t* __restrict__ code = v.flat + s0;
+  const uint64_t* code = v.flat + flat_base(v.slope, s0, b);
   const uint64_t xpre = pre_key(lo);
   uint32_t c = 0;  // keys (or output ranges) of the siblings left behind
   for (uint64_t kp = p.y;; kp = load_decoded(code)) {
     const uint32_t h = family_top32(xpre, kp);
     uint32_t unit, codes, part;  // of every child but the last; the key's child
     if constexpr (STEPS) {
-      if (m <= v.leaf) return s0 + c + __umulhi(h, RANGE ? m + static_cast<uint32_t>(v.extra) : m);
+      if (m <= v.leaf) return s0 + c + __umulhi(h, RANGE ? m + v.extra : m);
       const uint32_t val = __umulhi(h, m);
       const bool low = m <= v.lower;
       unit = low ? v.leaf : v.lower;
@@ -474,7 +521,7 @@ __device__ __forceinline__ uint64_t lookup_flat(const FlatView& v, uint64_t hi, 
     } else {
       const uint4 nd = __ldg(v.rec + m);
       const uint32_t fanout = nd.w >> 28;
-      if (fanout == 0) return s0 + c + __umulhi(h, RANGE ? m + static_cast<uint32_t>(v.extra) : m);
+      if (fanout == 0) return s0 + c + __umulhi(h, RANGE ? m + v.extra : m);
       const uint32_t val = __umulhi(h, m);
       unit = nd.x;
       codes = nd.w & ((1u << kLookupCodeBits) - 1);
@@ -685,17 +732,17 @@ int decode_views(View* views, uint32_t count, uint64_t q, cudaStream_t s, uint64
   *scratch = nullptr;
   *batch = FlatBatch{};
   // the buckets of every structure, or their parts
-  uint64_t buckets = 0, codes = 0, range = 0;
+  uint64_t buckets = 0, codes = 0, places = 0;
   bool fits = true, steps = true;
   for (uint32_t i = 0; i < count; i++) {
     buckets += views[i].nb;
     codes += views[i].codes;
-    range += views[i].range;
+    places += flat_places(views[i]);
     fits &= decode_fits(views[i].range, views[i].mmax);
     steps &= steps_computed(views[i]);
   }
   if (buckets == 0 || !decode_pays(q, buckets) || !fits) return RECSPLIT_OK;
-  bool flat = flat_pays(q, codes, buckets);
+  bool flat = flat_pays(q, codes, buckets, places);
   // one allocation: the views, the flat views, the first part of every view (one
   // copy), then the decoded buckets and, with the codes, their keys
   constexpr uint64_t kViewWords = sizeof(View) / 8, kFlatWords = sizeof(FlatView) / 8;
@@ -704,7 +751,7 @@ int decode_views(View* views, uint32_t count, uint64_t q, cudaStream_t s, uint64
   auto base_at = [&] { return flat_at() + (flat ? count * kFlatWords : 0); };
   auto so_at = [&] { return (base_at() + count + 2) & ~uint64_t(1); };
   void* d_scratch = nullptr;
-  if (flat && pool_alloc(&d_scratch, 8 * (so_at() + 2 * buckets + range), s) != RECSPLIT_OK) flat = false;
+  if (flat && pool_alloc(&d_scratch, 8 * (so_at() + 2 * buckets + places), s) != RECSPLIT_OK) flat = false;
   if (!flat && pool_alloc(&d_scratch, 8 * (so_at() + 2 * buckets), s) != RECSPLIT_OK)
     return RECSPLIT_OK;  // fall back to per-query selects
   uint64_t* const d = static_cast<uint64_t*>(d_scratch);
@@ -722,7 +769,7 @@ int decode_views(View* views, uint32_t count, uint64_t q, cudaStream_t s, uint64
       if (flat) {
         v.flat = keys;
         v.log_group = flat_log_group(v.codes, v.nb, codes_per_part(codes));
-        keys += v.range;
+        keys += flat_places(v);
       }
       total += v.nb << v.log_group;
     }
@@ -762,6 +809,7 @@ View make_view(const Handle& h) {
   View v;
   v.so = nullptr;
   v.flat = nullptr;
+  v.flat_slope = flat_slope(header_leaf(h.header));
   v.range = h.range_size;
   v.codes = h.ncodes;
   v.log_group = 0;
@@ -819,9 +867,10 @@ int lookup_structure(const Handle& h, const KeyInput& q, uint64_t* d_out, cudaSt
   // With enough queries every code is decoded once (flat_pays), or else the prefix
   // sums and offsets of all buckets (decode_pays) instead of selected per query (the
   // stored structure does not change).  The scratch is allocated only then.
+  const uint64_t places = flat_places(v);
   uint64_t* so = nullptr;
-  if (allow_scratch && v.nb && flat_pays(q.n, v.codes, v.nb) && decode_fits(v.range, v.mmax) &&
-      pool_alloc(reinterpret_cast<void**>(&so), 16 * v.nb + 8 * v.range, s) == RECSPLIT_OK) {
+  if (allow_scratch && v.nb && flat_pays(q.n, v.codes, v.nb, places) && decode_fits(v.range, v.mmax) &&
+      pool_alloc(reinterpret_cast<void**>(&so), 16 * v.nb + 8 * places, s) == RECSPLIT_OK) {
     View f = v;
     f.so = so;
     f.flat = so + 2 * v.nb;

@@ -62,3 +62,22 @@ def test_batched_lists(rs, orc, q):
         assert np.array_equal(got[ids == i], orc.lookup_u64(blob, qk[ids == i])), i
     for h in hs:
         rs.recsplit_free(h)
+
+
+@pytest.mark.parametrize("n", [76000000, 79000000])
+def test_codes_beyond_the_cache(rs, n):
+    """On either side of the size up to which the codes are decoded (2^24 places): the same
+    values as batches too small to decode anything, and all different."""
+    keys = inputs.device_splitmix64(11, n, device="cuda")
+    s = rs.Structure.build_u64(keys, 8, 100)
+    q = 3 * s.stats()["num_codes"] // 2 + 1
+    out = torch.empty(q, dtype=torch.int64, device="cuda")
+    s.lookup_u64(keys[:q], out)
+    want = torch.empty_like(out)
+    for a in range(0, q, 250000):
+        s.lookup_u64(keys[a:min(q, a + 250000)], want[a:min(q, a + 250000)])
+    assert torch.equal(out, want)
+    assert int(out.min()) >= 0 and int(out.max()) < n
+    seen = torch.zeros(n, dtype=torch.bool, device="cuda")
+    seen[out] = True
+    assert int(seen.sum()) == q
