@@ -342,6 +342,7 @@ int recsplit_lookup_batch(const recsplit_t* const* hs, uint32_t count, const uin
   for (uint32_t i = 0; i < count; i++) {
     if (!hs[i]) return fail(RECSPLIT_E_INVALID, "structure is NULL");
     views[i] = make_view(*as_handle(hs[i]));
+    if (q >= kDecodeQueries) view_for_decode(*as_handle(hs[i]), &views[i]);
   }
   const bool dev = on_device(keys);
   if (on_device(ids) != dev || on_device(out) != dev)

@@ -150,18 +150,22 @@ struct View {
                          // holds the first code's key in place of o_i
   uint64_t range;      // size of the output range
   uint64_t codes;      // stored codes
-  uint32_t flat_slope;  // places of `flat` per value of the output range, in units of 2^-32 (lookup.cu)
-  uint64_t log_group;  // parts that a bucket's codes are decoded in (lookup.cu), log2
   uint64_t tree_words32;  // 32-bit words of the tree section (code scans stop there)
   uint64_t mmax;       // largest bucket (the tables cover sizes 0 .. mmax)
   uint32_t extra;      // leaf range extra (0: minimal)
+  uint32_t flat_slope;  // places of `flat` per value of the output range, in units of 2^-32 (lookup.cu)
+  uint32_t log_group;  // parts that a bucket's codes are decoded in (lookup.cu), log2
+  uint32_t leaf;
   uint64_t nb;
   uint64_t beta;
   int64_t delta_a, delta_b;
   uint32_t low_a, low_b;
-  uint32_t leaf;
 };
 View make_view(const Handle& h);
+// Batches below this many queries decode nothing first (lookup.cu).
+constexpr uint64_t kDecodeQueries = 3ull << 16;
+// Fills in what only a batch that may decode first reads: range, codes, flat_slope.
+void view_for_decode(const Handle& h, View* v);
 
 // ---------------------------------------------------------------- memory
 // Stream-ordered pool of the current device that keeps freed memory for

@@ -416,7 +416,7 @@ constexpr uint64_t kFlatPlaces = 1ull << 24;
 // within 3 us, and buckets of a few codes have nothing to skip (l = 5, b = 5: 1.6 codes,
 // 517 us without and 546 with it for ten queries per code).
 bool flat_pays(uint64_t q, uint64_t codes, uint64_t nb, uint64_t places) {
-  return places <= kFlatPlaces && 2 * q >= 3 * codes && q >= 3 * (1u << 16) && codes >= 2 * nb;
+  return places <= kFlatPlaces && 2 * q >= 3 * codes && q >= kDecodeQueries && codes >= 2 * nb;
 }
 
 // Whether a batch of q queries decodes the buckets of the lists first: l = 8, b = 100,
@@ -731,6 +731,7 @@ int lookup_many(const View* d_views, uint32_t count, const uint32_t* d_ids, cons
 int decode_views(View* views, uint32_t count, uint64_t q, cudaStream_t s, uint64_t** scratch, FlatBatch* batch) {
   *scratch = nullptr;
   *batch = FlatBatch{};
+  if (q < kDecodeQueries) return RECSPLIT_OK;
   // the buckets of every structure, or their parts
   uint64_t buckets = 0, codes = 0, places = 0;
   bool fits = true, steps = true;
@@ -809,9 +810,8 @@ View make_view(const Handle& h) {
   View v;
   v.so = nullptr;
   v.flat = nullptr;
-  v.flat_slope = flat_slope(header_leaf(h.header));
-  v.range = h.range_size;
-  v.codes = h.ncodes;
+  v.flat_slope = 0;
+  v.range = v.codes = 0;
   v.log_group = 0;
   v.mmax = h.header[H_MMAX];
   v.extra = header_extra(h.header);
@@ -842,6 +842,10 @@ View make_view(const Handle& h) {
 // b = 100: 10^6 queries 37.0 -> 34.8 us).
 template <typename... P, typename... A>
 cudaError_t launch_lookup(bool early, void (*kernel)(P...), unsigned grid, int block, cudaStream_t s, A... args) {
+  if (!early) {
+    kernel<<<grid, block, 0, s>>>(P(args)...);
+    return cudaGetLastError();
+  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
@@ -850,14 +854,22 @@ cudaError_t launch_lookup(bool early, void (*kernel)(P...), unsigned grid, int b
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
-  cfg.numAttrs = early ? 1 : 0;
+  cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
+void view_for_decode(const Handle& h, View* v) {
+  v->flat_slope = flat_slope(v->leaf);
+  v->range = h.range_size;
+  v->codes = h.ncodes;
 }
 
 int lookup_structure(const Handle& h, const KeyInput& q, uint64_t* d_out, cudaStream_t s, bool allow_scratch) {
   if (q.n == 0) return RECSPLIT_OK;
   LookupRange range;
-  const View v = make_view(h);
+  View v = make_view(h);
+  allow_scratch = allow_scratch && v.nb && q.n >= kDecodeQueries;
+  if (allow_scratch) view_for_decode(h, &v);
   int dev = 0, sms = 0;
   RS_CUDA(cudaGetDevice(&dev));
   RS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -869,7 +881,7 @@ int lookup_structure(const Handle& h, const KeyInput& q, uint64_t* d_out, cudaSt
   // stored structure does not change).  The scratch is allocated only then.
   const uint64_t places = flat_places(v);
   uint64_t* so = nullptr;
-  if (allow_scratch && v.nb && flat_pays(q.n, v.codes, v.nb, places) && decode_fits(v.range, v.mmax) &&
+  if (allow_scratch && flat_pays(q.n, v.codes, v.nb, places) && decode_fits(v.range, v.mmax) &&
       pool_alloc(reinterpret_cast<void**>(&so), 16 * v.nb + 8 * places, s) == RECSPLIT_OK) {
     View f = v;
     f.so = so;
@@ -892,7 +904,7 @@ int lookup_structure(const Handle& h, const KeyInput& q, uint64_t* d_out, cudaSt
     if (e != cudaSuccess) return cuda_fail(e, "lookup launch");
     return RECSPLIT_OK;
   }
-  if (allow_scratch && v.nb && decode_pays(q.n, v.nb) && decode_fits(v.range, v.mmax) &&
+  if (allow_scratch && decode_pays(q.n, v.nb) && decode_fits(v.range, v.mmax) &&
       pool_alloc(reinterpret_cast<void**>(&so), 16 * v.nb, s) == RECSPLIT_OK) {
     View d = v;
     d.so = so;
