@@ -1069,7 +1069,8 @@ int build_sets(const SetInput* in, uint32_t count, const BuildOptions& opt, cuda
       a.cls = c;
       a.work_counter = leaf_work + 2 * c;
       if (share_leaves[c]) shared.epoch++;
-      int r = launch_leaves(a, class_leaf[c], class_extra[c], sm_count, ws, share_leaves[c] ? &shared : nullptr);
+      int r = launch_leaves(a, class_leaf[c], class_extra[c], h_cls_max[c], sm_count, ws,
+                            share_leaves[c] ? &shared : nullptr);
       if (r) return r;
     }
     if (!opt.use_graph) timer.mark();

@@ -326,7 +326,8 @@ int launch_split_level(const SearchArgs& a, uint64_t max_m, uint64_t trials, uin
 // Whether the full leaves of a class are searched shared (launch_leaves then
 // needs share).
 bool leaves_shared(uint32_t leaf, uint32_t extra);
-int launch_leaves(const SearchArgs& a, uint32_t leaf, uint32_t extra, int sm_count, cudaStream_t s,
+// largest: keys of the class's largest bucket, where its table ends
+int launch_leaves(const SearchArgs& a, uint32_t leaf, uint32_t extra, uint64_t largest, int sm_count, cudaStream_t s,
                   const SharedNodes* share = nullptr);
 
 // Launch shapes of the searches for one leaf size (see recsplit_tuning_t).

@@ -1951,11 +1951,14 @@ bool leaves_shared(uint32_t leaf, uint32_t extra) {
   return !extra && leaf >= uint32_t(kFifoLeaf) && tuning_for(leaf).leaf_two_phase;
 }
 
-int launch_leaves(const SearchArgs& a, uint32_t leaf, uint32_t extra, int sm_count, cudaStream_t s,
+int launch_leaves(const SearchArgs& a, uint32_t leaf, uint32_t extra, uint64_t largest, int sm_count, cudaStream_t s,
                   const SharedNodes* share) {
-  if (leaf < 2) return RECSPLIT_OK;
+  if (leaf < 2 || largest < 2) return RECSPLIT_OK;
   const recsplit_tuning_t t = tuning_for(leaf);
-  int rc = (extra ? kFullRange : kFull)[leaf](a, t, sm_count, s, share);
+  // The kernels of full leaves read the table's entry of `leaf` keys whether or
+  // not their queue is empty, so they are launched only where the table has it:
+  // a class whose buckets are all smaller has no full leaf.
+  int rc = largest >= leaf ? (extra ? kFullRange : kFull)[leaf](a, t, sm_count, s, share) : RECSPLIT_OK;
   if (rc || leaf == 2) return rc;  // no leaves between 2 and leaf - 1
   SearchArgs b = a;
   b.work_counter++;
