@@ -684,12 +684,35 @@ int ef_width(uint64_t u, uint64_t count) {
 
 uint64_t tiles(uint64_t items) { return (items + kTile - 1) / kTile; }
 
+// Parameter class of a set.
+uint32_t class_key(const SetInput& si) { return si.leaf | (si.leaf_extra << 8); }
+
+// Adds the profile of a pass to the call's.
+void add_profile(recsplit_profile_t* sum, const recsplit_profile_t& p) {
+  sum->ms_signature += p.ms_signature;
+  sum->ms_group += p.ms_group;
+  sum->ms_split += p.ms_split;
+  sum->ms_leaf += p.ms_leaf;
+  sum->ms_encode += p.ms_encode;
+  sum->ms_total += p.ms_total;
+  sum->split_nodes += p.split_nodes;
+  sum->split_trials += p.split_trials;
+  sum->split_evals += p.split_evals;
+  sum->leaf_nodes += p.leaf_nodes;
+  sum->leaf_trials += p.leaf_trials;
+  sum->leaf_evals += p.leaf_evals;
+  sum->launches += p.launches;
+  sum->split_levels += p.split_levels;
+  sum->leaf_evals_executed += p.leaf_evals_executed;
+  sum->split_evals_executed += p.split_evals_executed;
+}
+
 }  // namespace
 
-int build_sets(const SetInput* in, uint32_t count, const BuildOptions& opt, cudaStream_t s, Handle** out) {
-  for (uint32_t i = 0; i < count; i++) out[i] = nullptr;
-  if (count == 0) return RECSPLIT_OK;
-  const double t_call = steady_ms();
+// One pass over sets of at most kMaxClasses classes; t_call: start of the call
+// (time limit).
+static int build_pass(const SetInput* in, uint32_t count, const BuildOptions& opt, cudaStream_t s, double t_call,
+                      Handle** out) {
   int dev = 0, sm_count = 0;
   RS_CUDA(cudaGetDevice(&dev));
   RS_CUDA(cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev));
@@ -702,9 +725,8 @@ int build_sets(const SetInput* in, uint32_t count, const BuildOptions& opt, cuda
   uint64_t K = 0, NB = 0, key_tiles = 0, bucket_tiles = 0, elem_tiles = 0;
   for (uint32_t i = 0; i < count; i++) {
     const SetInput& si = in[i];
-    if (si.leaf_extra > 32 - si.leaf) return fail(RECSPLIT_E_INVALID, "leaf size + leaf range extra above 32");
     any_extra |= si.leaf_extra != 0;
-    const uint32_t key = si.leaf | (si.leaf_extra << 8);
+    const uint32_t key = class_key(si);
     auto it = cls_of_leaf.find(key);
     if (it == cls_of_leaf.end()) {
       it = cls_of_leaf.emplace(key, static_cast<uint32_t>(class_leaf.size())).first;
@@ -730,7 +752,6 @@ int build_sets(const SetInput* in, uint32_t count, const BuildOptions& opt, cuda
     bucket_tiles += tiles(d.nb);
     elem_tiles += tiles(d.nb + 1);
   }
-  if (K >= (1ull << 32)) return fail(RECSPLIT_E_INVALID, "at most 2^32 - 1 keys per build");
   const uint32_t nclass = static_cast<uint32_t>(class_leaf.size());
 
   // classes by key count (queue capacities): a split node has more keys than
@@ -1259,6 +1280,48 @@ int build_sets(const SetInput* in, uint32_t count, const BuildOptions& opt, cuda
     pr.split_levels = split_levels;
     store_profile(pr);
   }
+  return RECSPLIT_OK;
+}
+
+// The searches' arguments hold kMaxClasses classes, and there are more pairs of
+// leaf size and leaf range extra than that: sets of more classes are built in
+// passes of kMaxClasses classes, in the order in which the classes first occur.
+int build_sets(const SetInput* in, uint32_t count, const BuildOptions& opt, cudaStream_t s, Handle** out) {
+  const double t_call = steady_ms();
+  std::map<uint32_t, uint32_t> class_of;
+  uint64_t keys = 0;
+  for (uint32_t i = 0; i < count; i++) {
+    out[i] = nullptr;
+    if (in[i].leaf_extra > 32 - in[i].leaf) return fail(RECSPLIT_E_INVALID, "leaf size + leaf range extra above 32");
+    class_of.emplace(class_key(in[i]), static_cast<uint32_t>(class_of.size()));
+    keys += in[i].keys.n;
+  }
+  if (keys >= (1ull << 32)) return fail(RECSPLIT_E_INVALID, "at most 2^32 - 1 keys per build");
+  if (count == 0) return RECSPLIT_OK;
+  if (class_of.size() <= size_t(kMaxClasses)) return build_pass(in, count, opt, s, t_call, out);
+  recsplit_profile_t sum{};
+  for (uint32_t first = 0; first < class_of.size(); first += kMaxClasses) {
+    std::vector<SetInput> sets;
+    std::vector<uint32_t> at;
+    for (uint32_t i = 0; i < count; i++)
+      if (class_of[class_key(in[i])] - first < uint32_t(kMaxClasses)) {
+        sets.push_back(in[i]);
+        at.push_back(i);
+      }
+    std::vector<Handle*> built(sets.size(), nullptr);
+    const int rc = build_pass(sets.data(), static_cast<uint32_t>(sets.size()), opt, s, t_call, built.data());
+    for (size_t k = 0; k < at.size(); k++) out[at[k]] = built[k];
+    if (rc) {
+      for (uint32_t i = 0; i < count; i++) {
+        delete out[i];
+        out[i] = nullptr;
+      }
+      return rc;
+    }
+    recsplit_profile_t p;
+    if (profiling_enabled() && !recsplit_last_profile(&p)) add_profile(&sum, p);
+  }
+  if (profiling_enabled()) store_profile(sum);
   return RECSPLIT_OK;
 }
 

@@ -268,7 +268,7 @@ struct Node {
   uint32_t depth;  // depth | class << 8
 };
 constexpr uint32_t kDepthMask = 0xFF;
-constexpr int kMaxClasses = 25;
+constexpr int kMaxClasses = 25;  // classes of a pass (build_sets makes as many passes as it takes)
 
 struct SearchArgs {
   uint64_t* keys[2];                      // key arrays (x ^ x >> 30) by depth parity
