@@ -111,15 +111,18 @@ __device__ __forceinline__ uint64_t lookup_decoded(const View& v, const uint64_t
   return descend<RANGE>(v, s0, m, p.y, lo);
 }
 
-// Bit reads inside one bucket's code, with positions relative to the word `t` that
-// holds the code's first bit.  A bucket's code takes about two bits per key and
-// the build rejects one that reaches 2^32 bits, so positions fit 32-bit registers.
-// The descent reads 64-bit words: its loads are scattered over the lanes, a fixed part
-// lies in one such word nine times in ten and a window in two (32-bit words took two
-// and three).  With {s_b | size, o_b} of a decoded bucket in 16 bytes: l = 8, b =
-// 100, 10^7 keys, 10^6 queries 37.2 -> 37.0 us; with a leaf range extra, whose bucket
-// sizes each query searched for before, 43.8 -> 38.0.  Scans beyond the window
-// read the same bits as 32-bit little-endian words.
+// Bit reads inside one bucket's code.  The tree bits are read as 32-bit
+// little-endian words (bit k of the vector is bit k mod 32 of 32-bit word
+// k / 32, the same bits as the 64-bit layout), with positions relative to the
+// 32-bit word `t` that holds the code's first bit.  A bucket's code takes about
+// two bits per key and the build rejects one that reaches 2^32 bits, so
+// positions fit 32-bit registers.  32-bit words make every mask, shift, find
+// and count a single instruction.  (64-bit words, half the loads but more
+// instructions a level, were slower: from host call to end of 1000 queries, l = 12,
+// b = 2000, 10^6 keys 22.4 us with 32-bit words and 23.0 with 64-bit ones, l = 8, b =
+// 100 with a leaf range extra 19.3 and 19.6, without 17.1 and 17.2; 10^6 queries, l = 8,
+// 10^7 keys 34.0 and 35.0, l = 12, 3 * 10^6 keys 35.1 and 37.1.  Only l = 5, b = 5, 10^7
+// keys favours them: 3 * 10^5 queries 24.0 and 22.8, 10^6 55.5 and 55.0.)
 //
 // Scans stop at `end`, the 32-bit words from t to the end of the tree
 // section, and then return 2^32 - 1: the structure check of deserialize
@@ -170,21 +173,13 @@ __device__ __forceinline__ uint32_t select_in_word64(uint64_t x, uint32_t k) {
   return (up ? 32u : 0u) + select_in_word32(up ? static_cast<uint32_t>(x >> 32) : lo, up ? k - c : k);
 }
 
-// The 64 bits of the code from bit pos (relative to t), zero past the `end`
-// 64-bit words.
-__device__ __forceinline__ uint64_t window64(const uint64_t* __restrict__ t, uint32_t pos, uint32_t end) {
-  const uint32_t w = pos >> 6, sh = pos & 63;
-  const uint64_t a0 = w < end ? __ldg(t + w) : 0ull;
-  const uint64_t a1 = sh && w + 1 < end ? __ldg(t + w + 1) : 0ull;
-  return (a0 >> sh) | ((a1 << 1) << (63 - sh));
-}
-
-// The r < 32 bits of the code from bit pos on.
-__device__ __forceinline__ uint32_t code_bits(const uint64_t* __restrict__ t, uint32_t pos, uint32_t r, uint32_t end) {
-  const uint32_t w = pos >> 6, sh = pos & 63;
-  uint64_t x = __ldg(t + w) >> sh;
-  if (sh + r > 64 && w + 1 < end) x |= __ldg(t + w + 1) << (64 - sh);
-  return static_cast<uint32_t>(x) & ((1u << r) - 1u);
+// The 64 bits of the code from bit pos (relative to t), zero past `end`.
+__device__ __forceinline__ uint64_t window64(const uint32_t* __restrict__ t, uint32_t pos, uint32_t end) {
+  const uint32_t w = pos >> 5, sh = pos & 31;
+  const uint32_t a0 = w < end ? __ldg(t + w) : 0u;
+  const uint32_t a1 = w + 1 < end ? __ldg(t + w + 1) : 0u;
+  const uint32_t a2 = w + 2 < end ? __ldg(t + w + 2) : 0u;
+  return (uint64_t(__funnelshift_r(a1, a2, sh)) << 32) | __funnelshift_r(a0, a1, sh);
 }
 
 // (i * 64 + d) * W = i * (64 W) + d * W: the family key of index i at depth d
@@ -198,24 +193,25 @@ constexpr uint64_t kWeyl64 = kWeyl << 6;
 // subtree (to skip the earlier siblings).  The unary part of the bucket's
 // code (one code per node, about 1.5 bits each) is held in a 64-bit register
 // window from its first bit, so reading a unary code is a find-first-set and
-// skipping j * codes(unit) codes a select inside the window, which is shifted past
-// what is read.  Where the window runs out (buckets of thousands of keys), a scan of the code words
+// skipping j * codes(unit) codes a select inside the window.  Where the
+// window runs out (buckets of thousands of keys), a scan of the code words
 // finds the position and the window is reloaded there: the chosen subtree's
-// codes follow it, so the rest of the descent reads the new window.  With a leaf
+// codes follow it, so the rest of the descent reads the new window.  Fixed parts
+// are read with two loads and a funnel shift, without a branch.  With a leaf
 // range extra e (RANGE), a leaf of m keys maps into m + e values and the
 // siblings left behind contribute their output ranges (table word 3) instead
 // of their keys.
 template <bool RANGE>
 __device__ __forceinline__ uint64_t descend(const View& v, uint64_t s0, uint32_t m, uint64_t o, uint64_t lo) {
-  const uint64_t* __restrict__ t = v.tree + (o >> 6);
-  const uint32_t* __restrict__ t32 = reinterpret_cast<const uint32_t*>(t);
-  const uint64_t left = v.tree_words32 / 2 - (o >> 6);
-  const uint32_t end = left < 0x7FFFFFFFull ? static_cast<uint32_t>(left) : 0x7FFFFFFFu;
-  uint32_t fixed = static_cast<uint32_t>(o & 63);
+  const uint32_t* __restrict__ t = reinterpret_cast<const uint32_t*>(v.tree) + (o >> 5);
+  const uint64_t left = v.tree_words32 - (o >> 5);
+  const uint32_t end = left < 0xFFFFFFFFull ? static_cast<uint32_t>(left) : 0xFFFFFFFFu;
+  uint32_t fixed = static_cast<uint32_t>(o & 31);
   // the unary part starts after the fixed parts of all the bucket's codes
   const uint32_t u0 = fixed + static_cast<uint32_t>(__ldg(v.table + kTableWords * m));
-  uint32_t up = u0;  // bit of the next unary code
-  uint64_t win = window64(t, u0, end);  // bits from `up` on, zeros past the window
+  uint32_t wb = 0;  // first bit of the window, relative to u0
+  uint64_t win = window64(t, u0, end);
+  uint32_t up = 0;  // bit of the next unary code, relative to u0
   const uint64_t xpre = pre_key(lo);
   uint64_t dkey = 0;  // depth * W
   uint32_t c = 0;     // keys of the siblings left behind
@@ -223,22 +219,25 @@ __device__ __forceinline__ uint64_t descend(const View& v, uint64_t s0, uint32_t
   uint4 nd = __ldg(rec + m);
   for (;;) {
     const uint32_t r = (nd.w >> kLookupCodeBits) & 31, fanout = nd.w >> 28;
-    const uint32_t low = code_bits(t, fixed, r, end);
+    const uint32_t fw = fixed >> 5;
+    const uint32_t f0 = __ldg(t + fw);
+    const uint32_t f1 = fw + 1 < end ? __ldg(t + fw + 1) : 0u;
+    const uint32_t low = __funnelshift_r(f0, f1, fixed & 31) & ((1u << r) - 1u);
     fixed += r;
-    uint32_t unary;  // zeros of the unary code
-    if (!win) {
-      // no one bit is left in the window: the rest of the descent reads from the next one on
-      const uint32_t a = code_next_one(t32, up, 2 * end);
-      if (a == ~0u) return ~0ull;
-      unary = a - up;
-      win = window64(t, a, end);
+    const uint32_t rel = up - wb;
+    const uint64_t rest = rel < 64 ? win >> rel : 0ull;
+    uint32_t one;  // the unary code's one bit, relative to u0
+    if (rest) {
+      one = up + static_cast<uint32_t>(__ffsll(static_cast<long long>(rest)) - 1);
     } else {
-      unary = static_cast<uint32_t>(__ffsll(static_cast<long long>(win)) - 1);
-      win >>= unary;
+      const uint32_t a = code_next_one(t, u0 + up, end);
+      if (a == ~0u) return ~0ull;
+      one = a - u0;
+      wb = one;  // the rest of the descent reads from here on
+      win = window64(t, u0 + wb, end);
     }
-    win >>= 1;
-    const uint64_t seed = (uint64_t(unary) << r) | low;
-    up += unary + 1;
+    const uint64_t seed = (uint64_t(one - up) << r) | low;
+    up = one + 1;
     const uint64_t k = seed * kWeyl64 + dkey;
     const uint32_t h = family_top32(xpre, k ^ (k >> 30));
     if (fanout == 0) return s0 + c + __umulhi(h, RANGE ? m + v.extra : m);
@@ -251,15 +250,16 @@ __device__ __forceinline__ uint64_t descend(const View& v, uint64_t s0, uint32_t
       // one of rank part * codes(unit) - 1
       const uint32_t skip = part * (nd.w & ((1u << kLookupCodeBits) - 1));
       if (skip) {
-        if (static_cast<uint32_t>(__popcll(win)) >= skip) {
-          const uint32_t past = select_in_word64(win, skip - 1);
-          win = (win >> past) >> 1;
-          up += past + 1;
+        const uint32_t rel = up - wb;
+        const uint64_t x = rel < 64 ? win & (~0ull << rel) : 0ull;
+        if (static_cast<uint32_t>(__popcll(x)) >= skip) {
+          up = wb + select_in_word64(x, skip - 1) + 1;
         } else {
-          const uint32_t a = code_select(t32, up, skip - 1, 2 * end);
+          const uint32_t a = code_select(t, u0 + up, skip - 1, end);
           if (a == ~0u) return ~0ull;
-          up = a + 1;
-          win = window64(t, up, end);  // the chosen subtree's codes start here
+          up = a - u0 + 1;
+          wb = up;  // the chosen subtree's codes start here
+          win = window64(t, u0 + wb, end);
         }
       }
       // keys (or, with a leaf range extra, output ranges) of the siblings left behind
@@ -595,9 +595,8 @@ __global__ void k_ef_decode(View v) {
 }
 
 template <bool RANGE, bool DECODED>
-__global__ void __launch_bounds__(256, 6) k_lookup_u64(View v, const uint64_t* so,
-                                                       const uint64_t* __restrict__ keys, uint64_t q,
-                                                       uint64_t* __restrict__ out) {
+__global__ void __launch_bounds__(256) k_lookup_u64(View v, const uint64_t* so, const uint64_t* __restrict__ keys,
+                                                    uint64_t q, uint64_t* __restrict__ out) {
   for (uint64_t i = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; i < q; i += uint64_t(gridDim.x) * blockDim.x) {
     uint64_t hi, lo;
     signature_u64(__ldg(keys + i), hi, lo);
