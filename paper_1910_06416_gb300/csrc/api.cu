@@ -342,7 +342,6 @@ int recsplit_lookup_batch(const recsplit_t* const* hs, uint32_t count, const uin
   for (uint32_t i = 0; i < count; i++) {
     if (!hs[i]) return fail(RECSPLIT_E_INVALID, "structure is NULL");
     views[i] = make_view(*as_handle(hs[i]));
-    if (q >= kDecodeQueries) view_for_decode(*as_handle(hs[i]), &views[i]);
   }
   const bool dev = on_device(keys);
   if (on_device(ids) != dev || on_device(out) != dev)
@@ -352,11 +351,12 @@ int recsplit_lookup_batch(const recsplit_t* const* hs, uint32_t count, const uin
   // large batches: every bucket, or every code, decoded once (freed on return)
   uint64_t* d_so = nullptr;
   FlatBatch flat;
-  if ((rc = decode_views(views.data(), count, q, s, &d_so, &flat))) return rc;
+  if ((rc = decode_views(reinterpret_cast<const Handle* const*>(hs), views.data(), count, q, s, &d_so, &flat)))
+    return rc;
   so.dev = d_so;
   so.owned = d_so != nullptr;
   so.s = s;
-  if (flat.decoded)
+  if (flat.decoded || flat.views)
     v.dev = const_cast<View*>(flat.decoded);
   else if ((rc = v.from(views.data(), count * sizeof(View), false, s)))
     return rc;

@@ -135,7 +135,11 @@ struct Handle {
   int device = 0;
 };
 
-// Device-side view of a structure, passed by value to lookup kernels.
+// Device-side view of a structure, passed by value to lookup kernels, or in an
+// array that every batch over several structures uploads.  So it holds only what
+// a lookup reads (136 bytes): with what the decodes read as well (176), and one
+// kernel for decoded lists and others (k_lookup_many), 10^4 queries over 200
+// structures took 28.8 us, 26.5 so.
 struct View {
   const uint64_t* tree;
   const uint64_t* lower;
@@ -145,27 +149,19 @@ struct View {
   const uint16_t* subs;
   const uint64_t* table;  // kTableWords words per size
   const LookupRecord* rec;  // one lookup record per size
-  const uint64_t* so;  // s_i and size, o_i of every bucket decoded beforehand, or null
-  const uint64_t* flat;  // function key of every code decoded beforehand (lookup.cu), or null: so then
-                         // holds the first code's key in place of o_i
-  uint64_t range;      // size of the output range
-  uint64_t codes;      // stored codes
+  const uint64_t* so;  // s_i and size, o_i of every bucket decoded beforehand, or null; with the codes
+                       // decoded too (lookup.cu) the first code's key in place of o_i
   uint64_t tree_words32;  // 32-bit words of the tree section (code scans stop there)
   uint64_t mmax;       // largest bucket (the tables cover sizes 0 .. mmax)
-  uint32_t extra;      // leaf range extra (0: minimal)
-  uint32_t flat_slope;  // places of `flat` per value of the output range, in units of 2^-32 (lookup.cu)
-  uint32_t log_group;  // parts that a bucket's codes are decoded in (lookup.cu), log2
-  uint32_t leaf;
   uint64_t nb;
   uint64_t beta;
   int64_t delta_a, delta_b;
   uint32_t low_a, low_b;
+  uint32_t extra;      // leaf range extra (0: minimal)
 };
 View make_view(const Handle& h);
 // Batches below this many queries decode nothing first (lookup.cu).
 constexpr uint64_t kDecodeQueries = 3ull << 16;
-// Fills in what only a batch that may decode first reads: range, codes, flat_slope.
-void view_for_decode(const Handle& h, View* v);
 
 // ---------------------------------------------------------------- memory
 // Stream-ordered pool of the current device that keeps freed memory for
@@ -235,8 +231,9 @@ struct BuildOptions {
 int build_sets(const SetInput* sets, uint32_t count, const BuildOptions& opt, cudaStream_t s, Handle** out);
 // allow_scratch = false: allocate nothing (no per-batch decode of the lists)
 int lookup_structure(const Handle& h, const KeyInput& q, uint64_t* d_out, cudaStream_t s, bool allow_scratch = true);
-// A batch's structures on the device, decoded (lookup.cu): their views and, if
-// their codes are decoded too, their flat views; null otherwise.
+// A batch's structures on the device, decoded (lookup.cu): their views with the
+// lists decoded, or their flat views with the codes decoded too; both null
+// otherwise.
 struct FlatBatch {
   const View* decoded = nullptr;
   const void* views = nullptr;
@@ -255,7 +252,8 @@ int lookup_many(const View* d_views, uint32_t count, const uint32_t* d_ids, cons
 // every bucket alone (views[i].so).  Otherwise, or if the memory is
 // not available, *scratch stays null and the views are unchanged (the lookups
 // then select in the lists per query).
-int decode_views(View* views, uint32_t count, uint64_t q, cudaStream_t s, uint64_t** scratch, FlatBatch* flat);
+int decode_views(const Handle* const* hs, View* views, uint32_t count, uint64_t q, cudaStream_t s, uint64_t** scratch,
+                 FlatBatch* flat);
 int lookup_many_bytes(const View* d_views, uint32_t count, const uint32_t* d_ids, const uint8_t* d_bytes,
                       const uint64_t* d_offsets, uint64_t q, uint64_t* d_out, cudaStream_t s);
 

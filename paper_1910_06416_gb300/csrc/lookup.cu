@@ -311,9 +311,10 @@ uint32_t flat_slope(uint32_t leaf) {
 
 // Places of a structure; with at most kFlatPlaces of them s_b, b and the places fit
 // 32 bits (rho is at least 1 / 24).
-uint64_t flat_places(const View& v) {
-  const uint64_t range = std::min<uint64_t>(v.range, 1ull << 40), nb = std::min<uint64_t>(v.nb, 1ull << 40);
-  const uint64_t high = (range >> 16) * v.flat_slope, low = (range & 0xFFFF) * v.flat_slope;  // range * slope in halves
+uint64_t flat_places(const Handle& h) {
+  const uint64_t range = std::min<uint64_t>(h.range_size, 1ull << 40), nb = std::min<uint64_t>(h.header[H_NB], 1ull << 40);
+  const uint64_t slope = flat_slope(header_leaf(h.header));
+  const uint64_t high = (range >> 16) * slope, low = (range & 0xFFFF) * slope;  // range * slope in halves
   return (high >> 16) + (low >> 32) + 1 + kFlatSlack * nb;
 }
 
@@ -346,11 +347,23 @@ __device__ __forceinline__ uint64_t code_key(const View& v, const uint32_t* __re
   return family_key((uint64_t(un) << r) | low, depth);
 }
 
-// Part g of 2^log_group of the decode of bucket b: codes g, g + 2^log_group, ...
-// Every part reads the lists for itself and scans the unary part with a cursor
-// of its own, so parts need nothing from each other.
+// What the decode of the codes reads of a structure.
+struct DecodeView : View {
+  uint64_t* flat;      // function key of every code
+  uint32_t slope;      // flat_slope
+  uint32_t log_group;  // parts that a bucket's codes are decoded in, log2
+};
+
+// Part p of the decode of the structure's buckets, 2^log_group to a bucket: part g
+// of bucket b decodes codes g, g + 2^log_group, ...  Every part reads the lists for
+// itself and scans the unary part with a cursor of its own, so parts need
+// nothing from each other.
 template <bool RANGE>
-__device__ __forceinline__ void flat_bucket(const View& v, uint64_t b, uint32_t g, uint32_t log_group) {
+__device__ __forceinline__ void flat_part(const DecodeView& v, uint64_t p) {
+  const uint32_t log_group = v.log_group;
+  const uint64_t b = p >> log_group;
+  const uint32_t g = p & ((1u << log_group) - 1);
+  if (b >= v.nb) return;
   uint64_t* so = const_cast<uint64_t*>(v.so);
   uint32_t m;
   const uint64_t s0 = bucket_start<RANGE>(v, b, m);
@@ -364,7 +377,7 @@ __device__ __forceinline__ void flat_bucket(const View& v, uint64_t b, uint32_t 
   const uint64_t left = v.tree_words32 - (o >> 5);
   const uint32_t end = left < 0xFFFFFFFFull ? static_cast<uint32_t>(left) : 0xFFFFFFFFu;
   const uint32_t fixed = static_cast<uint32_t>(o & 31);
-  uint64_t* flat = const_cast<uint64_t*>(v.flat) + flat_base(v.flat_slope, s0, b);
+  uint64_t* flat = v.flat + flat_base(v.slope, s0, b);
   const uint32_t u0 = fixed + static_cast<uint32_t>(w0);  // first bit of the unary part
   // cursor: `rank` ones lie in [u0, word w), `word` holds the ones of word w
   // from u0 on
@@ -403,6 +416,16 @@ uint32_t flat_log_group(uint64_t codes, uint64_t nb, uint64_t per) {
 // threads the device holds).
 uint64_t codes_per_part(uint64_t codes) { return std::max<uint64_t>(2, codes >> 19); }
 
+// v (with so set) for a decode of the codes into `flat`, `per` codes or more to a part.
+DecodeView decode_view(const Handle& h, const View& v, uint64_t* flat, uint64_t per) {
+  DecodeView d;
+  static_cast<View&>(d) = v;
+  d.flat = flat;
+  d.slope = flat_slope(header_leaf(h.header));
+  d.log_group = v.nb ? flat_log_group(h.ncodes, v.nb, per) : 0;
+  return d;
+}
+
 // Most places of the flat keys, 128 MiB: beyond, they are read from HBM, while the code bits of the
 // same structures stay in L2.  l = 8, b = 100, three queries per code, lists alone and codes:
 // 4 * 10^7 keys (70 MB of flat keys) 0.52 and 0.38 ms, 10^8 (174 MB) 1.26 and 1.35,
@@ -425,30 +448,6 @@ bool flat_pays(uint64_t q, uint64_t codes, uint64_t nb, uint64_t places) {
 // 55.6 us, 3.2 * 10^6 150 and 87.
 bool decode_pays(uint64_t q, uint64_t nb) { return q >= nb / 2 + (1u << 18); }
 
-template <bool RANGE>
-__global__ void __launch_bounds__(256) k_flat_decode(const __grid_constant__ View v, uint32_t log_group) {
-  cudaTriggerProgrammaticLaunchCompletion();
-  const uint64_t i = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x;
-  if (i >> log_group < v.nb) flat_bucket<RANGE>(v, i >> log_group, i & ((1u << log_group) - 1), log_group);
-}
-
-// Buckets of every structure: part p of the global index space belongs to the
-// structure i with base[i] <= p < base[i + 1].
-__global__ void __launch_bounds__(256) k_flat_decode_views(const View* __restrict__ views,
-                                                           const uint64_t* __restrict__ base, uint32_t count,
-                                                           uint64_t total) {
-  const uint64_t p = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x;
-  if (p >= total) return;
-  uint32_t lo = 0, hi = count;  // last i with base[i] <= p
-  while (hi - lo > 1) {
-    const uint32_t mid = (lo + hi) / 2;
-    if (__ldg(base + mid) <= p) lo = mid; else hi = mid;
-  }
-  const View& v = views[lo];
-  const uint64_t i = p - __ldg(base + lo);
-  flat_bucket<true>(v, i >> v.log_group, i & ((1u << v.log_group) - 1), v.log_group);
-}
-
 // What a flat lookup reads of a structure (16-byte loads where it is read per
 // query).
 struct alignas(16) FlatView {
@@ -464,21 +463,43 @@ struct alignas(16) FlatView {
   uint32_t extra, slope;
 };
 
-FlatView flat_view(const View& v) {
-  const Strategy st = make_strategy(v.leaf);
+FlatView flat_view(const Handle& h, const DecodeView& v) {
+  const uint32_t leaf = header_leaf(h.header);
+  const Strategy st = make_strategy(leaf);
   auto magic = [](uint64_t u) { return static_cast<uint32_t>(((1ull << 32) + u - 1) / u); };
   const uint32_t lower_codes = static_cast<uint32_t>(1 + st.lower / st.leaf);
-  return FlatView{reinterpret_cast<const ulonglong2*>(v.so), v.flat, v.nb, v.table, v.leaf,
+  return FlatView{reinterpret_cast<const ulonglong2*>(v.so), v.flat, v.nb, v.table, leaf,
                   static_cast<uint32_t>(st.lower), static_cast<uint32_t>(st.upper),
-                  v.leaf >= 2 ? magic(st.leaf) : 0, magic(st.lower), magic(st.upper), lower_codes,
+                  leaf >= 2 ? magic(st.leaf) : 0, magic(st.lower), magic(st.upper), lower_codes,
                   static_cast<uint32_t>(1 + st.upper / st.lower * lower_codes),
-                  reinterpret_cast<const uint4*>(v.rec), v.extra, v.flat_slope};
+                  reinterpret_cast<const uint4*>(v.rec), v.extra, v.slope};
+}
+
+template <bool RANGE>
+__global__ void __launch_bounds__(256) k_flat_decode(const __grid_constant__ DecodeView v) {
+  cudaTriggerProgrammaticLaunchCompletion();
+  flat_part<RANGE>(v, blockIdx.x * uint64_t(blockDim.x) + threadIdx.x);
+}
+
+// Buckets of every structure: part p of the global index space belongs to the
+// structure i with base[i] <= p < base[i + 1].
+__global__ void __launch_bounds__(256) k_flat_decode_views(const DecodeView* __restrict__ views,
+                                                           const uint64_t* __restrict__ base, uint32_t count,
+                                                           uint64_t total) {
+  const uint64_t p = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x;
+  if (p >= total) return;
+  uint32_t lo = 0, hi = count;  // last i with base[i] <= p
+  while (hi - lo > 1) {
+    const uint32_t mid = (lo + hi) / 2;
+    if (__ldg(base + mid) <= p) lo = mid; else hi = mid;
+  }
+  flat_part<true>(views[lo], p - __ldg(base + lo));
 }
 
 // Whether the steps of a descent can be computed (lookup_flat): the
 // reciprocals are exact for values below 2^16, and leaves of one key have no
 // code.
-bool steps_computed(const View& v) { return v.mmax < 65536 && v.leaf >= 2; }
+bool steps_computed(const Handle& h) { return h.header[H_MMAX] < 65536 && header_leaf(h.header) >= 2; }
 
 // STEPS: the part, its size and the codes to step over are computed from the
 // strategy's sizes instead of loaded by node size.  About 12 instructions
@@ -642,7 +663,11 @@ __global__ void k_ef_decode_views(const View* __restrict__ views, const uint64_t
 // 32 registers like k_lookup_bytes (measured: 10.0 -> 8.6 ms per 10^8
 // batched lookups over 4096 structures).  A query whose structure id is not
 // below `count` gets the value 2^64 - 1 (no structure is read for it).
-template <bool ANY_RANGE>
+// DECODED: the lists of every structure are decoded.  (Both lookups in one kernel
+// spilled 64 and reloaded 104 bytes, the lookup without decoded lists alone 40 and
+// 64: with the smaller views, 10^4 queries over 40 structures of 1000 buckets 25.9 ->
+// 24.9 us.)
+template <bool ANY_RANGE, bool DECODED>
 __global__ void __launch_bounds__(256, 8) k_lookup_many(const View* __restrict__ views, uint32_t count,
                               const uint32_t* __restrict__ ids, const uint64_t* __restrict__ keys, uint64_t q,
                               uint64_t* __restrict__ out) {
@@ -655,11 +680,14 @@ __global__ void __launch_bounds__(256, 8) k_lookup_many(const View* __restrict__
     uint64_t hi, lo;
     signature_u64(__ldg(keys + i), hi, lo);
     const View& v = views[id];
-    out[i] = ANY_RANGE && v.extra ? (v.so ? lookup_decoded<true>(v, v.so, hi, lo) : lookup_one<true>(v, hi, lo))
-                                  : (v.so ? lookup_decoded<false>(v, v.so, hi, lo) : lookup_one<false>(v, hi, lo));
+    if constexpr (DECODED)
+      out[i] = ANY_RANGE && v.extra ? lookup_decoded<true>(v, v.so, hi, lo) : lookup_decoded<false>(v, v.so, hi, lo);
+    else
+      out[i] = ANY_RANGE && v.extra ? lookup_one<true>(v, hi, lo) : lookup_one<false>(v, hi, lo);
   }
 }
 
+// (The serving engine's: it decodes nothing.)
 __global__ void k_lookup_many_bytes(const View* __restrict__ views, uint32_t count, const uint32_t* __restrict__ ids,
                                     const uint8_t* __restrict__ bytes, const uint64_t* __restrict__ offsets,
                                     uint64_t q, uint64_t* __restrict__ out) {
@@ -675,8 +703,7 @@ __global__ void k_lookup_many_bytes(const View* __restrict__ views, uint32_t cou
     const bool ok = o0 <= o1 && o1 <= last;  // else read as the empty string
     signature_bytes(bytes + (ok ? o0 : 0), ok ? o1 - o0 : 0, hi, lo);
     const View& v = views[id];
-    out[i] = v.extra ? (v.so ? lookup_decoded<true>(v, v.so, hi, lo) : lookup_one<true>(v, hi, lo))
-                     : (v.so ? lookup_decoded<false>(v, v.so, hi, lo) : lookup_one<false>(v, hi, lo));
+    out[i] = v.extra ? lookup_one<true>(v, hi, lo) : lookup_one<false>(v, hi, lo);
   }
 }
 
@@ -719,15 +746,17 @@ int lookup_many(const View* d_views, uint32_t count, const uint32_t* d_ids, cons
                             : (any_range ? k_lookup_many_flat<true, false> : k_lookup_many_flat<false, false>);
     kern<<<grid, block, 0, s>>>(static_cast<const FlatView*>(flat->views), count, d_ids, d_keys, q, d_out);
   } else {
-    (any_range ? k_lookup_many<true> : k_lookup_many<false>)<<<grid, block, 0, s>>>(d_views, count, d_ids, d_keys, q,
-                                                                                    d_out);
+    auto kern = flat && flat->decoded ? (any_range ? k_lookup_many<true, true> : k_lookup_many<false, true>)
+                                      : (any_range ? k_lookup_many<true, false> : k_lookup_many<false, false>);
+    kern<<<grid, block, 0, s>>>(d_views, count, d_ids, d_keys, q, d_out);
   }
   count_launch();
   RS_CUDA(cudaGetLastError());
   return RECSPLIT_OK;
 }
 
-int decode_views(View* views, uint32_t count, uint64_t q, cudaStream_t s, uint64_t** scratch, FlatBatch* batch) {
+int decode_views(const Handle* const* hs, View* views, uint32_t count, uint64_t q, cudaStream_t s, uint64_t** scratch,
+                 FlatBatch* batch) {
   *scratch = nullptr;
   *batch = FlatBatch{};
   if (q < kDecodeQueries) return RECSPLIT_OK;
@@ -736,18 +765,20 @@ int decode_views(View* views, uint32_t count, uint64_t q, cudaStream_t s, uint64
   bool fits = true, steps = true;
   for (uint32_t i = 0; i < count; i++) {
     buckets += views[i].nb;
-    codes += views[i].codes;
-    places += flat_places(views[i]);
-    fits &= decode_fits(views[i].range, views[i].mmax);
-    steps &= steps_computed(views[i]);
+    codes += hs[i]->ncodes;
+    places += flat_places(*hs[i]);
+    fits &= decode_fits(hs[i]->range_size, views[i].mmax);
+    steps &= steps_computed(*hs[i]);
   }
   if (buckets == 0 || !decode_pays(q, buckets) || !fits) return RECSPLIT_OK;
   bool flat = flat_pays(q, codes, buckets, places);
   // one allocation: the views, the flat views, the first part of every view (one
   // copy), then the decoded buckets and, with the codes, their keys
-  constexpr uint64_t kViewWords = sizeof(View) / 8, kFlatWords = sizeof(FlatView) / 8;
-  static_assert(sizeof(View) % 8 == 0 && sizeof(FlatView) % 16 == 0, "views are copied as words");
-  auto flat_at = [&] { return (count * kViewWords + 1) & ~uint64_t(1); };  // 16-byte aligned
+  constexpr uint64_t kViewWords = sizeof(View) / 8, kDecodeWords = sizeof(DecodeView) / 8,
+                     kFlatWords = sizeof(FlatView) / 8;
+  static_assert(sizeof(View) % 8 == 0 && sizeof(DecodeView) % 8 == 0 && sizeof(FlatView) % 16 == 0,
+                "views are copied as words");
+  auto flat_at = [&] { return (count * (flat ? kDecodeWords : kViewWords) + 1) & ~uint64_t(1); };  // 16-byte aligned
   auto base_at = [&] { return flat_at() + (flat ? count * kFlatWords : 0); };
   auto so_at = [&] { return (base_at() + count + 2) & ~uint64_t(1); };
   void* d_scratch = nullptr;
@@ -763,20 +794,18 @@ int decode_views(View* views, uint32_t count, uint64_t q, cudaStream_t s, uint64
   for (uint32_t i = 0; i < count; i++) {
     View& v = views[i];
     base[i] = total;
-    if (v.nb) {
-      v.so = next_so;
-      next_so += 2 * v.nb;
-      if (flat) {
-        v.flat = keys;
-        v.log_group = flat_log_group(v.codes, v.nb, codes_per_part(codes));
-        keys += flat_places(v);
-      }
-      total += v.nb << v.log_group;
-    }
-    memcpy(host.data() + i * kViewWords, &v, sizeof(View));
+    if (v.nb) v.so = next_so;
+    next_so += 2 * v.nb;
     if (flat) {
-      const FlatView f = flat_view(v);
+      const DecodeView dv = decode_view(*hs[i], v, keys, codes_per_part(codes));
+      const FlatView f = flat_view(*hs[i], dv);
+      memcpy(host.data() + i * kDecodeWords, &dv, sizeof(DecodeView));
       memcpy(host.data() + flat_at() + i * kFlatWords, &f, sizeof(FlatView));
+      if (v.nb) keys += flat_places(*hs[i]);
+      total += v.nb << dv.log_group;
+    } else {
+      memcpy(host.data() + i * kViewWords, &v, sizeof(View));
+      total += v.nb;
     }
   }
   base[count] = total;
@@ -786,7 +815,8 @@ int decode_views(View* views, uint32_t count, uint64_t q, cudaStream_t s, uint64
   if (e == cudaSuccess) {
     const uint64_t blocks = (total + 255) / 256;
     if (flat)
-      k_flat_decode_views<<<static_cast<unsigned>(blocks), 256, 0, s>>>(d_views, d + base_at(), count, total);
+      k_flat_decode_views<<<static_cast<unsigned>(blocks), 256, 0, s>>>(
+          reinterpret_cast<const DecodeView*>(d), d + base_at(), count, total);
     else
       k_ef_decode_views<<<static_cast<unsigned>(blocks < 65535 ? blocks : 65535), 256, 0, s>>>(d_views, d + base_at(),
                                                                                               count, total);
@@ -794,13 +824,15 @@ int decode_views(View* views, uint32_t count, uint64_t q, cudaStream_t s, uint64
     e = cudaGetLastError();
   }
   if (e != cudaSuccess) {
-    for (uint32_t i = 0; i < count; i++) views[i].so = views[i].flat = nullptr;
+    for (uint32_t i = 0; i < count; i++) views[i].so = nullptr;
     cudaFreeAsync(d_scratch, s);
     return cuda_fail(e, "decode of the structures");
   }
   *scratch = d;
-  batch->decoded = d_views;
-  if (flat) batch->views = d + flat_at();
+  if (flat)
+    batch->views = d + flat_at();
+  else
+    batch->decoded = d_views;
   batch->steps = steps;
   return RECSPLIT_OK;
 }
@@ -808,10 +840,6 @@ int decode_views(View* views, uint32_t count, uint64_t q, cudaStream_t s, uint64
 View make_view(const Handle& h) {
   View v;
   v.so = nullptr;
-  v.flat = nullptr;
-  v.flat_slope = 0;
-  v.range = v.codes = 0;
-  v.log_group = 0;
   v.mmax = h.header[H_MMAX];
   v.extra = header_extra(h.header);
   const uint64_t* H = h.header;
@@ -830,7 +858,6 @@ View make_view(const Handle& h) {
   v.delta_b = static_cast<int64_t>(H[H_DELTA_B]);
   v.low_a = static_cast<uint32_t>(H[H_LOW_A]);
   v.low_b = static_cast<uint32_t>(H[H_LOW_B]);
-  v.leaf = header_leaf(H);
   return v;
 }
 
@@ -857,18 +884,11 @@ cudaError_t launch_lookup(bool early, void (*kernel)(P...), unsigned grid, int b
   return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
 }
 
-void view_for_decode(const Handle& h, View* v) {
-  v->flat_slope = flat_slope(v->leaf);
-  v->range = h.range_size;
-  v->codes = h.ncodes;
-}
-
 int lookup_structure(const Handle& h, const KeyInput& q, uint64_t* d_out, cudaStream_t s, bool allow_scratch) {
   if (q.n == 0) return RECSPLIT_OK;
   LookupRange range;
   View v = make_view(h);
-  allow_scratch = allow_scratch && v.nb && q.n >= kDecodeQueries;
-  if (allow_scratch) view_for_decode(h, &v);
+  allow_scratch = allow_scratch && v.nb && q.n >= kDecodeQueries && decode_fits(h.range_size, v.mmax);
   int dev = 0, sms = 0;
   RS_CUDA(cudaGetDevice(&dev));
   RS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -878,21 +898,20 @@ int lookup_structure(const Handle& h, const KeyInput& q, uint64_t* d_out, cudaSt
   // With enough queries every code is decoded once (flat_pays), or else the prefix
   // sums and offsets of all buckets (decode_pays) instead of selected per query (the
   // stored structure does not change).  The scratch is allocated only then.
-  const uint64_t places = flat_places(v);
+  const uint64_t places = allow_scratch ? flat_places(h) : 0;
   uint64_t* so = nullptr;
-  if (allow_scratch && flat_pays(q.n, v.codes, v.nb, places) && decode_fits(v.range, v.mmax) &&
+  if (allow_scratch && flat_pays(q.n, h.ncodes, v.nb, places) &&
       pool_alloc(reinterpret_cast<void**>(&so), 16 * v.nb + 8 * places, s) == RECSPLIT_OK) {
-    View f = v;
-    f.so = so;
-    f.flat = so + 2 * v.nb;
-    const FlatView fv = flat_view(f);
-    const uint32_t lg = flat_log_group(v.codes, v.nb, codes_per_part(v.codes));
-    const unsigned dg = static_cast<unsigned>(((v.nb << lg) + block - 1) / block);
-    (v.extra ? k_flat_decode<true> : k_flat_decode<false>)<<<dg, block, 0, s>>>(f, lg);
+    View d = v;
+    d.so = so;
+    const DecodeView dv = decode_view(h, d, so + 2 * v.nb, codes_per_part(h.ncodes));
+    const FlatView fv = flat_view(h, dv);
+    const unsigned dg = static_cast<unsigned>(((v.nb << dv.log_group) + block - 1) / block);
+    (v.extra ? k_flat_decode<true> : k_flat_decode<false>)<<<dg, block, 0, s>>>(dv);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess)
       e = q.u64 ? launch_lookup(true,
-                                steps_computed(v)
+                                steps_computed(h)
                                     ? (v.extra ? k_lookup_u64_flat<true, true> : k_lookup_u64_flat<false, true>)
                                     : (v.extra ? k_lookup_u64_flat<true, false> : k_lookup_u64_flat<false, false>),
                                 grid, block, s, fv, q.u64, q.n, d_out)
@@ -903,7 +922,7 @@ int lookup_structure(const Handle& h, const KeyInput& q, uint64_t* d_out, cudaSt
     if (e != cudaSuccess) return cuda_fail(e, "lookup launch");
     return RECSPLIT_OK;
   }
-  if (allow_scratch && decode_pays(q.n, v.nb) && decode_fits(v.range, v.mmax) &&
+  if (allow_scratch && decode_pays(q.n, v.nb) &&
       pool_alloc(reinterpret_cast<void**>(&so), 16 * v.nb, s) == RECSPLIT_OK) {
     View d = v;
     d.so = so;
