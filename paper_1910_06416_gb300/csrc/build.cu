@@ -956,7 +956,17 @@ static int build_pass(const SetInput* in, uint32_t count, const BuildOptions& op
       level_heavy.push_back(heavy);
     }
   }
-  const uint64_t heavy_cap = any_heavy ? split_cap : 0;
+  // heavy nodes of a level hold disjoint keys, each at least as many as the
+  // smallest heavy node of its class (with a queue as long as the light nodes', and
+  // its search state, a build of 2 * 10^7 keys at l = 12, b = 100 took 48.7 bytes per
+  // key, 45.3 so)
+  uint64_t heavy_cap = 0;
+  for (uint32_t c = 0; c < nclass; c++)
+    for (uint64_t m = class_leaf[c] + 1; m <= h_cls_max[c]; m++)
+      if (is_heavy(T[c].expected_trials[m], m, heavy_min)) {
+        heavy_cap += keys_c[c] / m;
+        break;
+      }
   qtotal += 2 * (split_cap + heavy_cap);
 
   // grouping; queues: two split levels (ping-pong) shared by all classes, full
