@@ -1164,7 +1164,7 @@ static int build_pass(const SetInput* in, uint32_t count, const BuildOptions& op
   }
   if (herr == RECSPLIT_E_DUPLICATE) return fail(herr, "two keys share their lower signature half (duplicate keys)");
   if (herr == RECSPLIT_E_SEARCH_LIMIT) return fail(herr, "seed search exceeded its limit");
-  if (herr) return fail(herr, "a queue capacity or bucket code length check failed");
+  if (herr) return fail(herr, "a queue capacity, bucket code length or prefix sum check failed");
 
   // headers and layouts; one arena for all structures (256-byte aligned each)
   std::vector<uint64_t> headers(uint64_t(count) * kHeaderWords, 0), blob_off(count + 1, 0);
