@@ -226,7 +226,8 @@ struct BuildOptions {
   bool use_graph = false;  // capture the search and length phases in a CUDA graph
 };
 
-// Builds one structure per set in one pass over all sets (out[i] for set i).
+// Builds one structure per set (out[i] for set i) in one pass over all sets, or one
+// per kMaxClasses parameter classes.
 // KeyInput pointers must be device memory.
 int build_sets(const SetInput* sets, uint32_t count, const BuildOptions& opt, cudaStream_t s, Handle** out);
 // allow_scratch = false: allocate nothing (no per-batch decode of the lists)
@@ -244,14 +245,13 @@ struct FlatBatch {
 // non-minimal variant); flat: from decode_views
 int lookup_many(const View* d_views, uint32_t count, const uint32_t* d_ids, const uint64_t* d_keys, uint64_t q,
                 uint64_t* d_out, cudaStream_t s, bool any_range = true, const FlatBatch* flat = nullptr);
-// Batched lookups over several structures with more queries than the structures
-// have codes: the function key of every code and s_i and the size of every
-// bucket of every structure are decoded into one pooled array *scratch (the
-// caller frees it, stream-ordered, after the lookups), and *flat describes
-// them.  With fewer queries, but enough for the buckets, s_i, the size and o_i of
-// every bucket alone (views[i].so).  Otherwise, or if the memory is
-// not available, *scratch stays null and the views are unchanged (the lookups
-// then select in the lists per query).
+// Batched lookups over several structures: from buckets / 2 + 2^18 queries on s_i,
+// the size and o_i of every bucket of every structure are decoded (views[i].so), or,
+// with at least 1.5 queries per code and two codes per bucket, the function key of every
+// code and s_i and the size of every bucket, into one pooled array *scratch (the
+// caller frees it, stream-ordered, after the lookups), and *flat describes them.
+// Otherwise, or if the memory is not available, *scratch stays null and the
+// views are unchanged (the lookups then select in the lists per query).
 int decode_views(const Handle* const* hs, View* views, uint32_t count, uint64_t q, cudaStream_t s, uint64_t** scratch,
                  FlatBatch* flat);
 int lookup_many_bytes(const View* d_views, uint32_t count, const uint32_t* d_ids, const uint8_t* d_bytes,

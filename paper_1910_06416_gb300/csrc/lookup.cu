@@ -97,8 +97,8 @@ __device__ __forceinline__ ulonglong2 load_decoded(const ulonglong2* p) {
   return x;
 }
 
-// The same lookup with s_i, the size and o_i of every bucket decoded beforehand:
-// for batches with at least as many queries as buckets.
+// The same lookup with s_i, the size and o_i of every bucket decoded beforehand
+// (decode_pays).
 template <bool RANGE>
 __device__ __forceinline__ uint64_t lookup_decoded(const View& v, const uint64_t* so, uint64_t hi,
                                                    uint64_t lo) {
@@ -273,7 +273,7 @@ __device__ __forceinline__ uint64_t descend(const View& v, uint64_t s0, uint32_t
 }
 
 // ---------------------------------------------------------------- flat codes
-// A batch with more queries than the structure has codes (flat_pays) decodes every
+// A batch of at least 1.5 queries per code of the structure (flat_pays) decodes every
 // code once: the function key K ^ (K >> 30) of code c (preorder) of bucket b is stored
 // at place flat_base(s_b, b) + c, and so holds s_b, the bucket's size and the key of its
 // first code in 16 bytes: {s_b | m << 40, key}.  A level of the
@@ -770,6 +770,10 @@ int decode_views(const Handle* const* hs, View* views, uint32_t count, uint64_t 
     fits &= decode_fits(hs[i]->range_size, views[i].mmax);
     steps &= steps_computed(*hs[i]);
   }
+  // Codes as well as lists are decoded from the lists' line on, later than for one
+  // structure: 40 structures of 100 buckets, l = 8, b = 100: 2.5 * 10^5 queries, below the
+  // line, 32.4 us, 3 * 10^5, with decoded codes, 32.7; of 20 buckets, l = 12, b = 2000:
+  // 43.7 and 38.8.
   if (buckets == 0 || !decode_pays(q, buckets) || !fits) return RECSPLIT_OK;
   bool flat = flat_pays(q, codes, buckets, places);
   // one allocation: the views, the flat views, the first part of every view (one
