@@ -442,10 +442,15 @@ bool flat_pays(uint64_t q, uint64_t codes, uint64_t nb, uint64_t places) {
   return places <= kFlatPlaces && 2 * q >= 3 * codes && q >= kDecodeQueries && codes >= 2 * nb;
 }
 
-// Whether a batch of q queries decodes the buckets of the lists first: l = 8, b = 100,
-// 10^5 buckets: without and with it 2 * 10^5 queries 16.5 and 16.2 us, 4 * 10^5 25.2
-// and 20.7, 10^6 51.5 and 34.7; l = 5, b = 5, 2 * 10^6 buckets: 10^6 queries 53.5 and
-// 55.6 us, 3.2 * 10^6 150 and 87.
+// Whether a batch of q queries decodes the buckets of the lists first.  From host
+// call to end, without the decode and with it:
+//   one structure, l = 8, b = 100, 1000 buckets: 2 * 10^5 queries 23.4 and 24.9 us,
+//     2.6 * 10^5 26.7 and 26.1, 4 * 10^5 31.8 and 28.6; 10^5 buckets 24.4 and 25.5, 29.4 and
+//     26.8, 33.4 and 30.4; 1000 with a leaf range extra 24.8 and 26.1, 28.3 and 27.3, 34.0
+//     and 30.2; l = 5, b = 5, 10^6 buckets: 4 * 10^5 33.3 and 40.5, 7 * 10^5 46.1 and 44.9;
+//   40 structures, l = 8, b = 100, 100 buckets each: 2 * 10^5 37.2 and 39.8, 4 * 10^5 47.4
+//     and 46.9, 7 * 10^5 60.4 and 53.7; 2500 each: 2.6 * 10^5 42.6 and 43.0, 4 * 10^5 53.6 and
+//     48.9.
 bool decode_pays(uint64_t q, uint64_t nb) { return q >= nb / 2 + (1u << 18); }
 
 // What a flat lookup reads of a structure (16-byte loads where it is read per

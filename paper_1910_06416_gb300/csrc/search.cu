@@ -556,8 +556,9 @@ __device__ __forceinline__ void partition_node(const SearchArgs& a, const Node& 
 // spread 4 against 1).  spread is 4 where a search takes several rounds of 32
 // indices (128 trials) and 2 below, where four warps mostly test past the
 // winner (l = 8, 10^5 keys: split 97 us with 2, 117 us with 4), and 32 where it
-// takes long (2048 trials, leaves from l = 10: 3 * 10^5 keys at l = 11, b = 100 take
-// 1.64 ms with one warp per leaf and 1.34 ms with four, 3 * 10^6 keys 10.8 and 11.3).
+// takes long (2048 trials, leaves from l = 10; leaf phase, b = 100, spread 4, 16 and 32: l =
+// 11, 10^5 keys 633, 559 and 561 us, 3 * 10^5 1719, 1539 and 1376, from 10^6 on equal; l = 12,
+// 10^5 1184, 1114 and 1120; but l = 10, 10^5 260, 295 and 300, 3 * 10^5 655, 616 and 631).
 __device__ __forceinline__ uint32_t group_warps(uint32_t gwarps, uint32_t items, uint32_t spread) {
   while (gwarps < kWarps && uint64_t(items) * gwarps * 2 <= spread * gridDim.x * kWarps) gwarps *= 2;
   return gwarps;
