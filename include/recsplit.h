@@ -133,9 +133,11 @@ typedef struct recsplit_keyset {
  * captured into one CUDA graph per call and launched as one).  outs[i]
  * receives the structure of
  * sets[i], identical to what recsplit_build_u64 / _bytes would build from it.
- * All key arrays must be device memory; at most 2^32 - 1 keys in total and
- * at most 25 distinct leaf sizes.  The structures share one device arena,
- * released when the last of them is freed. */
+ * All key arrays must be device memory; at most 2^32 - 1 keys in total.
+ * A pass holds 25 distinct pairs of leaf size and leaf range extra; sets of
+ * more pairs take several passes, whose profile is the sum of theirs.  The
+ * structures of a pass share one device arena, released when the last of
+ * them is freed. */
 int recsplit_build_batch(const recsplit_keyset_t* sets, uint32_t count, void* stream, recsplit_t** outs);
 
 /* Batched lookup over several structures: out[i] = lookup of keys[i] in
